@@ -62,7 +62,6 @@ struct lbm_handle {
     double *fil_par = nullptr;
     uint64_t *ibmask = nullptr;
     double *rd_f19 = nullptr, *rd_mac = nullptr;  // read-out scratch, largest instance (allocated on first use)
-    int32_t *cell_box_dev = nullptr;               // box index of every stored cell (allocated on first use)
     // stream-ordered 0D parameter updates: pinned staging ring, one event per slot
     static constexpr int PAR_RING = 64;
     BcParam *par_ring = nullptr, *par_ring_dev = nullptr;  // host and device addresses of the mapped ring
@@ -932,19 +931,9 @@ lbm_status lbm_read_fields(lbm_handle *h, int inst, double *P, double *jx, doubl
 lbm_status lbm_read_fields_device(lbm_handle *h, int inst, float *P, float *jx, float *jy, float *jz) {
     if (bad_inst(h, inst) || !P || !jx || !jy || !jz) return fail(h, LBM_ERR_ARG, "bad instance or array");
     CK(h, cudaSetDevice(h->device));
-    const Layout &L = h->L;
-    if (!h->cell_box_dev) {
-        std::vector<int32_t> box(L.cell_box.begin(), L.cell_box.end());
-        CK(h, upload(h, &h->cell_box_dev, box));
-    }
-    if (!h->rd_mac) CK(h, dalloc(h, &h->rd_mac, 4 * (size_t)h->max_inst_cells));
-    const int64_t c0 = L.inst_cell_begin[inst], c1 = L.inst_cell_end[inst];
     const lbm_instance_desc &d = h->inst[inst];
-    const size_t nbox = (size_t)d.nx * d.ny * d.nz;
-    float *outs[4] = {P, jx, jy, jz};
-    for (float *o : outs) CK(h, cudaMemsetAsync(o, 0, nbox * sizeof(float), h->stream));
-    CK(h, launch_gather(h->prec, h->f[h->parity], h->kp, (int)c0, (int)c1, nullptr, h->rd_mac, h->stream));
-    CK(h, launch_scatter_box(h->rd_mac, (int)(c1 - c0), h->cell_box_dev + c0, P, jx, jy, jz, h->stream));
+    CK(h, launch_fields_box(h->prec, h->f[h->parity], h->kp, h->rowid + h->L.inst[inst].rowid_off, d.nx,
+                            (int64_t)d.nx * d.ny * d.nz, P, jx, jy, jz, h->stream));
     return LBM_OK;
 }
 

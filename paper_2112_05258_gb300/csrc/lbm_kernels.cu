@@ -9,6 +9,7 @@
 //   k_bc_apply        the ghost populations of Eq. Non-equilibrium3 (per
 //                     link, in the compute type)
 //   k_gather          read-out of f(t_n), P and j for the host
+//   k_fields_box      FP32 read-out of P and j into box-order device arrays
 //   k_wall_shear      wall shear stress at the fluid cells next to rigid walls
 //   k_init, k_init_eq inverse of the pull: lays out a given f(t_0), or the
 //                     equilibrium of given macroscopic fields
@@ -542,22 +543,107 @@ cudaError_t launch_copy_words(const void *src, void *dst, size_t bytes, cudaStre
     return cudaGetLastError();
 }
 
-// compact -> box scatter of the gathered P, j into FP32 device arrays
-__global__ void k_scatter_box(const double *__restrict__ mac4, int M, const int32_t *__restrict__ box, float *P,
-                              float *jx, float *jy, float *jz) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    const int b = box[m];
-    P[b] = (float)mac4[m];
-    jx[b] = (float)mac4[M + m];
-    jy[b] = (float)mac4[2 * (size_t)M + m];
-    jz[b] = (float)mac4[3 * (size_t)M + m];
+// Sums of population deviations for the FP32 read-out, about as exact as FP64
+// ones: FP32 storage adds in pairs of FP32 (two-sum, error about 2^-46 of the
+// terms), FP64 storage in FP64.
+struct PairSum {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float s = h + x, t = s - h;
+        l += (h - (s - t)) + (x - t);
+        h = s;
+    }
+    // an infinity or NaN in h makes l a NaN: then h alone is the sum
+    __device__ __forceinline__ float low() const { return isfinite(l) ? l : 0.f; }
+    __device__ __forceinline__ float value() const { return h + low(); }
+    __device__ __forceinline__ float pressure() const {  // (1 + h + l) / 3 to the last bit or so
+        PairSum t;
+        t.h = 1.f;
+        t.add(h);
+        const float q = t.h * (1.f / 3.f);
+        const float r = (fmaf(-3.f, q, t.h) + (t.low() + low())) * (1.f / 3.f);
+        return isfinite(r) ? q + r : q;
+    }
+};
+struct WideSum {
+    double h = 0.0;
+    __device__ __forceinline__ void add(double x) { h += x; }
+    __device__ __forceinline__ float value() const { return (float)h; }
+    __device__ __forceinline__ float pressure() const { return (float)((1.0 + h) / 3.0); }
+};
+template <class R> struct ReadSum { using T = PairSum; };
+template <> struct ReadSum<double> { using T = WideSum; };
+
+// FP32 read-out of one instance in box order: thread b takes the box cells
+// b, so the four arrays are written once, coalesced, with the zeros off the
+// fluid, and the pulls of a row's cells are coalesced too.  Bound by memory:
+// 80 B read per fluid cell (FP32 storage) and 16 B written per box cell.  The
+// sums must not lose precision against FP64, whose pipe is narrow on this
+// part (68 FP64 operations a cell took the whole time before); pairs of FP32
+// cost about 350 FP32 operations a cell and stay below the memory time.
+// Aorta (16.8M box cells, 4.0M fluid, FP32): 1,315 us as FP64 gather, four
+// memsets and a scatter, 200 us in this kernel; the 96 uneven tubes of a batch
+// (33M box cells): 576 launches and 9.3 ms before, 96 launches and 1.2 ms now.
+template <class S>
+__global__ void __launch_bounds__(256) k_fields_box(const S *__restrict__ fin, KParams p, const int32_t *__restrict__ rowid,
+                                                    int nx, unsigned nbox, float *__restrict__ P, float *__restrict__ jx,
+                                                    float *__restrict__ jy, float *__restrict__ jz) {
+    using R = typename Storage<S>::R;
+    const unsigned b = blockIdx.x * 256u + threadIdx.x;
+    if (b >= nbox) return;
+    const unsigned line = b / (unsigned)nx;
+    const int x = (int)(b - line * (unsigned)nx);
+    const int r = __ldg(&rowid[line]);
+    float o[4] = {0.f, 0.f, 0.f, 0.f};
+    if (r >= 0) {
+        const int4 *row = reinterpret_cast<const int4 *>(p.rows + r);
+        const int4 h0 = __ldg(row), h1 = __ldg(row + 1), h2 = __ldg(row + 2), h3 = __ldg(row + 3);
+        const int k = x - h0.y, c = h0.x + k;
+        const uint32_t fl = k >= 0 && k < h0.z ? __ldg(&p.flags[c]) : 0u;
+        if (fl & FL_ACTIVE) {
+            const int N = (int)p.n;
+            const int ln[9] = {h1.z + x, h1.w + x, h2.x + x, h2.y + x, c, h2.w + x, h3.x + x, h3.y + x, h3.z + x};
+            R f[NQ];
+            f[0] = Storage<S>::ld(fin + c);
+#pragma unroll
+            for (int i = 1; i < NQ; i++) {
+                const int src = ln[nbk(i)] - cx(i), own = c + ((i & 1) ? N : -N);
+                f[i] = Storage<S>::ld(fin + (size_t)i * N + (((fl >> i) & 1u) ? own : src));
+            }
+            typename ReadSum<R>::T s, m[3];
+#pragma unroll
+            for (int i = 0; i < NQ; i++) {
+                s.add(f[i]);
+                if (cx(i)) m[0].add(cx(i) > 0 ? f[i] : -f[i]);
+                if (cy(i)) m[1].add(cy(i) > 0 ? f[i] : -f[i]);
+                if (cz(i)) m[2].add(cz(i) > 0 ? f[i] : -f[i]);
+            }
+            o[0] = s.pressure();
+#pragma unroll
+            for (int a = 0; a < 3; a++) o[1 + a] = m[a].value();
+            if (!isfinite(s.h)) {  // the plain sum of e_i f_i over all directions (0 times infinity is a NaN)
+#pragma unroll
+                for (int a = 0; a < 3; a++) {
+                    float t = 0.f;
+#pragma unroll
+                    for (int i = 0; i < NQ; i++)
+                        t = __fadd_rn(t, __fmul_rn((float)(a == 0 ? cx(i) : a == 1 ? cy(i) : cz(i)), (float)f[i]));
+                    o[1 + a] = t;
+                }
+            }
+        }
+    }
+    P[b] = o[0];
+    jx[b] = o[1];
+    jy[b] = o[2];
+    jz[b] = o[3];
 }
 
-cudaError_t launch_scatter_box(const double *mac4, int M, const int32_t *box, float *P, float *jx, float *jy,
-                               float *jz, cudaStream_t s) {
-    if (M == 0) return cudaSuccess;
-    k_scatter_box<<<(M + 255) / 256, 256, 0, s>>>(mac4, M, box, P, jx, jy, jz);
+cudaError_t launch_fields_box(int prec, const void *fin, const KParams &p, const int32_t *rowid, int nx, int64_t nbox,
+                              float *P, float *jx, float *jy, float *jz, cudaStream_t s) {
+    const unsigned grid = (unsigned)((nbox + 255) / 256);
+    DISPATCH(prec, (k_fields_box<S><<<grid, 256, 0, s>>>(static_cast<const S *>(fin), p, rowid, nx, (unsigned)nbox, P, jx,
+                                                         jy, jz)));
     return cudaGetLastError();
 }
 

@@ -114,8 +114,9 @@ cudaError_t launch_copy_words(const void *src, void *dst, size_t bytes, cudaStre
 cudaError_t launch_io_params(const double *params, int np, BcParam *par, const long long *cursor, cudaStream_t s);
 cudaError_t launch_io_state(const BcState *st, const BcParam *par, const double *etab, int b0, int nb, int nbc_total,
                             const long long *step, double *out8, long long *cursor, cudaStream_t s);
-cudaError_t launch_scatter_box(const double *mac4, int M, const int32_t *box, float *P, float *jx, float *jy,
-                               float *jz, cudaStream_t s);
+// P and j of f(t_n) of one instance as FP32 in box order (rowid: its table of rows)
+cudaError_t launch_fields_box(int prec, const void *fin, const KParams &p, const int32_t *rowid, int nx, int64_t nbox,
+                              float *P, float *jx, float *jy, float *jz, cudaStream_t s);
 cudaError_t launch_cycle_change(const BcKParams &q, const int *bc_first, const int *n_bc, const long long *period,
                                 long long steps, double *delta, int n_inst, cudaStream_t s);
 cudaError_t launch_init(int prec, void *fout, const KParams &p, const double *f19, int c0, int c1,
