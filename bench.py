@@ -70,9 +70,12 @@ def parse_args():
 
 
 def launches(info, steps):
-    """Kernel launches of `steps` steps taken as lbm_step does them: whole step
+    """Kernel launches of `steps` steps taken as lbm_step does them: small
+    lattices in one launch per steps_per_launch steps, others in whole step
     graphs, then single-step graphs for the rest; a graph's first step (and a
     single step) issues launches_first_step, its later steps launches_per_step."""
+    if getattr(info, "steps_per_launch", 0):
+        return -(-steps // info.steps_per_launch)
     g = info.graph_steps
     full, rest = divmod(steps, g)
     return full * (info.launches_first_step + (g - 1) * info.launches_per_step) + rest * info.launches_first_step

@@ -157,6 +157,8 @@ typedef struct {
                               launches beside the previous step's 0D boundary kernels) */
     int launches_first_step; /* kernel launches of a graph's first step and of a single step */
     int graph_steps;         /* steps per step graph */
+    int steps_per_launch;    /* small lattices take the steps of an lbm_step call in one kernel launch per this many
+                                steps, without step graphs; 0: step graphs as above */
 } lbm_info_t;
 
 /* Sizes of the layout lbm_create would build (see lbm_check_config). */
@@ -195,7 +197,8 @@ lbm_status lbm_init_populations(lbm_handle *h, int inst, const double *f);
 
 /* Advances all instances by n steps (Algorithm 1).  Asynchronous: returns
  * after enqueueing, as CUDA graphs of graph_steps steps and, for the
- * remainder, single-step graphs (each captured once per step parity). */
+ * remainder, single-step graphs (each captured once per step parity); small
+ * lattices without wall nodes as one kernel launch (lbm_info_t). */
 lbm_status lbm_step(lbm_handle *h, int64_t n);
 
 /* n steps with per-step 0D input and output and no host round trip: before

@@ -109,6 +109,10 @@ struct lbm_handle {
         cudaGraphExec_t exec;
     };
     std::vector<IoGraph> io_graphs;
+    // small lattices: many steps in one launch, a cluster of blocks per instance (0: one-step kernels)
+    int small_cluster = 0;
+    size_t small_smem = 0;
+    SmallKParams small{};
     // kernel timing
     bool timing = false;
     std::vector<cudaEvent_t> ev;
@@ -443,6 +447,98 @@ void drop_graphs(lbm_handle *h) {
     }
 }
 
+// Decides whether the lattice takes its steps in the multi-step kernel, and
+// with how many blocks per instance.
+cudaError_t set_up_small(lbm_handle *h) {
+    const Layout &L = h->L;
+    if (!L.ib_dA.empty() || L.n_fluid == 0) return cudaSuccess;
+    std::vector<int32_t> bulk, off;
+    int64_t worst_bulk[17] = {0};
+    size_t smem_b = 0;
+    int most_bc = 0, worst_xf = 0;
+    std::vector<uint8_t> seen((size_t)L.n_stored, 0);
+    for (size_t q = 0; q < L.inst.size(); q++) {
+        const InstParam &ip = L.inst[q];
+        most_bc = std::max(most_bc, ip.n_bc);
+        for (int k = 0; k < ip.n_bc; k++) {
+            const BcParam &b = L.bc[ip.bc_first + k];
+            if (b.n_red > SMALL_MAX_RED || b.n_nodes > 32767) return cudaSuccess;
+            worst_xf = std::max(worst_xf, b.n_xf);
+            smem_b = std::max(smem_b, small_smem_boundary(b.n_xf, b.n_links, b.n_nodes, h->prec == LBM_F64));
+            for (int a = 0; a < b.n_xf; a++) {
+                uint8_t &c = seen[(size_t)L.xf[b.xf_off + a]];
+                if (c) return cudaSuccess;  // a cell in two first layers
+                c = 1;
+            }
+        }
+        off.push_back((int32_t)bulk.size());
+        for (int64_t c = L.inst_cell_begin[q]; c < L.inst_cell_end[q]; c++)
+            if ((L.flags[(size_t)c] & FL_ACTIVE) && !seen[(size_t)c]) bulk.push_back((int32_t)c);
+        const int64_t n = (int64_t)bulk.size() - off.back();
+        for (int C = ip.n_bc + 1; C <= 16; C++)
+            worst_bulk[C] = std::max(worst_bulk[C], (n + C - ip.n_bc - 1) / (C - ip.n_bc));
+    }
+    off.push_back((int32_t)bulk.size());
+    // Times of a step in us, measured on GB300 over tubes of 2,400 to 110,000
+    // cells.  This kernel: as many rounds as the clusters need, each the longer
+    // of the boundary block (latency: 3.8 us and its first layer's share; FP64
+    // runs on a pipe of 2 lanes an SM) and of a bulk block's cells.  One-step
+    // kernels: launches and latencies of 12 us (FP64: 20), then bandwidth.
+    const bool f64 = h->prec == LBM_F64;
+    const double cells = (double)L.n_fluid;
+    const double one_step = std::max(f64 ? 20.0 : 12.0, (f64 ? 16.0 : 9.0) + cells * (f64 ? 240e-6 : 30e-6));
+    double best = 0.9 * one_step;
+    for (int C : {16, 8}) {
+        if (C <= most_bc) continue;
+        const size_t smem = std::max(smem_b, small_smem_bulk((int)worst_bulk[C]));
+        if (smem > SMALL_MAX_SMEM) continue;
+        const double owner = f64 ? 4.5 + 0.09 * worst_xf : 3.8 + 0.006 * worst_xf;
+        const double bulk = f64 ? 1.5 + 33e-3 * worst_bulk[C] : 0.7 + 3.2e-3 * worst_bulk[C];
+        if (std::max(owner, bulk) >= best) continue;
+        int clusters = 0;
+        if (prepare_small(h->prec, C, smem, &clusters) != cudaSuccess || clusters < 1) {
+            (void)cudaGetLastError();
+            continue;
+        }
+        const int rounds = ((int)L.inst.size() + clusters - 1) / clusters;
+        const double t = rounds * std::max(owner, bulk);
+        if (t >= best) continue;
+        best = t;
+        h->small_cluster = C;
+        h->small_smem = smem;
+    }
+    if (!h->small_cluster) return cudaSuccess;
+    int32_t *d_bulk = nullptr, *d_off = nullptr;
+    int *done = nullptr;
+    cudaError_t e = upload(h, &d_bulk, bulk);
+    if (e == cudaSuccess) e = upload(h, &d_off, off);
+    if (e == cudaSuccess) e = dalloc(h, &done, 1);
+    if (e == cudaSuccess) e = cudaMemset(done, 0, sizeof(int));
+    h->small.inst = h->inst_dev;
+    h->small.bulk = d_bulk;
+    h->small.bulk_off = d_off;
+    h->small.done = done;
+    h->small.par = h->bc_par;
+    return e;
+}
+
+// n steps in the multi-step kernel (launches of at most SMALL_MAX_STEPS
+// steps); io: per-step params and state rows of lbm_step_io, or null.
+lbm_status small_steps(lbm_handle *h, int64_t n, const SmallKParams *io = nullptr) {
+    SmallKParams sp = io ? *io : h->small;
+    while (n > 0) {
+        sp.n_steps = (int)std::min<int64_t>(n, SMALL_MAX_STEPS);
+        CK(h, launch_small(h->prec, h->f[h->parity], h->f[1 - h->parity], h->kp, h->bp, sp, (int)h->inst.size(),
+                           h->small_cluster, h->small_smem, h->stream));
+        if (sp.n_steps & 1) h->parity ^= 1;
+        h->steps += sp.n_steps;
+        n -= sp.n_steps;
+        if (sp.io_params) sp.io_params += (size_t)sp.n_steps * sp.io_np;
+        if (sp.io_states) sp.io_states += (size_t)sp.n_steps * 8 * sp.io_nb;
+    }
+    return LBM_OK;
+}
+
 bool bad_inst(lbm_handle *h, int inst) { return !h || inst < 0 || inst >= (int)h->inst.size(); }
 
 // validation of one set of boundary params (lbm_set_0d_params, lbm_step_io); null if valid
@@ -748,6 +844,7 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
         h->n_band_dep = (int)dep.size();
         h->overlap = true;
     }
+    if (!ck(set_up_small(h), "small-lattice tables")) return bail(LBM_ERR_CUDA, h->err);
     if (cudaDeviceSynchronize() != cudaSuccess) return bail(LBM_ERR_CUDA, "set-up failed");
     *out = h;
     return LBM_OK;
@@ -830,6 +927,7 @@ lbm_status lbm_step(lbm_handle *h, int64_t n) {
         }
         return LBM_OK;
     }
+    if (h->small_cluster) return small_steps(h, n);
     int64_t left = n;
     while (left >= h->graph_steps) {
         lbm_status s = ensure_graph(h);
@@ -871,6 +969,19 @@ lbm_status lbm_step_io(lbm_handle *h, int inst, int bc, int64_t n, const double 
         }
         pdev = static_cast<const double *>(a.devicePointer);
         sdev = static_cast<double *>(c.devicePointer);
+    }
+    if (h->small_cluster && !h->timing) {
+        SmallKParams sp = h->small;
+        sp.io_params = pdev;
+        sp.io_states = sdev;
+        sp.io_np = np;
+        sp.io_b = b;
+        sp.io_b0 = ip.bc_first;
+        sp.io_nb = ip.n_bc;
+        const lbm_status st = small_steps(h, n, &sp);
+        if (st != LBM_OK) return st;
+        for (int k = 0; k < np; k++) bp.par[k] = params[(n - 1) * np + k];  // the host copy: the last set
+        return LBM_OK;
     }
     if (!h->io_cursor) CK(h, dalloc(h, &h->io_cursor, 1));
     CK(h, cudaMemsetAsync(h->io_cursor, 0, sizeof(long long), h->stream));
@@ -1336,6 +1447,7 @@ lbm_status lbm_get_info(lbm_handle *h, lbm_info_t *info) {
     if (h->overlap)  // band velocities as the two lists (an empty list launches nothing)
         info->launches_per_step += (h->n_band_ind > 0) + (h->n_band_dep > 0) - 1;
     info->graph_steps = h->graph_steps;
+    info->steps_per_launch = h->small_cluster ? SMALL_MAX_STEPS : 0;
     return LBM_OK;
 }
 

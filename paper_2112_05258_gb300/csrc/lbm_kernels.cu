@@ -21,13 +21,9 @@
 // the 0D boundary nodes for t_{n+1} already in their slots, so one step is:
 // (immersed boundary) -> k_stream_collide -> k_bc_reduce -> k_bc_apply.
 #include "lbm_device.cuh"
-#include "lbm_zero_d.cuh"
+#include "lbm_boundary.cuh"
 
 namespace lbm {
-
-__constant__ signed char c_ex[NQ] = {0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 1, -1, 1, -1, 0, 0, 0, 0};
-__constant__ signed char c_ey[NQ] = {0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 0, 0, 0, 0, 1, -1, 1, -1};
-__constant__ signed char c_ez[NQ] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, -1, 1};
 
 // ---------------------------------------------------------------------------
 // 0D coupling.  The per-cell and per-link arithmetic runs in the compute type
@@ -47,39 +43,6 @@ __device__ __forceinline__ void forced_velocity(const KParams &p, int cf, R v[3]
         v[1] += R(0.5) * bb.y;
         v[2] += R(0.5) * bb.z;
     }
-}
-
-// The 0D step of boundary b from the sums over its first layer (taken by one
-// thread): the state of t_{n+1} and, if store, the state and the waveform row
-// written; returns what the ghost pass needs.
-static __device__ BcStepResult bc_step(const BcParam &P, int b, double Q, double Ps, long long n,
-                                       const BcKParams &q, bool store) {
-    const BcState old = q.state[(size_t)(n & 1) * q.n_bc_total + b];
-    int ptype, closed;
-    double Sm;
-    const double Psum = (double)P.n_xf / 3.0 + Ps;  // sum of P over the layer
-    const BcState st = zero_d_step(P, old, Q, Psum, (double)P.n_xf, n, q.etab, &ptype, &closed, &Sm);
-    if (store) {
-        q.state[(size_t)((n + 1) & 1) * q.n_bc_total + b] = st;
-        double *w = q.wave + ((size_t)(n % q.wave_cap) * q.n_bc_total + b) * 4;
-        w[0] = st.Qu;
-        w[1] = st.Pbar - 1.0 / 3.0;
-        w[2] = (P.kind == BC_RCR) ? st.Pw : (P.kind == BC_LV ? st.Pv : st.Pstar_gauge);
-        w[3] = st.valve_open;
-    }
-    BcStepResult r;
-    r.Pg = st.Pstar_gauge;
-    r.S = Sm;
-    r.cosp = r.sinp = 0.0;
-    if (P.kind == BC_VELOCITY) {  // the inlet's phase, once for every link of the boundary
-        const double wv = P.par[0], tn1 = (double)(n + 1);
-        r.cosp = cos(wv * tn1);
-        r.sinp = sin(wv * tn1);
-    }
-    r.ptype = ptype;
-    r.closed = closed;
-    r.pad0 = r.pad1 = 0;
-    return r;
 }
 
 // The boundary's partial sums added by one warp in a fixed order (lane k
@@ -207,43 +170,8 @@ __global__ void __launch_bounds__(BC_CHUNK) k_bc_apply(S *__restrict__ f, KParam
         if (!have) return;
         r = s_r;
     }
-    R dP, vs[3];  // P* - P(x_f) and v*
-    if (r.ptype) {  // pressure-type: (P_0D(t_{n+1}), v(x_f, t_n))
-        dP = (R)r.Pg - sdf / R(3);
-        vs[0] = vf[0];
-        vs[1] = vf[1];
-        vs[2] = vf[2];
-    } else {        // velocity-type: (P(x_f, t_n), v_0D(t_{n+1}))
-        dP = R(0);
-        vs[0] = vs[1] = vs[2] = R(0);
-        if (P.kind == BC_VELOCITY) {
-            vs[P.axis] = (R)((double)P.sign * (pr[0] + pr[1] * r.cosp - pr[2] * r.sinp));
-        } else if (P.kind == BC_LV) {  // closed valve: v_0(T_d) S(t, T_d, N_S)
-            R u0[3];
-            if (r.closed) {  // v_0(T_d) = v(x_f, T_d); links sharing x_f store the same value
-                double *v0 = q.v0 + 3 * (size_t)(P.xf_off + q.lk_xfi[P.link_off + L]);
-#pragma unroll
-                for (int a = 0; a < 3; a++) {
-                    u0[a] = vf[a];
-                    v0[a] = (double)vf[a];
-                }
-            } else {
-#pragma unroll
-                for (int a = 0; a < 3; a++) u0[a] = (R)v0o[a];
-            }
-            const R Sm = (R)r.S;
-            vs[0] = u0[0] * Sm;
-            vs[1] = u0[1] * Sm;
-            vs[2] = u0[2] * Sm;
-        }
-    }
-    const R ex = c_ex[i], ey = c_ey[i], ez = c_ez[i];
-    const R w = i == 0 ? R(1.0 / 3.0) : (i < 7 ? R(1.0 / 18.0) : R(1.0 / 36.0));
-    const R eus = ex * vs[0] + ey * vs[1] + ez * vs[2];
-    const R euf = ex * vf[0] + ey * vf[1] + ez * vf[2];
-    const R us2 = vs[0] * vs[0] + vs[1] * vs[1] + vs[2] * vs[2];
-    const R uf2 = vf[0] * vf[0] + vf[1] * vf[1] + vf[2] * vf[2];
-    const R dfeq = w * R(3) * dP + w * (R(3) * (eus - euf) + R(4.5) * (eus * eus - euf * euf) - R(1.5) * (us2 - uf2));
+    const R dfeq = ghost_change<R>(P, r, i, vf, sdf, pr, v0o,
+                                   P.kind == BC_LV ? q.v0 + 3 * (size_t)(P.xf_off + q.lk_xfi[P.link_off + L]) : nullptr);
     Storage<S>::st(f + pidx(i, (uint32_t)cb, (uint32_t)N), post + dfeq);
 }
 
@@ -461,30 +389,13 @@ cudaError_t launch_gather(int prec, const void *fin, const KParams &p, int c0, i
     return cudaGetLastError();
 }
 
-// 0D state rows of boundaries [b0, b0 + nb) for lbm_read_0d_state_async:
-// {t, Q, Q_u, Pbar_gauge, state, C_v P_v (LV), valve_open, T_d}
-// the 8-value state row of boundary b after `steps` steps
-__device__ __forceinline__ void state_row(const BcState *__restrict__ st, const BcParam *__restrict__ par,
-                                          const double *__restrict__ etab, int b, int nbc_total, long long steps,
-                                          double *o) {
-    const BcState s = st[(size_t)(steps & 1) * nbc_total + b];
-    const BcParam &P = par[b];
-    o[0] = (double)steps;
-    o[1] = s.Q;
-    o[2] = s.Qu;
-    o[3] = s.Pbar - 1.0 / 3.0;
-    o[4] = P.kind == BC_RCR ? s.Pw : (P.kind == BC_LV ? s.Pv : s.Pstar_gauge);
-    o[5] = P.kind == BC_LV ? s.Pv / etab[2 * (P.etab_off + (int)(steps % P.period))] : 0.0;
-    o[6] = s.valve_open;
-    o[7] = s.Td;
-}
-
+// 0D state rows of boundaries [b0, b0 + nb) for lbm_read_0d_state_async
 __global__ void k_state_rows(const BcState *__restrict__ st, const BcParam *__restrict__ par,
                              const double *__restrict__ etab, int b0, int nb, int nbc_total, long long steps,
                              double *out8) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nb) return;
-    state_row(st, par, etab, b0 + k, nbc_total, steps, out8 + 8 * (size_t)k);
+    state_row(st[(size_t)(steps & 1) * nbc_total + b0 + k], par[b0 + k], etab, steps, out8 + 8 * (size_t)k);
 }
 
 // Per-step 0D input and output of lbm_step_io, in stream order around each
@@ -504,7 +415,10 @@ __global__ void k_io_state(const BcState *__restrict__ st, const BcParam *__rest
                            const long long *__restrict__ step, double *out8, long long *cursor) {
     const long long c = *cursor;
     const int k = threadIdx.x;
-    if (k < nb) state_row(st, par, etab, b0 + k, nbc_total, *step + 1, out8 + 8 * ((size_t)c * nb + k));
+    const long long steps = *step + 1;
+    if (k < nb)
+        state_row(st[(size_t)(steps & 1) * nbc_total + b0 + k], par[b0 + k], etab, steps,
+                  out8 + 8 * ((size_t)c * nb + k));
     __syncthreads();
     if (threadIdx.x == 0) *cursor = c + 1;
 }

@@ -1,0 +1,464 @@
+// Many steps of small lattices in one launch (no wall nodes).  A thread-block
+// cluster takes one instance and advances it n steps, its populations staying
+// in L2; the hardware cluster barrier separates the steps, so a step costs
+// neither launches nor the gaps between them.
+//
+// Work of a cluster of C blocks on an instance with B 0D boundaries:
+//   * block k < B owns boundary k: it collides the cells of its first fluid
+//     layer, sums flow and pressure over them (from registers), takes the 0D
+//     step and writes the ghosts of t_{n+1}.  Ghosts are pulled only by
+//     first-layer cells, i.e. by the same block in the next step, and the
+//     moments never leave it;
+//   * the blocks k >= B share the other cells.
+// Both only need the other blocks' populations of the step before, so there is
+// one cluster barrier per step, and the 0D work runs beside the bulk.
+// The pull sources of every cell (18 offsets into the population buffer, the
+// bounce-back and the row lookup resolved) are laid out once per launch in
+// shared memory: the loop starts its loads without any other lookup.
+//
+// Same device functions and the same summation order as the one-step kernels
+// (collide_store, the 256-wide trees and partial sums, bc_step, ghost_change):
+// the trajectory is the same bit for bit.
+//
+// Bound by latency.  FP64 additions take 64 cycles each on this part and a
+// division about 700, so the boundary block's chain decides: for the 24x24x64
+// tube (12,896 cells, FP32) about 1,200 cycles for the pulls, 1,400 collision
+// and the layer's terms, 1,800 trees, 2,400 means and 0D step, 2,000 ghosts,
+// 1,800 barrier; what does not depend on the step's flow (inlet velocities,
+// elastance terms, state and waveform stores) runs while the block waits at the
+// barrier.  A step: 12.4 -> 5.1 us for that tube, 12.1 -> 4.1
+// us for 2,400 cells (FP32), 20.7 -> 11.6 us in FP64 (whose collision is bound
+// by the FP64 pipe); three such tubes side by side 5.0 -> 1.7 us a step each.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+#include "lbm_boundary.cuh"
+#include "lbm_collide.cuh"
+
+namespace lbm {
+
+namespace {
+
+// Populations are read with plain loads: they are written during the launch,
+// so not through the read-only path.
+template <class S> struct PlainLoad;
+template <> struct PlainLoad<float> {
+    static __device__ __forceinline__ float ld(const float *p) { return *p; }
+};
+template <> struct PlainLoad<double> {
+    static __device__ __forceinline__ double ld(const double *p) { return *p; }
+};
+template <> struct PlainLoad<__half> {
+    static __device__ __forceinline__ float ld(const __half *p) { return __half2float(*p); }
+};
+template <> struct PlainLoad<__nv_bfloat16> {
+    static __device__ __forceinline__ float ld(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
+};
+
+template <class S> struct OneBase {
+    S *f;
+    int N;
+    __device__ __forceinline__ S *operator()(int i, int c) const { return f + (i * N + c); }  // 19 N < 2^31
+};
+
+// offset in the population buffer that direction i of cell c is pulled from
+__device__ __forceinline__ void pull_offsets(const KParams &p, int c, uint32_t fl, int *tab, int stride) {
+    const int N = (int)p.n;
+    const int r = find_row(p, c);
+    const RowInfo &ri = p.rows[r];
+    const int x = ri.x0 + (c - ri.off);
+#pragma unroll
+    for (int i = 1; i < NQ; i++) {
+        const int src = (nbk(i) == 4 ? c : ri.nb[nbk(i)] + x) - cx(i);
+        tab[(i - 1) * stride] = ((fl >> i) & 1u) ? opp(i) * N + c : i * N + src;
+    }
+}
+
+template <class R> struct FirstLayer {  // of one first-layer cell: forced velocity and sum s; v_0 of its closure (LV)
+    R v[3], sd;
+};
+
+// What a step of the 0D model needs besides the flow and pressure of t_n, in
+// terms of zero_d_step's expressions (forward Euler).
+struct Ahead {
+    double area, third;  // n_xf and n_xf / 3
+    int order;           // marching scheme
+    double p0_rc;        // RCR: P_w / (R_d C)
+    double inv_cv, dcv;  // LV: 1 / C_v and dC_v/dt, C_v = 1/E
+};
+
+constexpr int PULLS = NQ - 1;
+
+}  // namespace
+
+// Shared memory of a block.  Boundary block: per first-layer cell the pull
+// table, the cell, its moments and its closure velocity; per link its
+// destination offset and {direction, first-layer index, node}; per boundary
+// node the prescribed velocity.  Bulk block: pull table and cell per cell.
+size_t small_smem_boundary(int n_xf, int n_links, int n_nodes, bool f64) {
+    const size_t r = f64 ? 8 : 4;
+    return (size_t)n_xf * (PULLS * 4 + 4 + 8 * r) + (size_t)n_links * 8 + (size_t)n_nodes * r + 64;
+}
+size_t small_smem_bulk(int cells) { return (size_t)cells * (PULLS * 4 + 4) + 64; }
+
+template <class S, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParams p, BcKParams q, SmallKParams sp) {
+    using R = typename Storage<S>::R;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ double sQ[THREADS], sP[THREADS], s_part[2 * SMALL_MAX_RED], s_cos, s_sin;
+    __shared__ BcStepResult s_r;
+    __shared__ BcParam s_P;
+    __shared__ BcState s_st;
+    __shared__ Ahead s_a;
+    const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int inst = blockIdx.x / C;
+    const InstParam &ip = sp.inst[inst];
+    const int nb = ip.n_bc, N = (int)p.n;
+    const int tid = threadIdx.x;
+    const R omega = omega_of<R>(p, inst);
+    const bool owner = rank < nb;
+    const int b = ip.bc_first + rank;
+    const long long first = *p.step + 1;  // t_n of the first step of the launch
+
+    // cells of this block and their pull tables
+    int n_cells, cell0 = 0;
+    if (owner) {
+        for (int k = tid; k < (int)(sizeof(BcParam) / 4); k += THREADS)
+            reinterpret_cast<int *>(&s_P)[k] = reinterpret_cast<const int *>(q.par + b)[k];
+        __syncthreads();
+        n_cells = s_P.n_xf;
+    } else {
+        const int lo = sp.bulk_off[inst], n = sp.bulk_off[inst + 1] - lo, w = C - nb, k = rank - nb;
+        const int per = (n + w - 1) / w;
+        cell0 = lo + min(k * per, n);
+        n_cells = lo + min((k + 1) * per, n) - cell0;
+    }
+    int *tab = reinterpret_cast<int *>(smem);       // [18][n_cells]
+    int *cell = tab + PULLS * n_cells;              // [n_cells]
+    FirstLayer<R> *xf = reinterpret_cast<FirstLayer<R> *>((reinterpret_cast<uintptr_t>(cell + n_cells) + 15) & ~(uintptr_t)15);
+    FirstLayer<R> *v0s = xf + (owner ? n_cells : 0);  // closure velocities
+    int2 *link = reinterpret_cast<int2 *>(v0s + (owner ? n_cells : 0));
+    R *unode = reinterpret_cast<R *>(link + (owner ? s_P.n_links : 0));
+    for (int k = tid; k < n_cells; k += THREADS) {
+        const int c = owner ? q.xf[s_P.xf_off + k] : sp.bulk[cell0 + k];
+        cell[k] = c;
+        pull_offsets(p, c, p.flags[c], tab + k, n_cells);
+        if (owner) {
+            const double *v0 = q.v0 + 3 * (size_t)(s_P.xf_off + k);
+            v0s[k] = FirstLayer<R>{{(R)v0[0], (R)v0[1], (R)v0[2]}, R(0)};
+        }
+    }
+    if (owner) {
+        for (int L = tid; L < s_P.n_links; L += THREADS) {
+            const int g = s_P.link_off + L, i = q.lk_i[g];
+            link[L] = make_int2(i * N + q.lk_xb[g], i | (q.lk_xfi[g] << 5) | (q.lk_node[g] << 16));
+        }
+        if (tid == 0) {
+            s_st = q.state[(size_t)(first & 1) * q.n_bc_total + b];
+            s_a.area = (double)s_P.n_xf;
+            s_a.third = (double)s_P.n_xf / 3.0;
+            s_a.order = (int)s_P.par[4];
+        }
+    }
+    __syncthreads();
+    const bool io_in = owner && sp.io_params && b == sp.io_b;
+    const bool io_out = owner && sp.io_states && b >= sp.io_b0 && b < sp.io_b0 + sp.io_nb;
+
+    // The last AHEAD threads of a boundary block prepare step s while the others
+    // wait at the cluster barrier and collide: its params (io), and the parts of
+    // its 0D model that do not depend on its flow.
+    constexpr int AHEAD = 128;
+    const int ta = tid - (THREADS - AHEAD);
+    double given = 0.0;
+    if (io_in && ta >= 0 && ta < sp.io_np) given = __ldcv(sp.io_params + ta);
+    auto ahead = [&](int s) {
+        const BcParam &P = s_P;
+        const long long n = first + s;
+        auto meet = [] { asm volatile("bar.sync 1, %0;" ::"n"(AHEAD) : "memory"); };
+        if (io_in) {
+            if (ta < sp.io_np) {
+                s_P.par[ta] = given;
+                sp.par[b].par[ta] = given;
+                if (ta == 4) s_a.order = (int)given;
+                if (s + 1 < sp.n_steps) given = __ldcv(sp.io_params + (size_t)(s + 1) * sp.io_np + ta);
+            }
+            meet();
+        }
+        if (P.kind == BC_VELOCITY) {
+            const double wt = P.par[0] * (double)(n + 1);
+            if (ta == 0) s_cos = cos(wt);
+            if (ta == 32) s_sin = sin(wt);
+            meet();
+            const double cosp = s_cos, sinp = s_sin;
+            for (int a = ta; a < P.n_nodes; a += AHEAD) {  // the nodes' velocities at t_{n+1}
+                const double *pr = q.profile + 3 * (size_t)(P.node_off + a);
+                unode[a] = (R)((double)P.sign * (pr[0] + pr[1] * cosp - pr[2] * sinp));
+            }
+        } else if (ta == 0) {
+            if (P.kind == BC_RCR) s_a.p0_rc = s_st.Pw / (P.par[2] * P.par[1]);
+            if (P.kind == BC_LV) {
+                const double E = q.etab[2 * (P.etab_off + (int)(n % P.period))];
+                const double Ed = q.etab[2 * (P.etab_off + (int)(n % P.period)) + 1];
+                const double Cv = 1.0 / E;
+                s_a.dcv = -Ed / (E * E);
+                s_a.inv_cv = 1.0 / Cv;
+            }
+        }
+    };
+    if (owner && ta >= 0) ahead(0);
+    __syncthreads();
+
+    const S *fin = f0;
+    S *fout = f1;
+    for (int s = 0; s < sp.n_steps; s++) {
+        const OneBase<S> out{fout, N};
+        if (!owner) {
+            for (int k = tid; k < n_cells; k += THREADS) {
+                const int c = cell[k];
+                R f[NQ];
+                f[0] = PlainLoad<S>::ld(fin + c);
+#pragma unroll
+                for (int i = 1; i < NQ; i++) f[i] = PlainLoad<S>::ld(fin + tab[(i - 1) * n_cells + k]);
+                collide_store<S, R, false>(out, p, f, omega, 0u, c);
+            }
+        } else {
+            const BcParam &P = s_P;
+            const long long n = first + s;
+            for (int k0 = 0; k0 < P.n_red * BC_CHUNK; k0 += THREADS) {
+                const int k = k0 + tid;
+                double Q = 0.0, Ps = 0.0;
+                if (k < n_cells) {
+                    const int c = cell[k];
+                    R f[NQ];
+                    f[0] = PlainLoad<S>::ld(fin + c);
+#pragma unroll
+                    for (int i = 1; i < NQ; i++) f[i] = PlainLoad<S>::ld(fin + tab[(i - 1) * n_cells + k]);
+                    const Moments<R> m = collide_store<S, R, false>(out, p, f, omega, 0u, c);
+                    const R j = P.axis == 0 ? m.jx : P.axis == 1 ? m.jy : m.jz;
+                    Q = (double)((R)P.sign * j / (R(1) + m.sd));
+                    Ps = (double)(m.sd / R(3));
+                    xf[k] = FirstLayer<R>{{m.jx, m.jy, m.jz}, m.sd};
+                }
+                if (k < P.n_red * BC_CHUNK) {
+                    sQ[tid] = Q;
+                    sP[tid] = Ps;
+                }
+                __syncthreads();
+                // one warp per quantity and chunk of 256 cells: the tree of
+                // k_bc_reduce (128, 64, 32, then within the warp)
+                constexpr int CH = THREADS / BC_CHUNK;
+                const int w = tid >> 5, ch = k0 / BC_CHUNK + (w & (CH - 1));
+                if (w < 2 * CH && ch < P.n_red) {
+                    const double *v = (w < CH ? sQ : sP) + (w & (CH - 1)) * BC_CHUNK + (tid & 31);
+                    double a[4];
+#pragma unroll
+                    for (int h = 0; h < 4; h++) a[h] = v[32 * h] + v[32 * (h + 4)];
+                    a[0] = (a[0] + a[2]) + (a[1] + a[3]);
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) a[0] += __shfl_down_sync(0xffffffffu, a[0], o);
+                    if ((tid & 31) == 0) s_part[2 * ch + (w < CH ? 0 : 1)] = a[0];
+                }
+                __syncthreads();
+            }
+            // the thread's first link, its population in flight beside the 0D step
+            int2 lk0 = make_int2(0, 0);
+            R post0 = R(0);
+            if (tid < P.n_links) {
+                lk0 = link[tid];
+                post0 = PlainLoad<S>::ld(fout + ((lk0.y & 31) * N + cell[(lk0.y >> 5) & 0x7ff]));
+            }
+            if (tid < 32) {
+                // lane 0 takes the flow, lane 1 the pressure: partials in the order of bc_sum_partials
+                double a[SMALL_MAX_RED];
+                const double *sp_ = s_part + (tid & 1);
+                a[0] = 0.0 + sp_[0];
+                if (P.n_red > 1) {
+#pragma unroll
+                    for (int k = 1; k < SMALL_MAX_RED; k++) a[k] = k < P.n_red ? 0.0 + sp_[2 * k] : 0.0;
+                    if (P.n_red > 4)
+#pragma unroll
+                        for (int k = 0; k < 4; k++) a[k] += a[k + 4];
+                    if (P.n_red > 2) {
+                        a[0] += a[2];
+                        a[1] += a[3];
+                    }
+                    a[0] += a[1];
+                }
+                const int order = s_a.order;
+                if ((P.kind == BC_RCR || P.kind == BC_LV) && (order == 2 || order == 4)) {
+                    const double Ps = __shfl_sync(0xffffffffu, a[0], 1);
+                    if (tid == 0) {
+                        BcStepResult r;
+                        const BcState old = s_st;
+                        s_st = zero_d_step(P, old, a[0], s_a.third + Ps, s_a.area, n, q.etab, &r.ptype, &r.closed, &r.S);
+                        r.Pg = s_st.Pstar_gauge;
+                        s_r = r;
+                    }
+                } else {  // zero_d_step with forward Euler, its Q-independent parts taken above
+                    const double mean = ((tid & 1) ? s_a.third + a[0] : a[0]) / s_a.area;
+                    const double Pbar = __shfl_sync(0xffffffffu, mean, 1);
+                    if (tid == 0) {
+                        BcState st = s_st;
+                        st.Q = a[0];
+                        st.Qu = P.q_scale ? mean : a[0];
+                        st.Pbar = Pbar;
+                        BcStepResult r;
+                        r.ptype = 1;
+                        r.closed = 0;
+                        r.S = 0.0;
+                        if (P.kind == BC_RCR) {
+                            const double Qout = -st.Qu;
+                            const double Pw = s_st.Pw + (Qout / P.par[1] - s_a.p0_rc);
+                            st.Pw = Pw;
+                            st.Pstar_gauge = Pw + P.par[0] * Qout;
+                        } else if (P.kind == BC_PRESSURE) {
+                            st.Pstar_gauge = P.par[0];
+                        } else if (P.kind == BC_LV) {
+                            const double Qin = (st.valve_open != 0.0) ? st.Qu : 0.0;
+                            double Pv = st.Pv - s_a.inv_cv * (s_a.dcv * st.Pv + Qin);
+                            if (st.valve_open != 0.0) {
+                                if (st.Qu < 0.0) {  // closure: the inflow has reversed
+                                    st.valve_open = 0.0;
+                                    st.Td = (double)n;
+                                    r.closed = 1;
+                                }
+                            } else {
+                                if (Pv < P.par[1]) Pv = P.par[1];
+                                if (Pv > st.Pbar - 1.0 / 3.0) st.valve_open = 1.0;
+                            }
+                            st.Pv = Pv;
+                            st.Pstar_gauge = Pv;
+                            r.ptype = st.valve_open != 0.0;
+                            if (!r.ptype) r.S = smooth_to_zero((double)(n + 1), st.Td, P.par[2]);
+                        } else {
+                            r.ptype = 0;
+                        }
+                        r.Pg = st.Pstar_gauge;
+                        s_r = r;
+                        s_st = st;
+                    }
+                }
+            }
+            __syncthreads();
+            const BcStepResult &r = s_r;
+            const bool closed = r.closed != 0, ptype = r.ptype != 0;
+            const R Pg = (R)r.Pg, Sm = (R)r.S;
+            for (int L = tid; L < P.n_links; L += THREADS) {
+                const int2 lk = L == tid ? lk0 : link[L];
+                const int i = lk.y & 31, xfi = (lk.y >> 5) & 0x7ff;
+                const FirstLayer<R> m = xf[xfi];
+                const R post = L == tid ? post0 : PlainLoad<S>::ld(fout + (i * N + cell[xfi]));
+                R dP = R(0), vs[3] = {R(0), R(0), R(0)};
+                if (ptype) {
+                    dP = Pg - m.sd / R(3);
+                    vs[0] = m.v[0];
+                    vs[1] = m.v[1];
+                    vs[2] = m.v[2];
+                } else if (P.kind == BC_VELOCITY) {
+                    vs[P.axis] = unode[lk.y >> 16];
+                } else if (P.kind == BC_LV) {  // v_0(T_d) S(t, T_d, N_S); closing now, v_0 = v(x_f, T_d)
+                    const FirstLayer<R> &u = closed ? xf[xfi] : v0s[xfi];
+                    vs[0] = u.v[0] * Sm;
+                    vs[1] = u.v[1] * Sm;
+                    vs[2] = u.v[2] * Sm;
+                }
+                Storage<S>::st(fout + lk.x, post + feq_change<R>(i, dP, vs, m.v));
+            }
+            if (closed && P.kind == BC_LV) {
+                __syncthreads();
+                for (int k = tid; k < n_cells; k += THREADS) {
+                    double *v0 = q.v0 + 3 * (size_t)(P.xf_off + k);
+                    v0s[k] = xf[k];
+                    for (int a = 0; a < 3; a++) v0[a] = (double)xf[k].v[a];
+                }
+            }
+        }
+        const S *t = fin;
+        fin = fout;
+        fout = const_cast<S *>(t);
+        __syncwarp();
+        cluster.barrier_arrive();  // this step's populations are visible to the cluster after the wait
+        if (owner) {
+            if (tid == THREADS - AHEAD - 32) {  // the state of t_{n+1} and the waveform row, as bc_step stores them
+                const long long n = first + s;
+                const BcState st = s_st;
+                q.state[(size_t)((n + 1) & 1) * q.n_bc_total + b] = st;
+                double *wv = q.wave + ((size_t)(n % q.wave_cap) * q.n_bc_total + b) * 4;
+                wv[0] = st.Qu;
+                wv[1] = st.Pbar - 1.0 / 3.0;
+                wv[2] = (s_P.kind == BC_RCR) ? st.Pw : (s_P.kind == BC_LV ? st.Pv : st.Pstar_gauge);
+                wv[3] = st.valve_open;
+                if (io_out)
+                    state_row(st, s_P, q.etab, n + 1, sp.io_states + 8 * ((size_t)s * sp.io_nb + (b - sp.io_b0)));
+            }
+            if (ta >= 0 && s + 1 < sp.n_steps) ahead(s + 1);
+        }
+        __syncwarp();
+        cluster.barrier_wait();
+    }
+    // the last cluster to finish advances the step counter (all have read it)
+    if (rank == 0 && tid == 0) {
+        __threadfence();
+        if (atomicAdd(sp.done, 1) == (int)(gridDim.x / C) - 1) {
+            *sp.done = 0;
+            *p.step = first + sp.n_steps - 1;
+        }
+    }
+}
+
+namespace {
+
+template <class S> constexpr int small_threads() { return sizeof(typename Storage<S>::R) == 8 ? 512 : 1024; }
+
+template <class S> cudaError_t prepare(int cluster, size_t smem, int *clusters) {
+    auto k = k_small_steps<S, small_threads<S>()>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && cluster > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim = {(unsigned)cluster, 1, 1};
+    cfg.gridDim = dim3(cluster);
+    cfg.blockDim = dim3(small_threads<S>());
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(clusters, k, &cfg);
+}
+
+template <class S> cudaError_t launch(void *f0, void *f1, const KParams &p, const BcKParams &q, const SmallKParams &sp,
+                                      int n_inst, int cluster, size_t smem, cudaStream_t st) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim = {(unsigned)cluster, 1, 1};
+    cfg.gridDim = dim3((unsigned)(n_inst * cluster));
+    cfg.blockDim = dim3(small_threads<S>());
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_small_steps<S, small_threads<S>()>, static_cast<S *>(f0), static_cast<S *>(f1), p,
+                              q, sp);
+}
+
+}  // namespace
+
+cudaError_t prepare_small(int prec, int cluster, size_t smem, int *clusters) {
+    cudaError_t e = cudaSuccess;
+    DISPATCH(prec, e = prepare<S>(cluster, smem, clusters));
+    return e;
+}
+
+cudaError_t launch_small(int prec, void *f0, void *f1, const KParams &p, const BcKParams &q, const SmallKParams &sp,
+                         int n_inst, int cluster, size_t smem, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    DISPATCH(prec, e = launch<S>(f0, f1, p, q, sp, n_inst, cluster, smem, st));
+    return e;
+}
+
+}  // namespace lbm

@@ -1,0 +1,115 @@
+"""The multi-step kernel of small lattices against the one-step kernels (taken
+while kernel timing is on): the same trajectory bit for bit, for every kind of
+0D boundary, marching order, storage type, first layers of one to five chunks
+of 256 cells, batches, per-step 0D input, and launches split at the step limit.
+"""
+import numpy as np
+import pytest
+
+from workloads import batch, configs, geometry
+from workloads.spec import BC_VELOCITY, Instance
+
+pytestmark = pytest.mark.gpu
+
+
+def _box():
+    return Instance(node=geometry.closed_box(17, 9, 13), tau=0.7, name="box")
+
+
+def _lv(radius, length):
+    return batch.lv_tube_instance(batch.draw_params(np.random.default_rng(0), 1)[0], radius, length)
+
+
+def _order(inst, order):
+    for b in inst.boundaries:
+        if len(b.params) == 4:
+            b.params = list(b.params) + [float(order)]
+    return inst
+
+
+CASES = {
+    "velocity": lambda: [configs.rigid_tube()],
+    "lv": lambda: [configs.lv_tube(period=300)],
+    "lv_order2": lambda: [_order(configs.lv_tube(period=300), 2)],
+    "lv_order4": lambda: [_order(configs.lv_tube(period=300), 4)],
+    "lv_along_x": lambda: [configs.lv_tube_x(31)],
+    "pressure": lambda: [configs.pressure_tube(15, 15, 24, 5.2, 0.8, 2e-3, 0.0)],
+    "box": lambda: [_box()],
+    "two_chunks": lambda: [configs.rigid_tube(27, 27, 20, radius=10.3)],
+    "five_chunks": lambda: [configs.rigid_tube(41, 41, 12, radius=18.3)],
+    "batch": lambda: [configs.lv_tube(period=300), _box(), _lv(6.3, 41), configs.rigid_tube(16, 16, 24, radius=5.0)],
+}
+
+
+def _pair(insts, precision, steps):
+    from paper_2112_05258_gb300 import Lattice
+    a, b = (Lattice(insts, precision=precision) for _ in range(2))
+    for q, inst in enumerate(insts):
+        f = configs.random_populations(inst, seed=q, amp=2e-3)
+        a.init_populations(q, f)
+        b.init_populations(q, f)
+    b.set_kernel_timing(True)
+    for n in steps:
+        a.step(n)
+        b.step(n)
+    a.sync()
+    b.sync()
+    return a, b
+
+
+def _same(a, b, insts):
+    for q, inst in enumerate(insts):
+        assert np.array_equal(a.populations(q), b.populations(q))
+        assert np.array_equal(a.waves(q), b.waves(q))
+        for k in range(len(inst.boundaries)):
+            assert np.array_equal(a.state_0d(q, k), b.state_0d(q, k))
+
+
+@pytest.mark.parametrize("precision", ["f32", "f16"])
+@pytest.mark.parametrize("name", list(CASES))
+def test_multi_step_kernel_equals_one_step_kernels(name, precision):
+    insts = CASES[name]()
+    a, b = _pair(insts, precision, (1, 2, 350, 61))
+    assert a.info().steps_per_launch > 0      # the case takes the multi-step kernel
+    _same(a, b, insts)
+    a.step(7)                                 # and goes on after a switch of the path
+    b.set_kernel_timing(False)
+    b.step(7)
+    _same(a, b, insts)
+
+
+def test_multi_step_kernel_fp64_and_long_calls():
+    insts = [configs.lv_tube(period=300)]
+    a, b = _pair(insts, "f64", (4 * 300 + 1, 3001))   # the second call goes past the steps of one launch
+    n = a.info().steps_per_launch
+    a.step(n + 5)
+    b.step(n + 5)
+    _same(a, b, insts)
+
+
+def test_step_io_of_a_velocity_inlet_equals_per_step_calls():
+    import torch
+    from paper_2112_05258_gb300 import Lattice
+    inst = configs.rigid_tube()
+    n = 90
+    omega = torch.tensor(2 * np.pi / (1000.0 + 5.0 * np.arange(n)).reshape(n, 1)).pin_memory()
+    rows = torch.zeros((n, 16), dtype=torch.float64, pin_memory=True)
+    want = torch.zeros((n, 16), dtype=torch.float64, pin_memory=True)
+    a, b = (Lattice([inst], precision="f32") for _ in range(2))
+    assert inst.boundaries[0].kind == BC_VELOCITY and a.info().steps_per_launch > 0
+    a.step_io(0, 0, n, omega.data_ptr(), 1, rows.data_ptr())
+    a.sync()
+    b.set_kernel_timing(True)
+    for k in range(n):
+        b.set_0d_params(0, 0, omega[k].numpy())
+        b.step(1)
+        b.state_0d_async(0, want[k].data_ptr())
+    b.sync()
+    assert np.array_equal(rows.numpy(), want.numpy())
+    _same(a, b, [inst])
+
+
+def test_large_or_elastic_lattices_keep_the_step_graphs():
+    from paper_2112_05258_gb300 import Lattice
+    for inst in (configs.ib_tube(), _lv(13.0, 200)):
+        assert Lattice([inst]).info().steps_per_launch == 0
