@@ -452,6 +452,8 @@ void drop_graphs(lbm_handle *h) {
 cudaError_t set_up_small(lbm_handle *h) {
     const Layout &L = h->L;
     if (!L.ib_dA.empty() || L.n_fluid == 0) return cudaSuccess;
+    for (int64_t n : L.inst_fluid)
+        if (small_smem_bulk((int)std::min<int64_t>(n / 16, 1 << 20)) > SMALL_MAX_SMEM) return cudaSuccess;
     std::vector<int32_t> bulk, off;
     int64_t worst_bulk[17] = {0};
     size_t smem_b = 0;

@@ -25,6 +25,7 @@
 // Populations are stored as deviations s = f - w (FP32 or FP64), in SoA
 // order f[i][j nx + x]; the resident state is f*(t_n) with the ghosts of
 // t_{n+1} in the 0D boundary nodes' slots, as in the 3D lattice.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -99,6 +100,7 @@ struct BcDev {
     const int32_t *lk_off, *lk_n;           // links per boundary
     const int32_t *lk_xf, *lk_ieff, *lk_xb, *lk_ib, *lk_node, *lk_xfi;
     const int32_t *node_off;                // first profile row per boundary
+    const int32_t *node_n;                  // boundary nodes
     double *v0;                             // 2 per first-layer node
     double *wave;                           // ring [cap][1 + 4 n_bc]
     int wave_cap;
@@ -114,29 +116,18 @@ struct BcDev {
     int n_red_blocks, n_app_blocks;
 };
 
-// grid: (x-blocks, nr) of 256 nodes of a row, one row of the (x, r) grid per
-// blockIdx.y; the launch covers the x-blocks xb0 .. xb0 + gridDim.x - 1
-template <class S>
-__global__ void __launch_bounds__(256, 8) k_axi_collide(const S *__restrict__ fin, S *__restrict__ fout, Params p,
-                                                       int xb0) {
-    using R = typename Storage<S>::R;
-    const int x = (blockIdx.x + xb0) * blockDim.x + threadIdx.x, j = blockIdx.y;
-    if (p.step && x == 0 && j == 0) *p.step += 1;  // the step index t_n seen by the boundary kernels
-    if (x >= p.nx) return;
-    const int c = j * p.nx + x;
-    const uint32_t fl = __ldg(&p.flags[c]);
-    if (!(fl & AF_FLUID)) return;
+// First-layer moments of a node: s_sum + m/2, j_x, j_r, v_x, v_r, s_sum.
+template <class R> struct AxiMoments {
+    R sp, jx, jr, vx, vr, sd;
+};
+
+// Moments, axisymmetric sources, Guo forcing and BGK collision of node c
+// (inv_r = 1/r of its row) from its pulled populations; stores f*(t_n), and
+// the moments of a node flagged AF_XF in aux.
+template <class S, class R>
+__device__ __forceinline__ AxiMoments<R> axi_collide_store(S *__restrict__ fout, const Params &p, const R (&s)[Q9], R omega,
+                                                           R k, R nu, R inv_r, int c, uint32_t fl) {
     const int n = p.n;
-    R s[Q9];
-#pragma unroll
-    for (int i = 0; i < Q9; i++) {
-        uint32_t src;
-        if (i == 0) src = (uint32_t)c;
-        else if (fl & (1u << i)) src = (uint32_t)(opp(i) * n + c);
-        else if (j - er(i) < 0) src = (uint32_t)(mir(i) * n + (x - ex(i)));  // mirror at the axis (row 0)
-        else src = (uint32_t)(i * n + c - ex(i) - er(i) * p.nx);
-        s[i] = Storage<S>::ld(fin + src);
-    }
     // moments from the sums and differences of the four opposite pairs
     // (1, 2) = +-e_x, (3, 4) = +-e_r, (5, 6) = +-(e_x + e_r), (7, 8) = +-(e_x - e_r)
     R Sp[4], Dp[4];
@@ -148,8 +139,6 @@ __global__ void __launch_bounds__(256, 8) k_axi_collide(const S *__restrict__ fi
     const R sd = s[0] + ((Sp[0] + Sp[1]) + (Sp[2] + Sp[3]));
     const R jx = Dp[0] + Dp[2] + Dp[3], jr = Dp[1] + Dp[2] - Dp[3];
     const R pxr = Sp[2] - Sp[3], prr = Sp[1] + Sp[2] + Sp[3];
-    R omega, k, nu, inv_r;
-    Consts<R>::get(p, j, &omega, &k, &nu, &inv_r);
     const R m = -jr * inv_r;
     const R sp = sd + R(0.5) * m;                       // 3P - 1
     // non-equilibrium stress of f against f^eq(c_s^2 sum f, j): Pi^eq_xr = j_x j_r,
@@ -191,6 +180,35 @@ __global__ void __launch_bounds__(256, 8) k_axi_collide(const S *__restrict__ fi
         Storage<S>::st(fout + ((uint32_t)i * (uint32_t)n + (uint32_t)c), om1 * s[i] + w * (A + B));  // 9 n < 2^31
         Storage<S>::st(fout + ((uint32_t)(i + 1) * (uint32_t)n + (uint32_t)c), om1 * s[i + 1] + w * (A - B));
     }
+    return AxiMoments<R>{sp, jx, jr, vx, vr, sd};
+}
+
+// grid: (x-blocks, nr) of 256 nodes of a row, one row of the (x, r) grid per
+// blockIdx.y; the launch covers the x-blocks xb0 .. xb0 + gridDim.x - 1
+template <class S>
+__global__ void __launch_bounds__(256, 8) k_axi_collide(const S *__restrict__ fin, S *__restrict__ fout, Params p,
+                                                       int xb0) {
+    using R = typename Storage<S>::R;
+    const int x = (blockIdx.x + xb0) * blockDim.x + threadIdx.x, j = blockIdx.y;
+    if (p.step && x == 0 && j == 0) *p.step += 1;  // the step index t_n seen by the boundary kernels
+    if (x >= p.nx) return;
+    const int c = j * p.nx + x;
+    const uint32_t fl = __ldg(&p.flags[c]);
+    if (!(fl & AF_FLUID)) return;
+    const int n = p.n;
+    R s[Q9];
+#pragma unroll
+    for (int i = 0; i < Q9; i++) {
+        uint32_t src;
+        if (i == 0) src = (uint32_t)c;
+        else if (fl & (1u << i)) src = (uint32_t)(opp(i) * n + c);
+        else if (j - er(i) < 0) src = (uint32_t)(mir(i) * n + (x - ex(i)));  // mirror at the axis (row 0)
+        else src = (uint32_t)(i * n + c - ex(i) - er(i) * p.nx);
+        s[i] = Storage<S>::ld(fin + src);
+    }
+    R omega, k, nu, inv_r;
+    Consts<R>::get(p, j, &omega, &k, &nu, &inv_r);
+    axi_collide_store<S, R>(fout, p, s, omega, k, nu, inv_r, c, fl);
 }
 
 // f(t_n) (pulled) and P, u_x, u_r at every node; zero off the fluid
@@ -385,6 +403,299 @@ __global__ void __launch_bounds__(BC2) k_axi_bc_apply(S *__restrict__ f, Params 
     Storage<S>::st(f + (size_t)q.lk_ib[g] * n + q.lk_xb[g], ghost);
 }
 
+// Many steps of a small grid in one launch by one cluster of blocks, as the 3D
+// lattice's multi-step kernel does (lbm_small.cu, where the reasons stand):
+// block k < n_bc owns the first layer and the 0D model of boundary k, the other
+// blocks the rest, one cluster barrier per step.  Same device functions and
+// summation orders as the one-step kernels.
+// A step, FP32: 258 x 32 grid 12.6 -> 4.1 us, 762 x 95 grid 14.7 -> 7.8 us; FP64: 82 x 10 grid
+// 17.2 -> 7.9 us (the FP64 pipe bounds larger ones, which keep the one-step kernels).
+constexpr int AXI_PULLS = Q9 - 1;
+constexpr int AXI_MAX_RED = 8;
+constexpr int AXI_MAX_STEPS = 4096;
+constexpr size_t AXI_MAX_SMEM = 212000;
+
+size_t axi_smem_bulk(int nodes, int r) { return (size_t)nodes * (AXI_PULLS * 4 + 4 + r) + 64; }
+size_t axi_smem_boundary(int n_xf, int n_links, int n_nodes, int r) {
+    return (size_t)n_xf * (AXI_PULLS * 4 + 4 + r + r + 6 * r + 16) + (size_t)n_links * 8 + (size_t)n_nodes * r + 128;
+}
+
+struct AxiSmall {
+    const int32_t *bulk;  // fluid nodes outside the first layers
+    int n_bulk, n_steps;
+};
+
+template <class S, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Params p, BcDev q, AxiSmall sp) {
+    using R = typename Storage<S>::R;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ double sQ[THREADS], sP[THREADS], s_part[2 * AXI_MAX_RED], s_cos, s_sin, s_p0_rc, s_inv_cv, s_dcv;
+    __shared__ double s_area, s_third, s_S;
+    __shared__ BcParam s_P;
+    __shared__ BcState s_st;
+    __shared__ R s_3p;
+    __shared__ int s_ptype, s_closed;
+    const int C = (int)cluster.num_blocks(), b = (int)cluster.block_rank(), nb = q.n_bc, n = p.n, tid = threadIdx.x;
+    const bool owner = b < nb;
+    const long long first = *q.step + 1;
+    R omega, kk, nu, ir0;
+    Consts<R>::get(p, 0, &omega, &kk, &nu, &ir0);
+    int n_cells, cell0 = 0, n_links = 0, n_red = 0, n_nodes = 0;
+    if (owner) {
+        for (int k = tid; k < (int)(sizeof(BcParam) / 4); k += THREADS)
+            reinterpret_cast<int *>(&s_P)[k] = reinterpret_cast<const int *>(q.par + b)[k];
+        n_cells = q.xf_n[b];
+        n_links = q.lk_n[b];
+        n_red = q.red_n[b];
+        n_nodes = q.node_n[b];
+        if (tid == 0) {
+            s_st = q.state[(size_t)(first & 1) * nb + b];
+            s_area = q.area_sum[b];
+            s_third = q.area_sum[b] / 3.0;
+        }
+    } else {
+        const int w = C - nb, per = (sp.n_bulk + w - 1) / w;
+        cell0 = min((b - nb) * per, sp.n_bulk);
+        n_cells = min((b - nb + 1) * per, sp.n_bulk) - cell0;
+    }
+    // shared memory: 8-byte words first
+    double *v0s = reinterpret_cast<double *>(smem);                   // [2 n_xf] closure velocities
+    AxiMoments<R> *mom = reinterpret_cast<AxiMoments<R> *>(v0s + (owner ? 2 * n_cells : 0));
+    R *area = reinterpret_cast<R *>(mom + (owner ? n_cells : 0));      // [n_xf]
+    R *unode = area + (owner ? n_cells : 0);                           // [n_nodes]
+    R *ir = unode + n_nodes;                                           // [n_cells] 1/r
+    int2 *link = reinterpret_cast<int2 *>((reinterpret_cast<uintptr_t>(ir + n_cells) + 7) & ~(uintptr_t)7);
+    int *cell = reinterpret_cast<int *>(link + n_links);
+    int *tab = cell + n_cells;                                         // [8][n_cells]
+    for (int k = tid; k < n_cells; k += THREADS) {
+        const int c = owner ? q.xf[q.xf_off[b] + k] : sp.bulk[cell0 + k];
+        const int x = c % p.nx, j = c / p.nx;
+        const uint32_t fl = p.flags[c];
+        cell[k] = c;
+        R a, d, e;
+        Consts<R>::get(p, j, &a, &d, &e, &ir[k]);
+#pragma unroll
+        for (int i = 1; i < Q9; i++)
+            tab[(i - 1) * n_cells + k] = (fl & (1u << i)) ? opp(i) * n + c
+                                         : j - er(i) < 0  ? mir(i) * n + (x - ex(i))
+                                                          : i * n + c - ex(i) - er(i) * p.nx;
+        if (owner) {
+            area[k] = (R)q.area[q.xf_off[b] + k];
+            v0s[2 * k] = q.v0[2 * (size_t)(q.xf_off[b] + k)];
+            v0s[2 * k + 1] = q.v0[2 * (size_t)(q.xf_off[b] + k) + 1];
+        }
+    }
+    for (int L = tid; L < n_links; L += THREADS) {
+        const int g = q.lk_off[b] + L;
+        link[L] = make_int2(q.lk_ib[g] * n + q.lk_xb[g], q.lk_ieff[g] | (q.lk_xfi[g] << 4) | (q.lk_node[g] << 16));
+    }
+    __syncthreads();
+    // beside the cluster barrier: what does not depend on the step's flow
+    constexpr int AHEAD = 128;
+    const int ta = tid - (THREADS - AHEAD);
+    auto ahead = [&](int s) {
+        const BcParam &P = s_P;
+        const long long t = first + s;
+        if (P.kind == BC_VELOCITY) {
+            const double wt = P.par[0] * (double)(t + 1);
+            if (ta == 0) s_cos = cos(wt);
+            if (ta == 32) s_sin = sin(wt);
+            asm volatile("bar.sync 1, %0;" ::"n"(AHEAD) : "memory");
+            const double cosp = s_cos, sinp = s_sin;
+            for (int a = ta; a < n_nodes; a += AHEAD) {
+                const double *pr = q.profile + 3 * (size_t)(q.node_off[b] + a);
+                unode[a] = (R)((double)P.sign * (pr[0] + pr[1] * cosp - pr[2] * sinp));
+            }
+        } else if (ta == 0) {
+            if (P.kind == BC_RCR) s_p0_rc = s_st.Pw / (P.par[2] * P.par[1]);
+            if (P.kind == BC_LV) {
+                const double E = q.etab[2 * (P.etab_off + (int)(t % P.period))];
+                const double Ed = q.etab[2 * (P.etab_off + (int)(t % P.period)) + 1];
+                const double Cv = 1.0 / E;
+                s_dcv = -Ed / (E * E);
+                s_inv_cv = 1.0 / Cv;
+            }
+        }
+    };
+    if (owner && ta >= 0) ahead(0);
+    __syncthreads();
+
+    const S *fin = f0;
+    S *fout = f1;
+    for (int s = 0; s < sp.n_steps; s++) {
+        if (!owner) {
+            for (int k = tid; k < n_cells; k += THREADS) {
+                const int c = cell[k];
+                R f[Q9];
+                f[0] = fin[c];
+#pragma unroll
+                for (int i = 1; i < Q9; i++) f[i] = fin[tab[(i - 1) * n_cells + k]];
+                axi_collide_store<S, R>(fout, p, f, omega, kk, nu, ir[k], c, 0u);
+            }
+        } else {
+            const BcParam &P = s_P;
+            const long long t = first + s;
+            for (int k0 = 0; k0 < n_red * BC2; k0 += THREADS) {
+                const int k = k0 + tid;
+                double Q = 0.0, Ps = 0.0;
+                if (k < n_cells) {
+                    const int c = cell[k];
+                    R f[Q9];
+                    f[0] = fin[c];
+#pragma unroll
+                    for (int i = 1; i < Q9; i++) f[i] = fin[tab[(i - 1) * n_cells + k]];
+                    const AxiMoments<R> m = axi_collide_store<S, R>(fout, p, f, omega, kk, nu, ir[k], c, 0u);
+                    const R A = area[k];
+                    Q = (double)(A * (R)P.sign * m.jx / (R(1) + m.sd));
+                    Ps = (double)(A * m.sp / R(3));
+                    mom[k] = m;
+                }
+                if (k < n_red * BC2) {
+                    sQ[tid] = Q;
+                    sP[tid] = Ps;
+                }
+                __syncthreads();
+                // the tree of k_axi_bc_reduce, one warp per quantity and chunk
+                constexpr int CH = THREADS / BC2;
+                const int w = tid >> 5, ch = k0 / BC2 + (w & (CH - 1));
+                if (w < 2 * CH && ch < n_red) {
+                    const double *v = (w < CH ? sQ : sP) + (w & (CH - 1)) * BC2 + (tid & 31);
+                    double a[4];
+#pragma unroll
+                    for (int h = 0; h < 4; h++) a[h] = v[32 * h] + v[32 * (h + 4)];
+                    a[0] = (a[0] + a[2]) + (a[1] + a[3]);
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) a[0] += __shfl_down_sync(0xffffffffu, a[0], o);
+                    if ((tid & 31) == 0) s_part[2 * ch + (w < CH ? 0 : 1)] = a[0];
+                }
+                __syncthreads();
+            }
+            int2 lk0 = make_int2(0, 0);  // the thread's first link, its population in flight beside the 0D step
+            R post0 = R(0);
+            if (tid < n_links) {
+                lk0 = link[tid];
+                post0 = fout[(lk0.y & 15) * n + cell[(lk0.y >> 4) & 0xfff]];
+            }
+            if (tid < 32) {
+                double a = 0.0;  // lane 0 the flow, lane 1 the pressure: the partials in their fixed order
+                for (int k = 0; k < n_red; k++) a += s_part[2 * k + (tid & 1)];
+                const int order = (int)P.par[4];
+                if ((P.kind == BC_RCR || P.kind == BC_LV) && (order == 2 || order == 4)) {
+                    const double Ps = __shfl_sync(0xffffffffu, a, 1);
+                    if (tid == 0) {
+                        const BcState old = s_st;
+                        double Sm;
+                        s_st = zero_d_step(P, old, a, s_third + Ps, s_area, t, q.etab, &s_ptype, &s_closed, &Sm);
+                        s_S = Sm;
+                        s_3p = (R)(3.0 * s_st.Pstar_gauge);
+                    }
+                } else {  // zero_d_step with forward Euler, its flow-independent parts taken above
+                    const double mean = ((tid & 1) ? s_third + a : a) / s_area;
+                    const double Pbar = __shfl_sync(0xffffffffu, mean, 1);
+                    if (tid == 0) {
+                        BcState st = s_st;
+                        st.Q = a;
+                        st.Qu = P.q_scale ? mean : a;
+                        st.Pbar = Pbar;
+                        int ptype = 1, closed = 0;
+                        double Sm = 0.0;
+                        if (P.kind == BC_RCR) {
+                            const double Qout = -st.Qu;
+                            const double Pw = s_st.Pw + (Qout / P.par[1] - s_p0_rc);
+                            st.Pw = Pw;
+                            st.Pstar_gauge = Pw + P.par[0] * Qout;
+                        } else if (P.kind == BC_PRESSURE) {
+                            st.Pstar_gauge = P.par[0];
+                        } else if (P.kind == BC_LV) {
+                            const double Qin = (st.valve_open != 0.0) ? st.Qu : 0.0;
+                            double Pv = st.Pv - s_inv_cv * (s_dcv * st.Pv + Qin);
+                            if (st.valve_open != 0.0) {
+                                if (st.Qu < 0.0) {
+                                    st.valve_open = 0.0;
+                                    st.Td = (double)t;
+                                    closed = 1;
+                                }
+                            } else {
+                                if (Pv < P.par[1]) Pv = P.par[1];
+                                if (Pv > st.Pbar - 1.0 / 3.0) st.valve_open = 1.0;
+                            }
+                            st.Pv = Pv;
+                            st.Pstar_gauge = Pv;
+                            ptype = st.valve_open != 0.0;
+                            if (!ptype) Sm = smooth_to_zero((double)(t + 1), st.Td, P.par[2]);
+                        } else {
+                            ptype = 0;
+                        }
+                        s_st = st;
+                        s_ptype = ptype;
+                        s_closed = closed;
+                        s_S = Sm;
+                        s_3p = (R)(3.0 * st.Pstar_gauge);
+                    }
+                }
+            }
+            __syncthreads();
+            const bool ptype = s_ptype != 0, closed = s_closed != 0;
+            for (int L = tid; L < n_links; L += THREADS) {
+                const int2 lk = L == tid ? lk0 : link[L];
+                const int ie = lk.y & 15, xfi = (lk.y >> 4) & 0xfff;
+                const AxiMoments<R> m = mom[xfi];
+                const R post = L == tid ? post0 : (R)fout[ie * n + cell[xfi]];
+                R sps, vxs, vrs;
+                if (ptype) {
+                    sps = s_3p;
+                    vxs = m.vx;
+                    vrs = m.vr;
+                } else if (P.kind == BC_VELOCITY) {
+                    sps = m.sp;
+                    vxs = unode[lk.y >> 16];
+                    vrs = R(0);
+                } else {
+                    const double u0x = closed ? (double)m.vx : v0s[2 * xfi];
+                    const double u0r = closed ? (double)m.vr : v0s[2 * xfi + 1];
+                    sps = m.sp;
+                    vxs = (R)(u0x * s_S);
+                    vrs = (R)(u0r * s_S);
+                }
+                fout[lk.x] = post + dfeq_dev<R>(ie, sps, vxs, vrs, m.sp, m.vx, m.vr);
+            }
+            if (closed) {
+                __syncthreads();
+                for (int k = tid; k < n_cells; k += THREADS) {
+                    double *v0 = q.v0 + 2 * (size_t)(q.xf_off[b] + k);
+                    v0s[2 * k] = v0[0] = (double)mom[k].vx;
+                    v0s[2 * k + 1] = v0[1] = (double)mom[k].vr;
+                }
+            }
+        }
+        const S *tmp = fin;
+        fin = fout;
+        fout = const_cast<S *>(tmp);
+        __syncwarp();
+        cluster.barrier_arrive();
+        if (owner) {
+            if (tid == THREADS - AHEAD - 32) {
+                const long long t = first + s;
+                const BcState st = s_st;
+                q.state[(size_t)((t + 1) & 1) * nb + b] = st;
+                double *row = q.wave + (size_t)(t % q.wave_cap) * (1 + 4 * nb);
+                if (b == 0) row[0] = (double)t;
+                row[1 + 4 * b] = st.Qu;
+                row[2 + 4 * b] = st.Pbar - 1.0 / 3.0;
+                row[3 + 4 * b] = s_P.kind == BC_RCR ? st.Pw : (s_P.kind == BC_LV ? st.Pv : st.Pstar_gauge);
+                row[4 + 4 * b] = st.valve_open;
+            }
+            if (ta >= 0 && s + 1 < sp.n_steps) ahead(s + 1);
+        }
+        __syncwarp();
+        cluster.barrier_wait();
+    }
+    // every block has read the counter: the last barrier is behind all of them
+    if (b == 0 && tid == 0) *q.step = first + sp.n_steps - 1;
+}
+
 }  // namespace axi
 }  // namespace lbm
 
@@ -406,6 +717,10 @@ struct lbm_axi_handle {
     int xb_lo = 0, xb_hi = 0;
     cudaStream_t s_bc = nullptr;
     cudaEvent_t ev_f = nullptr, ev_d = nullptr;
+    // small grids: many steps in one launch by a cluster of blocks (0: one-step kernels)
+    int small_cluster = 0;
+    size_t small_smem = 0;
+    AxiSmall small{};
     int parity = 0;
     int64_t steps = 0;
     void *f[2] = {nullptr, nullptr};
@@ -523,6 +838,81 @@ cudaError_t launch_step(lbm_axi_handle *h, bool pre = false, bool next = false) 
     return h->prec == LBM_F64 ? launch_step_t<double>(h, pre, next) : launch_step_t<float>(h, pre, next);
 }
 
+template <class S> constexpr int axi_small_threads() { return sizeof(S) == 8 ? 512 : 1024; }
+
+template <class S> cudaError_t small_launch(lbm_axi_handle *h, int *clusters, int n_steps) {
+    auto k = k_axi_small_steps<S, axi_small_threads<S>()>;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim = {(unsigned)h->small_cluster, 1, 1};
+    cfg.gridDim = dim3((unsigned)h->small_cluster);
+    cfg.blockDim = dim3(axi_small_threads<S>());
+    cfg.dynamicSmemBytes = h->small_smem;
+    cfg.stream = h->stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    if (clusters) {  // admit the shared memory and cluster size, and ask how many clusters run at once
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AXI_MAX_SMEM);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        return e == cudaSuccess ? cudaOccupancyMaxActiveClusters(clusters, k, &cfg) : e;
+    }
+    AxiSmall sp = h->small;
+    sp.n_steps = n_steps;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<S *>(h->f[h->parity]), static_cast<S *>(h->f[1 - h->parity]), params(h),
+                              h->bd, sp);
+}
+
+cudaError_t small_launch(lbm_axi_handle *h, int *clusters, int n_steps) {
+    return h->prec == LBM_F64 ? small_launch<double>(h, clusters, n_steps) : small_launch<float>(h, clusters, n_steps);
+}
+
+// Decides whether the grid takes its steps in the multi-step kernel.  Times of
+// a step in us, measured on GB300: this kernel the longer of a boundary block
+// (latency, and its first layer) and a bulk block; the one-step kernels 13.4
+// (FP64 21) and then bandwidth (FP64: the narrow FP64 pipe).
+cudaError_t set_up_small(lbm_axi_handle *h, const std::vector<uint16_t> &flags, const std::vector<int32_t> &xf,
+                         const std::vector<int32_t> &xf_n, const std::vector<int32_t> &lk_n,
+                         const std::vector<int32_t> &node_n) {
+    constexpr int C = 16;
+    const int nb = (int)xf_n.size(), r = h->prec == LBM_F64 ? 8 : 4;
+    if (h->n > 16 * 6000 || nb >= C) return cudaSuccess;
+    std::vector<uint8_t> first((size_t)h->n, 0);
+    for (int32_t c : xf) {
+        if (first[(size_t)c]) return cudaSuccess;  // a node in two first layers
+        first[(size_t)c] = 1;
+    }
+    size_t smem = 0;
+    int worst = 0;
+    for (int k = 0; k < nb; k++) {
+        if (xf_n[k] > AXI_MAX_RED * BC2 || node_n[k] > 32767) return cudaSuccess;
+        worst = std::max(worst, xf_n[k]);
+        smem = std::max(smem, axi_smem_boundary(xf_n[k], lk_n[k], node_n[k], r));
+    }
+    std::vector<int32_t> bulk;
+    for (int c = 0; c < h->n; c++)
+        if ((flags[(size_t)c] & AF_FLUID) && !first[(size_t)c]) bulk.push_back(c);
+    const int per = ((int)bulk.size() + C - nb - 1) / (C - nb);
+    smem = std::max(smem, axi_smem_bulk(per, r));
+    if (smem > AXI_MAX_SMEM) return cudaSuccess;
+    const double small = r == 8 ? std::max(4.5 + 0.09 * worst, 1.5 + 16e-3 * per) : std::max(3.8 + 0.006 * worst, 0.7 + 1.6e-3 * per);
+    const double one = r == 8 ? std::max(21.0, 16.0 + 120e-6 * h->n) : 13.4;
+    if (small > 0.9 * one) return cudaSuccess;
+    h->small_cluster = C;
+    h->small_smem = smem;
+    int clusters = 0;
+    if (small_launch(h, &clusters, 0) != cudaSuccess || clusters < 1) {
+        (void)cudaGetLastError();
+        h->small_cluster = 0;
+        return cudaSuccess;
+    }
+    int32_t *d = nullptr;
+    const cudaError_t e = aupload(h, &d, bulk);
+    h->small.bulk = d;
+    h->small.n_bulk = (int)bulk.size();
+    return e;
+}
+
 // step counter for graph-free steps (the boundary kernel advances it when
 // there are boundaries; without boundaries nothing reads it)
 void count_step(lbm_axi_handle *h) { h->steps++; }
@@ -603,7 +993,7 @@ lbm_status lbm_axi_create(const lbm_axi_config *cfg, lbm_axi_handle **out) {
         }
     // boundaries: nodes, links, first layer
     std::vector<BcParam> bcp;
-    std::vector<int32_t> xf_off, xf_n, xf, lk_off, lk_n, lk_xf, lk_ieff, lk_xb, lk_ib, lk_node, lk_xfi, node_off;
+    std::vector<int32_t> xf_off, xf_n, xf, lk_off, lk_n, lk_xf, lk_ieff, lk_xb, lk_ib, lk_node, lk_xfi, node_off, node_n;
     std::vector<double> area, area_sum, profile, etab;
     for (int k = 0; k < cfg->n_bc; k++) {
         const lbm_boundary_desc &b = cfg->bc[k];
@@ -614,6 +1004,7 @@ lbm_status lbm_axi_create(const lbm_axi_config *cfg, lbm_axi_handle **out) {
             for (int x = 0; x < nx; x++)
                 if (node[j * nx + x] == code) nodes_of[j * nx + x] = cnt++;
         node_off.push_back((int32_t)(profile.size() / 3));
+        node_n.push_back(b.kind == LBM_BC_VELOCITY ? cnt : 0);
         if (b.kind == LBM_BC_VELOCITY)
             for (int a = 0; a < 3 * cnt; a++) profile.push_back(b.profile[a]);
         struct Lk { int xf, ie, xb, ib, nd; };
@@ -763,6 +1154,7 @@ lbm_status lbm_axi_create(const lbm_axi_config *cfg, lbm_axi_handle **out) {
               aupload(h, (int32_t **)&bd.lk_node, lk_node) == cudaSuccess &&
               aupload(h, (int32_t **)&bd.lk_xfi, lk_xfi) == cudaSuccess &&
               aupload(h, (int32_t **)&bd.node_off, node_off) == cudaSuccess &&
+              aupload(h, (int32_t **)&bd.node_n, node_n) == cudaSuccess &&
               aalloc(h, &dv0, 2 * std::max<size_t>(xf.size(), 1)) == cudaSuccess &&
               cudaMemset(dv0, 0, 2 * std::max<size_t>(xf.size(), 1) * sizeof(double)) == cudaSuccess &&
               aalloc(h, &dwave, (size_t)h->wave_cap * width) == cudaSuccess &&
@@ -799,6 +1191,7 @@ lbm_status lbm_axi_create(const lbm_axi_config *cfg, lbm_axi_handle **out) {
             h->xb_hi = hi;
         }
     }
+    if (set_up_small(h, flags, xf, xf_n, lk_n, node_n) != cudaSuccess) return bail("out of memory (small-grid tables)");
     if (cudaDeviceSynchronize() != cudaSuccess) return bail("initialisation failed");
     *out = h;
     return LBM_OK;
@@ -808,6 +1201,13 @@ lbm_status lbm_axi_step(lbm_axi_handle *h, int64_t nsteps) {
     if (!h || nsteps < 0) return afail(h, LBM_ERR_ARG, "bad arguments");
     ACK(h, cudaSetDevice(h->device));
     int64_t done = 0;
+    while (h->small_cluster && done < nsteps) {
+        const int k = (int)std::min<int64_t>(nsteps - done, AXI_MAX_STEPS);
+        ACK(h, small_launch(h, nullptr, k));
+        if (k & 1) h->parity ^= 1;
+        done += k;
+        h->steps += k;
+    }
     while (done < nsteps) {
         const int64_t left = nsteps - done;
         if (h->parity == 0 && left >= h->graph_steps) {

@@ -124,3 +124,34 @@ def test_f32_womersley_waveforms(Axi):
     wg, wo = lat.waves(), o.waves()
     for col in (1, 2, 5, 6):
         assert np.abs(wg[:, col] - wo[:, col]).max() < 1e-4 * np.abs(wo[:, col]).max() + 1e-9
+
+
+def _wide(kind):
+    """A grid small enough for the multi-step kernel whose first layers span
+    two chunks of 256 nodes; LV and RCR ends, or a constant pressure."""
+    inst = axw.lv_tube(nr=300, nx=12, radius=290.0, period=60)
+    if kind == "order4":
+        for b in inst.boundaries:
+            b.params = list(b.params) + [4.0]
+    if kind == "pressure":
+        inst.boundaries[1] = Boundary(BC_PRESSURE, 0, -1, [1e-4])
+    return inst
+
+
+@pytest.mark.parametrize("kind", ["order1", "order4", "pressure"])
+def test_wide_first_layers_match_oracle(Axi, kind):
+    lat, o = _run(Axi, _wide(kind), 150)
+    _compare(lat, o)
+
+
+def test_step_calls_of_any_length_give_the_same_bits(Axi):
+    # one call, many short calls and calls past the steps of one launch
+    inst = axw.lv_tube(period=60)
+    a, b = Axi(inst, precision="f32"), Axi(inst, precision="f32")
+    a.step(4500)
+    for n in (1, 2, 97, 4097, 303):
+        b.step(n)
+    a.sync()
+    b.sync()
+    assert np.array_equal(a.populations(), b.populations())
+    assert np.array_equal(a.waves()[-200:], b.waves()[-200:])
