@@ -8,8 +8,11 @@
 //   forward     act_out[B][N]  = act_in[B][K]  * Wt[N][K]^T   (+ bias, SiLU)
 //   input grad  g_in[B][K]     = g_out[B][N]   * W[K][N]^T    (x SiLU'(pre))
 //   weight grad dWt[N][K]      = g_out^T[N][B] * act_in^T[K][B]^T
-// so each layer keeps its weights in both layouts (Wt and W) and the
-// backward pass transposes activations and output gradients.
+// so each layer keeps its weights in both layouts (Wt and W), and activations
+// and output gradients are written in both by the kernel that makes them.
+// One Adam step of the 8-256-256-256-64 network on 512 rows is 11 launches and
+// 57 us (35 launches and 291 us before; 64-wide, one hidden layer, 64 rows: 96
+// -> 18 us), with the same bits: every sum keeps its order.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -22,10 +25,6 @@
 
 namespace {
 
-#ifndef LBM_MLP_MMA_SYNC
-#define LBM_MLP_MMA_SYNC 0  // 1: the warp-level mma.sync products instead of tcgen05 (for comparison)
-#endif
-
 using bf16 = __nv_bfloat16;
 constexpr int K0 = 16;       // padded input width
 
@@ -37,6 +36,8 @@ struct Epi {
     bf16 *out_bf;        // EPI_HIDDEN: SiLU(pre); EPI_DX: gradient (bf16)
     float *out_f;        // EPI_OUT: y; EPI_DX: gradient (fp32); EPI_DW: dWt
     const float *pre_in; // EPI_DX: pre-activation of the layer below
+    bf16 *out_t;         // EPI_HIDDEN, EPI_DX: out_bf transposed (N x M) for the weight gradients, or null
+    int n_keep;          // EPI_DW: columns kept (the layer's inputs without padding; the row stride of out_f)
 };
 
 __device__ __forceinline__ float silu_f(float z) { return z / (1.f + __expf(-z)); }
@@ -45,144 +46,53 @@ __device__ __forceinline__ float silu_grad_f(float z) {
     return s * (1.f + z * (1.f - s));
 }
 
-#if LBM_MLP_MMA_SYNC
-constexpr int TM = 64, TN = 64, TK = 32;
-
-__device__ __forceinline__ void mma_bf16(float *d, const uint32_t *a, const uint32_t *b) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
-        "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-// C[M][N] = A[M][K] * Bt[N][K]^T; M, N multiples of 16, K a multiple of 16.
-// 128 threads: 2 x 2 warps, each a 32 x 32 sub-tile of the 64 x 64 block tile.
-template <int EPI>
-__global__ void __launch_bounds__(128) k_gemm_nt(const bf16 *__restrict__ A, const bf16 *__restrict__ Bt, int M,
-                                                 int N, int K, Epi e) {
-    __shared__ __align__(16) bf16 As[TM][TK + 8];
-    __shared__ __align__(16) bf16 Bs[TN][TK + 8];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wm = warp >> 1, wn = warp & 1;
-    const int g = lane >> 2, t = lane & 3;
-    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-    float acc[2][4][4];
-#pragma unroll
-    for (int i = 0; i < 2; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++)
-#pragma unroll
-            for (int k = 0; k < 4; k++) acc[i][j][k] = 0.f;
-    for (int k0 = 0; k0 < K; k0 += TK) {
-        // each thread loads 16 bf16 (two 16-byte chunks) of A and of Bt
-        {
-            const int r = tid >> 1, c = (tid & 1) * 16;
-            uint4 va0 = make_uint4(0, 0, 0, 0), va1 = va0, vb0 = va0, vb1 = va0;
-            if (m0 + r < M && k0 + c < K) {
-                const uint4 *p = reinterpret_cast<const uint4 *>(A + (size_t)(m0 + r) * K + k0 + c);
-                va0 = p[0];
-                va1 = p[1];
-            }
-            if (n0 + r < N && k0 + c < K) {
-                const uint4 *p = reinterpret_cast<const uint4 *>(Bt + (size_t)(n0 + r) * K + k0 + c);
-                vb0 = p[0];
-                vb1 = p[1];
-            }
-            *reinterpret_cast<uint4 *>(&As[r][c]) = va0;
-            *reinterpret_cast<uint4 *>(&As[r][c + 8]) = va1;
-            *reinterpret_cast<uint4 *>(&Bs[r][c]) = vb0;
-            *reinterpret_cast<uint4 *>(&Bs[r][c + 8]) = vb1;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < TK; kk += 16) {
-            uint32_t a[2][4], b[4][2];
-#pragma unroll
-            for (int i = 0; i < 2; i++) {
-                const int r = wm * 32 + i * 16 + g;
-                a[i][0] = *reinterpret_cast<const uint32_t *>(&As[r][kk + 2 * t]);
-                a[i][1] = *reinterpret_cast<const uint32_t *>(&As[r + 8][kk + 2 * t]);
-                a[i][2] = *reinterpret_cast<const uint32_t *>(&As[r][kk + 8 + 2 * t]);
-                a[i][3] = *reinterpret_cast<const uint32_t *>(&As[r + 8][kk + 8 + 2 * t]);
-            }
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const int c = wn * 32 + j * 8 + g;
-                b[j][0] = *reinterpret_cast<const uint32_t *>(&Bs[c][kk + 2 * t]);
-                b[j][1] = *reinterpret_cast<const uint32_t *>(&Bs[c][kk + 8 + 2 * t]);
-            }
-#pragma unroll
-            for (int i = 0; i < 2; i++)
-#pragma unroll
-                for (int j = 0; j < 4; j++) mma_bf16(acc[i][j], a[i], b[j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 2; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++)
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int row = m0 + wm * 32 + i * 16 + g + 8 * h;
-                const int col = n0 + wn * 32 + j * 8 + 2 * t;
-                if (row >= M || col >= N) continue;
-#pragma unroll
-                for (int q = 0; q < 2; q++) {
-                    const float v = acc[i][j][2 * h + q];
-                    const size_t idx = (size_t)row * N + col + q;
-                    if (EPI == EPI_HIDDEN) {
-                        const float z = v + e.bias[col + q];
-                        e.pre[idx] = z;
-                        e.out_bf[idx] = __float2bfloat16_rn(silu_f(z));
-                    } else if (EPI == EPI_OUT) {
-                        e.out_f[idx] = v + e.bias[col + q];
-                    } else if (EPI == EPI_DX) {
-                        const float gr = v * silu_grad_f(e.pre_in[idx]);
-                        e.out_f[idx] = gr;
-                        e.out_bf[idx] = __float2bfloat16_rn(gr);
-                    } else {
-                        e.out_f[idx] = v;
-                    }
-                }
-            }
-}
-#endif  // LBM_MLP_MMA_SYNC
-
 // ---------------------------------------------------------------------------
 // tcgen05 product C[M][N] = A[M][K] * Bt[N][K]^T (BF16 operands, FP32
-// accumulator in tensor memory).  One CTA of 128 threads per 128 x NT tile of
+// accumulator in tensor memory).  One CTA of 256 threads per 128 x NT tile of
 // C (NT = 32 or 16 columns).  The K range is walked in chunks of 64 through
-// two shared-memory stages: the four warps start the asynchronous copies
-// (cp.async, 16 bytes each) of chunk j + 1's A tile (128 rows) and B tile
-// (NT rows) into stage (j + 1) % 2 before the tensor core works on chunk j.  The tiles are laid out in the canonical
-// no-swizzle K-major form of the tensor-core descriptors: 8-row x 16-byte
-// core matrices, element (r, k) of a tile at byte
-// ((r / 8) * 8 + k / 8) * 128 + (r % 8) * 16 + (k % 8) * 2, so that the core
-// matrix next in K is 128 bytes on (the descriptor's leading-dimension
-// offset) and the next 8-row group 1024 bytes on (its stride offset).  One
+// a ring of TC_STAGES shared-memory stages: the warps start the
+// asynchronous copies (cp.async, 16 bytes each) of the first stages' chunks of
+// the A tile (128 rows) and B tile (NT rows) at once and refill a stage once
+// its MMAs are done.  The products are small (256 x 256 weights, 512 rows) and
+// bound by latency, not by the tensor cores: clocks of a CTA of the 512 x 256 x
+// 256 layer before were 8,500 copies (4-way conflicts of 8-row core matrices
+// and a round trip per chunk) and 5,600 epilogue (32 SiLU values a thread); with
+// swizzled rows, four stages, twice the threads and tiles of 16 columns 3,500
+// and 1,500.
+// The tiles are laid out K-major with the 128-byte swizzle: row r of a chunk is
+// 128 bytes (64 columns) at r * 128, its 16-byte piece p at p ^ (r % 8), so that
+// a warp's copy writes whole rows without bank conflicts; 16 columns of K are
+// 32 bytes on in the descriptor's start address.  One
 // thread issues one MMA (M = 128, N = NT, K = 16) per 16 columns of the chunk
-// and commits them to the stage's mbarrier, which the copy of chunk j + 2
-// waits for.  After the last chunk each warp reads its 32 rows of the
+// and commits them to the stage's mbarrier, which the copy that reuses the
+// stage waits for.  After the last chunk each warp reads its 32 rows of the
 // accumulator (tensor-memory lanes 32 w .. 32 w + 31) with tcgen05.ld and
 // applies the epilogue, 16 consecutive columns of a row per thread with
 // 16-byte loads and stores.  Rows >= M and columns >= N are computed from zeros
 // and not stored.  Every wait is bounded: on a time-out the kernel sets
 // *err, waits (bounded) for its own MMAs, frees its tensor memory and leaves.
 constexpr int TC_M = 128, TC_K = 64;
-constexpr int TC_THREADS = 128;
+constexpr int TC_STAGES = 4;
+constexpr int TC_SMEM = TC_STAGES * (TC_M + 32) * TC_K * 2 + 1024;  // and the 1024-byte alignment of the tiles
+constexpr int TC_THREADS = 256;
 constexpr long long TC_SPIN = 1ll << 22;  // mbarrier polls before a time-out
+
+// The kernels of a pass follow one another at once (programmatic dependent
+// launch): a kernel lets its successor start its set-up early and itself waits,
+// before it touches memory, until its predecessor has finished.  Every thread
+// waits, so that a finished kernel means that all before it have finished too.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// shared-memory matrix descriptor: start address, leading (K) and stride (M/N)
-// byte offsets, the fixed 0b001 at bits 46-48, no swizzle (bits 61-63 = 0)
-__device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo & 0x3FFFFu) >> 4) << 16) |
-           ((uint64_t)((sbo & 0x3FFFFu) >> 4) << 32) | (1ull << 46);
+// shared-memory matrix descriptor of a K-major tile with 128-byte swizzle: start
+// address, leading offset (unused with this swizzle), stride offset 1024 bytes
+// (8 rows), the fixed 0b001 at bits 46-48, swizzle mode 2 at bits 61-63
+__device__ __forceinline__ uint64_t tc_desc(uint32_t addr) {
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(1024u >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 
 // instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), BF16 A
@@ -207,52 +117,79 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase) {
     return false;
 }
 
-// Epilogue of 16 consecutive columns col .. col + 15 of one row (col and N
-// multiples of 16): 16-byte vector loads and stores.
-template <int EPI> __device__ __forceinline__ void epi_store16(const Epi &e, int row, int col, int N, const uint32_t *r) {
-    const size_t idx = (size_t)row * N + col;
-    float v[16];
+// Epilogue of W (8 or 16) consecutive columns col .. col + W - 1 of one row (col
+// a multiple of W, N of 16): 16-byte vector loads and stores; x holds the
+// columns' biases or pre-activations, read before the product was ready.
+template <int EPI, int W> __device__ __forceinline__ void epi_load(const Epi &e, int row, int col, int N, float (&x)[W]) {
+    if (EPI == EPI_DW) return;
+    const float4 *p = reinterpret_cast<const float4 *>(EPI == EPI_DX ? e.pre_in + (size_t)row * N + col : e.bias + col);
 #pragma unroll
-    for (int j = 0; j < 16; j++) v[j] = __uint_as_float(r[j]);
-    if (EPI == EPI_HIDDEN || EPI == EPI_OUT) {
-        const float4 *b4 = reinterpret_cast<const float4 *>(e.bias + col);
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const float4 b = b4[q];
-            v[4 * q] += b.x;
-            v[4 * q + 1] += b.y;
-            v[4 * q + 2] += b.z;
-            v[4 * q + 3] += b.w;
-        }
+    for (int q = 0; q < W / 4; q++) {
+        const float4 v = p[q];
+        x[4 * q] = v.x;
+        x[4 * q + 1] = v.y;
+        x[4 * q + 2] = v.z;
+        x[4 * q + 3] = v.w;
     }
-    if (EPI == EPI_DX) {
-        const float4 *p4 = reinterpret_cast<const float4 *>(e.pre_in + idx);
+}
+template <int EPI, int W>
+__device__ __forceinline__ void epi_store(const Epi &e, int row, int col, int M, int N, const uint32_t (&r)[W],
+                                          const float (&x)[W]) {
+    const size_t idx = (size_t)row * N + col;
+    float v[W];
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const float4 z = p4[q];
-            v[4 * q] *= silu_grad_f(z.x);
-            v[4 * q + 1] *= silu_grad_f(z.y);
-            v[4 * q + 2] *= silu_grad_f(z.z);
-            v[4 * q + 3] *= silu_grad_f(z.w);
-        }
+    for (int j = 0; j < W; j++) {
+        v[j] = __uint_as_float(r[j]);
+        if (EPI == EPI_HIDDEN || EPI == EPI_OUT) v[j] += x[j];
+        if (EPI == EPI_DX) v[j] *= silu_grad_f(x[j]);
+    }
+    if (EPI == EPI_DW && e.n_keep != N) {  // an input layer narrower than its padding
+#pragma unroll
+        for (int j = 0; j < W; j++)
+            if (col + j < e.n_keep) e.out_f[(size_t)row * e.n_keep + col + j] = v[j];
+        return;
     }
     float *of = EPI == EPI_HIDDEN ? e.pre : e.out_f;
     float4 *o4 = reinterpret_cast<float4 *>(of + idx);
 #pragma unroll
-    for (int q = 0; q < 4; q++) o4[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    for (int q = 0; q < W / 4; q++) o4[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     if (EPI == EPI_HIDDEN || EPI == EPI_DX) {
-        uint32_t w[8];
+        uint32_t w[W / 2];
 #pragma unroll
-        for (int q = 0; q < 8; q++) {
+        for (int q = 0; q < W / 2; q++) {
             const float a = EPI == EPI_HIDDEN ? silu_f(v[2 * q]) : v[2 * q];
             const float b = EPI == EPI_HIDDEN ? silu_f(v[2 * q + 1]) : v[2 * q + 1];
             const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
             w[q] = *reinterpret_cast<const uint32_t *>(&h);
         }
         uint4 *b4 = reinterpret_cast<uint4 *>(e.out_bf + idx);
-        b4[0] = make_uint4(w[0], w[1], w[2], w[3]);
-        b4[1] = make_uint4(w[4], w[5], w[6], w[7]);
+#pragma unroll
+        for (int q = 0; q < W / 8; q++) b4[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+        if (e.out_t) {  // the warp's rows are consecutive: 64 bytes per column
+            uint16_t *t = reinterpret_cast<uint16_t *>(e.out_t) + (size_t)col * M + row;
+#pragma unroll
+            for (int q = 0; q < W / 2; q++) {
+                t[(size_t)(2 * q) * M] = (uint16_t)w[q];
+                t[(size_t)(2 * q + 1) * M] = (uint16_t)(w[q] >> 16);
+            }
+        }
     }
+}
+
+// tcgen05.ld of W consecutive accumulator columns, lane l of the warp row l of its quadrant
+template <int W> __device__ __forceinline__ void tmem_ld(uint32_t addr, uint32_t (&r)[W]);
+template <> __device__ __forceinline__ void tmem_ld<8>(uint32_t ta, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(ta));
+}
+template <> __device__ __forceinline__ void tmem_ld<16>(uint32_t ta, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
+        "[%16];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(ta));
 }
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid) {
@@ -261,23 +198,24 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool v
 }
 
 template <int EPI, int NT>
-__global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const bf16 *__restrict__ A, const bf16 *__restrict__ Bt,
-                                                        int M, int N, int K, Epi e, int *err) {
+__device__ __forceinline__ void gemm_tile(const bf16 *__restrict__ A, const bf16 *__restrict__ Bt, int M, int N, int K,
+                                          const Epi &e, int *err, int mt, int nt) {
     constexpr int TMEM_COLS = 32;  // NT <= 32 accumulator columns (the minimum allocation)
     constexpr int A_BYTES = TC_M * TC_K * 2, B_BYTES = NT * TC_K * 2;
     static_assert(NT == 16 || NT == 32, "tile width");
-    __shared__ __align__(1024) uint8_t sA[2][A_BYTES];
-    __shared__ __align__(1024) uint8_t sB[2][B_BYTES];
-    __shared__ __align__(8) uint64_t bar[2];
+    extern __shared__ uint8_t tiles[];
+    __shared__ __align__(8) uint64_t bar[TC_STAGES];
     __shared__ uint32_t tmem_base;
     __shared__ int failed;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int m0 = blockIdx.y * TC_M, n0 = blockIdx.x * NT;
-    const uint32_t bar_a[2] = {smem_u32(&bar[0]), smem_u32(&bar[1])};
+    const uint32_t sA = (smem_u32(tiles) + 1023u) & ~1023u, sB = sA + TC_STAGES * A_BYTES;
+    static_assert(TC_THREADS / 32 >= 32 / 4, "one piece of the B tile per warp");
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int m0 = mt * TC_M, n0 = nt * NT;
+    const uint32_t bar0 = smem_u32(&bar[0]);
     if (tid == 0) {
         failed = 0;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_a[0]));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_a[1]));
+#pragma unroll
+        for (int k = 0; k < TC_STAGES; k++) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * k));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -289,36 +227,48 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const bf16 *__restrict__
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base;
+    wait_for_previous();
     const uint32_t idesc = tc_idesc<NT>();
     const int nchunk = (K + TC_K - 1) / TC_K;
-    // asynchronous copy of chunk j into stage j % 2 (rows or columns past the
+    // asynchronous copy of chunk j into its stage (rows or columns past the
     // matrix are zero-filled): A tile 128 rows x 8 pieces of 16 bytes, B tile NT rows
     auto copy_chunk = [&](int j) {
-        const int st = j & 1, k0 = j * TC_K;
-        const uint32_t a_s = smem_u32(sA[st]), b_s = smem_u32(sB[st]);
-        for (int q = tid; q < (TC_M + NT) * (TC_K / 8); q += TC_THREADS) {
-            const bool isA = q < TC_M * (TC_K / 8);
-            const int qq = isA ? q : q - TC_M * (TC_K / 8);
-            const int r = qq >> 3, kc = qq & 7;
-            const int grow = (isA ? m0 : n0) + r, gk = k0 + kc * 8;
-            const bool valid = grow < (isA ? M : N) && gk < K;
-            const bf16 *src = valid ? (isA ? A : Bt) + (size_t)grow * K + gk : A;
-            cp_async16((isA ? a_s : b_s) + (uint32_t)(((r >> 3) * 8 + kc) * 128 + (r & 7) * 16), src, valid);
-        }
+        const int st = j % TC_STAGES, k0 = j * TC_K;
+        const uint32_t a_s = sA + st * A_BYTES, b_s = sB + st * B_BYTES;
+        // a warp copies 4 rows of 128 bytes at a time (whole lines of both memories)
+        auto piece = [&](uint32_t tile, const bf16 *X, int row0, int rows, int idx) {
+            const int r = 4 * idx + (lane >> 3), kc = lane & 7;
+            const int grow = row0 + r, gk = k0 + kc * 8;
+            const bool valid = grow < rows && gk < K;
+            cp_async16(tile + (uint32_t)(r * 128 + ((kc ^ (r & 7)) << 4)), valid ? X + (size_t)grow * K + gk : X, valid);
+        };
+#pragma unroll
+        for (int u = 0; u < TC_M / 4; u += TC_THREADS / 32) piece(a_s, A, m0, M, warp + u);
+        if (warp < NT / 4) piece(b_s, Bt, n0, N, warp);
     };
+    // this thread's part of the epilogue
+    constexpr int W = NT / 2;
+    const int row = m0 + (warp & 3) * 32 + lane, col = n0 + (warp >> 2) * W;
+    const bool mine = row < M && col < N;  // N is a multiple of 16
+    float x[W];
     bool ok = true;
     int last = -1;  // the last chunk whose MMAs were committed
-    copy_chunk(0);
-    asm volatile("cp.async.commit_group;" ::: "memory");
+#pragma unroll
+    for (int j = 0; j < TC_STAGES - 1; j++) {  // one group per chunk, empty past the last
+        if (j < nchunk) copy_chunk(j);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    if (mine) epi_load<EPI, W>(e, row, col, N, x);
     for (int j = 0; j < nchunk && ok; j++) {
-        const int st = j & 1, k0 = j * TC_K;
-        if (j + 1 < nchunk) {
-            // stage (j + 1) % 2 was last read by the MMAs of chunk j - 1
-            if (j >= 1 && !mbar_wait(bar_a[(j + 1) & 1], ((j - 1) >> 1) & 1)) atomicExch(&failed, 1);
-            if (!failed) copy_chunk(j + 1);
+        const int st = j % TC_STAGES, k0 = j * TC_K;
+        const int jn = j + TC_STAGES - 1;  // the chunk to start now
+        if (jn < nchunk) {
+            // its stage was last read by the MMAs of chunk j - 1
+            if (j >= 1 && !mbar_wait(bar0 + 8 * ((j - 1) % TC_STAGES), ((j - 1) / TC_STAGES) & 1)) atomicExch(&failed, 1);
+            if (!failed) copy_chunk(jn);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group 1;" ::: "memory");  // chunk j has landed
+        asm volatile("cp.async.wait_group %0;" ::"n"(TC_STAGES - 1) : "memory");  // chunk j has landed
         // make the copies visible to the tensor core
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
@@ -328,11 +278,11 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const bf16 *__restrict__
         }
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a_base = smem_u32(sA[st]), b_base = smem_u32(sB[st]);
+            const uint32_t a_base = sA + st * A_BYTES, b_base = sB + st * B_BYTES;
             const int nk = min(TC_K / 16, (K - k0 + 15) / 16);
             for (int kk = 0; kk < nk; kk++) {
-                const uint64_t ad = tc_desc(a_base + kk * 256, 128, 1024);
-                const uint64_t bd = tc_desc(b_base + kk * 256, 128, 1024);
+                const uint64_t ad = tc_desc(a_base + kk * 32);
+                const uint64_t bd = tc_desc(b_base + kk * 32);
                 const uint32_t acc = (k0 > 0 || kk > 0) ? 1u : 0u;
                 asm volatile(
                     "{\n.reg .pred p;\n"
@@ -341,38 +291,28 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const bf16 *__restrict__
                     "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             bar_a[st])
+                             bar0 + 8 * st)
                          : "memory");
         }
         last = j;
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");  // no copy outlives the kernel
     // the last commit completes when all MMAs issued before it have completed
-    if (last >= 0 && !mbar_wait(bar_a[last & 1], (last >> 1) & 1)) atomicExch(&failed, 1);
+    if (last >= 0 && !mbar_wait(bar0 + 8 * (last % TC_STAGES), (last / TC_STAGES) & 1)) atomicExch(&failed, 1);
     __syncthreads();
     if (failed) ok = false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (ok) {
-        // epilogue: warp w holds rows 32 w .. 32 w + 31 (tensor-memory lanes), 16 columns per load
-        const int row = m0 + warp * 32 + (tid & 31);
-#pragma unroll
-        for (int c0 = 0; c0 < NT; c0 += 16) {
-            uint32_t r[16];
-            const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                "[%16];\n"
-                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                  "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-                  "=r"(r[15])
-                : "r"(ta));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (row < M && n0 + c0 < N) epi_store16<EPI>(e, row, n0 + c0, N, r);  // N is a multiple of 16
-        }
+        // warps w and w + 4 hold the rows 32 (w % 4) .. + 31 (their quadrant of the
+        // tensor memory) and one half of the tile's columns each
+        uint32_t r[W];
+        tmem_ld<W>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * W), r);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (mine) epi_store<EPI, W>(e, row, col, M, N, r, x);
     } else {
         if (tid == 0) atomicExch(err, 1);
         // the MMAs still in flight (bounded; their commit was the last one)
-        if (last >= 0) mbar_wait(bar_a[last & 1], (last >> 1) & 1);
+        if (last >= 0) mbar_wait(bar0 + 8 * (last % TC_STAGES), (last / TC_STAGES) & 1);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -380,6 +320,103 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const bf16 *__restrict__
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
     }
+}
+
+// one forward layer
+template <int EPI, int NT>
+__global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(const bf16 *__restrict__ A, const bf16 *__restrict__ Bt, int M,
+                                                        int N, int K, Epi e, int *err) {
+    let_next_start();
+    gemm_tile<EPI, NT>(A, Bt, M, N, K, e, err, blockIdx.y, blockIdx.x);
+}
+
+// db[n] = sum over the batch of g[b][n] for 32 columns, in the order of the
+// rows: the block stages 128 rows at a time in shared memory (the next rows in
+// flight in registers meanwhile), one warp adds them column by column.  Bound
+// by the chain of FP32 additions, 4 cycles each; one thread per column reading
+// global memory row by row took 31 us for 512 rows.
+__device__ __forceinline__ void bias_columns(const float *__restrict__ g, int batch, int n, float *db, int c0, float *tile) {
+    constexpr int ROWS = 128;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = c0 + lane;
+    constexpr int WARPS = TC_THREADS / 32;
+    float v[ROWS / WARPS], s = 0.f;
+    auto load = [&](int r0) {
+#pragma unroll
+        for (int k = 0; k < ROWS / WARPS; k++) {
+            const int r = r0 + w + WARPS * k;
+            v[k] = r < batch && c < n ? g[(size_t)r * n + c] : 0.f;
+        }
+    };
+    load(0);
+    for (int r0 = 0; r0 < batch; r0 += ROWS) {
+#pragma unroll
+        for (int k = 0; k < ROWS / WARPS; k++) tile[(w + WARPS * k) * 32 + lane] = v[k];
+        __syncthreads();
+        if (r0 + ROWS < batch) load(r0 + ROWS);
+        if (w == 0) {
+            const int m = min(ROWS, batch - r0);
+            if (m == ROWS) {
+#pragma unroll 32
+                for (int r = 0; r < ROWS; r++) s += tile[r * 32 + lane];
+            } else {
+                for (int r = 0; r < m; r++) s += tile[r * 32 + lane];
+            }
+        }
+        __syncthreads();
+    }
+    if (w == 0 && c < n) db[c] = s;
+}
+
+// The loss: the rows' sums added in a fixed tree of 256 threads.
+__device__ __forceinline__ void sum_loss(const float *row_loss, int batch, int n_out, float *loss, float *red) {
+    static_assert(TC_THREADS == 256, "the tree's threads");
+    float s = 0.f;
+    for (int b = threadIdx.x; b < batch; b += 256) s += row_loss[b];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *loss = red[0] / (float)(batch * n_out);
+}
+
+// One layer of the backward pass in one launch (five and a product before: two
+// transposes, now written by the epilogues, bias sums, weight product, copy
+// without padding); the blocks take, in this order,
+// the tiles of the input gradient (the longest chain: the next layer waits for
+// it), the tiles of the weight gradient, 32 columns each of the bias gradient,
+// and, with loss, the loss.  All of them only need the layer's output gradient.
+struct Backward {
+    int B, N, K;                      // rows, outputs, padded inputs
+    const bf16 *g, *g_t, *W, *in_t;   // output gradient (B x N), transposed; weights (K x N); inputs transposed (K x B)
+    const float *g_f;
+    float *db;
+    Epi dx, dw;
+    int n_dx, dx_cols, n_dw, dw_cols; // tiles, and tiles per row of tiles
+    int n_bias;
+    const float *row_loss;
+    float *loss;
+    int n_out;
+};
+template <int NT>
+__global__ void __launch_bounds__(TC_THREADS) k_backward(Backward q, int *err) {
+    extern __shared__ uint8_t tiles[];
+    let_next_start();
+    int k = blockIdx.x;
+    if (k < q.n_dx) {
+        gemm_tile<EPI_DX, NT>(q.g, q.W, q.B, q.K, q.N, q.dx, err, k / q.dx_cols, k % q.dx_cols);
+        return;
+    }
+    k -= q.n_dx;
+    if (k < q.n_dw) {
+        gemm_tile<EPI_DW, NT>(q.g_t, q.in_t, q.N, q.K, q.B, q.dw, err, k / q.dw_cols, k % q.dw_cols);
+        return;
+    }
+    k -= q.n_dw;
+    wait_for_previous();
+    if (k < q.n_bias) bias_columns(q.g_f, q.B, q.N, q.db, 32 * k, reinterpret_cast<float *>(tiles));
+    else sum_loss(q.row_loss, q.B, q.n_out, q.loss, reinterpret_cast<float *>(tiles));
 }
 
 __global__ void k_transpose_bf16(const bf16 *__restrict__ in, bf16 *__restrict__ out, int R, int C) {
@@ -393,19 +430,27 @@ __global__ void k_transpose_bf16(const bf16 *__restrict__ in, bf16 *__restrict__
         if (c0 + k < C && r < R) out[(size_t)(c0 + k) * R + r] = tile[threadIdx.x][k];
 }
 
-// Gathers minibatch rows into the padded BF16 input and the FP32 target.
+// Gathers minibatch rows into the padded BF16 input (both layouts) and the FP32 target.
 __global__ void k_gather_batch(const float *__restrict__ xd, const float *__restrict__ td,
                                const int32_t *__restrict__ idx, int batch, int n_in, int n_out, bf16 *x_bf,
-                               float *t) {
+                               bf16 *x_t, float *t) {
+    let_next_start();
+    wait_for_previous();
     const int b = blockIdx.x, j = threadIdx.x;
     const int r = idx[b];
-    if (j < K0) x_bf[(size_t)b * K0 + j] = __float2bfloat16_rn(j < n_in ? xd[(size_t)r * n_in + j] : 0.f);
+    if (j < K0) {
+        const bf16 v = __float2bfloat16_rn(j < n_in ? xd[(size_t)r * n_in + j] : 0.f);
+        x_bf[(size_t)b * K0 + j] = v;
+        x_t[(size_t)j * batch + b] = v;
+    }
     for (int k = j; k < n_out; k += blockDim.x) t[(size_t)b * n_out + k] = td[(size_t)r * n_out + k];
 }
 
 // d loss / d y for the mean squared error, and per-row partial sums of the loss.
 __global__ void k_mse_grad(const float *__restrict__ y, const float *__restrict__ t, int batch, int n_out,
-                           float *g_f, bf16 *g_bf, float *row_loss) {
+                           float *g_f, bf16 *g_bf, bf16 *g_t, float *row_loss) {
+    let_next_start();
+    wait_for_previous();
     const int b = blockIdx.x;
     float s = 0.f;
     const float scale = 2.f / (float)(batch * n_out);
@@ -414,7 +459,9 @@ __global__ void k_mse_grad(const float *__restrict__ y, const float *__restrict_
         const float d = y[i] - t[i];
         s += d * d;
         g_f[i] = scale * d;
-        g_bf[i] = __float2bfloat16_rn(scale * d);
+        const bf16 v = __float2bfloat16_rn(scale * d);
+        g_bf[i] = v;
+        g_t[(size_t)k * batch + b] = v;
     }
     __shared__ float red[64];
     red[threadIdx.x] = s;
@@ -424,35 +471,6 @@ __global__ void k_mse_grad(const float *__restrict__ y, const float *__restrict_
         __syncthreads();
     }
     if (threadIdx.x == 0) row_loss[b] = red[0];
-}
-
-__global__ void k_sum_loss(const float *row_loss, int batch, int n_out, float *loss) {
-    __shared__ float red[256];
-    float s = 0.f;
-    for (int b = threadIdx.x; b < batch; b += 256) s += row_loss[b];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *loss = red[0] / (float)(batch * n_out);
-}
-
-// db[n] = sum over the batch of g[b][n]; one thread per column, fixed order.
-__global__ void k_bias_grad(const float *__restrict__ g, int batch, int n, float *db) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    float s = 0.f;
-    for (int b = 0; b < batch; b++) s += g[(size_t)b * n + c];
-    db[c] = s;
-}
-
-// Copies a (rows x cols_pad) FP32 block into (rows x cols) at dst (drops padding).
-__global__ void k_unpad(const float *__restrict__ src, int rows, int cols_pad, int cols, float *dst) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * cols) return;
-    dst[i] = src[(size_t)(i / cols) * cols_pad + i % cols];
 }
 
 // Master FP32 layer weights (flat, n_out x n_in) -> BF16 Wt (n_out x K pad) and W (K pad x n_out).
@@ -466,8 +484,17 @@ __global__ void k_refresh_bf16(const float *__restrict__ wt, int n_out, int n_in
     W_bf[(size_t)c * n_out + r] = v;
 }
 
+// Adam on the flat parameters, and the BF16 copies of the new weights in both
+// layouts (their padding stays zero).
+struct LayerTab {
+    int64_t woff, boff;  // weights, biases in the flat vector
+    int n_in, n_out, kpad;
+    bf16 *Wt, *W;
+};
 __global__ void k_adam(float *theta, const float *g, float *m, float *v, int64_t n, float lr, float b1, float b2,
-                       float c1, float c2, float eps) {
+                       float c1, float c2, float eps, const LayerTab *tab) {
+    let_next_start();
+    wait_for_previous();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float gi = g[i];
@@ -475,7 +502,16 @@ __global__ void k_adam(float *theta, const float *g, float *m, float *v, int64_t
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    theta[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    const float t = theta[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    theta[i] = t;
+    int l = 0;
+    while (i >= tab[l].boff + tab[l].n_out) l++;
+    const LayerTab &q = tab[l];
+    if (i >= q.boff) return;
+    const int k = (int)(i - q.woff), r = k / q.n_in, c = k - r * q.n_in;
+    const bf16 h = __float2bfloat16_rn(t);
+    q.Wt[(size_t)r * q.kpad + c] = h;
+    q.W[(size_t)c * q.n_out + r] = h;
 }
 
 }  // namespace
@@ -496,7 +532,10 @@ struct lbm_mlp {
     float *y = nullptr, *t = nullptr, *row_loss = nullptr, *losses = nullptr;
     std::vector<float *> gf;              // gradient w.r.t. layer l output (B x nout[l]), fp32
     std::vector<bf16 *> gbf, gT;          // bf16 copy and transpose
-    float *dw = nullptr;                  // padded dWt scratch (max nout x kpad)
+    LayerTab *tab = nullptr;
+    int32_t *ord = nullptr;               // training: order of the rows and losses of a call (grown as needed)
+    float *dl = nullptr;
+    size_t ord_cap = 0, dl_cap = 0;
     float *xd = nullptr, *td = nullptr;   // training set
     int n_data = 0;
     int32_t *idx = nullptr;
@@ -518,6 +557,20 @@ template <class T> cudaError_t dal(lbm_mlp *h, T **p, size_t n) {
     return e;
 }
 
+// a workspace of at least n entries (the stream must not be using the old one)
+template <class T> cudaError_t grow(T **p, size_t *cap, size_t n) {
+    if (n <= *cap) return cudaSuccess;
+    if (*p) cudaFree(*p);
+    *p = nullptr;
+    *cap = 0;
+    void *q = nullptr;
+    const cudaError_t e = cudaMalloc(&q, n * sizeof(T));
+    if (e != cudaSuccess) return e;
+    *p = static_cast<T *>(q);
+    *cap = n;
+    return cudaSuccess;
+}
+
 #define MCK(call)                                                                   \
     do {                                                                            \
         cudaError_t e_ = (call);                                                    \
@@ -527,20 +580,43 @@ template <class T> cudaError_t dal(lbm_mlp *h, T **p, size_t n) {
         }                                                                           \
     } while (0)
 
+// a launch that may start while its predecessor on the stream finishes
+template <class... P, class... A>
+cudaError_t follow(lbm_mlp *h, void (*k)(P...), dim3 grid, int threads, size_t smem, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = h->stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
+// Tile width of a product of mt tiles of rows and N columns: 16 while tiles of
+// 32 would leave SMs idle (the epilogue, whose SiLU divisions take longer than
+// the product, then spreads over twice as many CTAs), else 32.
+int tile_cols(int mt, int N) { return N % 32 == 0 && mt * (N / 32) >= 148 ? 32 : 16; }
+
 template <int EPI> cudaError_t gemm(lbm_mlp *h, const bf16 *A, const bf16 *Bt, int M, int N, int K, const Epi &e) {
-#if LBM_MLP_MMA_SYNC
-    dim3 grid((N + TN - 1) / TN, (M + TM - 1) / TM);
-    k_gemm_nt<EPI><<<grid, 128, 0, h->stream>>>(A, Bt, M, N, K, e);
-#else
-    if (N % 32 == 0) {
-        dim3 grid(N / 32, (M + TC_M - 1) / TC_M);
-        k_gemm_tc<EPI, 32><<<grid, TC_THREADS, 0, h->stream>>>(A, Bt, M, N, K, e, h->err);
-    } else {
-        dim3 grid((N + 15) / 16, (M + TC_M - 1) / TC_M);
-        k_gemm_tc<EPI, 16><<<grid, TC_THREADS, 0, h->stream>>>(A, Bt, M, N, K, e, h->err);
-    }
-#endif
-    return cudaGetLastError();
+    const int mt = (M + TC_M - 1) / TC_M;
+    if (tile_cols(mt, N) == 32)
+        return follow(h, k_gemm_tc<EPI, 32>, dim3(N / 32, mt), TC_THREADS, TC_SMEM, A, Bt, M, N, K, e, h->err);
+    return follow(h, k_gemm_tc<EPI, 16>, dim3(N / 16, mt), TC_THREADS, TC_SMEM, A, Bt, M, N, K, e, h->err);
+}
+
+// the products' shared memory exceeds the 48 KB that need no request
+cudaError_t prepare_products() {
+    const void *k[] = {(const void *)k_gemm_tc<EPI_HIDDEN, 32>, (const void *)k_gemm_tc<EPI_HIDDEN, 16>,
+                       (const void *)k_gemm_tc<EPI_OUT, 32>,    (const void *)k_gemm_tc<EPI_OUT, 16>,
+                       (const void *)k_backward<32>,            (const void *)k_backward<16>};
+    cudaError_t e = cudaSuccess;
+    for (const void *f : k)
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+    return e;
 }
 
 cudaError_t transpose(lbm_mlp *h, const bf16 *in, bf16 *out, int R, int C) {
@@ -558,14 +634,16 @@ cudaError_t refresh(lbm_mlp *h) {
     return cudaGetLastError();
 }
 
-// forward pass from act[0] (already filled, B x 16); output in h->y
-cudaError_t forward(lbm_mlp *h, int B) {
+// forward pass from act[0] (already filled, B x 16); output in h->y; with
+// train, the activations' transposes for the backward pass too
+cudaError_t forward(lbm_mlp *h, int B, bool train) {
     for (int l = 0; l < h->n_layers; l++) {
         Epi e{};
         e.bias = h->theta + h->boff[l];
         if (l < h->n_layers - 1) {
             e.pre = h->pre[l];
             e.out_bf = h->act[l + 1];
+            e.out_t = train ? h->actT[l + 1] : nullptr;
             cudaError_t r = gemm<EPI_HIDDEN>(h, h->act[l], h->Wt[l], B, h->nout[l], h->kpad[l], e);
             if (r != cudaSuccess) return r;
         } else {
@@ -577,30 +655,45 @@ cudaError_t forward(lbm_mlp *h, int B) {
     return cudaSuccess;
 }
 
-// backward pass from gf/gbf[L-1] (gradient w.r.t. the output); fills h->grad
-cudaError_t backward(lbm_mlp *h, int B) {
+// backward pass from gf, gbf and gT of the output layer; fills h->grad and,
+// where loss is given, *loss from h->row_loss
+cudaError_t backward(lbm_mlp *h, int B, float *loss) {
     for (int l = h->n_layers - 1; l >= 0; l--) {
-        const int N = h->nout[l], K = h->kpad[l];
-        k_bias_grad<<<(N + 127) / 128, 128, 0, h->stream>>>(h->gf[l], B, N, h->grad + h->boff[l]);
-        cudaError_t r = transpose(h, h->gbf[l], h->gT[l], B, N);
-        if (r == cudaSuccess) r = transpose(h, h->act[l], h->actT[l], B, K);
-        if (r != cudaSuccess) return r;
-        Epi e{};
-        e.out_f = h->dw;
-        r = gemm<EPI_DW>(h, h->gT[l], h->actT[l], N, K, B, e);
-        if (r != cudaSuccess) return r;
-        const int cnt = N * h->nin[l];
-        k_unpad<<<(cnt + 255) / 256, 256, 0, h->stream>>>(h->dw, N, K, h->nin[l], h->grad + h->woff[l]);
+        Backward q{};
+        q.B = B;
+        q.N = h->nout[l];
+        q.K = h->kpad[l];
+        q.g = h->gbf[l];
+        q.g_t = h->gT[l];
+        q.W = h->W[l];
+        q.in_t = h->actT[l];
+        q.g_f = h->gf[l];
+        q.db = h->grad + h->boff[l];
+        q.dw.out_f = h->grad + h->woff[l];
+        q.dw.n_keep = h->nin[l];
+        const int nt = tile_cols((B + TC_M - 1) / TC_M + (q.N + TC_M - 1) / TC_M, q.K);
+        q.dw_cols = q.K / nt;
+        q.n_dw = q.dw_cols * ((q.N + TC_M - 1) / TC_M);
+        q.n_bias = (q.N + 31) / 32;
         if (l > 0) {
-            Epi d{};
-            d.out_f = h->gf[l - 1];
-            d.out_bf = h->gbf[l - 1];
-            d.pre_in = h->pre[l - 1];
-            r = gemm<EPI_DX>(h, h->gbf[l], h->W[l], B, K, N, d);
-            if (r != cudaSuccess) return r;
+            q.dx.out_f = h->gf[l - 1];
+            q.dx.out_bf = h->gbf[l - 1];
+            q.dx.out_t = h->gT[l - 1];
+            q.dx.pre_in = h->pre[l - 1];
+            q.dx_cols = q.dw_cols;
+            q.n_dx = q.dx_cols * ((B + TC_M - 1) / TC_M);
         }
+        const bool with_loss = loss && l == h->n_layers - 1;
+        if (with_loss) {
+            q.row_loss = h->row_loss;
+            q.loss = loss;
+            q.n_out = h->n_out;
+        }
+        const int grid = q.n_dx + q.n_dw + q.n_bias + (with_loss ? 1 : 0);
+        const cudaError_t e = follow(h, nt == 32 ? k_backward<32> : k_backward<16>, dim3(grid), TC_THREADS, TC_SMEM, q, h->err);
+        if (e != cudaSuccess) return e;
     }
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 lbm_status load_input(lbm_mlp *h, const float *x, int B) {
@@ -653,7 +746,6 @@ lbm_status lbm_mlp_create(int n_in, int hidden, int n_hidden, int n_out, int max
         h->own_stream = true;
     }
     int64_t off = 0;
-    int maxw = 0;
     for (int l = 0; l < h->n_layers; l++) {
         const int ni = l == 0 ? n_in : hidden, no = l == h->n_layers - 1 ? n_out : hidden;
         h->nin.push_back(ni);
@@ -663,12 +755,11 @@ lbm_status lbm_mlp_create(int n_in, int hidden, int n_hidden, int n_out, int max
         off += (int64_t)ni * no;
         h->boff.push_back(off);
         off += no;
-        maxw = std::max(maxw, no * h->kpad[l]);
     }
     h->np = off;
     bool ok = dal(h, &h->theta, off) == cudaSuccess && dal(h, &h->grad, off) == cudaSuccess &&
               dal(h, &h->m, off) == cudaSuccess && dal(h, &h->v, off) == cudaSuccess &&
-              dal(h, &h->dw, maxw) == cudaSuccess && dal(h, &h->y, (size_t)max_batch * n_out) == cudaSuccess &&
+              dal(h, &h->tab, h->n_layers) == cudaSuccess && dal(h, &h->y, (size_t)max_batch * n_out) == cudaSuccess &&
               dal(h, &h->t, (size_t)max_batch * n_out) == cudaSuccess &&
               dal(h, &h->row_loss, max_batch) == cudaSuccess && dal(h, &h->idx, max_batch) == cudaSuccess &&
               dal(h, &h->err, 1) == cudaSuccess;
@@ -694,6 +785,14 @@ lbm_status lbm_mlp_create(int n_in, int hidden, int n_hidden, int n_out, int max
     if (!ok) {
         lbm_mlp_destroy(h);
         return LBM_ERR_OOM;
+    }
+    std::vector<LayerTab> tab;
+    for (int l = 0; l < h->n_layers; l++)
+        tab.push_back({h->woff[l], h->boff[l], h->nin[l], h->nout[l], h->kpad[l], h->Wt[l], h->W[l]});
+    if (cudaMemcpy(h->tab, tab.data(), tab.size() * sizeof(LayerTab), cudaMemcpyHostToDevice) != cudaSuccess ||
+        prepare_products() != cudaSuccess) {
+        lbm_mlp_destroy(h);
+        return LBM_ERR_CUDA;
     }
     *out = h;
     return LBM_OK;
@@ -728,7 +827,7 @@ lbm_status lbm_mlp_forward(lbm_mlp *h, const float *x, int B, float *y) {
     MCK(cudaSetDevice(h->device));
     lbm_status s = load_input(h, x, B);
     if (s != LBM_OK) return s;
-    MCK(forward(h, B));
+    MCK(forward(h, B, false));
     MCK(cudaMemcpyAsync(y, h->y, (size_t)B * h->n_out * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
     MCK(cudaStreamSynchronize(h->stream));
     return check_err(h);
@@ -739,14 +838,16 @@ lbm_status lbm_mlp_grad(lbm_mlp *h, const float *x, const float *dy, int B, floa
     MCK(cudaSetDevice(h->device));
     lbm_status s = load_input(h, x, B);
     if (s != LBM_OK) return s;
-    MCK(forward(h, B));
+    MCK(forward(h, B, true));
     const int L = h->n_layers - 1;
     const size_t n = (size_t)B * h->n_out;
     std::vector<bf16> db(n);
     for (size_t i = 0; i < n; i++) db[i] = __float2bfloat16_rn(dy[i]);
     MCK(cudaMemcpyAsync(h->gf[L], dy, n * sizeof(float), cudaMemcpyHostToDevice, h->stream));
     MCK(cudaMemcpyAsync(h->gbf[L], db.data(), n * sizeof(bf16), cudaMemcpyHostToDevice, h->stream));
-    MCK(backward(h, B));
+    MCK(transpose(h, h->gbf[L], h->gT[L], B, h->n_out));
+    MCK(transpose(h, h->act[0], h->actT[0], B, K0));
+    MCK(backward(h, B, nullptr));
     MCK(cudaMemcpyAsync(g, h->grad, h->np * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
     MCK(cudaStreamSynchronize(h->stream));
     return check_err(h);
@@ -772,35 +873,33 @@ lbm_status lbm_mlp_train(lbm_mlp *h, const int32_t *order, int n_steps, int B, f
     for (int64_t i = 0; i < (int64_t)n_steps * B; i++)
         if (order[i] < 0 || order[i] >= h->n_data) return LBM_ERR_ARG;
     MCK(cudaSetDevice(h->device));
-    int32_t *ord = nullptr;
-    float *dl = nullptr;
-    MCK(cudaMalloc(&ord, (size_t)n_steps * B * sizeof(int32_t)));
-    MCK(cudaMalloc(&dl, (size_t)n_steps * sizeof(float)));
-    MCK(cudaMemcpy(ord, order, (size_t)n_steps * B * sizeof(int32_t), cudaMemcpyHostToDevice));
+    MCK(grow(&h->ord, &h->ord_cap, (size_t)n_steps * B));
+    MCK(grow(&h->dl, &h->dl_cap, (size_t)n_steps));
+    int32_t *ord = h->ord;
+    float *dl = h->dl;
+    MCK(cudaMemcpyAsync(ord, order, (size_t)n_steps * B * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream));
     const int L = h->n_layers - 1;
     const float b1 = 0.9f, b2 = 0.999f;
     cudaError_t e = cudaSuccess;
     for (int s = 0; s < n_steps && e == cudaSuccess; s++) {
-        k_gather_batch<<<B, 64, 0, h->stream>>>(h->xd, h->td, ord + (size_t)s * B, B, h->n_in, h->n_out, h->act[0], h->t);
-        e = forward(h, B);
-        if (e != cudaSuccess) break;
-        k_mse_grad<<<B, 64, 0, h->stream>>>(h->y, h->t, B, h->n_out, h->gf[L], h->gbf[L], h->row_loss);
-        k_sum_loss<<<1, 256, 0, h->stream>>>(h->row_loss, B, h->n_out, dl + s);
-        e = backward(h, B);
+        e = follow(h, k_gather_batch, dim3(B), 64, 0, h->xd, h->td, ord + (size_t)s * B, B, h->n_in, h->n_out, h->act[0],
+                   h->actT[0], h->t);
+        if (e == cudaSuccess) e = forward(h, B, true);
+        if (e == cudaSuccess)
+            e = follow(h, k_mse_grad, dim3(B), 64, 0, h->y, h->t, B, h->n_out, h->gf[L], h->gbf[L], h->gT[L], h->row_loss);
+        if (e == cudaSuccess) e = backward(h, B, dl + s);
         if (e != cudaSuccess) break;
         h->adam_steps++;
         const float c1 = 1.f - powf(b1, (float)h->adam_steps), c2 = 1.f - powf(b2, (float)h->adam_steps);
-        k_adam<<<(int)((h->np + 255) / 256), 256, 0, h->stream>>>(h->theta, h->grad, h->m, h->v, h->np, lr, b1, b2, c1,
-                                                                    c2, 1e-8f);
-        e = refresh(h);
+        e = follow(h, k_adam, dim3((unsigned)((h->np + 255) / 256)), 256, 0, h->theta, h->grad, h->m, h->v, h->np, lr, b1,
+                   b2, c1, c2, 1e-8f, h->tab);
     }
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess && losses)
         e = cudaMemcpyAsync(losses, dl, (size_t)n_steps * sizeof(float), cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    cudaFree(ord);
-    cudaFree(dl);
+    const cudaError_t es = cudaStreamSynchronize(h->stream);  // also before the host's arrays may go
     MCK(e);
+    MCK(es);
     return check_err(h);
 }
 
@@ -809,6 +908,8 @@ void lbm_mlp_destroy(lbm_mlp *h) {
     cudaSetDevice(h->device);
     if (h->stream) cudaStreamSynchronize(h->stream);
     for (void *p : h->allocs) cudaFree(p);
+    if (h->ord) cudaFree(h->ord);
+    if (h->dl) cudaFree(h->dl);
     if (h->xd) cudaFree(h->xd);
     if (h->td) cudaFree(h->td);
     if (h->own_stream) cudaStreamDestroy(h->stream);

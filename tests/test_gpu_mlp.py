@@ -103,3 +103,36 @@ def test_ragged_batches_match_oracle(MLP, batch):
     g = net.grad(x, dy).astype(np.float64)
     go = omlp.grad_from_output(theta_b, shapes, bf16_round(x), bf16_round(dy))
     assert g @ go / (np.linalg.norm(g) * np.linalg.norm(go)) > 0.999
+
+
+@pytest.mark.parametrize("n_in,hidden,n_hidden,batch", [(16, 64, 1, 16), (6, 128, 2, 2064), (1, 320, 3, 144)])
+def test_training_step_follows_the_gradient(MLP, n_in, hidden, n_hidden, batch):
+    # one Adam step from zero moments moves every parameter by lr in the
+    # direction of -gradient (wherever the gradient is not tiny), for the tile
+    # widths 16 and 32, ragged row tiles, an input layer with and without
+    # padding, and biases summed over whole and partial groups of rows; the loss
+    # is the mean squared error of the forward pass
+    rng = np.random.default_rng(11)
+    n_out, lr = 48, 1e-3
+    shapes = omlp.layer_shapes(n_in, hidden, n_hidden, n_out)
+    theta = np.concatenate([np.concatenate([rng.standard_normal(r * c) / np.sqrt(c), 0.1 * rng.standard_normal(r)])
+                            for r, c in shapes]).astype(np.float32)
+    net = MLP(n_in, hidden, n_hidden, n_out, max_batch=(batch + 63) // 64 * 64)
+    net.set_params(theta)
+    x = rng.standard_normal((batch, n_in)).astype(np.float32)
+    t = rng.standard_normal((batch, n_out)).astype(np.float32)
+    net.set_data(x, t)
+    y = net.forward(x)
+    g = net.grad(x, (2.0 / (batch * n_out)) * (y - t))
+    order = np.arange(batch, dtype=np.int32)
+    loss = net.train(order, batch, lr)
+    assert loss.size == 1 and abs(loss[0] - np.mean((y - t).astype(np.float64) ** 2)) < 1e-5 * loss[0]
+    moved = net.params().astype(np.float64) - theta
+    big = np.abs(g) > 1e-2 * np.abs(g).max()
+    assert big.sum() > 100
+    # lr g / (|g| + eps) up to the FP32 rounding of theta and of the two corrections
+    assert np.abs(moved[big] + lr * np.sign(g[big])).max() < 1e-3 * lr + 2.0 ** -23 * np.abs(theta).max()
+    # the BF16 copies in use are those of the new parameters
+    fresh = MLP(n_in, hidden, n_hidden, n_out, max_batch=(batch + 63) // 64 * 64)
+    fresh.set_params(net.params())
+    assert np.array_equal(fresh.forward(x), net.forward(x))
