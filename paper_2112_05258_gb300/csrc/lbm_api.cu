@@ -271,7 +271,7 @@ lbm_status launch_step_slabs(lbm_handle *h) {
     }
     CK(h, cudaStreamWaitEvent(h->stream, h->ev_node[0], 0));
     CK(h, cudaStreamWaitEvent(h->stream, h->ev_sc[0], 0));
-    CK(h, launch_boundary(h->prec, fout, h->kp, h->bp, h->stream));
+    CK(h, launch_boundary(h->prec, fout, h->kp, h->bp, BcIo{}, h->stream));
     h->parity ^= 1;
     return LBM_OK;
 }
@@ -280,7 +280,7 @@ lbm_status launch_step_slabs(lbm_handle *h) {
 // previous step (next = true there); next: issue the next step's band
 // velocities beside this step's boundary kernels (graph capture only; the
 // last step of a graph leaves them to the next graph's first step).
-lbm_status launch_step(lbm_handle *h, bool timed, bool band_done = false, bool next = false) {
+lbm_status launch_step(lbm_handle *h, bool timed, bool band_done = false, bool next = false, const BcIo &io = BcIo{}) {
     if (h->n_slab && !timed) return launch_step_slabs(h);
     void *fin = h->f[h->parity], *fout = h->f[1 - h->parity];
     if (h->ibp.n_nodes) CK(h, launch_ib(h->prec, fin, h->kp, h->ibp, h->stream, !band_done));
@@ -304,7 +304,8 @@ lbm_status launch_step(lbm_handle *h, bool timed, bool band_done = false, bool n
     // starts on the lines the step before finished on (the band-velocity
     // kernel takes that role when there are wall nodes)
     const int desc = h->ibp.n_nodes ? 0 : h->parity;
-    CK(h, launch_stream_collide(h->prec, fin, fout, h->kp, h->block, h->variant, h->stream, desc));
+    CK(h, launch_stream_collide(h->prec, fin, fout, h->kp, h->block, h->variant, h->stream, desc, 0, -1, 1,
+                                h->bp.cluster && !timed));
     if (timed) {
         CK(h, cudaEventRecord(e1, h->stream));
         h->timed_launches++;
@@ -317,14 +318,14 @@ lbm_status launch_step(lbm_handle *h, bool timed, bool band_done = false, bool n
         ib.band = h->band_ind;
         CK(h, launch_band_moments(h->prec, fout, h->kp, ib, 0, h->n_band_ind, h->s_band));
         CK(h, cudaEventRecord(h->ev_oband, h->s_band));
-        CK(h, launch_boundary(h->prec, fout, h->kp, h->bp, h->s_bc));
+        CK(h, launch_boundary(h->prec, fout, h->kp, h->bp, BcIo{}, h->s_bc));
         ib.band = h->band_dep;
         CK(h, launch_band_moments(h->prec, fout, h->kp, ib, 0, h->n_band_dep, h->s_bc));
         CK(h, cudaEventRecord(h->ev_obc, h->s_bc));
         CK(h, cudaStreamWaitEvent(h->stream, h->ev_oband, 0));
         CK(h, cudaStreamWaitEvent(h->stream, h->ev_obc, 0));
     } else {
-        CK(h, launch_boundary(h->prec, fout, h->kp, h->bp, h->stream));
+        CK(h, launch_boundary(h->prec, fout, h->kp, h->bp, io, h->stream));
     }
     h->parity ^= 1;
     return LBM_OK;
@@ -371,11 +372,15 @@ lbm_status ensure_graph1(lbm_handle *h) {
     return LBM_OK;
 }
 
-// One step of lbm_step_io: the params of step *io_cursor, the step, the
-// state rows written after it.  band_done / next as in launch_step.
+// One step of lbm_step_io: the params of its row, the step, the state rows
+// written after it (rows count from step *io_cursor in the one-launch boundary
+// kernel; otherwise *io_cursor counts the call's steps).  band_done / next as in launch_step.
 lbm_status launch_io_step(lbm_handle *h, const double *params_dev, int np, int b, double *states_dev, int inst,
                           bool timed, bool band_done, bool next) {
     const InstParam &ip = h->L.inst[inst];
+    if (h->bp.cluster)  // the boundary kernel reads and writes the host arrays itself
+        return launch_step(h, timed, band_done, next,
+                           BcIo{params_dev, states_dev, h->bc_par, h->io_cursor, np, b, ip.bc_first, ip.n_bc});
     CK(h, launch_io_params(params_dev, np, &h->bc_par[b], h->io_cursor, h->stream));
     lbm_status st = launch_step(h, timed, band_done, next);
     if (st != LBM_OK) return st;
@@ -767,6 +772,18 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
         h->bp.step_in_reduce = (int)L.app_bc.size() > 4 * sms ? 1 : 0;
     }
     h->bp.result = h->bc_result;
+    h->bp.cluster = h->bp.wide = 0;
+    if (L.ib_dA.empty()) {
+        // one launch for the boundary work: blocks enough that a thread has one
+        // link (at most 8 blocks of 512 per boundary), as long as all clusters
+        // run at once; the figures for the line stand at k_boundary
+        int links = 0;
+        for (auto &b : L.bc) links = std::max(links, b.n_links);
+        h->bp.wide = links > 4 * 256;
+        int c = 1;
+        while (c < 8 && c * (h->bp.wide ? 512 : 256) < links) c *= 2;
+        if (h->prec != LBM_F64 && links > 0 && links <= 4096 && c * (int)L.bc.size() <= 300) h->bp.cluster = c;
+    }
     h->bp.n_red_blocks = (int)L.red_bc.size();
     h->bp.n_app_blocks = (int)L.app_bc.size();
     h->bp.red_bc = h->red_bc;
@@ -986,7 +1003,8 @@ lbm_status lbm_step_io(lbm_handle *h, int inst, int bc, int64_t n, const double 
         return LBM_OK;
     }
     if (!h->io_cursor) CK(h, dalloc(h, &h->io_cursor, 1));
-    CK(h, cudaMemsetAsync(h->io_cursor, 0, sizeof(long long), h->stream));
+    if (h->bp.cluster) CK(h, launch_io_base(h->step_dev, h->io_cursor, h->stream));
+    else CK(h, cudaMemsetAsync(h->io_cursor, 0, sizeof(long long), h->stream));
     if (h->timing) {
         for (int64_t k = 0; k < n; k++) {
             lbm_status s = launch_io_step(h, pdev, np, b, sdev, inst, true, false, false);
@@ -1444,7 +1462,7 @@ lbm_status lbm_get_info(lbm_handle *h, lbm_info_t *info) {
     } else {
         n = (L.n_stored > 0) + (L.ib_dA.empty() ? 0 : (L.band.empty() ? 0 : 1) + 1 + (L.fil_start.empty() ? 0 : 1));
     }
-    info->launches_per_step = n + (L.bc.empty() ? 0 : 2);
+    info->launches_per_step = n + (L.bc.empty() ? 0 : h->bp.cluster ? 1 : 2);
     info->launches_first_step = info->launches_per_step;
     if (h->overlap)  // band velocities as the two lists (an empty list launches nothing)
         info->launches_per_step += (h->n_band_ind > 0) + (h->n_band_dep > 0) - 1;

@@ -37,7 +37,7 @@
 
 #include "../../include/lbm_axi.h"
 #include "lbm_device.cuh"
-#include "lbm_zero_d.cuh"
+#include "lbm_boundary.cuh"
 
 namespace lbm {
 namespace axi {
@@ -431,7 +431,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Pa
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ __align__(16) uint8_t smem[];
-    __shared__ double sQ[THREADS], sP[THREADS], s_part[2 * AXI_MAX_RED], s_cos, s_sin, s_p0_rc, s_inv_cv, s_dcv;
+    __shared__ double sQ[THREADS], sP[THREADS], s_part[2 * AXI_MAX_RED], s_cos, s_sin;
+    __shared__ Ahead s_a;
     __shared__ double s_area, s_third, s_S;
     __shared__ BcParam s_P;
     __shared__ BcState s_st;
@@ -509,14 +510,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Pa
                 unode[a] = (R)((double)P.sign * (pr[0] + pr[1] * cosp - pr[2] * sinp));
             }
         } else if (ta == 0) {
-            if (P.kind == BC_RCR) s_p0_rc = s_st.Pw / (P.par[2] * P.par[1]);
-            if (P.kind == BC_LV) {
-                const double E = q.etab[2 * (P.etab_off + (int)(t % P.period))];
-                const double Ed = q.etab[2 * (P.etab_off + (int)(t % P.period)) + 1];
-                const double Cv = 1.0 / E;
-                s_dcv = -Ed / (E * E);
-                s_inv_cv = 1.0 / Cv;
-            }
+            ahead_terms(P, s_st, t, q.etab, &s_a);
         }
     };
     if (owner && ta >= 0) ahead(0);
@@ -561,14 +555,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Pa
                 constexpr int CH = THREADS / BC2;
                 const int w = tid >> 5, ch = k0 / BC2 + (w & (CH - 1));
                 if (w < 2 * CH && ch < n_red) {
-                    const double *v = (w < CH ? sQ : sP) + (w & (CH - 1)) * BC2 + (tid & 31);
-                    double a[4];
-#pragma unroll
-                    for (int h = 0; h < 4; h++) a[h] = v[32 * h] + v[32 * (h + 4)];
-                    a[0] = (a[0] + a[2]) + (a[1] + a[3]);
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) a[0] += __shfl_down_sync(0xffffffffu, a[0], o);
-                    if ((tid & 31) == 0) s_part[2 * ch + (w < CH ? 0 : 1)] = a[0];
+                    const double a = tree_256((w < CH ? sQ : sP) + (w & (CH - 1)) * BC2);
+                    if ((tid & 31) == 0) s_part[2 * ch + (w < CH ? 0 : 1)] = a;
                 }
                 __syncthreads();
             }
@@ -581,59 +569,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Pa
             if (tid < 32) {
                 double a = 0.0;  // lane 0 the flow, lane 1 the pressure: the partials in their fixed order
                 for (int k = 0; k < n_red; k++) a += s_part[2 * k + (tid & 1)];
-                const int order = (int)P.par[4];
-                if ((P.kind == BC_RCR || P.kind == BC_LV) && (order == 2 || order == 4)) {
-                    const double Ps = __shfl_sync(0xffffffffu, a, 1);
-                    if (tid == 0) {
-                        const BcState old = s_st;
-                        double Sm;
-                        s_st = zero_d_step(P, old, a, s_third + Ps, s_area, t, q.etab, &s_ptype, &s_closed, &Sm);
-                        s_S = Sm;
-                        s_3p = (R)(3.0 * s_st.Pstar_gauge);
-                    }
-                } else {  // zero_d_step with forward Euler, its flow-independent parts taken above
-                    const double mean = ((tid & 1) ? s_third + a : a) / s_area;
-                    const double Pbar = __shfl_sync(0xffffffffu, mean, 1);
-                    if (tid == 0) {
-                        BcState st = s_st;
-                        st.Q = a;
-                        st.Qu = P.q_scale ? mean : a;
-                        st.Pbar = Pbar;
-                        int ptype = 1, closed = 0;
-                        double Sm = 0.0;
-                        if (P.kind == BC_RCR) {
-                            const double Qout = -st.Qu;
-                            const double Pw = s_st.Pw + (Qout / P.par[1] - s_p0_rc);
-                            st.Pw = Pw;
-                            st.Pstar_gauge = Pw + P.par[0] * Qout;
-                        } else if (P.kind == BC_PRESSURE) {
-                            st.Pstar_gauge = P.par[0];
-                        } else if (P.kind == BC_LV) {
-                            const double Qin = (st.valve_open != 0.0) ? st.Qu : 0.0;
-                            double Pv = st.Pv - s_inv_cv * (s_dcv * st.Pv + Qin);
-                            if (st.valve_open != 0.0) {
-                                if (st.Qu < 0.0) {
-                                    st.valve_open = 0.0;
-                                    st.Td = (double)t;
-                                    closed = 1;
-                                }
-                            } else {
-                                if (Pv < P.par[1]) Pv = P.par[1];
-                                if (Pv > st.Pbar - 1.0 / 3.0) st.valve_open = 1.0;
-                            }
-                            st.Pv = Pv;
-                            st.Pstar_gauge = Pv;
-                            ptype = st.valve_open != 0.0;
-                            if (!ptype) Sm = smooth_to_zero((double)(t + 1), st.Td, P.par[2]);
-                        } else {
-                            ptype = 0;
-                        }
-                        s_st = st;
-                        s_ptype = ptype;
-                        s_closed = closed;
-                        s_S = Sm;
-                        s_3p = (R)(3.0 * st.Pstar_gauge);
-                    }
+                const double mean = ((tid & 1) ? s_third + a : a) / s_area;
+                const double Ps = __shfl_sync(0xffffffffu, a, 1), Pbar = __shfl_sync(0xffffffffu, mean, 1);
+                if (tid == 0) {
+                    const BcState old = s_st;
+                    double Sm;
+                    s_st = boundary_euler(P)
+                               ? zero_d_euler(P, old, s_a, a, mean, Pbar, t, &s_ptype, &s_closed, &Sm)
+                               : zero_d_step(P, old, a, s_third + Ps, s_area, t, q.etab, &s_ptype, &s_closed, &Sm);
+                    s_S = Sm;
+                    s_3p = (R)(3.0 * s_st.Pstar_gauge);
                 }
             }
             __syncthreads();

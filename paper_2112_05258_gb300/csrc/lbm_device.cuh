@@ -48,6 +48,28 @@ template <> __device__ __forceinline__ double omega_of<double>(const KParams &p,
 
 template <class S> static S *as(void *p) { return static_cast<S *>(p); }
 
+// Programmatic dependent launch: a kernel lets its successor on the stream start
+// its set-up, and waits for its predecessor's end before it touches what that
+// one writes.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// a launch that may start before its predecessor on the stream has finished (its
+// kernel calls wait_for_previous)
+template <class... P, class... A>
+cudaError_t launch_early(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s, const A &...args) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
 #define DISPATCH(prec, CALL)                                   \
     switch (prec) {                                            \
     case 0: { using S = float; CALL; } break;                  \

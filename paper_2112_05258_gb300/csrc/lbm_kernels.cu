@@ -8,6 +8,7 @@
 //                     Section 2.2.1)
 //   k_bc_apply        the ghost populations of Eq. Non-equilibrium3 (per
 //                     link, in the compute type)
+//   k_boundary        both in one launch, a cluster of blocks per boundary
 //   k_gather          read-out of f(t_n), P and j for the host
 //   k_fields_box      FP32 read-out of P and j into box-order device arrays
 //   k_wall_shear      wall shear stress at the fluid cells next to rigid walls
@@ -20,8 +21,10 @@
 // steps is the post-collision field f*(t_n) with the ghost populations of
 // the 0D boundary nodes for t_{n+1} already in their slots, so one step is:
 // (immersed boundary) -> k_stream_collide -> k_bc_reduce -> k_bc_apply.
-#include "lbm_device.cuh"
+#include <cooperative_groups.h>
+
 #include "lbm_boundary.cuh"
+#include "lbm_device.cuh"
 
 namespace lbm {
 
@@ -173,6 +176,165 @@ __global__ void __launch_bounds__(BC_CHUNK) k_bc_apply(S *__restrict__ f, KParam
     const R dfeq = ghost_change<R>(P, r, i, vf, sdf, pr, v0o,
                                    P.kind == BC_LV ? q.v0 + 3 * (size_t)(P.xf_off + q.lk_xfi[P.link_off + L]) : nullptr);
     Storage<S>::st(f + pidx(i, (uint32_t)cb, (uint32_t)N), post + dfeq);
+}
+
+// The whole boundary work of a step in one launch (lattices without wall nodes):
+// one cluster of blocks per boundary.  The blocks sum their chunks of 256
+// first-layer cells (the tree of k_bc_reduce); after a cluster barrier the
+// first block adds the partials, takes the 0D step and hands the result to the
+// others' shared memory; after another every block writes its links' ghosts,
+// whose inputs it has read beside all this.  Per-step 0D input and output
+// (lbm_step_io) is part of it: the params come straight from the host's memory
+// while the sums run, the state rows go there after the ghosts.  Same
+// expressions and orders as k_bc_reduce and k_bc_apply, the same bits.
+// Bound by latency (two cluster barriers, the trees, FP64 divisions of 700
+// cycles).  One launch and its start hidden behind stream-collide's end: tube
+// of 172k cells 14.5 -> 12.4 us per step (FP16 14.2 -> 12.4), 20.1 -> 14.6 with
+// per-step 0D input and output (three launches and two of one warp before),
+// 64 tubes of 14k cells 36.6 -> 30.1.  A boundary of more links than its blocks
+// have threads (12.5 -> 13.0 us at 6,100 links), FP64 (whose ghosts need the FP64
+// pipes of many SMs: 25 -> 33 us) and batches with more clusters than SMs
+// take at once (96 uneven tubes 528 -> 617 us) keep the two kernels.
+template <class S, int BS>
+__global__ void __launch_bounds__(BS) k_boundary(S *__restrict__ f, KParams p, BcKParams q, BcIo io) {
+    using R = typename Storage<S>::R;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ double sQ[BS], sP[BS], s_area, s_third, s_cos, s_sin;
+    __shared__ BcParam s_P;
+    __shared__ BcState s_st;
+    __shared__ BcStepResult s_r;
+    __shared__ Ahead s_a;
+    __shared__ int s_euler;
+    cluster.barrier_arrive();  // waited for before the first block writes into the others
+    let_next_start();
+    const int CL = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), b = blockIdx.x / CL;
+    const int tid = threadIdx.x;
+    const size_t N = (size_t)p.n;
+    const R *aux = static_cast<const R *>(p.aux);
+    for (int k = tid; k < (int)(sizeof(BcParam) / 4); k += BS)
+        reinterpret_cast<int *>(&s_P)[k] = reinterpret_cast<const int *>(q.par + b)[k];
+    wait_for_previous();  // stream-collide of this step
+    const long long n = *p.step;
+    const bool io_in = rank == 0 && io.params && b == io.b;
+    __syncthreads();
+    if (io_in && tid < io.np) {
+        const double v = __ldcv(io.params + (n - *io.base) * io.np + tid);
+        s_P.par[tid] = v;
+        io.par[b].par[tid] = v;
+    }
+    if (io_in) __syncthreads();
+    const BcParam &P = s_P;
+    // the thread's first link: read before the sums, used after the 0D step
+    struct Link {
+        int cb, cf, i;
+        R vf[3], sd, post;
+        double pr[3], v0[3];
+    };
+    auto load_link = [&](int L, Link &k) {
+        k.cb = q.lk_xb[P.link_off + L];
+        k.cf = q.lk_xf[P.link_off + L];
+        k.i = q.lk_i[P.link_off + L];
+        forced_velocity<R>(p, k.cf, k.vf);
+        k.sd = aux[k.cf];
+        k.post = Storage<S>::ld(f + pidx(k.i, (uint32_t)k.cf, (uint32_t)N));
+        if (P.kind == BC_VELOCITY) {
+            const double *prof = q.profile + 3 * (size_t)(P.node_off + q.lk_node[P.link_off + L]);
+            k.pr[0] = prof[0];
+            k.pr[1] = prof[1];
+            k.pr[2] = prof[2];
+        } else if (P.kind == BC_LV) {
+            const double *v0 = q.v0 + 3 * (size_t)(P.xf_off + q.lk_xfi[P.link_off + L]);
+            k.v0[0] = v0[0];
+            k.v0[1] = v0[1];
+            k.v0[2] = v0[2];
+        }
+    };
+    const int L0 = rank * BS + tid;
+    Link first;
+    if (L0 < P.n_links) load_link(L0, first);
+    if (rank == 0) {  // beside the sums, on warps of their own
+        if (P.kind == BC_VELOCITY) {
+            const double wt = P.par[0] * (double)(n + 1);
+            if (tid == BS - 32) s_cos = cos(wt);
+            if (tid == BS - 64) s_sin = sin(wt);
+        } else if (tid == BS - 32) {
+            const BcState st = q.state[(size_t)(n & 1) * q.n_bc_total + b];
+            ahead_terms(P, st, n, q.etab, &s_a);
+        }
+        if (tid == BS - 96) s_st = q.state[(size_t)(n & 1) * q.n_bc_total + b];
+        if (tid == BS - 128) {
+            s_area = (double)P.n_xf;
+            s_third = (double)P.n_xf / 3.0;
+            s_euler = boundary_euler(P);
+        }
+    }
+    for (int k0 = rank * BS; k0 < P.n_red * BC_CHUNK; k0 += CL * BS) {
+        const int a = k0 + tid;
+        double Q = 0.0, Ps = 0.0;
+        if (a < P.n_xf) {
+            const int cf = q.xf[P.xf_off + a];
+            const R sd = aux[cf];
+            Q = (double)((R)P.sign * aux[(size_t)(1 + P.axis) * N + cf] / (R(1) + sd));
+            Ps = (double)(sd / R(3));
+        }
+        sQ[tid] = Q;
+        sP[tid] = Ps;
+        __syncthreads();
+        constexpr int CH = BS / BC_CHUNK;
+        const int w = tid >> 5, ch = k0 / BC_CHUNK + (w & (CH - 1));
+        if (w < 2 * CH && ch < P.n_red) {  // one warp per quantity and chunk
+            const double t = tree_256((w < CH ? sQ : sP) + (w & (CH - 1)) * BC_CHUNK);
+            if ((tid & 31) == 0) q.partial[2 * (P.red_off + ch) + (w < CH ? 0 : 1)] = t;
+        }
+        __syncthreads();
+    }
+    __syncwarp();
+    cluster.barrier_wait();
+    cluster.sync();  // the partials are visible to the cluster
+    if (rank == 0) {
+        if (tid < 32) {
+            const double a = sum_partials_pair(q.partial + 2 * P.red_off, P.n_red);
+            const double mean = ((tid & 1) ? s_third + a : a) / s_area;
+            const double Ps = __shfl_sync(0xffffffffu, a, 1), Pbar = __shfl_sync(0xffffffffu, mean, 1);
+            if (tid == 0) {
+                BcStepResult r;
+                const BcState old = s_st;
+                s_st = s_euler ? zero_d_euler(P, old, s_a, a, mean, Pbar, n, &r.ptype, &r.closed, &r.S)
+                               : zero_d_step(P, old, a, s_third + Ps, s_area, n, q.etab, &r.ptype, &r.closed, &r.S);
+                r.Pg = s_st.Pstar_gauge;
+                r.cosp = s_cos;
+                r.sinp = s_sin;
+                r.pad0 = r.pad1 = 0;
+                s_r = r;
+            }
+            __syncwarp();
+            constexpr int W = (int)(sizeof(BcStepResult) / 8);
+            for (int k = tid; k < W * (CL - 1); k += 32)
+                reinterpret_cast<unsigned long long *>(cluster.map_shared_rank(&s_r, 1 + k / W))[k % W] =
+                    reinterpret_cast<const unsigned long long *>(&s_r)[k % W];
+        }
+    }
+    __syncwarp();
+    cluster.sync();  // the result is in every block's shared memory
+    const BcStepResult r = s_r;
+    for (int L = L0; L < P.n_links; L += CL * BS) {
+        if (L != L0) load_link(L, first);
+        const R d = ghost_change<R>(P, r, first.i, first.vf, first.sd, first.pr, first.v0,
+                                    P.kind == BC_LV ? q.v0 + 3 * (size_t)(P.xf_off + q.lk_xfi[P.link_off + L]) : nullptr);
+        Storage<S>::st(f + pidx(first.i, (uint32_t)first.cb, (uint32_t)N), first.post + d);
+    }
+    if (rank == 0 && tid == BS - 32) {  // the state of t_{n+1} and the waveform row, as bc_step stores them
+        const BcState st = s_st;
+        q.state[(size_t)((n + 1) & 1) * q.n_bc_total + b] = st;
+        double *w = q.wave + ((size_t)(n % q.wave_cap) * q.n_bc_total + b) * 4;
+        w[0] = st.Qu;
+        w[1] = st.Pbar - 1.0 / 3.0;
+        w[2] = (P.kind == BC_RCR) ? st.Pw : (P.kind == BC_LV ? st.Pv : st.Pstar_gauge);
+        w[3] = st.valve_open;
+        if (io.states && b >= io.b0 && b < io.b0 + io.nb)
+            state_row(st, P, q.etab, n + 1, io.states + 8 * ((size_t)(n - *io.base) * io.nb + (b - io.b0)));
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -368,8 +530,33 @@ __global__ void k_cycle_change(BcKParams q, const int *bc_first, const int *n_bc
 // ---------------------------------------------------------------------------
 // launchers
 
-cudaError_t launch_boundary(int prec, void *f, const KParams &p, const BcKParams &q, cudaStream_t s) {
+template <class S, int BS>
+static cudaError_t boundary_in_one(void *f, const KParams &p, const BcKParams &q, const BcIo &io, cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {(unsigned)q.cluster, 1, 1};
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_early
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)(q.n_bc_total * q.cluster));
+    cfg.blockDim = dim3(BS);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, k_boundary<S, BS>, as<S>(f), p, q, io);
+}
+
+cudaError_t launch_boundary(int prec, void *f, const KParams &p, const BcKParams &q, const BcIo &io, cudaStream_t s) {
     if (q.n_bc_total == 0) return cudaSuccess;
+    if (q.cluster) {
+        cudaError_t e = cudaSuccess;
+        if (q.wide) {
+            DISPATCH(prec, (e = boundary_in_one<S, 512>(f, p, q, io, s)));
+        } else {
+            DISPATCH(prec, (e = boundary_in_one<S, 256>(f, p, q, io, s)));
+        }
+        return e;
+    }
     if (prec == 3) k_bc_reduce<double><<<q.n_red_blocks, BC_CHUNK, 0, s>>>(p, q);
     else k_bc_reduce<float><<<q.n_red_blocks, BC_CHUNK, 0, s>>>(p, q);
     if (q.step_in_reduce) {
@@ -421,6 +608,14 @@ __global__ void k_io_state(const BcState *__restrict__ st, const BcParam *__rest
                   out8 + 8 * ((size_t)c * nb + k));
     __syncthreads();
     if (threadIdx.x == 0) *cursor = c + 1;
+}
+
+// the step count after the steps so far: the first row of lbm_step_io's arrays
+__global__ void k_io_base(const long long *step, long long *base) { *base = *step + 1; }
+
+cudaError_t launch_io_base(const long long *step, long long *base, cudaStream_t s) {
+    k_io_base<<<1, 1, 0, s>>>(step, base);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_io_params(const double *params, int np, BcParam *par, const long long *cursor, cudaStream_t s) {

@@ -59,9 +59,21 @@ struct BcKParams {
     int step_in_reduce;         // 1: the 0D step once per boundary in k_bc_reduce; 0: in every k_bc_apply block
     int *arrived;               // per boundary: reduce CTAs done in this step (back to 0 after it)
     BcStepResult *result;       // per boundary
+    int cluster, wide;          // blocks per boundary of k_boundary (0: the two kernels), and whether they have 512 threads
     int n_red_blocks, n_app_blocks;
     const int32_t *red_bc, *red_chunk;  // per reduce block
     const int32_t *app_bc, *app_chunk;  // per apply block
+};
+
+// Per-step 0D input and output of lbm_step_io in k_boundary (null pointers:
+// none): np params of boundary b, state rows of boundaries b0 .. b0 + nb - 1; the
+// arrays' rows count from step *base.
+struct BcIo {
+    const double *params;
+    double *states;
+    BcParam *par;
+    const long long *base;
+    int np, b, b0, nb;
 };
 
 // Immersed-boundary tables (device memory).
@@ -121,11 +133,14 @@ cudaError_t launch_small(int prec, void *f0, void *f1, const KParams &p, const B
 constexpr int SC_VARIANTS = 5;
 int stream_collide_min_blocks(int variant);
 int stream_collide_cells_per_thread(int variant);
+// early: may start while the boundary kernel before it on the stream runs (its
+// set-up, the row tables, beside that kernel's latency); variant 0 only
 // stream-collide of the stored cells [c0, c1) (c1 < 0: all cells); bump: the
 // launch advances the step counter (one launch per step does)
 cudaError_t launch_stream_collide(int prec, const void *fin, void *fout, const KParams &p, int block,
-                                  int variant, cudaStream_t s, int desc = 0, int c0 = 0, int c1 = -1, int bump = 1);
-cudaError_t launch_boundary(int prec, void *f, const KParams &p, const BcKParams &q, cudaStream_t s);
+                                  int variant, cudaStream_t s, int desc = 0, int c0 = 0, int c1 = -1, int bump = 1,
+                                  bool early = false);
+cudaError_t launch_boundary(int prec, void *f, const KParams &p, const BcKParams &q, const BcIo &io, cudaStream_t s);
 cudaError_t launch_gather(int prec, const void *fin, const KParams &p, int c0, int c1, double *f19, double *mac4,
                           cudaStream_t s);
 cudaError_t launch_init_eq(int prec, void *fout, const KParams &p, const double *mac, int c0, int c1,
@@ -135,7 +150,8 @@ cudaError_t launch_wall_shear(int prec, const void *fin, const KParams &p, int c
 cudaError_t launch_state_rows(const BcState *st, const BcParam *par, const double *etab, int b0, int nb,
                               int nbc_total, long long steps, double *out8, cudaStream_t s);
 cudaError_t launch_copy_words(const void *src, void *dst, size_t bytes, cudaStream_t s);
-// per-step 0D input and output of lbm_step_io (see k_io_params, k_io_state)
+// per-step 0D input and output of lbm_step_io (see k_io_params, k_io_state, k_io_base)
+cudaError_t launch_io_base(const long long *step, long long *base, cudaStream_t s);
 cudaError_t launch_io_params(const double *params, int np, BcParam *par, const long long *cursor, cudaStream_t s);
 cudaError_t launch_io_state(const BcState *st, const BcParam *par, const double *etab, int b0, int nb, int nbc_total,
                             const long long *step, double *out8, long long *cursor, cudaStream_t s);

@@ -79,15 +79,6 @@ template <class R> struct FirstLayer {  // of one first-layer cell: forced veloc
     R v[3], sd;
 };
 
-// What a step of the 0D model needs besides the flow and pressure of t_n, in
-// terms of zero_d_step's expressions (forward Euler).
-struct Ahead {
-    double area, third;  // n_xf and n_xf / 3
-    int order;           // marching scheme
-    double p0_rc;        // RCR: P_w / (R_d C)
-    double inv_cv, dcv;  // LV: 1 / C_v and dC_v/dt, C_v = 1/E
-};
-
 constexpr int PULLS = NQ - 1;
 
 }  // namespace
@@ -113,6 +104,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
     __shared__ BcParam s_P;
     __shared__ BcState s_st;
     __shared__ Ahead s_a;
+    __shared__ double s_area, s_third;  // n_xf and n_xf / 3
+    __shared__ int s_euler;
     const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const int inst = blockIdx.x / C;
     const InstParam &ip = sp.inst[inst];
@@ -158,9 +151,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
         }
         if (tid == 0) {
             s_st = q.state[(size_t)(first & 1) * q.n_bc_total + b];
-            s_a.area = (double)s_P.n_xf;
-            s_a.third = (double)s_P.n_xf / 3.0;
-            s_a.order = (int)s_P.par[4];
+            s_area = (double)s_P.n_xf;
+            s_third = (double)s_P.n_xf / 3.0;
+            s_euler = boundary_euler(s_P);
         }
     }
     __syncthreads();
@@ -182,10 +175,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
             if (ta < sp.io_np) {
                 s_P.par[ta] = given;
                 sp.par[b].par[ta] = given;
-                if (ta == 4) s_a.order = (int)given;
                 if (s + 1 < sp.n_steps) given = __ldcv(sp.io_params + (size_t)(s + 1) * sp.io_np + ta);
             }
             meet();
+            if (ta == 0) s_euler = boundary_euler(P);
         }
         if (P.kind == BC_VELOCITY) {
             const double wt = P.par[0] * (double)(n + 1);
@@ -198,14 +191,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
                 unode[a] = (R)((double)P.sign * (pr[0] + pr[1] * cosp - pr[2] * sinp));
             }
         } else if (ta == 0) {
-            if (P.kind == BC_RCR) s_a.p0_rc = s_st.Pw / (P.par[2] * P.par[1]);
-            if (P.kind == BC_LV) {
-                const double E = q.etab[2 * (P.etab_off + (int)(n % P.period))];
-                const double Ed = q.etab[2 * (P.etab_off + (int)(n % P.period)) + 1];
-                const double Cv = 1.0 / E;
-                s_a.dcv = -Ed / (E * E);
-                s_a.inv_cv = 1.0 / Cv;
-            }
+            ahead_terms(P, s_st, n, q.etab, &s_a);
         }
     };
     if (owner && ta >= 0) ahead(0);
@@ -252,14 +238,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
                 constexpr int CH = THREADS / BC_CHUNK;
                 const int w = tid >> 5, ch = k0 / BC_CHUNK + (w & (CH - 1));
                 if (w < 2 * CH && ch < P.n_red) {
-                    const double *v = (w < CH ? sQ : sP) + (w & (CH - 1)) * BC_CHUNK + (tid & 31);
-                    double a[4];
-#pragma unroll
-                    for (int h = 0; h < 4; h++) a[h] = v[32 * h] + v[32 * (h + 4)];
-                    a[0] = (a[0] + a[2]) + (a[1] + a[3]);
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) a[0] += __shfl_down_sync(0xffffffffu, a[0], o);
-                    if ((tid & 31) == 0) s_part[2 * ch + (w < CH ? 0 : 1)] = a[0];
+                    const double a = tree_256((w < CH ? sQ : sP) + (w & (CH - 1)) * BC_CHUNK);
+                    if ((tid & 31) == 0) s_part[2 * ch + (w < CH ? 0 : 1)] = a;
                 }
                 __syncthreads();
             }
@@ -271,75 +251,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
                 post0 = PlainLoad<S>::ld(fout + ((lk0.y & 31) * N + cell[(lk0.y >> 5) & 0x7ff]));
             }
             if (tid < 32) {
-                // lane 0 takes the flow, lane 1 the pressure: partials in the order of bc_sum_partials
-                double a[SMALL_MAX_RED];
-                const double *sp_ = s_part + (tid & 1);
-                a[0] = 0.0 + sp_[0];
-                if (P.n_red > 1) {
-#pragma unroll
-                    for (int k = 1; k < SMALL_MAX_RED; k++) a[k] = k < P.n_red ? 0.0 + sp_[2 * k] : 0.0;
-                    if (P.n_red > 4)
-#pragma unroll
-                        for (int k = 0; k < 4; k++) a[k] += a[k + 4];
-                    if (P.n_red > 2) {
-                        a[0] += a[2];
-                        a[1] += a[3];
-                    }
-                    a[0] += a[1];
-                }
-                const int order = s_a.order;
-                if ((P.kind == BC_RCR || P.kind == BC_LV) && (order == 2 || order == 4)) {
-                    const double Ps = __shfl_sync(0xffffffffu, a[0], 1);
-                    if (tid == 0) {
-                        BcStepResult r;
-                        const BcState old = s_st;
-                        s_st = zero_d_step(P, old, a[0], s_a.third + Ps, s_a.area, n, q.etab, &r.ptype, &r.closed, &r.S);
-                        r.Pg = s_st.Pstar_gauge;
-                        s_r = r;
-                    }
-                } else {  // zero_d_step with forward Euler, its Q-independent parts taken above
-                    const double mean = ((tid & 1) ? s_a.third + a[0] : a[0]) / s_a.area;
-                    const double Pbar = __shfl_sync(0xffffffffu, mean, 1);
-                    if (tid == 0) {
-                        BcState st = s_st;
-                        st.Q = a[0];
-                        st.Qu = P.q_scale ? mean : a[0];
-                        st.Pbar = Pbar;
-                        BcStepResult r;
-                        r.ptype = 1;
-                        r.closed = 0;
-                        r.S = 0.0;
-                        if (P.kind == BC_RCR) {
-                            const double Qout = -st.Qu;
-                            const double Pw = s_st.Pw + (Qout / P.par[1] - s_a.p0_rc);
-                            st.Pw = Pw;
-                            st.Pstar_gauge = Pw + P.par[0] * Qout;
-                        } else if (P.kind == BC_PRESSURE) {
-                            st.Pstar_gauge = P.par[0];
-                        } else if (P.kind == BC_LV) {
-                            const double Qin = (st.valve_open != 0.0) ? st.Qu : 0.0;
-                            double Pv = st.Pv - s_a.inv_cv * (s_a.dcv * st.Pv + Qin);
-                            if (st.valve_open != 0.0) {
-                                if (st.Qu < 0.0) {  // closure: the inflow has reversed
-                                    st.valve_open = 0.0;
-                                    st.Td = (double)n;
-                                    r.closed = 1;
-                                }
-                            } else {
-                                if (Pv < P.par[1]) Pv = P.par[1];
-                                if (Pv > st.Pbar - 1.0 / 3.0) st.valve_open = 1.0;
-                            }
-                            st.Pv = Pv;
-                            st.Pstar_gauge = Pv;
-                            r.ptype = st.valve_open != 0.0;
-                            if (!r.ptype) r.S = smooth_to_zero((double)(n + 1), st.Td, P.par[2]);
-                        } else {
-                            r.ptype = 0;
-                        }
-                        r.Pg = st.Pstar_gauge;
-                        s_r = r;
-                        s_st = st;
-                    }
+                const double a = sum_partials_pair(s_part, P.n_red);
+                const double mean = ((tid & 1) ? s_third + a : a) / s_area;
+                const double Ps = __shfl_sync(0xffffffffu, a, 1), Pbar = __shfl_sync(0xffffffffu, mean, 1);
+                if (tid == 0) {
+                    BcStepResult r;
+                    const BcState old = s_st;
+                    s_st = s_euler ? zero_d_euler(P, old, s_a, a, mean, Pbar, n, &r.ptype, &r.closed, &r.S)
+                                   : zero_d_step(P, old, a, s_third + Ps, s_area, n, q.etab, &r.ptype, &r.closed, &r.S);
+                    r.Pg = s_st.Pstar_gauge;
+                    s_r = r;
                 }
             }
             __syncthreads();

@@ -45,7 +45,10 @@ template <class S> struct PopDirs {
 // launch starts on the lines the previous kernel touched last (still in L2).
 // The launch covers the stored cells [c0, c1); the launch with bump = 1
 // advances the step counter.
-template <class S, int MINB, int CPT>
+// EARLY: launched while its predecessor, the boundary kernel, still runs (see
+// launch_stream_collide); only tables that no step writes are read before the
+// wait.
+template <class S, int MINB, int CPT, bool EARLY = false>
 __global__ void __launch_bounds__(256, MINB)
     k_stream_collide(const __grid_constant__ PopDirs<S> d, const __grid_constant__ KParams p, int desc, int c0,
                      int c1, int bump) {
@@ -53,7 +56,7 @@ __global__ void __launch_bounds__(256, MINB)
     const int bid = desc ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
     const int t = c0 + bid * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
-    if (bump && t == c0 && p.step) *p.step += 1;  // the step index t_n seen by the boundary kernels
+    if (!EARLY && bump && t == c0 && p.step) *p.step += 1;  // the step index t_n seen by the boundary kernels
     const int N = (int)p.n;  // 19 N < 2^31 is checked at creation
     R f[CPT][NQ];
     R om[CPT];
@@ -63,10 +66,22 @@ __global__ void __launch_bounds__(256, MINB)
         const int c = t + u * stride;
         fl[u] = c < c1 ? __ldg(&p.flags[c]) : 0u;
         om[u] = R(0);
-        if (!(fl[u] & FL_ACTIVE)) continue;
-        const int r = find_row(p, c);
-        const int4 *row = reinterpret_cast<const int4 *>(p.rows + r);
-        const int4 h0 = __ldg(row), h1 = __ldg(row + 1), h2 = __ldg(row + 2), h3 = __ldg(row + 3);
+        const bool active = (fl[u] & FL_ACTIVE) != 0;
+        if (!EARLY && !active) continue;
+        int4 h0 = {}, h1 = {}, h2 = {}, h3 = {};
+        if (!EARLY || active) {
+            const int4 *row = reinterpret_cast<const int4 *>(p.rows + find_row(p, c));
+            h0 = __ldg(row);
+            h1 = __ldg(row + 1);
+            h2 = __ldg(row + 2);
+            h3 = __ldg(row + 3);
+        }
+        if (EARLY) {
+            wait_for_previous();
+            let_next_start();
+            if (bump && t == c0 && p.step) *p.step += 1;
+            if (!active) continue;
+        }
         // h0 = {off, x0, len, inst}, h1 = {y, z, nb0, nb1}, h2 = {nb2..nb5}, h3 = {nb6, nb7, nb8, pad}
         om[u] = omega_of<R>(p, h0.w);
         const int x = h0.y + (c - h0.x);
@@ -111,12 +126,18 @@ template <class S> static PopDirs<S> pop_dirs(const void *fin, void *fout, long 
 }
 
 cudaError_t launch_stream_collide(int prec, const void *fin, void *fout, const KParams &p, int block,
-                                  int variant, cudaStream_t s, int desc, int c0, int c1, int bump) {
+                                  int variant, cudaStream_t s, int desc, int c0, int c1, int bump, bool early) {
     if (c1 < 0) c1 = (int)p.n;
     if (c1 <= c0) return cudaSuccess;
     if (block % 32) return cudaErrorInvalidValue;  // whole warps: the forcing branch is a warp vote
     const int cpt = kVariants[variant][1];
     const int grid = (int)((c1 - c0 + (long long)block * cpt - 1) / ((long long)block * cpt));
+    if (early && variant == 0) {
+        cudaError_t e = cudaSuccess;
+        DISPATCH(prec, (e = launch_early(k_stream_collide<S, 6, 1, true>, dim3(grid), dim3(block), s,
+                                         pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump)));
+        return e;
+    }
     switch (variant) {
     case 1:
         DISPATCH(prec, (k_stream_collide<S, 8, 1><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump)));

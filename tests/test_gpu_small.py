@@ -113,3 +113,61 @@ def test_large_or_elastic_lattices_keep_the_step_graphs():
     from paper_2112_05258_gb300 import Lattice
     for inst in (configs.ib_tube(), _lv(13.0, 200)):
         assert Lattice([inst]).info().steps_per_launch == 0
+
+
+WIDE = {
+    "lv": lambda: _lv(13.0, 200),
+    "lv_order4": lambda: _order(_lv(12.2, 190), 4),
+    "velocity": lambda: configs.rigid_tube(31, 31, 170, radius=11.4),
+    "pressure": lambda: configs.pressure_tube(30, 30, 150, 12.6, 0.8, 2e-3, 0.0),
+}
+
+
+@pytest.mark.parametrize("precision", ["f32", "bf16"])
+@pytest.mark.parametrize("name", list(WIDE))
+def test_one_launch_boundary_equals_two_kernels(name, precision):
+    # a tube too large for the multi-step kernel takes its boundary work in one
+    # launch of clusters (started while stream-collide ends); many copies in one
+    # lattice have too many boundary blocks for it and take the two kernels
+    from paper_2112_05258_gb300 import Lattice
+    inst = WIDE[name]()
+    copies = 40
+    one, many = Lattice([inst], precision=precision), Lattice([inst] * copies, precision=precision)
+    assert one.info().steps_per_launch == 0 and one.info().launches_per_step == 2
+    assert many.info().launches_per_step == 3
+    f = configs.random_populations(inst, seed=5, amp=2e-3)
+    one.init_populations(0, f)
+    many.init_populations(7, f)
+    for n in (1, 130, 71):
+        one.step(n)
+        many.step(n)
+    assert np.array_equal(one.populations(0), many.populations(7))
+    assert np.array_equal(one.waves(0), many.waves(7))
+    for k in range(2):
+        assert np.array_equal(one.state_0d(0, k), many.state_0d(7, k))
+
+
+@pytest.mark.parametrize("name,bc,cols", [("lv", 1, 4), ("velocity", 0, 1)])
+def test_step_io_in_the_one_launch_boundary(name, bc, cols):
+    import torch
+    from paper_2112_05258_gb300 import Lattice
+    inst = WIDE[name]()
+    n = 150
+    base = np.array(inst.boundaries[bc].params[:cols], dtype=np.float64)
+    par = torch.from_numpy(np.tile(base, (n, 1)) * (1.0 + 0.2 * np.sin(np.arange(n) / 9.0))[:, None]).pin_memory()
+    par[:, 1:] = torch.from_numpy(base[1:])
+    rows = torch.zeros((n, 16), dtype=torch.float64, pin_memory=True)
+    want = torch.zeros((n, 16), dtype=torch.float64, pin_memory=True)
+    a, b = (Lattice([inst], precision="f32") for _ in range(2))
+    a.step(3)
+    b.step(3)
+    a.step_io(0, bc, n, par.data_ptr(), cols, rows.data_ptr())
+    a.sync()
+    for k in range(n):
+        b.set_0d_params(0, bc, par[k].numpy())
+        b.step(1)
+        b.state_0d_async(0, want[k].data_ptr())
+    b.sync()
+    assert np.array_equal(rows.numpy(), want.numpy())
+    assert np.array_equal(rows.numpy()[:, 0], np.arange(4, 154))
+    assert np.array_equal(a.populations(0), b.populations(0))
