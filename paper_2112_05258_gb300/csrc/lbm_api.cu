@@ -488,7 +488,7 @@ cudaError_t set_up_small(lbm_handle *h) {
     off.push_back((int32_t)bulk.size());
     // Times of a step in us, measured on GB300 over tubes of 2,400 to 110,000
     // cells.  This kernel: as many rounds as the clusters need, each the longer
-    // of the boundary block (latency: 3.8 us and its first layer's share; FP64
+    // of the boundary block (latency: 3.1 us and its first layer's share; FP64
     // runs on a pipe of 2 lanes an SM) and of a bulk block's cells.  One-step
     // kernels: launches and latencies of 12 us (FP64: 20), then bandwidth.
     const bool f64 = h->prec == LBM_F64;
@@ -499,7 +499,7 @@ cudaError_t set_up_small(lbm_handle *h) {
         if (C <= most_bc) continue;
         const size_t smem = std::max(smem_b, small_smem_bulk((int)worst_bulk[C]));
         if (smem > SMALL_MAX_SMEM) continue;
-        const double owner = f64 ? 4.5 + 0.09 * worst_xf : 3.8 + 0.006 * worst_xf;
+        const double owner = f64 ? 3.5 + 0.085 * worst_xf : 3.1 + 0.0058 * worst_xf;
         const double bulk = f64 ? 1.5 + 33e-3 * worst_bulk[C] : 0.7 + 3.2e-3 * worst_bulk[C];
         if (std::max(owner, bulk) >= best) continue;
         int clusters = 0;

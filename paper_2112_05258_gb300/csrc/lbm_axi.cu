@@ -408,8 +408,8 @@ __global__ void __launch_bounds__(BC2) k_axi_bc_apply(S *__restrict__ f, Params 
 // block k < n_bc owns the first layer and the 0D model of boundary k, the other
 // blocks the rest, one cluster barrier per step.  Same device functions and
 // summation orders as the one-step kernels.
-// A step, FP32: 258 x 32 grid 12.6 -> 4.1 us, 762 x 95 grid 14.7 -> 7.8 us; FP64: 82 x 10 grid
-// 17.2 -> 7.9 us (the FP64 pipe bounds larger ones, which keep the one-step kernels).
+// A step, FP32: 258 x 32 grid 12.6 -> 3.1 us, 762 x 95 grid 14.7 -> 8.0 us; FP64: 82 x 10 grid
+// 17.2 -> 7.3 us (the FP64 pipe bounds larger ones, which keep the one-step kernels).
 constexpr int AXI_PULLS = Q9 - 1;
 constexpr int AXI_MAX_RED = 8;
 constexpr int AXI_MAX_STEPS = 4096;
@@ -417,7 +417,7 @@ constexpr size_t AXI_MAX_SMEM = 212000;
 
 size_t axi_smem_bulk(int nodes, int r) { return (size_t)nodes * (AXI_PULLS * 4 + 4 + r) + 64; }
 size_t axi_smem_boundary(int n_xf, int n_links, int n_nodes, int r) {
-    return (size_t)n_xf * (AXI_PULLS * 4 + 4 + r + r + 6 * r + 16) + (size_t)n_links * 8 + (size_t)n_nodes * r + 128;
+    return (size_t)n_xf * (AXI_PULLS * 4 + 4 + r + r + 6 * r + 16) + (size_t)n_links * 8 + (size_t)n_nodes * (24 + 2 * r) + 128;
 }
 
 struct AxiSmall {
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Pa
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ double sQ[THREADS], sP[THREADS], s_part[2 * AXI_MAX_RED], s_cos, s_sin;
     __shared__ Ahead s_a;
-    __shared__ double s_area, s_third, s_S;
+    __shared__ double s_area, s_inv_area, s_third, s_S;
     __shared__ BcParam s_P;
     __shared__ BcState s_st;
     __shared__ R s_3p;
@@ -454,6 +454,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Pa
         if (tid == 0) {
             s_st = q.state[(size_t)(first & 1) * nb + b];
             s_area = q.area_sum[b];
+            s_inv_area = 1.0 / q.area_sum[b];
             s_third = q.area_sum[b] / 3.0;
         }
     } else {
@@ -463,10 +464,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Pa
     }
     // shared memory: 8-byte words first
     double *v0s = reinterpret_cast<double *>(smem);                   // [2 n_xf] closure velocities
-    AxiMoments<R> *mom = reinterpret_cast<AxiMoments<R> *>(v0s + (owner ? 2 * n_cells : 0));
+    double *prof = v0s + (owner ? 2 * n_cells : 0);                   // [3 n_nodes] inlet profile
+    AxiMoments<R> *mom = reinterpret_cast<AxiMoments<R> *>(prof + 3 * n_nodes);
     R *area = reinterpret_cast<R *>(mom + (owner ? n_cells : 0));      // [n_xf]
-    R *unode = area + (owner ? n_cells : 0);                           // [n_nodes]
-    R *ir = unode + n_nodes;                                           // [n_cells] 1/r
+    R *unode = area + (owner ? n_cells : 0);                           // [2 n_nodes] of this and the next step
+    R *ir = unode + 2 * n_nodes;                                       // [n_cells] 1/r
     int2 *link = reinterpret_cast<int2 *>((reinterpret_cast<uintptr_t>(ir + n_cells) + 7) & ~(uintptr_t)7);
     int *cell = reinterpret_cast<int *>(link + n_links);
     int *tab = cell + n_cells;                                         // [8][n_cells]
@@ -488,14 +490,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Pa
             v0s[2 * k + 1] = q.v0[2 * (size_t)(q.xf_off[b] + k) + 1];
         }
     }
+    for (int k = tid; k < 3 * n_nodes; k += THREADS) prof[k] = q.profile[3 * (size_t)q.node_off[b] + k];
     for (int L = tid; L < n_links; L += THREADS) {
         const int g = q.lk_off[b] + L;
         link[L] = make_int2(q.lk_ib[g] * n + q.lk_xb[g], q.lk_ieff[g] | (q.lk_xfi[g] << 4) | (q.lk_node[g] << 16));
     }
     __syncthreads();
-    // beside the cluster barrier: what does not depend on the step's flow
-    constexpr int AHEAD = 128;
-    const int ta = tid - (THREADS - AHEAD);
+    // the threads' roles as in k_small_steps
+    constexpr int AHEAD = THREADS / 4, WORK = THREADS - AHEAD, LAYER = WORK / BC2 * BC2, PREP = AHEAD - 32;
+    const int ta = tid - WORK;
     auto ahead = [&](int s) {
         const BcParam &P = s_P;
         const long long t = first + s;
@@ -503,17 +506,18 @@ __global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Pa
             const double wt = P.par[0] * (double)(t + 1);
             if (ta == 0) s_cos = cos(wt);
             if (ta == 32) s_sin = sin(wt);
-            asm volatile("bar.sync 1, %0;" ::"n"(AHEAD) : "memory");
+            asm volatile("bar.sync 1, %0;" ::"n"(PREP) : "memory");
             const double cosp = s_cos, sinp = s_sin;
-            for (int a = ta; a < n_nodes; a += AHEAD) {
-                const double *pr = q.profile + 3 * (size_t)(q.node_off[b] + a);
-                unode[a] = (R)((double)P.sign * (pr[0] + pr[1] * cosp - pr[2] * sinp));
+            R *u = unode + (s & 1) * n_nodes;
+            for (int a = ta; a < n_nodes; a += PREP) {
+                const double *pr = prof + 3 * a;
+                u[a] = (R)((double)P.sign * (pr[0] + pr[1] * cosp - pr[2] * sinp));
             }
         } else if (ta == 0) {
             ahead_terms(P, s_st, t, q.etab, &s_a);
         }
     };
-    if (owner && ta >= 0) ahead(0);
+    if (owner && ta >= 0 && ta < PREP) ahead(0);
     __syncthreads();
 
     const S *fin = f0;
@@ -528,13 +532,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Pa
                 for (int i = 1; i < Q9; i++) f[i] = fin[tab[(i - 1) * n_cells + k]];
                 axi_collide_store<S, R>(fout, p, f, omega, kk, nu, ir[k], c, 0u);
             }
+            __syncwarp();
+            cluster.barrier_arrive();
         } else {
             const BcParam &P = s_P;
             const long long t = first + s;
-            for (int k0 = 0; k0 < n_red * BC2; k0 += THREADS) {
+            for (int k0 = 0; k0 < n_red * BC2; k0 += LAYER) {
                 const int k = k0 + tid;
                 double Q = 0.0, Ps = 0.0;
-                if (k < n_cells) {
+                if (tid < LAYER && k < n_cells) {
                     const int c = cell[k];
                     R f[Q9];
                     f[0] = fin[c];
@@ -546,83 +552,87 @@ __global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Pa
                     Ps = (double)(A * m.sp / R(3));
                     mom[k] = m;
                 }
-                if (k < n_red * BC2) {
+                if (tid < LAYER) {
                     sQ[tid] = Q;
                     sP[tid] = Ps;
                 }
                 __syncthreads();
-                // the tree of k_axi_bc_reduce, one warp per quantity and chunk
-                constexpr int CH = THREADS / BC2;
-                const int w = tid >> 5, ch = k0 / BC2 + (w & (CH - 1));
+                const bool last = k0 + LAYER >= n_red * BC2;
+                constexpr int CH = LAYER / BC2;  // one warp per quantity and chunk
+                const int w = tid >> 5, h = w < CH ? w : w - CH, ch = k0 / BC2 + h;
                 if (w < 2 * CH && ch < n_red) {
-                    const double a = tree_256((w < CH ? sQ : sP) + (w & (CH - 1)) * BC2);
+                    const double a = tree_256((w < CH ? sQ : sP) + h * BC2);
                     if ((tid & 31) == 0) s_part[2 * ch + (w < CH ? 0 : 1)] = a;
                 }
+                __syncwarp();
+                if (last && w >= 2 * CH) cluster.barrier_arrive();
                 __syncthreads();
+                if (last && w > 0 && w < 2 * CH) cluster.barrier_arrive();
             }
+            constexpr int LINKS = WORK - 32;
+            const int tl = tid - 32;
             int2 lk0 = make_int2(0, 0);  // the thread's first link, its population in flight beside the 0D step
             R post0 = R(0);
-            if (tid < n_links) {
-                lk0 = link[tid];
+            if (tl >= 0 && tid < WORK && tl < n_links) {
+                lk0 = link[tl];
                 post0 = fout[(lk0.y & 15) * n + cell[(lk0.y >> 4) & 0xfff]];
             }
             if (tid < 32) {
                 double a = 0.0;  // lane 0 the flow, lane 1 the pressure: the partials in their fixed order
                 for (int k = 0; k < n_red; k++) a += s_part[2 * k + (tid & 1)];
-                const double mean = ((tid & 1) ? s_third + a : a) / s_area;
+                const double mean = quotient((tid & 1) ? s_third + a : a, s_area, s_inv_area);
                 const double Ps = __shfl_sync(0xffffffffu, a, 1), Pbar = __shfl_sync(0xffffffffu, mean, 1);
                 if (tid == 0) {
                     const BcState old = s_st;
                     double Sm;
-                    s_st = boundary_euler(P)
-                               ? zero_d_euler(P, old, s_a, a, mean, Pbar, t, &s_ptype, &s_closed, &Sm)
-                               : zero_d_step(P, old, a, s_third + Ps, s_area, t, q.etab, &s_ptype, &s_closed, &Sm);
+                    const BcState st =
+                        boundary_euler(P)
+                            ? zero_d_euler(P, old, s_a, a, mean, Pbar, t, &s_ptype, &s_closed, &Sm)
+                            : zero_d_step(P, old, a, s_third + Ps, s_area, t, q.etab, &s_ptype, &s_closed, &Sm);
                     s_S = Sm;
-                    s_3p = (R)(3.0 * s_st.Pstar_gauge);
+                    s_3p = (R)(3.0 * st.Pstar_gauge);
+                    s_st = st;
                 }
             }
             __syncthreads();
-            const bool ptype = s_ptype != 0, closed = s_closed != 0;
-            for (int L = tid; L < n_links; L += THREADS) {
-                const int2 lk = L == tid ? lk0 : link[L];
-                const int ie = lk.y & 15, xfi = (lk.y >> 4) & 0xfff;
-                const AxiMoments<R> m = mom[xfi];
-                const R post = L == tid ? post0 : (R)fout[ie * n + cell[xfi]];
-                R sps, vxs, vrs;
-                if (ptype) {
-                    sps = s_3p;
-                    vxs = m.vx;
-                    vrs = m.vr;
-                } else if (P.kind == BC_VELOCITY) {
-                    sps = m.sp;
-                    vxs = unode[lk.y >> 16];
-                    vrs = R(0);
-                } else {
-                    const double u0x = closed ? (double)m.vx : v0s[2 * xfi];
-                    const double u0r = closed ? (double)m.vr : v0s[2 * xfi + 1];
-                    sps = m.sp;
-                    vxs = (R)(u0x * s_S);
-                    vrs = (R)(u0r * s_S);
+            if (tid < 32) cluster.barrier_arrive();
+            if (tid < WORK) {
+                const bool ptype = s_ptype != 0, closed = s_closed != 0;
+                for (int L = tl >= 0 ? tl : n_links; L < n_links; L += LINKS) {
+                    const int2 lk = L == tl ? lk0 : link[L];
+                    const int ie = lk.y & 15, xfi = (lk.y >> 4) & 0xfff;
+                    const AxiMoments<R> m = mom[xfi];
+                    const R post = L == tl ? post0 : (R)fout[ie * n + cell[xfi]];
+                    R sps, vxs, vrs;
+                    if (ptype) {
+                        sps = s_3p;
+                        vxs = m.vx;
+                        vrs = m.vr;
+                    } else if (P.kind == BC_VELOCITY) {
+                        sps = m.sp;
+                        vxs = unode[(s & 1) * n_nodes + (lk.y >> 16)];
+                        vrs = R(0);
+                    } else {
+                        const double u0x = closed ? (double)m.vx : v0s[2 * xfi];
+                        const double u0r = closed ? (double)m.vr : v0s[2 * xfi + 1];
+                        sps = m.sp;
+                        vxs = (R)(u0x * s_S);
+                        vrs = (R)(u0r * s_S);
+                    }
+                    fout[lk.x] = post + dfeq_dev<R>(ie, sps, vxs, vrs, m.sp, m.vx, m.vr);
                 }
-                fout[lk.x] = post + dfeq_dev<R>(ie, sps, vxs, vrs, m.sp, m.vx, m.vr);
-            }
-            if (closed) {
-                __syncthreads();
-                for (int k = tid; k < n_cells; k += THREADS) {
-                    double *v0 = q.v0 + 2 * (size_t)(q.xf_off[b] + k);
-                    v0s[2 * k] = v0[0] = (double)mom[k].vx;
-                    v0s[2 * k + 1] = v0[1] = (double)mom[k].vr;
+                asm volatile("bar.sync 2, %0;" ::"n"(WORK) : "memory");
+                if (closed) {
+                    for (int k = tid; k < n_cells; k += WORK) {
+                        double *v0 = q.v0 + 2 * (size_t)(q.xf_off[b] + k);
+                        v0s[2 * k] = v0[0] = (double)mom[k].vx;
+                        v0s[2 * k + 1] = v0[1] = (double)mom[k].vr;
+                    }
+                    asm volatile("bar.sync 2, %0;" ::"n"(WORK) : "memory");
                 }
-            }
-        }
-        const S *tmp = fin;
-        fin = fout;
-        fout = const_cast<S *>(tmp);
-        __syncwarp();
-        cluster.barrier_arrive();
-        if (owner) {
-            if (tid == THREADS - AHEAD - 32) {
-                const long long t = first + s;
+            } else if (ta < PREP) {
+                if (s + 1 < sp.n_steps) ahead(s + 1);
+            } else if (ta == PREP) {
                 const BcState st = s_st;
                 q.state[(size_t)((t + 1) & 1) * nb + b] = st;
                 double *row = q.wave + (size_t)(t % q.wave_cap) * (1 + 4 * nb);
@@ -632,8 +642,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_axi_small_steps(S *f0, S *f1, Pa
                 row[3 + 4 * b] = s_P.kind == BC_RCR ? st.Pw : (s_P.kind == BC_LV ? st.Pv : st.Pstar_gauge);
                 row[4 + 4 * b] = st.valve_open;
             }
-            if (ta >= 0 && s + 1 < sp.n_steps) ahead(s + 1);
         }
+        const S *tmp = fin;
+        fin = fout;
+        fout = const_cast<S *>(tmp);
         __syncwarp();
         cluster.barrier_wait();
     }
@@ -840,7 +852,7 @@ cudaError_t set_up_small(lbm_axi_handle *h, const std::vector<uint16_t> &flags, 
     const int per = ((int)bulk.size() + C - nb - 1) / (C - nb);
     smem = std::max(smem, axi_smem_bulk(per, r));
     if (smem > AXI_MAX_SMEM) return cudaSuccess;
-    const double small = r == 8 ? std::max(4.5 + 0.09 * worst, 1.5 + 16e-3 * per) : std::max(3.8 + 0.006 * worst, 0.7 + 1.6e-3 * per);
+    const double small = r == 8 ? std::max(3.5 + 0.085 * worst, 1.5 + 16e-3 * per) : std::max(2.9 + 0.006 * worst, 0.7 + 1.6e-3 * per);
     const double one = r == 8 ? std::max(21.0, 16.0 + 120e-6 * h->n) : 13.4;
     if (small > 0.9 * one) return cudaSuccess;
     h->small_cluster = C;

@@ -38,12 +38,26 @@ static __device__ BcStepResult bc_step(const BcParam &P, int b, double Q, double
     return r;
 }
 
+// a / b, rounded to nearest, from inv_b = 1 / b rounded to nearest: Markstein's
+// correction (P. Markstein, IBM J. Res. Dev. 34, 1990): with q within an ulp of
+// a / b, q + (a - b q) inv_b is the correctly rounded quotient.  The first step
+// brings a inv_b within an ulp.  Five dependent operations, half the latency of a
+// division; magnitudes near the ends of the range are divided.
+static __device__ __forceinline__ double quotient(double a, double b, double inv_b) {
+    // binary exponents within +-500 of one (integer tests: an FP64 comparison waits as long as an addition)
+    const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ffu, eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu;
+    if (ea - 523u > 1000u || eb - 823u > 400u) return a / b;
+    double q = a * inv_b;
+    q = fma(fma(-b, q, a), inv_b, q);
+    return fma(fma(-b, q, a), inv_b, q);
+}
+
 // zero_d_step with forward Euler in two parts, in the same expressions: what
 // does not depend on the step's flow, taken beside other work (an FP64 division
 // is about 700 cycles on this part), and the rest.  boundary_euler: whether the
 // boundary marches so.
 struct Ahead {
-    double p0_rc;        // RCR: P_w / (R_d C)
+    double p0_rc, inv_c; // RCR: P_w / (R_d C) and 1 / C
     double inv_cv, dcv;  // LV: 1 / C_v and dC_v/dt, C_v = 1/E
 };
 static __device__ __forceinline__ bool boundary_euler(const BcParam &P) {
@@ -52,7 +66,10 @@ static __device__ __forceinline__ bool boundary_euler(const BcParam &P) {
 }
 static __device__ __forceinline__ void ahead_terms(const BcParam &P, const BcState &st, long long n, const double *etab,
                                                    Ahead *a) {
-    if (P.kind == BC_RCR) a->p0_rc = st.Pw / (P.par[2] * P.par[1]);
+    if (P.kind == BC_RCR) {
+        a->p0_rc = st.Pw / (P.par[2] * P.par[1]);
+        a->inv_c = 1.0 / P.par[1];
+    }
     if (P.kind == BC_LV) {
         const double E = etab[2 * (P.etab_off + (int)(n % P.period))];
         const double Ed = etab[2 * (P.etab_off + (int)(n % P.period)) + 1];
@@ -74,7 +91,7 @@ static __device__ __forceinline__ BcState zero_d_euler(const BcParam &P, const B
     *Smooth = 0.0;
     if (P.kind == BC_RCR) {
         const double Qout = -st.Qu;
-        const double Pw = old.Pw + (Qout / P.par[1] - a.p0_rc);
+        const double Pw = old.Pw + (quotient(Qout, P.par[1], a.inv_c) - a.p0_rc);
         st.Pw = Pw;
         st.Pstar_gauge = Pw + P.par[0] * Qout;
     } else if (P.kind == BC_PRESSURE) {
@@ -136,6 +153,16 @@ static __device__ __forceinline__ double sum_partials_pair(const double *part, i
     return (lane & 1) ? c : a;
 }
 
+// s / 3, rounded to nearest, by the same correction in the arithmetic type
+static __device__ __forceinline__ float third_of(float s) {
+    const unsigned e = (__float_as_uint(s) >> 23) & 0xffu;
+    if (e - 40u > 200u) return s / 3.0f;
+    const float q = s * (1.0f / 3.0f);
+    const float q1 = fmaf(fmaf(-3.0f, q, s), 1.0f / 3.0f, q);
+    return fmaf(fmaf(-3.0f, q1, s), 1.0f / 3.0f, q1);
+}
+static __device__ __forceinline__ double third_of(double s) { return quotient(s, 3.0, 1.0 / 3.0); }
+
 // Sum of 256 values of shared memory by one warp, in the order of the tree of
 // k_bc_reduce (128, 64, 32, then within the warp); lane 0 gets it.
 static __device__ __forceinline__ double tree_256(const double *v) {
@@ -168,10 +195,8 @@ static __constant__ signed char c_ex[NQ] = {0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 
 static __constant__ signed char c_ey[NQ] = {0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 0, 0, 0, 0, 1, -1, 1, -1};
 static __constant__ signed char c_ez[NQ] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, -1, 1};
 
-// f^eq_i(P + dP, vs) - f^eq_i(P, vf)
-template <class R> __device__ __forceinline__ R feq_change(int i, R dP, const R vs[3], const R vf[3]) {
-    const R ex = c_ex[i], ey = c_ey[i], ez = c_ez[i];
-    const R w = i == 0 ? R(1.0 / 3.0) : (i < 7 ? R(1.0 / 18.0) : R(1.0 / 36.0));
+// f^eq_i(P + dP, vs) - f^eq_i(P, vf), (ex, ey, ez) = e_i and w = w_i
+template <class R> __device__ __forceinline__ R feq_change(R ex, R ey, R ez, R w, R dP, const R vs[3], const R vf[3]) {
     const R eus = ex * vs[0] + ey * vs[1] + ez * vs[2];
     const R euf = ex * vf[0] + ey * vf[1] + ez * vf[2];
     const R us2 = vs[0] * vs[0] + vs[1] * vs[1] + vs[2] * vs[2];
@@ -215,7 +240,8 @@ __device__ __forceinline__ R ghost_change(const BcParam &P, const BcStepResult &
             vs[2] = u0[2] * Sm;
         }
     }
-    return feq_change<R>(i, dP, vs, vf);
+    const R w = i == 0 ? R(1.0 / 3.0) : (i < 7 ? R(1.0 / 18.0) : R(1.0 / 36.0));
+    return feq_change<R>((R)c_ex[i], (R)c_ey[i], (R)c_ez[i], w, dP, vs, vf);
 }
 
 }  // namespace lbm

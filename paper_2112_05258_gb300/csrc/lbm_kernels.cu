@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(BS) k_boundary(S *__restrict__ f, KParams p, B
     using R = typename Storage<S>::R;
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    __shared__ double sQ[BS], sP[BS], s_area, s_third, s_cos, s_sin;
+    __shared__ double sQ[BS], sP[BS], s_area, s_inv_area, s_third, s_cos, s_sin;
     __shared__ BcParam s_P;
     __shared__ BcState s_st;
     __shared__ BcStepResult s_r;
@@ -265,7 +265,8 @@ __global__ void __launch_bounds__(BS) k_boundary(S *__restrict__ f, KParams p, B
         if (tid == BS - 96) s_st = q.state[(size_t)(n & 1) * q.n_bc_total + b];
         if (tid == BS - 128) {
             s_area = (double)P.n_xf;
-            s_third = (double)P.n_xf / 3.0;
+            s_inv_area = 1.0 / s_area;
+            s_third = s_area / 3.0;
             s_euler = boundary_euler(P);
         }
     }
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(BS) k_boundary(S *__restrict__ f, KParams p, B
     if (rank == 0) {
         if (tid < 32) {
             const double a = sum_partials_pair(q.partial + 2 * P.red_off, P.n_red);
-            const double mean = ((tid & 1) ? s_third + a : a) / s_area;
+            const double mean = quotient((tid & 1) ? s_third + a : a, s_area, s_inv_area);
             const double Ps = __shfl_sync(0xffffffffu, a, 1), Pbar = __shfl_sync(0xffffffffu, mean, 1);
             if (tid == 0) {
                 BcStepResult r;

@@ -20,15 +20,17 @@
 // (collide_store, the 256-wide trees and partial sums, bc_step, ghost_change):
 // the trajectory is the same bit for bit.
 //
-// Bound by latency.  FP64 additions take 64 cycles each on this part and a
-// division about 700, so the boundary block's chain decides: for the 24x24x64
-// tube (12,896 cells, FP32) about 1,200 cycles for the pulls, 1,400 collision
-// and the layer's terms, 1,800 trees, 2,400 means and 0D step, 2,000 ghosts,
-// 1,800 barrier; what does not depend on the step's flow (inlet velocities,
-// elastance terms, state and waveform stores) runs while the block waits at the
-// barrier.  A step: 12.4 -> 5.1 us for that tube, 12.1 -> 4.1
-// us for 2,400 cells (FP32), 20.7 -> 11.6 us in FP64 (whose collision is bound
-// by the FP64 pipe); three such tubes side by side 5.0 -> 1.7 us a step each.
+// Bound by latency: the boundary block's chain decides.  An FP64 operation takes
+// 64 cycles on this part, a division about 700.  For the 24x24x64 tube (12,896
+// cells, FP32) about 1,500 cycles for the pulls, 1,600 collision and the layer's
+// terms, 1,400 trees, 2,300 means and 0D step, 1,300 ghosts.  Kept out of the
+// chain: the cluster barrier (arrival, which waits for a warp's stores, as soon
+// as a warp is not needed for the sums; the ghosts are written after it), all
+// that does not depend on the step's flow (inlet velocities, elastance terms,
+// state and waveform stores: on threads of their own), divisions by the layer's
+// area and the compliance (quotient).
+// A step: 12.4 -> 4.1 us for that tube, 12.1 -> 3.5 us for 2,400 cells (FP32), 20.7
+// -> 10.1 us in FP64 (whose collision is bound by the FP64 pipe).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -75,8 +77,8 @@ __device__ __forceinline__ void pull_offsets(const KParams &p, int c, uint32_t f
     }
 }
 
-template <class R> struct FirstLayer {  // of one first-layer cell: forced velocity and sum s; v_0 of its closure (LV)
-    R v[3], sd;
+template <class R> struct FirstLayer {  // of one first-layer cell: velocity and (sum s) / 3; v_0 of its closure (LV)
+    R v[3], p;
 };
 
 constexpr int PULLS = NQ - 1;
@@ -86,10 +88,10 @@ constexpr int PULLS = NQ - 1;
 // Shared memory of a block.  Boundary block: per first-layer cell the pull
 // table, the cell, its moments and its closure velocity; per link its
 // destination offset and {direction, first-layer index, node}; per boundary
-// node the prescribed velocity.  Bulk block: pull table and cell per cell.
+// node its profile and the prescribed velocity.  Bulk block: pull table and cell per cell.
 size_t small_smem_boundary(int n_xf, int n_links, int n_nodes, bool f64) {
     const size_t r = f64 ? 8 : 4;
-    return (size_t)n_xf * (PULLS * 4 + 4 + 8 * r) + (size_t)n_links * 8 + (size_t)n_nodes * r + 64;
+    return (size_t)n_xf * (PULLS * 4 + 4 + 8 * r) + (size_t)n_links * 8 + (size_t)n_nodes * (24 + 2 * r) + 64;
 }
 size_t small_smem_bulk(int cells) { return (size_t)cells * (PULLS * 4 + 4) + 64; }
 
@@ -104,8 +106,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
     __shared__ BcParam s_P;
     __shared__ BcState s_st;
     __shared__ Ahead s_a;
-    __shared__ double s_area, s_third;  // n_xf and n_xf / 3
+    __shared__ double s_area, s_inv_area, s_third;  // n_xf, 1 / n_xf and n_xf / 3
     __shared__ int s_euler;
+    __shared__ R s_dir[NQ][4];  // e_i and w_i
     const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const int inst = blockIdx.x / C;
     const InstParam &ip = sp.inst[inst];
@@ -134,7 +137,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
     FirstLayer<R> *xf = reinterpret_cast<FirstLayer<R> *>((reinterpret_cast<uintptr_t>(cell + n_cells) + 15) & ~(uintptr_t)15);
     FirstLayer<R> *v0s = xf + (owner ? n_cells : 0);  // closure velocities
     int2 *link = reinterpret_cast<int2 *>(v0s + (owner ? n_cells : 0));
-    R *unode = reinterpret_cast<R *>(link + (owner ? s_P.n_links : 0));
+    double *prof = reinterpret_cast<double *>(link + (owner ? s_P.n_links : 0));  // velocity inlet: 3 per node
+    const int n_prof = owner && s_P.kind == BC_VELOCITY ? s_P.n_nodes : 0;
+    R *unode = reinterpret_cast<R *>(prof + 3 * n_prof);
     for (int k = tid; k < n_cells; k += THREADS) {
         const int c = owner ? q.xf[s_P.xf_off + k] : sp.bulk[cell0 + k];
         cell[k] = c;
@@ -145,6 +150,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
         }
     }
     if (owner) {
+        for (int k = tid; k < 3 * n_prof; k += THREADS) prof[k] = q.profile[3 * (size_t)s_P.node_off + k];
         for (int L = tid; L < s_P.n_links; L += THREADS) {
             const int g = s_P.link_off + L, i = q.lk_i[g];
             link[L] = make_int2(i * N + q.lk_xb[g], i | (q.lk_xfi[g] << 5) | (q.lk_node[g] << 16));
@@ -152,6 +158,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
         if (tid == 0) {
             s_st = q.state[(size_t)(first & 1) * q.n_bc_total + b];
             s_area = (double)s_P.n_xf;
+            s_inv_area = 1.0 / s_area;
             s_third = (double)s_P.n_xf / 3.0;
             s_euler = boundary_euler(s_P);
         }
@@ -160,17 +167,18 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
     const bool io_in = owner && sp.io_params && b == sp.io_b;
     const bool io_out = owner && sp.io_states && b >= sp.io_b0 && b < sp.io_b0 + sp.io_nb;
 
-    // The last AHEAD threads of a boundary block prepare step s while the others
-    // wait at the cluster barrier and collide: its params (io), and the parts of
-    // its 0D model that do not depend on its flow.
-    constexpr int AHEAD = 128;
-    const int ta = tid - (THREADS - AHEAD);
+    // Threads of a boundary block: the first WORK collide its first layer and write
+    // the ghosts; the next PREP prepare step s while those finish step s - 1 and
+    // collide: its params (io), and the parts of its 0D model that do not depend
+    // on its flow; the last warp stores states and waveforms.
+    constexpr int AHEAD = THREADS / 4, WORK = THREADS - AHEAD, LAYER = WORK / BC_CHUNK * BC_CHUNK, PREP = AHEAD - 32;
+    const int ta = tid - WORK;
     double given = 0.0;
     if (io_in && ta >= 0 && ta < sp.io_np) given = __ldcv(sp.io_params + ta);
     auto ahead = [&](int s) {
         const BcParam &P = s_P;
         const long long n = first + s;
-        auto meet = [] { asm volatile("bar.sync 1, %0;" ::"n"(AHEAD) : "memory"); };
+        auto meet = [] { asm volatile("bar.sync 1, %0;" ::"n"(PREP) : "memory"); };
         if (io_in) {
             if (ta < sp.io_np) {
                 s_P.par[ta] = given;
@@ -186,15 +194,22 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
             if (ta == 32) s_sin = sin(wt);
             meet();
             const double cosp = s_cos, sinp = s_sin;
-            for (int a = ta; a < P.n_nodes; a += AHEAD) {  // the nodes' velocities at t_{n+1}
-                const double *pr = q.profile + 3 * (size_t)(P.node_off + a);
-                unode[a] = (R)((double)P.sign * (pr[0] + pr[1] * cosp - pr[2] * sinp));
+            R *u = unode + (s & 1) * n_prof;  // the workers may still be reading step s - 1's
+            for (int a = ta; a < n_prof; a += PREP) {  // the nodes' velocities at t_{n+1}
+                const double *pr = prof + 3 * a;
+                u[a] = (R)((double)P.sign * (pr[0] + pr[1] * cosp - pr[2] * sinp));
             }
         } else if (ta == 0) {
             ahead_terms(P, s_st, n, q.etab, &s_a);
         }
     };
-    if (owner && ta >= 0) ahead(0);
+    if (tid < NQ) {
+        s_dir[tid][0] = c_ex[tid];
+        s_dir[tid][1] = c_ey[tid];
+        s_dir[tid][2] = c_ez[tid];
+        s_dir[tid][3] = tid == 0 ? R(1.0 / 3.0) : (tid < 7 ? R(1.0 / 18.0) : R(1.0 / 36.0));
+    }
+    if (owner && ta >= 0 && ta < PREP) ahead(0);
     __syncthreads();
 
     const S *fin = f0;
@@ -210,13 +225,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
                 for (int i = 1; i < NQ; i++) f[i] = PlainLoad<S>::ld(fin + tab[(i - 1) * n_cells + k]);
                 collide_store<S, R, false>(out, p, f, omega, 0u, c);
             }
+            __syncwarp();
+            cluster.barrier_arrive();
         } else {
             const BcParam &P = s_P;
             const long long n = first + s;
-            for (int k0 = 0; k0 < P.n_red * BC_CHUNK; k0 += THREADS) {
+            for (int k0 = 0; k0 < P.n_red * BC_CHUNK; k0 += LAYER) {
                 const int k = k0 + tid;
                 double Q = 0.0, Ps = 0.0;
-                if (k < n_cells) {
+                if (tid < LAYER && k < n_cells) {
                     const int c = cell[k];
                     R f[NQ];
                     f[0] = PlainLoad<S>::ld(fin + c);
@@ -224,76 +241,114 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
                     for (int i = 1; i < NQ; i++) f[i] = PlainLoad<S>::ld(fin + tab[(i - 1) * n_cells + k]);
                     const Moments<R> m = collide_store<S, R, false>(out, p, f, omega, 0u, c);
                     const R j = P.axis == 0 ? m.jx : P.axis == 1 ? m.jy : m.jz;
+                    const R third = third_of(m.sd);
                     Q = (double)((R)P.sign * j / (R(1) + m.sd));
-                    Ps = (double)(m.sd / R(3));
-                    xf[k] = FirstLayer<R>{{m.jx, m.jy, m.jz}, m.sd};
+                    Ps = (double)third;
+                    xf[k] = FirstLayer<R>{{m.jx, m.jy, m.jz}, third};
                 }
-                if (k < P.n_red * BC_CHUNK) {
+                if (tid < LAYER) {
                     sQ[tid] = Q;
                     sP[tid] = Ps;
                 }
                 __syncthreads();
-                // one warp per quantity and chunk of 256 cells: the tree of
-                // k_bc_reduce (128, 64, 32, then within the warp)
-                constexpr int CH = THREADS / BC_CHUNK;
-                const int w = tid >> 5, ch = k0 / BC_CHUNK + (w & (CH - 1));
+                // one warp per quantity and chunk of 256 cells.  The populations the
+                // other blocks wait for are stored: a warp arrives at the cluster
+                // barrier, which holds it until its stores are out, once the sums
+                // and the 0D step no longer wait for it
+                constexpr int CH = LAYER / BC_CHUNK;
+                const int w = tid >> 5, h = w < CH ? w : w - CH, ch = k0 / BC_CHUNK + h;
+                const bool last = k0 + LAYER >= P.n_red * BC_CHUNK;
                 if (w < 2 * CH && ch < P.n_red) {
-                    const double a = tree_256((w < CH ? sQ : sP) + (w & (CH - 1)) * BC_CHUNK);
+                    const double a = tree_256((w < CH ? sQ : sP) + h * BC_CHUNK);
                     if ((tid & 31) == 0) s_part[2 * ch + (w < CH ? 0 : 1)] = a;
                 }
+                __syncwarp();
+                if (last && w >= 2 * CH) cluster.barrier_arrive();
                 __syncthreads();
+                if (last && w > 0 && w < 2 * CH) cluster.barrier_arrive();
             }
-            // the thread's first link, its population in flight beside the 0D step
-            int2 lk0 = make_int2(0, 0);
-            R post0 = R(0);
-            if (tid < P.n_links) {
-                lk0 = link[tid];
-                post0 = PlainLoad<S>::ld(fout + ((lk0.y & 31) * N + cell[(lk0.y >> 5) & 0x7ff]));
+            // the thread's first two links (from the second warp on), their
+            // populations in flight beside the 0D step
+            constexpr int LINKS = WORK - 32;
+            const int tl = tid - 32;
+            int2 lk0 = make_int2(0, 0), lk1 = lk0;
+            R post0 = R(0), post1 = R(0);
+            auto post_of = [&](const int2 &lk) {
+                return PlainLoad<S>::ld(fout + ((lk.y & 31) * N + cell[(lk.y >> 5) & 0x7ff]));
+            };
+            if (tl >= 0 && tid < WORK && tl < P.n_links) {
+                lk0 = link[tl];
+                post0 = post_of(lk0);
+            }
+            if (tl >= 0 && tid < WORK && tl + LINKS < P.n_links) {
+                lk1 = link[tl + LINKS];
+                post1 = post_of(lk1);
             }
             if (tid < 32) {
                 const double a = sum_partials_pair(s_part, P.n_red);
-                const double mean = ((tid & 1) ? s_third + a : a) / s_area;
+                const double mean = quotient((tid & 1) ? s_third + a : a, s_area, s_inv_area);
                 const double Ps = __shfl_sync(0xffffffffu, a, 1), Pbar = __shfl_sync(0xffffffffu, mean, 1);
                 if (tid == 0) {
                     BcStepResult r;
                     const BcState old = s_st;
-                    s_st = s_euler ? zero_d_euler(P, old, s_a, a, mean, Pbar, n, &r.ptype, &r.closed, &r.S)
-                                   : zero_d_step(P, old, a, s_third + Ps, s_area, n, q.etab, &r.ptype, &r.closed, &r.S);
-                    r.Pg = s_st.Pstar_gauge;
+                    const BcState st =
+                        s_euler ? zero_d_euler(P, old, s_a, a, mean, Pbar, n, &r.ptype, &r.closed, &r.S)
+                                : zero_d_step(P, old, a, s_third + Ps, s_area, n, q.etab, &r.ptype, &r.closed, &r.S);
+                    r.Pg = st.Pstar_gauge;
                     s_r = r;
+                    s_st = st;
                 }
             }
             __syncthreads();
-            const BcStepResult &r = s_r;
-            const bool closed = r.closed != 0, ptype = r.ptype != 0;
-            const R Pg = (R)r.Pg, Sm = (R)r.S;
-            for (int L = tid; L < P.n_links; L += THREADS) {
-                const int2 lk = L == tid ? lk0 : link[L];
-                const int i = lk.y & 31, xfi = (lk.y >> 5) & 0x7ff;
-                const FirstLayer<R> m = xf[xfi];
-                const R post = L == tid ? post0 : PlainLoad<S>::ld(fout + (i * N + cell[xfi]));
-                R dP = R(0), vs[3] = {R(0), R(0), R(0)};
-                if (ptype) {
-                    dP = Pg - m.sd / R(3);
-                    vs[0] = m.v[0];
-                    vs[1] = m.v[1];
-                    vs[2] = m.v[2];
-                } else if (P.kind == BC_VELOCITY) {
-                    vs[P.axis] = unode[lk.y >> 16];
-                } else if (P.kind == BC_LV) {  // v_0(T_d) S(t, T_d, N_S); closing now, v_0 = v(x_f, T_d)
-                    const FirstLayer<R> &u = closed ? xf[xfi] : v0s[xfi];
-                    vs[0] = u.v[0] * Sm;
-                    vs[1] = u.v[1] * Sm;
-                    vs[2] = u.v[2] * Sm;
+            if (tid < 32) cluster.barrier_arrive();
+            if (tid < WORK) {
+                const BcStepResult &r = s_r;
+                const bool closed = r.closed != 0, ptype = r.ptype != 0;
+                const R Pg = (R)r.Pg, Sm = (R)r.S;
+                for (int L = tl >= 0 ? tl : P.n_links; L < P.n_links; L += LINKS) {
+                    const int2 lk = L == tl ? lk0 : L == tl + LINKS ? lk1 : link[L];
+                    const int i = lk.y & 31, xfi = (lk.y >> 5) & 0x7ff;
+                    const FirstLayer<R> m = xf[xfi];
+                    const R post = L == tl ? post0 : L == tl + LINKS ? post1 : post_of(lk);
+                    R dP = R(0), vs[3] = {R(0), R(0), R(0)};
+                    if (ptype) {
+                        dP = Pg - m.p;
+                        vs[0] = m.v[0];
+                        vs[1] = m.v[1];
+                        vs[2] = m.v[2];
+                    } else if (P.kind == BC_VELOCITY) {
+                        vs[P.axis] = unode[(s & 1) * n_prof + (lk.y >> 16)];
+                    } else if (P.kind == BC_LV) {  // v_0(T_d) S(t, T_d, N_S); closing now, v_0 = v(x_f, T_d)
+                        const FirstLayer<R> &u = closed ? xf[xfi] : v0s[xfi];
+                        vs[0] = u.v[0] * Sm;
+                        vs[1] = u.v[1] * Sm;
+                        vs[2] = u.v[2] * Sm;
+                    }
+                    Storage<S>::st(fout + lk.x, post + feq_change<R>(s_dir[i][0], s_dir[i][1], s_dir[i][2], s_dir[i][3], dP, vs, m.v));
                 }
-                Storage<S>::st(fout + lk.x, post + feq_change<R>(i, dP, vs, m.v));
-            }
-            if (closed && P.kind == BC_LV) {
-                __syncthreads();
-                for (int k = tid; k < n_cells; k += THREADS) {
-                    double *v0 = q.v0 + 3 * (size_t)(P.xf_off + k);
-                    v0s[k] = xf[k];
-                    for (int a = 0; a < 3; a++) v0[a] = (double)xf[k].v[a];
+                // the ghosts are pulled, and xf rewritten, by these threads only
+                asm volatile("bar.sync 2, %0;" ::"n"(WORK) : "memory");
+                if (closed && P.kind == BC_LV) {
+                    for (int k = tid; k < n_cells; k += WORK) {
+                        double *v0 = q.v0 + 3 * (size_t)(P.xf_off + k);
+                        v0s[k] = xf[k];
+                        for (int a = 0; a < 3; a++) v0[a] = (double)xf[k].v[a];
+                    }
+                    asm volatile("bar.sync 2, %0;" ::"n"(WORK) : "memory");
+                }
+            } else if (ta < PREP) {
+                if (s + 1 < sp.n_steps) ahead(s + 1);
+            } else {
+                if (ta == PREP) {  // the state of t_{n+1} and the waveform row, as bc_step stores them
+                    const BcState st = s_st;
+                    q.state[(size_t)((n + 1) & 1) * q.n_bc_total + b] = st;
+                    double *wv = q.wave + ((size_t)(n % q.wave_cap) * q.n_bc_total + b) * 4;
+                    wv[0] = st.Qu;
+                    wv[1] = st.Pbar - 1.0 / 3.0;
+                    wv[2] = (P.kind == BC_RCR) ? st.Pw : (P.kind == BC_LV ? st.Pv : st.Pstar_gauge);
+                    wv[3] = st.valve_open;
+                    if (io_out)
+                        state_row(st, P, q.etab, n + 1, sp.io_states + 8 * ((size_t)s * sp.io_nb + (b - sp.io_b0)));
                 }
             }
         }
@@ -301,24 +356,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
         fin = fout;
         fout = const_cast<S *>(t);
         __syncwarp();
-        cluster.barrier_arrive();  // this step's populations are visible to the cluster after the wait
-        if (owner) {
-            if (tid == THREADS - AHEAD - 32) {  // the state of t_{n+1} and the waveform row, as bc_step stores them
-                const long long n = first + s;
-                const BcState st = s_st;
-                q.state[(size_t)((n + 1) & 1) * q.n_bc_total + b] = st;
-                double *wv = q.wave + ((size_t)(n % q.wave_cap) * q.n_bc_total + b) * 4;
-                wv[0] = st.Qu;
-                wv[1] = st.Pbar - 1.0 / 3.0;
-                wv[2] = (s_P.kind == BC_RCR) ? st.Pw : (s_P.kind == BC_LV ? st.Pv : st.Pstar_gauge);
-                wv[3] = st.valve_open;
-                if (io_out)
-                    state_row(st, s_P, q.etab, n + 1, sp.io_states + 8 * ((size_t)s * sp.io_nb + (b - sp.io_b0)));
-            }
-            if (ta >= 0 && s + 1 < sp.n_steps) ahead(s + 1);
-        }
-        __syncwarp();
-        cluster.barrier_wait();
+        cluster.barrier_wait();  // the other blocks' populations of this step are visible
     }
     // the last cluster to finish advances the step counter (all have read it)
     if (rank == 0 && tid == 0) {
