@@ -90,6 +90,16 @@ __device__ __forceinline__ void vec_atomic_add(double4a *a, double4a v) {
 // of a ring.  The group's partial velocities are summed with butterfly
 // shuffles, which every lane evaluates in the same order, so all lanes
 // compute the same penalty force; lane 0 writes the node state.
+//
+// The kernel is bound by the L1 (73 % busy on the aorta: a load of 32 cells in
+// 32 different lines takes 32 tag cycles).  With four threads per node and FP32
+// arithmetic the gather therefore goes across the planes' lanes: lane q takes
+// cell dx = q of every line, four lanes one 64-byte run, the line bases and masks
+// by shuffle from the lane that owns the plane.  Aorta step 222.6 -> 217.5 us
+// (FP32), 191.9 -> 186.9 (FP16); in FP64, bound by its pipe, it was slower (2,202
+// -> 2,216 us).  The spreading keeps the planes on the lanes: neighbouring
+// nodes' atomics then rarely meet in one instruction.
+//
 // The kernel takes the wall nodes ib.order[k0 .. k1) (all nodes in index
 // order when ib.order is null).
 //
@@ -109,6 +119,7 @@ __global__ void __launch_bounds__(128) k_ib_nodes(KParams p, IbKParams ib, int k
     using V = typename Vec4<R>::T;
     constexpr int PL = 4 / TPN;
     constexpr bool PAIRED = TPN >= 2;
+    constexpr bool ACROSS = TPN == 4 && sizeof(R) == 4;  // the gather takes the cells of a line on neighbouring lanes
     const int gt = blockIdx.x * blockDim.x + threadIdx.x;
     const int kk = k0 + gt / TPN, q = gt % TPN;
     // the lanes of a node leave together; with pairs, those of a pair (a
@@ -196,6 +207,7 @@ __global__ void __launch_bounds__(128) k_ib_nodes(KParams p, IbKParams ib, int k
                     const uint64_t word = bit < 64 ? m0 : bit < 128 ? m1 : bit < 192 ? m2 : m3;
                     const bool ok = (word >> (bit & 63)) & 1ull;  // else a wall or boundary slot: no fluid
                     valid |= (uint64_t)ok << (dx + 4 * (dy + 4 * j));
+                    if (ACROSS) continue;
                     // branch-free, so that the loads can all be in flight: a
                     // missing cell reads slot 0 (zeroed at creation, finite)
                     // with weight 0
@@ -209,8 +221,29 @@ __global__ void __launch_bounds__(128) k_ib_nodes(KParams p, IbKParams ib, int k
         }
     }
     if (out_of_band && !dead) atomicOr(p.status, 2u);
-    if (dead) valid = 0;
     const unsigned grp = TPN > 1 ? ((1u << TPN) - 1u) << ((threadIdx.x & 31) & ~(TPN - 1)) : 0u;
+    if (ACROSS && !out_of_band) {
+        // lane q takes cell dx = q of all 16 support lines, whose bases and masks
+        // come from the lane that owns their plane
+        const R wx = q == 0 ? w[0][0] : q == 1 ? w[0][1] : q == 2 ? w[0][2] : w[0][3];
+        const int x = i0[0] + q - 1;
+#pragma unroll
+        for (int dz = 0; dz < 4; dz++) {
+            const uint32_t m = __shfl_sync(grp, (uint32_t)valid, dz, TPN) >> q;
+#pragma unroll
+            for (int dy = 0; dy < 4; dy++) {
+                const int base = __shfl_sync(grp, lb[dy], dz, TPN);
+                const bool ok = (m >> (4 * dy)) & 1u;
+                // a missing cell reads slot 0 (finite) with weight 0
+                const V v = vb[ok ? base + x : 0];
+                const R dd = ok ? wx * (w[1][dy] * w[2][dz]) : R(0);
+                vx += v.x * dd;
+                vy += v.y * dd;
+                vz += v.z * dd;
+            }
+        }
+    }
+    if (dead) valid = 0;
     if (TPN > 1) {
 #pragma unroll
         for (int o = 1; o < TPN; o <<= 1) {
