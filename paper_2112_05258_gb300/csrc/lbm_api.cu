@@ -748,6 +748,7 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
     h->kp.aux = h->aux;
     h->kp.step = h->step_dev;
     h->kp.status = h->status;
+    h->kp.keep = exceeds_l2((size_t)NQ * n * h->sbytes, h->device);
     h->bp.n_bc_total = (int)L.bc.size();
     h->bp.par = h->bc_par;
     h->bp.state = h->bc_state;

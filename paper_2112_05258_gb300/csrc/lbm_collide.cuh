@@ -53,6 +53,7 @@ __device__ __forceinline__ Moments<R> collide_store(const Out &out, const KParam
     const R vv = vx * vx + vy * vy + vz * vz;
     if (!(sd - sd == R(0)) || !(vv <= R(0.09))) atomicOr(p.status, 1u);
 
+    const uint64_t keep = keep_in_l2(p.keep);
     const R om1 = R(1) - omega;
     const R K = sd - R(1.5) * vv;
     // per weight class (1/18 faces, 1/36 edges): omega w K, 9/2 omega w, 3 omega w
@@ -69,7 +70,7 @@ __device__ __forceinline__ Moments<R> collide_store(const Out &out, const KParam
     }
     R post0 = om1 * f[0] + omega * R(1.0 / 3.0) * K;
     if (FORCED) post0 -= (R(1) - R(0.5) * omega) * vb;  // w_0 (1 - omega/2) (-3 v.b), w_0 = 1/3
-    Storage<S>::st(out(0, c), post0);
+    st_keep(out(0, c), post0, keep);
 #pragma unroll
     for (int q = 0; q < NP; q++) {
         const int i = 2 * q + 1;
@@ -94,8 +95,8 @@ __device__ __forceinline__ Moments<R> collide_store(const Out &out, const KParam
             A += kw * (R(9) * eu * eb - R(3) * vb);
             B += R(3) * kw * eb;
         }
-        Storage<S>::st(out(i, c), om1 * f[i] + (A + B));
-        Storage<S>::st(out(i + 1, c), om1 * f[i + 1] + (A - B));
+        st_keep(out(i, c), om1 * f[i] + (A + B), keep);
+        st_keep(out(i + 1, c), om1 * f[i + 1] + (A - B), keep);
     }
     return Moments<R>{sd, jx, jy, jz};
 }

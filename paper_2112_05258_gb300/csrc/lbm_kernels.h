@@ -25,7 +25,12 @@ struct KParams {
     void *aux;                  // first-layer macros (sum s, jx, jy, jz), compute type, 4 x n
     long long *step;            // index t_n of the step in progress
     unsigned *status;           // bit 0: NaN/Inf or |v| > 0.3 seen
+    bool keep;                  // one buffer of populations exceeds the L2 (keep_in_l2)
 };
+inline bool exceeds_l2(size_t bytes, int device) {
+    int l2 = 0;
+    return cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, device) == cudaSuccess && bytes > (size_t)l2;
+}
 
 // 0D boundary tables (device memory).  The boundary work of a step runs as
 // two kernels: k_bc_reduce (one CTA per chunk of BC_CHUNK first-layer cells
