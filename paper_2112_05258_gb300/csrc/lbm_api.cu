@@ -652,7 +652,8 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
         if (ok) ok = ck(cudaMemset(h->f[k], 0, pop_bytes), "memset");
     }
     if (ok) ok = ck(dalloc_bytes(h, &h->b, 4 * n * h->rbytes), "b") && ck(cudaMemset(h->b, 0, 4 * n * h->rbytes), "memset");
-    if (ok) ok = ck(dalloc_bytes(h, &h->aux, 4 * n * h->rbytes), "aux") && ck(cudaMemset(h->aux, 0, 4 * n * h->rbytes), "memset");
+    if (ok) ok = ck(dalloc_bytes(h, &h->aux, 4 * (size_t)population_cells((int64_t)n) * h->rbytes), "aux") &&
+                 ck(cudaMemset(h->aux, 0, 4 * (size_t)population_cells((int64_t)n) * h->rbytes), "memset");
     if (ok) ok = ck(upload(h, &h->flags, L.flags), "flags");
     if (ok) ok = ck(upload(h, &h->rows, L.rows), "rows");
     if (ok) ok = ck(upload(h, &h->chunk_row, L.chunk_row), "chunks");
@@ -738,7 +739,8 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
         lbm_status s = h->err.find("out of memory") != std::string::npos ? LBM_ERR_OOM : LBM_ERR_CUDA;
         return bail(s, h->err);
     }
-    h->kp.n = (long long)n;
+    h->kp.n = (long long)population_cells((int64_t)n);
+    h->kp.cells = (int)n;
     h->kp.flags = h->flags;
     h->kp.rows = h->rows;
     h->kp.chunk_row = h->chunk_row;
@@ -1258,15 +1260,21 @@ struct CkptHeader {
     char magic[8];
     int64_t version, prec, n_stored, n_bc, n_ib, n_xf, wave_cap, steps, parity;
 };
-struct CkptSection {
+struct CkptSection {  // rows of row_bytes on the device, pitch apart; packed in the checkpoint
     void *dev;
-    size_t bytes;
+    size_t row_bytes, rows = 1, pitch = 0;
+    size_t bytes() const { return row_bytes * rows; }
+    cudaError_t copy(void *packed, bool save) const {
+        const size_t p = rows > 1 ? pitch : row_bytes;
+        return save ? cudaMemcpy2D(packed, row_bytes, dev, p, row_bytes, rows, cudaMemcpyDeviceToHost)
+                    : cudaMemcpy2D(dev, p, packed, row_bytes, row_bytes, rows, cudaMemcpyHostToDevice);
+    }
 };
 std::vector<CkptSection> ckpt_sections(lbm_handle *h) {
     const Layout &L = h->L;
     const size_t n = (size_t)L.n_stored, nb = L.bc.size(), ns = L.ib_dA.size();
     std::vector<CkptSection> v = {
-        {h->f[h->parity], (size_t)NQ * (size_t)population_cells((int64_t)n) * h->sbytes},
+        {h->f[h->parity], n * (size_t)h->sbytes, NQ, (size_t)population_cells((int64_t)n) * h->sbytes},
         {h->b, 4 * n * (size_t)h->rbytes},
         {h->bc_state, 2 * std::max<size_t>(nb, 1) * sizeof(BcState)},
         {h->v0, 3 * std::max<size_t>(1, L.xf.size()) * sizeof(double)},
@@ -1305,7 +1313,7 @@ CkptHeader ckpt_header(const lbm_handle *h) {
 lbm_status lbm_checkpoint_size(lbm_handle *h, int64_t *bytes) {
     if (!h || !bytes) return fail(h, LBM_ERR_ARG, "bad arguments");
     size_t total = sizeof(CkptHeader);
-    for (auto &sct : ckpt_sections(h)) total += sct.bytes;
+    for (auto &sct : ckpt_sections(h)) total += sct.bytes();
     *bytes = (int64_t)total;
     return LBM_OK;
 }
@@ -1321,8 +1329,8 @@ lbm_status lbm_checkpoint_save(lbm_handle *h, void *buf, int64_t bytes) {
     memcpy(p, &hd, sizeof hd);
     p += sizeof hd;
     for (auto &sct : ckpt_sections(h)) {
-        CK(h, cudaMemcpy(p, sct.dev, sct.bytes, cudaMemcpyDeviceToHost));
-        p += sct.bytes;
+        if (sct.bytes()) CK(h, sct.copy(p, true));
+        p += sct.bytes();
     }
     return LBM_OK;
 }
@@ -1343,8 +1351,8 @@ lbm_status lbm_checkpoint_load(lbm_handle *h, const void *buf, int64_t bytes) {
     h->steps = hd.steps;
     const uint8_t *p = static_cast<const uint8_t *>(buf) + sizeof hd;
     for (auto &sct : ckpt_sections(h)) {
-        CK(h, cudaMemcpy(sct.dev, p, sct.bytes, cudaMemcpyHostToDevice));
-        p += sct.bytes;
+        if (sct.bytes()) CK(h, sct.copy(const_cast<uint8_t *>(p), false));
+        p += sct.bytes();
     }
     return LBM_OK;
 }

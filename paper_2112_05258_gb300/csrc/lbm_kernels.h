@@ -15,7 +15,8 @@ template <> struct Vec4<double> { using T = double4a; };
 
 // Lattice-wide pointers shared by the kernels (device memory).
 struct KParams {
-    long long n;                // stored cells = population stride
+    long long n;                // stride of the population and aux arrays (population_cells)
+    int cells;                  // stored cells
     const uint32_t *flags;      // per cell
     const RowInfo *rows;        // rows + sentinel
     const int32_t *chunk_row;   // per 32-cell chunk: {row of its first cell, new-row lane mask}

@@ -127,7 +127,7 @@ template <class S> static PopDirs<S> pop_dirs(const void *fin, void *fout, long 
 
 cudaError_t launch_stream_collide(int prec, const void *fin, void *fout, const KParams &p, int block,
                                   int variant, cudaStream_t s, int desc, int c0, int c1, int bump, bool early) {
-    if (c1 < 0) c1 = (int)p.n;
+    if (c1 < 0) c1 = p.cells;
     if (c1 <= c0) return cudaSuccess;
     if (block % 32) return cudaErrorInvalidValue;  // whole warps: the forcing branch is a warp vote
     const int cpt = kVariants[variant][1];
