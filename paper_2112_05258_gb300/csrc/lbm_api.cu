@@ -433,7 +433,6 @@ lbm_status read_gather(lbm_handle *h, int inst, bool with_f) {
     const int c0 = (int)h->L.inst_cell_begin[inst], c1 = (int)h->L.inst_cell_end[inst];
     CK(h, launch_gather(h->prec, h->f[h->parity], h->kp, c0, c1, with_f ? h->rd_f19 : nullptr, h->rd_mac,
                         h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
     return LBM_OK;
 }
 
@@ -1051,12 +1050,13 @@ lbm_status lbm_read_fields(lbm_handle *h, int inst, double *P, double *jx, doubl
     const int64_t c0 = L.inst_cell_begin[inst], c1 = L.inst_cell_end[inst];
     const size_t M = (size_t)(c1 - c0);
     std::vector<double> mac(4 * M);
-    CK(h, cudaMemcpy(mac.data(), h->rd_mac, 4 * M * sizeof(double), cudaMemcpyDeviceToHost));
     const lbm_instance_desc &d = h->inst[inst];
     const size_t nbox = (size_t)d.nx * d.ny * d.nz;
     double *outs[4] = {P, jx, jy, jz};
+    for (double *o : outs) std::fill(o, o + nbox, 0.0);  // while the GPU finishes
+    CK(h, cudaStreamSynchronize(h->stream));
+    CK(h, cudaMemcpy(mac.data(), h->rd_mac, 4 * M * sizeof(double), cudaMemcpyDeviceToHost));
     for (int k = 0; k < 4; k++) {
-        std::fill(outs[k], outs[k] + nbox, 0.0);
         for (size_t m = 0; m < M; m++) outs[k][L.cell_box[c0 + m]] = mac[k * M + m];
     }
     return LBM_OK;
@@ -1082,10 +1082,11 @@ lbm_status lbm_read_populations(lbm_handle *h, int inst, double *f) {
     const lbm_instance_desc &d = h->inst[inst];
     const size_t nbox = (size_t)d.nx * d.ny * d.nz;
     std::vector<double> tmp(M);
+    std::fill(f, f + NQ * nbox, 0.0);  // while the GPU finishes
+    CK(h, cudaStreamSynchronize(h->stream));
     for (int i = 0; i < NQ; i++) {
         CK(h, cudaMemcpy(tmp.data(), h->rd_f19 + i * M, M * sizeof(double), cudaMemcpyDeviceToHost));
         double *o = f + i * nbox;
-        std::fill(o, o + nbox, 0.0);
         for (size_t m = 0; m < M; m++) o[L.cell_box[c0 + m]] = tmp[m];
     }
     return LBM_OK;
@@ -1222,11 +1223,11 @@ lbm_status lbm_wall_shear(lbm_handle *h, int inst, double *wss) {
     if (!h->rd_mac) CK(h, dalloc(h, &h->rd_mac, 4 * (size_t)h->max_inst_cells));
     CK(h, launch_wall_shear(h->prec, h->f[h->parity], h->kp, (int)c0, (int)c1, h->rd_mac, h->stream));
     std::vector<double> tmp(3 * M);
-    CK(h, cudaMemcpyAsync(tmp.data(), h->rd_mac, 3 * M * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
     const lbm_instance_desc &d = h->inst[inst];
     const size_t nbox = (size_t)d.nx * d.ny * d.nz;
-    std::fill(wss, wss + 3 * nbox, 0.0);
+    std::fill(wss, wss + 3 * nbox, 0.0);  // while the GPU finishes
+    CK(h, cudaMemcpyAsync(tmp.data(), h->rd_mac, 3 * M * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    CK(h, cudaStreamSynchronize(h->stream));
     for (size_t m = 0; m < M; m++)
         for (int a = 0; a < 3; a++) wss[3 * (size_t)L.cell_box[c0 + m] + a] = tmp[a * M + m];
     return LBM_OK;

@@ -220,7 +220,8 @@ __global__ void k_axi_gather(const S *__restrict__ fin, Params p, double *f9, do
     const uint32_t fl = p.flags[c];
     const int n = p.n, x = c % p.nx, j = c / p.nx;
     if (!(fl & AF_FLUID)) {
-        for (int i = 0; i < Q9; i++) f9[(size_t)i * n + c] = 0.0;
+        if (f9)
+            for (int i = 0; i < Q9; i++) f9[(size_t)i * n + c] = 0.0;
         mac3[c] = mac3[n + c] = mac3[2 * n + c] = 0.0;
         return;
     }
@@ -232,7 +233,7 @@ __global__ void k_axi_gather(const S *__restrict__ fin, Params p, double *f9, do
         else if (j - er(i) < 0) src = mir(i) * n + (x - ex(i));
         else src = i * n + c - ex(i) - er(i) * p.nx;
         s[i] = (double)Storage<S>::ld(fin + src);
-        f9[(size_t)i * n + c] = s[i] + wgt(i);
+        if (f9) f9[(size_t)i * n + c] = s[i] + wgt(i);
         sd += s[i];
         jx += ex(i) * s[i];
         jr += er(i) * s[i];
@@ -1205,26 +1206,28 @@ lbm_status lbm_axi_sync(lbm_axi_handle *h) {
     return LBM_OK;
 }
 
-static lbm_status gather(lbm_axi_handle *h) {
+// f(t_n) (with_f) and P, u_x, u_r into the read-out scratch, in stream order
+static lbm_status gather(lbm_axi_handle *h, bool with_f) {
     ACK(h, cudaSetDevice(h->device));
     const Params p = params(h);
     const int grid = (h->n + 255) / 256;
     if (h->prec == LBM_F64)
-        k_axi_gather<double><<<grid, 256, 0, h->stream>>>(static_cast<const double *>(h->f[h->parity]), p, h->rd,
+        k_axi_gather<double><<<grid, 256, 0, h->stream>>>(static_cast<const double *>(h->f[h->parity]), p, with_f ? h->rd : nullptr,
                                                           h->rd + (size_t)Q9 * h->n);
     else
-        k_axi_gather<float><<<grid, 256, 0, h->stream>>>(static_cast<const float *>(h->f[h->parity]), p, h->rd,
+        k_axi_gather<float><<<grid, 256, 0, h->stream>>>(static_cast<const float *>(h->f[h->parity]), p, with_f ? h->rd : nullptr,
                                                          h->rd + (size_t)Q9 * h->n);
     ACK(h, cudaGetLastError());
-    ACK(h, cudaStreamSynchronize(h->stream));
     return LBM_OK;
 }
 
 lbm_status lbm_axi_read_fields(lbm_axi_handle *h, double *P, double *ux, double *ur) {
     if (!h || !P || !ux || !ur) return afail(h, LBM_ERR_ARG, "null array");
-    lbm_status s = gather(h);
+    lbm_status s = gather(h, false);
     if (s != LBM_OK) return s;
     const size_t n = h->n, o = (size_t)Q9 * n;
+    for (double *a : {P, ux, ur}) touch_pages(a, n * sizeof(double));
+    ACK(h, cudaStreamSynchronize(h->stream));
     ACK(h, cudaMemcpy(P, h->rd + o, n * sizeof(double), cudaMemcpyDeviceToHost));
     ACK(h, cudaMemcpy(ux, h->rd + o + n, n * sizeof(double), cudaMemcpyDeviceToHost));
     ACK(h, cudaMemcpy(ur, h->rd + o + 2 * n, n * sizeof(double), cudaMemcpyDeviceToHost));
@@ -1233,8 +1236,10 @@ lbm_status lbm_axi_read_fields(lbm_axi_handle *h, double *P, double *ux, double 
 
 lbm_status lbm_axi_read_populations(lbm_axi_handle *h, double *f) {
     if (!h || !f) return afail(h, LBM_ERR_ARG, "null array");
-    lbm_status s = gather(h);
+    lbm_status s = gather(h, true);
     if (s != LBM_OK) return s;
+    touch_pages(f, (size_t)Q9 * h->n * sizeof(double));
+    ACK(h, cudaStreamSynchronize(h->stream));
     ACK(h, cudaMemcpy(f, h->rd, (size_t)Q9 * h->n * sizeof(double), cudaMemcpyDeviceToHost));
     return LBM_OK;
 }

@@ -13,6 +13,14 @@ template <> struct Vec4<float> { using T = float4; };
 struct alignas(32) double4a { double x, y, z, w; };
 template <> struct Vec4<double> { using T = double4a; };
 
+// Writes a byte into every page of a host array that is about to be filled, so
+// that its page faults (10 ms for 300 MB) pass while the GPU still works.
+inline void touch_pages(void *p, size_t bytes) {
+    volatile char *c = static_cast<volatile char *>(p);
+    for (size_t k = 0; k < bytes; k += 4096) c[k] = 0;
+    if (bytes) c[bytes - 1] = 0;
+}
+
 // Lattice-wide pointers shared by the kernels (device memory).
 struct KParams {
     long long n;                // stride of the population and aux arrays (population_cells)
