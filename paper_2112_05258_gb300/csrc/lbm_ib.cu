@@ -500,17 +500,19 @@ cudaError_t launch_ib_nodes(int prec, const KParams &p, const IbKParams &ib, int
     return cudaGetLastError();
 }
 
+cudaError_t launch_filaments(int prec, const KParams &p, const IbKParams &ib, cudaStream_t st) {
+    if (ib.n_fil == 0) return cudaSuccess;
+    if (prec == 3)
+        k_filament<false><<<ib.n_fil, FIL_THREADS, filament_smem(ib.max_fil), st>>>(p, ib);
+    else
+        k_filament<true><<<ib.n_fil, FIL_THREADS, filament_smem(ib.max_fil), st>>>(p, ib);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_ib(int prec, const void *fin, const KParams &p, const IbKParams &ib, cudaStream_t st, bool band) {
     if (ib.n_nodes == 0) return cudaSuccess;
     cudaError_t e = band ? launch_band_moments(prec, fin, p, ib, 0, ib.n_band, st) : cudaSuccess;
     if (e == cudaSuccess) e = launch_ib_nodes(prec, p, ib, 0, ib.n_nodes, st);
-    if (e == cudaSuccess && ib.n_fil) {
-        if (prec == 3)
-            k_filament<false><<<ib.n_fil, FIL_THREADS, filament_smem(ib.max_fil), st>>>(p, ib);
-        else
-            k_filament<true><<<ib.n_fil, FIL_THREADS, filament_smem(ib.max_fil), st>>>(p, ib);
-        e = cudaGetLastError();
-    }
     return e;
 }
 
