@@ -116,8 +116,9 @@ struct lbm_handle {
         cudaGraphExec_t exec;
     };
     std::vector<IoGraph> io_graphs;
-    // small lattices: many steps in one launch, a cluster of blocks per instance (0: one-step kernels)
-    int small_cluster = 0;
+    // small lattices: many steps in one launch of so many blocks, clusters or a
+    // grid (0: one-step kernels)
+    int small_blocks = 0;
     size_t small_smem = 0;
     SmallKParams small{};
     // kernel timing
@@ -473,8 +474,7 @@ void drop_graphs(lbm_handle *h) {
 cudaError_t set_up_small(lbm_handle *h) {
     const Layout &L = h->L;
     if (!L.ib_dA.empty() || L.n_fluid == 0) return cudaSuccess;
-    for (int64_t n : L.inst_fluid)
-        if (small_smem_bulk((int)std::min<int64_t>(n / 16, 1 << 20)) > SMALL_MAX_SMEM) return cudaSuccess;
+    if (L.n_fluid > 160 * 2700) return cudaSuccess;  // beyond the shared memory of all blocks
     std::vector<int32_t> bulk, off;
     int64_t worst_bulk[17] = {0};
     size_t smem_b = 0;
@@ -502,14 +502,14 @@ cudaError_t set_up_small(lbm_handle *h) {
             worst_bulk[C] = std::max(worst_bulk[C], (n + C - ip.n_bc - 1) / (C - ip.n_bc));
     }
     off.push_back((int32_t)bulk.size());
-    // Times of a step in us, measured on GB300 over tubes of 2,400 to 110,000
+    // Times of a step in us, measured on GB300 over tubes of 900 to 320,000
     // cells.  This kernel: as many rounds as the clusters need, each the longer
     // of the boundary block (latency: 3.1 us and its first layer's share; FP64
     // runs on a pipe of 2 lanes an SM) and of a bulk block's cells.  One-step
-    // kernels: launches and latencies of 12 us (FP64: 20), then bandwidth.
+    // kernels: launches and latencies of 12 us (FP64: 21), then bandwidth.
     const bool f64 = h->prec == LBM_F64;
     const double cells = (double)L.n_fluid;
-    const double one_step = std::max(f64 ? 20.0 : 12.0, (f64 ? 16.0 : 9.0) + cells * (f64 ? 240e-6 : 30e-6));
+    const double one_step = std::max(f64 ? 21.0 : 12.0, (f64 ? 16.0 : 9.0) + cells * (f64 ? 240e-6 : 30e-6));
     double best = 0.9 * one_step;
     for (int C : {16, 8}) {
         if (C <= most_bc) continue;
@@ -527,13 +527,44 @@ cudaError_t set_up_small(lbm_handle *h) {
         const double t = rounds * std::max(owner, bulk);
         if (t >= best) continue;
         best = t;
-        h->small_cluster = C;
+        h->small.cluster = C;
+        h->small_blocks = C * (int)L.inst.size();
         h->small_smem = smem;
     }
-    if (!h->small_cluster) return cudaSuccess;
+    // One grid over all instances, if that beats the better of the two (by 5 %, as
+    // it takes more SMs): a boundary block as above (FP32: another pass beyond 768
+    // cells), and as many bulk blocks as are done a little earlier, if the shared
+    // memory of those takes their cells; the other SMs stay free for other streams.
+    // (Three FP32 tubes of 176,407 cells stepped at once on three streams take turns:
+    // 7.3 to 8.7 us a step of one of them, where one-step kernels overlap to 7.1;
+    // one alone 7.2 instead of 12.4, beside a stream of long kernels 16 instead of 328.)
+    int sms = 0, per_sm = 0;
+    const int nb = (int)L.bc.size();
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    if (e == cudaSuccess && nb < sms) {
+        const double owner = f64 ? std::max(6.6 + 0.048 * worst_xf, 1.7 + 0.084 * worst_xf)
+                                 : 3.1 + 0.0071 * worst_xf + 1.4 * (std::max(worst_xf - 1, 0) / 768);
+        const double b0 = f64 ? 1.5 : 2.05, b1 = f64 ? 34.5e-3 : 2.63e-3, n = (double)bulk.size();
+        const double fit = std::min((0.9 * owner - b0) / b1, f64 ? 2500.0 : 2600.0);
+        const int w = (int)std::max(1.0, std::min((double)(sms - nb), std::ceil(n / fit)));
+        const double per = std::ceil(n / w), t = std::max(owner, b0 + b1 * per);
+        const size_t smem = std::max(smem_b, small_smem_grid((int)per, f64));
+        if (t < 0.95 * (h->small_blocks ? best : one_step) && smem <= SMALL_MAX_SMEM) {
+            if (prepare_small(h->prec, 0, smem, &per_sm) == cudaSuccess && per_sm >= 1) {
+                h->small.cluster = 0;
+                h->small_blocks = nb + w;
+                h->small_smem = smem;
+            }
+            (void)cudaGetLastError();
+        }
+    }
+    if (e != cudaSuccess || !h->small_blocks) return e;
     int32_t *d_bulk = nullptr, *d_off = nullptr;
     int *done = nullptr;
-    cudaError_t e = upload(h, &d_bulk, bulk);
+    unsigned *meet = nullptr;
+    if (e == cudaSuccess) e = upload(h, &d_bulk, bulk);
+    if (e == cudaSuccess) e = dalloc(h, &meet, 1);
+    if (e == cudaSuccess) e = cudaMemset(meet, 0, sizeof(unsigned));
     if (e == cudaSuccess) e = upload(h, &d_off, off);
     if (e == cudaSuccess) e = dalloc(h, &done, 1);
     if (e == cudaSuccess) e = cudaMemset(done, 0, sizeof(int));
@@ -541,6 +572,8 @@ cudaError_t set_up_small(lbm_handle *h) {
     h->small.bulk = d_bulk;
     h->small.bulk_off = d_off;
     h->small.done = done;
+    h->small.meet = meet;
+    h->small.n_inst = (int)L.inst.size();
     h->small.par = h->bc_par;
     return e;
 }
@@ -549,10 +582,14 @@ cudaError_t set_up_small(lbm_handle *h) {
 // steps); io: per-step params and state rows of lbm_step_io, or null.
 lbm_status small_steps(lbm_handle *h, int64_t n, const SmallKParams *io = nullptr) {
     SmallKParams sp = io ? *io : h->small;
+    // refused as the step graphs of the other lattices are: a replay would pass the host's step count by
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    CK(h, cudaStreamIsCapturing(h->stream, &capture));
+    if (capture != cudaStreamCaptureStatusNone) return fail(h, LBM_ERR_CUDA, "the stream is being captured");
     while (n > 0) {
         sp.n_steps = (int)std::min<int64_t>(n, SMALL_MAX_STEPS);
-        CK(h, launch_small(h->prec, h->f[h->parity], h->f[1 - h->parity], h->kp, h->bp, sp, (int)h->inst.size(),
-                           h->small_cluster, h->small_smem, h->stream));
+        CK(h, launch_small(h->prec, h->f[h->parity], h->f[1 - h->parity], h->kp, h->bp, sp, h->small_blocks,
+                           h->small_smem, h->stream));
         if (sp.n_steps & 1) h->parity ^= 1;
         h->steps += sp.n_steps;
         n -= sp.n_steps;
@@ -969,7 +1006,7 @@ lbm_status lbm_step(lbm_handle *h, int64_t n) {
         }
         return LBM_OK;
     }
-    if (h->small_cluster) return small_steps(h, n);
+    if (h->small_blocks) return small_steps(h, n);
     int64_t left = n;
     while (left >= h->graph_steps) {
         lbm_status s = ensure_graph(h);
@@ -1012,7 +1049,7 @@ lbm_status lbm_step_io(lbm_handle *h, int inst, int bc, int64_t n, const double 
         pdev = static_cast<const double *>(a.devicePointer);
         sdev = static_cast<double *>(c.devicePointer);
     }
-    if (h->small_cluster && !h->timing) {
+    if (h->small_blocks && !h->timing) {
         SmallKParams sp = h->small;
         sp.io_params = pdev;
         sp.io_states = sdev;
@@ -1058,6 +1095,7 @@ lbm_status lbm_sync(lbm_handle *h) {
     unsigned s = 0;
     CK(h, cudaMemcpy(&s, h->status, sizeof s, cudaMemcpyDeviceToHost));
     if (s & 1u) return fail(h, LBM_ERR_UNSTABLE, "NaN/Inf or |v| > 0.3 in the lattice");
+    if (s & 4u) return fail(h, LBM_ERR_CUDA, "the blocks of a multi-step kernel did not meet in time");
     if (s & 2u) return fail(h, LBM_ERR_UNSTABLE, "a wall node moved outside its immersed-boundary band");
     return LBM_OK;
 }
@@ -1498,7 +1536,7 @@ lbm_status lbm_get_info(lbm_handle *h, lbm_info_t *info) {
     if (h->overlap)  // band velocities as the two lists (an empty list launches nothing)
         info->launches_per_step += (h->n_band_ind > 0) + (h->n_band_dep > 0) - 1;
     info->graph_steps = h->graph_steps;
-    info->steps_per_launch = h->small_cluster ? SMALL_MAX_STEPS : 0;
+    info->steps_per_launch = h->small_blocks ? SMALL_MAX_STEPS : 0;
     return LBM_OK;
 }
 

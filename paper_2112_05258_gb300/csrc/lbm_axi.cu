@@ -1159,6 +1159,12 @@ lbm_status lbm_axi_step(lbm_axi_handle *h, int64_t nsteps) {
     if (!h || nsteps < 0) return afail(h, LBM_ERR_ARG, "bad arguments");
     ACK(h, cudaSetDevice(h->device));
     int64_t done = 0;
+    if (h->small_cluster) {  // refused where the step graph of the other grids is
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        ACK(h, cudaStreamIsCapturing(h->stream, &capture));
+        if (capture != cudaStreamCaptureStatusNone && nsteps - h->parity >= h->graph_steps)
+            return afail(h, LBM_ERR_CUDA, "the stream is being captured");
+    }
     while (h->small_cluster && done < nsteps) {
         const int k = (int)std::min<int64_t>(nsteps - done, AXI_MAX_STEPS);
         ACK(h, small_launch(h, nullptr, k));

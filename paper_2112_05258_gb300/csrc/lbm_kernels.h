@@ -118,7 +118,7 @@ struct IbKParams {
 };
 
 // Small lattices: n_steps steps of every instance in one launch, one cluster
-// of blocks per instance (lbm_small.cu).
+// of blocks per instance or one grid over all (lbm_small.cu).
 constexpr int SMALL_MAX_RED = 8;          // chunks of a boundary's first layer
 constexpr int SMALL_MAX_STEPS = 4096;     // steps per launch
 constexpr size_t SMALL_MAX_SMEM = 212000; // dynamic shared memory of a block, beside 17 KB of static
@@ -126,7 +126,10 @@ struct SmallKParams {
     const InstParam *inst;
     const int32_t *bulk;      // fluid cells outside the first layers, instance by instance
     const int32_t *bulk_off;  // per instance, and the end
-    int *done;                // clusters finished (back to 0 after the launch)
+    int *done;                // blocks finished (back to 0 after the launch)
+    unsigned *meet;           // grid: arrivals at the barrier (back to 0 after the launch)
+    int cluster;              // blocks per instance, or 0: one grid over all instances
+    int n_inst;
     int n_steps;
     // per-step 0D input and output of lbm_step_io (null: none): np params of
     // boundary io_b per step, state rows of boundaries io_b0 .. io_b0 + io_nb - 1
@@ -137,10 +140,12 @@ struct SmallKParams {
 };
 size_t small_smem_boundary(int n_xf, int n_links, int n_nodes, bool f64);
 size_t small_smem_bulk(int cells);
-// admits the kernel's shared memory and cluster size; *clusters: how many run at once
-cudaError_t prepare_small(int prec, int cluster, size_t smem, int *clusters);
+size_t small_smem_grid(int cells, bool f64);
+// admits the kernel's shared memory and cluster size; *at_once: how many clusters
+// run at once, or (cluster = 0) blocks of the grid per SM
+cudaError_t prepare_small(int prec, int cluster, size_t smem, int *at_once);
 cudaError_t launch_small(int prec, void *f0, void *f1, const KParams &p, const BcKParams &q, const SmallKParams &sp,
-                         int n_inst, int cluster, size_t smem, cudaStream_t st);
+                         int blocks, size_t smem, cudaStream_t st);
 
 // variants {min resident 256-thread blocks per SM, cells per thread}:
 // 0 {6, 1} (40 registers), 1 {8, 1} (32), 2 {5, 1} (48), 3 {4, 2}, 4 {3, 2}

@@ -1,9 +1,11 @@
 // Many steps of small lattices in one launch (no wall nodes).  A thread-block
 // cluster takes one instance and advances it n steps, its populations staying
 // in L2; the hardware cluster barrier separates the steps, so a step costs
-// neither launches nor the gaps between them.
+// neither launches nor the gaps between them.  Lattices that are too large for
+// clusters of 16 blocks, up to what the shared memory of all SMs takes (about
+// 390,000 cells), are one cooperative grid with a barrier in global memory.
 //
-// Work of a cluster of C blocks on an instance with B 0D boundaries:
+// Work of the C blocks of an instance (grid: of all instances) with B 0D boundaries:
 //   * block k < B owns boundary k: it collides the cells of its first fluid
 //     layer, sums flow and pressure over them (from registers), takes the 0D
 //     step and writes the ghosts of t_{n+1}.  Ghosts are pulled only by
@@ -31,6 +33,16 @@
 // area and the compliance (quotient).
 // A step: 12.4 -> 4.1 us for that tube, 12.1 -> 3.5 us for 2,400 cells (FP32), 20.7
 // -> 10.1 us in FP64 (whose collision is bound by the FP64 pipe).
+//
+// The grid: its barrier makes a step 0.4 us longer than a cluster's (3.9 against
+// 3.5 us for 14,112 cells).  Its latency is kept out of the boundary block's
+// chain: one thread outside the 0D step announces the layer's populations as soon
+// as they are stored, and polls beside the ghosts (a fence in each thread and a
+// poll after the ghosts: 5.1 us).  Bulk blocks take about 2.05 us and 2.6 ns a
+// cell (L2 and issue).
+// A step of one-step kernels -> of the grid, FP32: 49,928 cells 9.4 -> 5.6 us,
+// 106,920 11.6 -> 6.8, 176,407 12.4 -> 7.2, 323,176 14.5 -> 10.8; 16 instances of
+// 14,112 10.4 (clusters) -> 6.9; FP64: 12,896 21.7 -> 18.1, 176,407 64.8 -> 47.4.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -83,6 +95,74 @@ template <class R> struct FirstLayer {  // of one first-layer cell: velocity and
 
 constexpr int PULLS = NQ - 1;
 
+// The barrier between the steps, arrived at by every warp and waited for later:
+// the hardware barrier of a cluster, or, for a whole grid (cooperative launch:
+// all blocks are resident), a counter in global memory.  There one thread
+// outside the 0D step adds the block, after a __syncthreads() behind its stores,
+// polls the counter and releases the block's warps through an mbarrier.  Every
+// wait is bounded: when one runs out (seconds; a step takes microseconds) the
+// status word says so and the block leaves its loop.
+template <bool GRID, int THREADS> struct StepBarrier;
+template <int THREADS> struct StepBarrier<false, THREADS> {
+    struct Shared {};
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    __device__ StepBarrier(Shared &, const SmallKParams &, unsigned *) {}
+    __device__ __forceinline__ void arrive() { cluster.barrier_arrive(); }
+    __device__ __forceinline__ bool wait() {
+        cluster.barrier_wait();
+        return true;
+    }
+};
+template <int THREADS> struct StepBarrier<true, THREADS> {
+    struct Shared {
+        unsigned long long bar;
+        int failed;
+    };
+    static constexpr int POLLER = THREADS - 32;
+    static constexpr int POLLS = 1 << 22, TRIES = 1 << 30;  // a warp never gives up before the polling thread has
+    Shared &s;
+    unsigned *count, *status, target = 0, phase = 0;
+    __device__ StepBarrier(Shared &sh, const SmallKParams &sp, unsigned *st) : s(sh), count(sp.meet), status(st) {
+        if (threadIdx.x == 0) {
+            s.failed = 0;
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(address()) : "memory");
+        }
+    }
+    __device__ __forceinline__ uint32_t address() const { return (uint32_t)__cvta_generic_to_shared(&s.bar); }
+    // after a __syncthreads() behind the block's stores
+    __device__ __forceinline__ void arrive() {
+        if (threadIdx.x == POLLER) {
+            __threadfence();
+            atomicAdd(count, 1u);
+        }
+    }
+    __device__ __forceinline__ bool wait() {
+        target += gridDim.x;
+        if (threadIdx.x == POLLER) {
+            unsigned v = 0;
+            int k = 0;
+            do asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+            while ((int)(v - target) < 0 && ++k < POLLS);
+            if (k == POLLS) {
+                atomicOr(status, 4u);
+                s.failed = 1;
+            }
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(address()) : "memory");
+        }
+        uint32_t done = 0;
+        for (int k = 0; k < TRIES && !done; k++)
+            asm volatile(
+                "{\n.reg .pred p;\n"
+                "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                "selp.u32 %0, 1, 0, p;\n}\n"
+                : "=r"(done)
+                : "r"(address()), "r"(phase)
+                : "memory");
+        phase ^= 1u;
+        return done && !*(volatile int *)&s.failed;
+    }
+};
+
 }  // namespace
 
 // Shared memory of a block.  Boundary block: per first-layer cell the pull
@@ -94,12 +174,15 @@ size_t small_smem_boundary(int n_xf, int n_links, int n_nodes, bool f64) {
     return (size_t)n_xf * (PULLS * 4 + 4 + 8 * r) + (size_t)n_links * 8 + (size_t)n_nodes * (24 + 2 * r) + 64;
 }
 size_t small_smem_bulk(int cells) { return (size_t)cells * (PULLS * 4 + 4) + 64; }
+size_t small_smem_grid(int cells, bool f64) { return (size_t)cells * (PULLS * 4 + 4 + (f64 ? 8 : 4)) + 64; }
 
-template <class S, int THREADS>
+// GRID: one grid over all instances instead of a cluster per instance (larger
+// lattices): block b < n_bc_total owns boundary b, the others share the bulk.
+template <class S, int THREADS, bool GRID>
 __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParams p, BcKParams q, SmallKParams sp) {
     using R = typename Storage<S>::R;
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ typename StepBarrier<GRID, THREADS>::Shared s_bar;
+    StepBarrier<GRID, THREADS> barrier(s_bar, sp, p.status);
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ double sQ[THREADS], sP[THREADS], s_part[2 * SMALL_MAX_RED], s_cos, s_sin;
     __shared__ BcStepResult s_r;
@@ -109,14 +192,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
     __shared__ double s_area, s_inv_area, s_third;  // n_xf, 1 / n_xf and n_xf / 3
     __shared__ int s_euler;
     __shared__ R s_dir[NQ][4];  // e_i and w_i
-    const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-    const int inst = blockIdx.x / C;
-    const InstParam &ip = sp.inst[inst];
-    const int nb = ip.n_bc, N = (int)p.n;
-    const int tid = threadIdx.x;
-    const R omega = omega_of<R>(p, inst);
+    // C blocks share the instances inst .. of which the first nb own boundaries b0 ..
+    const int C = GRID ? (int)gridDim.x : sp.cluster, rank = (int)blockIdx.x % C, inst = (int)blockIdx.x / C;
+    const int nb = GRID ? q.n_bc_total : sp.inst[inst].n_bc, b0 = GRID ? 0 : sp.inst[inst].bc_first;
+    const int N = (int)p.n, tid = threadIdx.x;
     const bool owner = rank < nb;
-    const int b = ip.bc_first + rank;
+    const int b = b0 + rank;
     const long long first = *p.step + 1;  // t_n of the first step of the launch
 
     // cells of this block and their pull tables
@@ -127,14 +208,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
         __syncthreads();
         n_cells = s_P.n_xf;
     } else {
-        const int lo = sp.bulk_off[inst], n = sp.bulk_off[inst + 1] - lo, w = C - nb, k = rank - nb;
+        const int lo = sp.bulk_off[inst], n = sp.bulk_off[GRID ? sp.n_inst : inst + 1] - lo, w = C - nb, k = rank - nb;
         const int per = (n + w - 1) / w;
         cell0 = lo + min(k * per, n);
         n_cells = lo + min((k + 1) * per, n) - cell0;
     }
+    const R omega = omega_of<R>(p, !GRID ? inst : owner ? s_P.inst : 0);
     int *tab = reinterpret_cast<int *>(smem);       // [18][n_cells]
     int *cell = tab + PULLS * n_cells;              // [n_cells]
     FirstLayer<R> *xf = reinterpret_cast<FirstLayer<R> *>((reinterpret_cast<uintptr_t>(cell + n_cells) + 15) & ~(uintptr_t)15);
+    R *om = reinterpret_cast<R *>(xf);                // bulk of a grid: 1/tau of each cell
     FirstLayer<R> *v0s = xf + (owner ? n_cells : 0);  // closure velocities
     int2 *link = reinterpret_cast<int2 *>(v0s + (owner ? n_cells : 0));
     double *prof = reinterpret_cast<double *>(link + (owner ? s_P.n_links : 0));  // velocity inlet: 3 per node
@@ -144,6 +227,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
         const int c = owner ? q.xf[s_P.xf_off + k] : sp.bulk[cell0 + k];
         cell[k] = c;
         pull_offsets(p, c, p.flags[c], tab + k, n_cells);
+        if (GRID && !owner) om[k] = omega_of<R>(p, p.rows[find_row(p, c)].inst);
         if (owner) {
             const double *v0 = q.v0 + 3 * (size_t)(s_P.xf_off + k);
             v0s[k] = FirstLayer<R>{{(R)v0[0], (R)v0[1], (R)v0[2]}, R(0)};
@@ -216,6 +300,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
     S *fout = f1;
     for (int s = 0; s < sp.n_steps; s++) {
         const OneBase<S> out{fout, N};
+        const bool end = GRID && s + 1 == sp.n_steps;  // a grid needs no barrier after the last step
         if (!owner) {
             for (int k = tid; k < n_cells; k += THREADS) {
                 const int c = cell[k];
@@ -223,10 +308,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
                 f[0] = PlainLoad<S>::ld(fin + c);
 #pragma unroll
                 for (int i = 1; i < NQ; i++) f[i] = PlainLoad<S>::ld(fin + tab[(i - 1) * n_cells + k]);
-                collide_store<S, R, false>(out, p, f, omega, 0u, c);
+                collide_store<S, R, false>(out, p, f, GRID ? om[k] : omega, 0u, c);
             }
+            if (GRID) __syncthreads();
             __syncwarp();
-            cluster.barrier_arrive();
+            if (!end) barrier.arrive();
         } else {
             const BcParam &P = s_P;
             const long long n = first + s;
@@ -263,9 +349,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
                     if ((tid & 31) == 0) s_part[2 * ch + (w < CH ? 0 : 1)] = a;
                 }
                 __syncwarp();
-                if (last && w >= 2 * CH) cluster.barrier_arrive();
+                if (!GRID && last && w >= 2 * CH) barrier.arrive();
                 __syncthreads();
-                if (last && w > 0 && w < 2 * CH) cluster.barrier_arrive();
+                if (last && (GRID || (w > 0 && w < 2 * CH)) && !end) barrier.arrive();
             }
             // the thread's first two links (from the second warp on), their
             // populations in flight beside the 0D step
@@ -300,7 +386,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
                 }
             }
             __syncthreads();
-            if (tid < 32) cluster.barrier_arrive();
+            if (!GRID && tid < 32) barrier.arrive();
             if (tid < WORK) {
                 const BcStepResult &r = s_r;
                 const bool closed = r.closed != 0, ptype = r.ptype != 0;
@@ -356,13 +442,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
         fin = fout;
         fout = const_cast<S *>(t);
         __syncwarp();
-        cluster.barrier_wait();  // the other blocks' populations of this step are visible
+        if (!end && !barrier.wait()) break;  // the other blocks' populations of this step are visible
     }
-    // the last cluster to finish advances the step counter (all have read it)
-    if (rank == 0 && tid == 0) {
+    // the last block to finish advances the step counter (all have read it; in a
+    // grid, none still polls)
+    __syncthreads();
+    if (tid == 0) {
         __threadfence();
-        if (atomicAdd(sp.done, 1) == (int)(gridDim.x / C) - 1) {
+        if (atomicAdd(sp.done, 1) == (int)gridDim.x - 1) {
             *sp.done = 0;
+            if (GRID) *sp.meet = 0u;
             *p.step = first + sp.n_steps - 1;
         }
     }
@@ -372,51 +461,57 @@ namespace {
 
 template <class S> constexpr int small_threads() { return sizeof(typename Storage<S>::R) == 8 ? 512 : 1024; }
 
-template <class S> cudaError_t prepare(int cluster, size_t smem, int *clusters) {
-    auto k = k_small_steps<S, small_threads<S>()>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess && cluster > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
+// cluster blocks per instance, or (cluster = 0) one cooperative grid
+template <class S>
+cudaLaunchConfig_t config(int cluster, int blocks, size_t smem, cudaStream_t st, cudaLaunchAttribute *at) {
     cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim = {(unsigned)cluster, 1, 1};
-    cfg.gridDim = dim3(cluster);
-    cfg.blockDim = dim3(small_threads<S>());
-    cfg.dynamicSmemBytes = smem;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    return cudaOccupancyMaxActiveClusters(clusters, k, &cfg);
-}
-
-template <class S> cudaError_t launch(void *f0, void *f1, const KParams &p, const BcKParams &q, const SmallKParams &sp,
-                                      int n_inst, int cluster, size_t smem, cudaStream_t st) {
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim = {(unsigned)cluster, 1, 1};
-    cfg.gridDim = dim3((unsigned)(n_inst * cluster));
+    if (cluster) {
+        at->id = cudaLaunchAttributeClusterDimension;
+        at->val.clusterDim = {(unsigned)cluster, 1, 1};
+    } else {
+        at->id = cudaLaunchAttributeCooperative;
+        at->val.cooperative = 1;
+    }
+    cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(small_threads<S>());
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cfg.attrs = &at;
+    cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_small_steps<S, small_threads<S>()>, static_cast<S *>(f0), static_cast<S *>(f1), p,
-                              q, sp);
+    return cfg;
+}
+
+template <class S> cudaError_t prepare(int cluster, size_t smem, int *at_once) {
+    const auto k = cluster ? k_small_steps<S, small_threads<S>(), false> : k_small_steps<S, small_threads<S>(), true>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_MAX_SMEM);
+    if (e == cudaSuccess && cluster > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    if (!cluster) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(at_once, k, small_threads<S>(), smem);
+    cudaLaunchAttribute at{};
+    const cudaLaunchConfig_t cfg = config<S>(cluster, cluster, smem, nullptr, &at);
+    return cudaOccupancyMaxActiveClusters(at_once, k, &cfg);
+}
+
+template <class S> cudaError_t launch(void *f0, void *f1, const KParams &p, const BcKParams &q, const SmallKParams &sp,
+                                      int blocks, size_t smem, cudaStream_t st) {
+    const auto k = sp.cluster ? k_small_steps<S, small_threads<S>(), false> : k_small_steps<S, small_threads<S>(), true>;
+    cudaLaunchAttribute at{};
+    const cudaLaunchConfig_t cfg = config<S>(sp.cluster, blocks, smem, st, &at);
+    return cudaLaunchKernelEx(&cfg, k, static_cast<S *>(f0), static_cast<S *>(f1), p, q, sp);
 }
 
 }  // namespace
 
-cudaError_t prepare_small(int prec, int cluster, size_t smem, int *clusters) {
+cudaError_t prepare_small(int prec, int cluster, size_t smem, int *at_once) {
     cudaError_t e = cudaSuccess;
-    DISPATCH(prec, e = prepare<S>(cluster, smem, clusters));
+    DISPATCH(prec, e = prepare<S>(cluster, smem, at_once));
     return e;
 }
 
 cudaError_t launch_small(int prec, void *f0, void *f1, const KParams &p, const BcKParams &q, const SmallKParams &sp,
-                         int n_inst, int cluster, size_t smem, cudaStream_t st) {
+                         int blocks, size_t smem, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
-    DISPATCH(prec, e = launch<S>(f0, f1, p, q, sp, n_inst, cluster, smem, st));
+    DISPATCH(prec, e = launch<S>(f0, f1, p, q, sp, blocks, smem, st));
     return e;
 }
 

@@ -1,7 +1,8 @@
 """The multi-step kernel of small lattices against the one-step kernels (taken
 while kernel timing is on): the same trajectory bit for bit, for every kind of
 0D boundary, marching order, storage type, first layers of one to five chunks
-of 256 cells, batches, per-step 0D input, and launches split at the step limit.
+of 256 cells, batches, per-step 0D input, and launches split at the step limit;
+with a cluster of blocks per instance and with one grid over all instances.
 """
 import numpy as np
 import pytest
@@ -39,6 +40,19 @@ CASES = {
     "five_chunks": lambda: [configs.rigid_tube(41, 41, 12, radius=18.3)],
     "batch": lambda: [configs.lv_tube(period=300), _box(), _lv(6.3, 41), configs.rigid_tube(16, 16, 24, radius=5.0)],
 }
+# sizes at which the rule takes one grid: a few blocks, all of them, instances of
+# different sizes and relaxation times, no boundary at all
+GRID = {
+    "lv": lambda: [_lv(8.0, 131)],
+    "lv_order4": lambda: [_order(_lv(13.0, 203), 4)],
+    "velocity": lambda: [configs.rigid_tube(31, 31, 170, radius=11.4)],
+    "pressure": lambda: [configs.pressure_tube(30, 30, 150, 12.6, 0.8, 2e-3, 0.0)],
+    "two_passes": lambda: [_lv(16.2, 310)],
+    "box": lambda: [Instance(node=geometry.closed_box(61, 47, 53), tau=0.7, name="box")],
+    "uneven": lambda: [_lv(6.0, 128), Instance(node=geometry.closed_box(31, 17, 53), tau=0.7, name="box"),
+                       _lv(12.0, 200), configs.rigid_tube()],
+}
+CASES.update({"grid_" + k: v for k, v in GRID.items()})
 
 
 def _pair(insts, precision, steps):
@@ -78,8 +92,9 @@ def test_multi_step_kernel_equals_one_step_kernels(name, precision):
     _same(a, b, insts)
 
 
-def test_multi_step_kernel_fp64_and_long_calls():
-    insts = [configs.lv_tube(period=300)]
+@pytest.mark.parametrize("inst", [lambda: configs.lv_tube(period=300), lambda: configs.rigid_tube()])
+def test_multi_step_kernel_fp64_and_long_calls(inst):
+    insts = [inst()]
     a, b = _pair(insts, "f64", (4 * 300 + 1, 3001))   # the second call goes past the steps of one launch
     n = a.info().steps_per_launch
     a.step(n + 5)
@@ -87,10 +102,12 @@ def test_multi_step_kernel_fp64_and_long_calls():
     _same(a, b, insts)
 
 
-def test_step_io_of_a_velocity_inlet_equals_per_step_calls():
+@pytest.mark.parametrize("inst", [lambda: configs.rigid_tube(), GRID["velocity"]])
+def test_step_io_of_a_velocity_inlet_equals_per_step_calls(inst):
     import torch
     from paper_2112_05258_gb300 import Lattice
-    inst = configs.rigid_tube()
+    inst = inst()
+    inst = inst[0] if isinstance(inst, list) else inst
     n = 90
     omega = torch.tensor(2 * np.pi / (1000.0 + 5.0 * np.arange(n)).reshape(n, 1)).pin_memory()
     rows = torch.zeros((n, 16), dtype=torch.float64, pin_memory=True)
@@ -111,15 +128,15 @@ def test_step_io_of_a_velocity_inlet_equals_per_step_calls():
 
 def test_large_or_elastic_lattices_keep_the_step_graphs():
     from paper_2112_05258_gb300 import Lattice
-    for inst in (configs.ib_tube(), _lv(13.0, 200)):
+    for inst in (configs.ib_tube(), _lv(13.0, 800)):
         assert Lattice([inst]).info().steps_per_launch == 0
 
 
 WIDE = {
-    "lv": lambda: _lv(13.0, 200),
-    "lv_order4": lambda: _order(_lv(12.2, 190), 4),
-    "velocity": lambda: configs.rigid_tube(31, 31, 170, radius=11.4),
-    "pressure": lambda: configs.pressure_tube(30, 30, 150, 12.6, 0.8, 2e-3, 0.0),
+    "lv": lambda: _lv(13.0, 770),
+    "lv_order4": lambda: _order(_lv(12.2, 881), 4),
+    "velocity": lambda: configs.rigid_tube(31, 31, 1003, radius=11.4),
+    "pressure": lambda: configs.pressure_tube(30, 30, 818, 12.6, 0.8, 2e-3, 0.0),
 }
 
 
