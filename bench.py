@@ -73,12 +73,15 @@ def launches(info, steps):
     """Kernel launches of `steps` steps taken as lbm_step does them: small
     lattices in one launch per steps_per_launch steps, others in whole step
     graphs, then single-step graphs for the rest; a graph's first step (and a
-    single step) issues launches_first_step, its later steps launches_per_step."""
+    single step) issues launches_first_step, its later steps launches_per_step; a
+    batch's graphs do so once per part, after one launch more."""
     if getattr(info, "steps_per_launch", 0):
         return -(-steps // info.steps_per_launch)
     g = info.graph_steps
     full, rest = divmod(steps, g)
-    return full * (info.launches_first_step + (g - 1) * info.launches_per_step) + rest * info.launches_first_step
+    parts = getattr(info, "parts", 1)
+    graph = parts * (info.launches_first_step + (g - 1) * info.launches_per_step) + (parts > 1)
+    return full * graph + rest * info.launches_first_step
 
 
 def dist_env():

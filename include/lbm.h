@@ -159,6 +159,8 @@ typedef struct {
     int graph_steps;         /* steps per step graph */
     int steps_per_launch;    /* small lattices take the steps of an lbm_step call in one kernel launch per this many
                                 steps, without step graphs; 0: step graphs as above */
+    int parts;               /* a batch's step graphs advance so many parts of its instances beside one another,
+                              each with launches of its own, after one launch per graph (1: whole) */
 } lbm_info_t;
 
 /* Sizes of the layout lbm_create would build (see lbm_check_config). */

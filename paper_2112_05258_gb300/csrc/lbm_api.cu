@@ -102,6 +102,30 @@ struct lbm_handle {
     // membrane tube of 64 x 64 x 512 with 151 filaments 109.6 -> 95.9 us per step
     // (FP16 99.2 -> 85.7, FP64 776 -> 761).
     cudaStream_t s_fil = nullptr;
+    // A batch's step graphs advance up to four parts of its instances, each a chain
+    // of its own (the instances do not meet): while one part's boundary kernels
+    // run, bound by latency, the others' stream-collide uses the memory.  A part
+    // counts its steps itself.  The boundary kernels have the higher priority:
+    // without it they wait until the other parts' stream-collide blocks are all
+    // dispatched, and the gain is lost (64 tubes of 14,112 cells in two parts 31.2 us
+    // per step, with it 28.8, in one part 30.2).  In 1, 2, 3, 4, 6 parts: those
+    // tubes 30.2, 28.7, 26.8, 26.2, 27.6 us per step (FP16 23.0, 22.3, 19.4, 17.7, 18.2;
+    // FP64 230, 227, 215, 210, 210), 96 uneven tubes 486, 474, 474, 476, 478 (FP16 370,
+    // 357, 356, 356, 358), 8 tubes of 106,920 cells 35.7, 29.0, 27.1, 27.4.
+    static constexpr int MAX_PARTS = 4;
+    struct Part {
+        int c0 = 0, c1 = 0;
+        KParams kp{};
+        BcKParams bp{};
+        cudaStream_t stream = nullptr;  // the first: the lattice's
+        cudaEvent_t done = nullptr;
+    };
+    // (64 tubes of 14,112 cells: building a graph of 100 steps in four parts takes
+    // 1.3 ms more than of whole steps, one of 20 less; the rejoining costs 0.3 us a step)
+    std::vector<Part> parts;     // empty: one chain
+    int part_steps = 0;          // steps of their graph: the first even divisor of graph_steps from 16 on
+    cudaEvent_t ev_parts = nullptr;
+    long long *step_parts = nullptr;
     cudaEvent_t ev_nodes = nullptr, ev_fil = nullptr;
     cudaEvent_t ev_ofork = nullptr, ev_oband = nullptr, ev_obc = nullptr;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
@@ -349,13 +373,36 @@ lbm_status launch_step(lbm_handle *h, bool timed, bool band_done = false, bool n
     return LBM_OK;
 }
 
+// part_steps steps of a lattice's parts, each on a stream of its own (captured)
+lbm_status launch_parts(lbm_handle *h) {
+    CK(h, launch_spread_step(h->step_dev, h->step_parts, (int)h->parts.size(), h->stream));
+    CK(h, cudaEventRecord(h->ev_parts, h->stream));
+    for (size_t q = 1; q < h->parts.size(); q++) CK(h, cudaStreamWaitEvent(h->parts[q].stream, h->ev_parts, 0));
+    for (int k = 0; k < h->part_steps; k++) {
+        for (auto &a : h->parts) {
+            cudaStream_t st = a.stream ? a.stream : h->stream;
+            void *fin = h->f[h->parity], *fout = h->f[1 - h->parity];
+            CK(h, launch_stream_collide(h->prec, fin, fout, a.kp, h->block, h->variant, st, h->parity, a.c0, a.c1, 1,
+                                        a.bp.cluster != 0));
+            CK(h, launch_boundary(h->prec, fout, a.kp, a.bp, BcIo{}, st));
+        }
+        h->parity ^= 1;
+    }
+    for (size_t q = 1; q < h->parts.size(); q++) {
+        CK(h, cudaEventRecord(h->parts[q].done, h->parts[q].stream));
+        CK(h, cudaStreamWaitEvent(h->stream, h->parts[q].done, 0));
+    }
+    return LBM_OK;
+}
+
 lbm_status ensure_graph(lbm_handle *h) {
     const int par = h->parity;
     if (h->graph[par]) return LBM_OK;
     cudaGraph_t g = nullptr;
     CK(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
     lbm_status st = LBM_OK;
-    for (int k = 0; k < h->graph_steps && st == LBM_OK; k++)
+    if (!h->parts.empty()) st = launch_parts(h);
+    for (int k = 0; k < h->graph_steps && st == LBM_OK && h->parts.empty(); k++)
         st = launch_step(h, false, k > 0 && h->overlap, k + 1 < h->graph_steps && h->overlap);
     cudaError_t e = cudaStreamEndCapture(h->stream, &g);
     h->parity = par;  // capture does not run anything
@@ -804,7 +851,7 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
     h->kp.step = h->step_dev;
     h->kp.status = h->status;
     h->kp.keep = exceeds_l2((size_t)NQ * n * h->sbytes, h->device);
-    h->bp.n_bc_total = (int)L.bc.size();
+    h->bp.n_bc_total = h->bp.n_bc = (int)L.bc.size();
     h->bp.par = h->bc_par;
     h->bp.state = h->bc_state;
     h->bp.xf = h->xf;
@@ -920,6 +967,51 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
         h->overlap = true;
     }
     if (!ck(set_up_small(h), "small-lattice tables")) return bail(LBM_ERR_CUDA, h->err);
+    if (!ns && !h->small_blocks && L.inst.size() > 1) {
+        const int K = (int)std::min<size_t>(L.inst.size(), lbm_handle::MAX_PARTS);
+        int lo = 0, hi = 0;
+        if (!(ck(dalloc(h, &h->step_parts, K), "step") &&
+              ck(cudaDeviceGetStreamPriorityRange(&lo, &hi), "stream priorities") &&
+              ck(cudaEventCreateWithFlags(&h->ev_parts, cudaEventDisableTiming), "events")))
+            return bail(LBM_ERR_CUDA, h->err);
+        h->parts.reserve(K);
+        h->part_steps = std::min(16, h->graph_steps);
+        while (h->graph_steps % h->part_steps || h->part_steps % 2) h->part_steps++;
+        size_t m = 0;  // part k: the instances [m, e), its end where about k + 1 of K cells are
+        for (int k = 0; k < K; k++) {
+            size_t e = m + 1;
+            auto off = [&](size_t q) { return std::llabs(K * L.inst_cell_end[q - 1] - (k + 1) * (int64_t)n); };
+            while (e + (K - 1 - k) < L.inst.size() && off(e + 1) < off(e)) e++;
+            if (k == K - 1) e = L.inst.size();
+            h->parts.emplace_back();
+            lbm_handle::Part &a = h->parts.back();
+            a.c0 = (int)L.inst_cell_begin[m];
+            a.c1 = (int)L.inst_cell_end[e - 1];
+            a.kp = h->kp;
+            a.bp = h->bp;
+            a.bp.priority = hi;
+            a.bp.bc0 = L.inst[m].bc_first;
+            const int b1 = L.inst[e - 1].bc_first + L.inst[e - 1].n_bc;
+            a.bp.n_bc = b1 - a.bp.bc0;
+            auto at = [](const std::vector<int32_t> &v, int bc) {
+                return (int)(std::lower_bound(v.begin(), v.end(), bc) - v.begin());
+            };
+            const int r0 = at(L.red_bc, a.bp.bc0), a0 = at(L.app_bc, a.bp.bc0);
+            a.bp.n_red_blocks = at(L.red_bc, b1) - r0;
+            a.bp.n_app_blocks = at(L.app_bc, b1) - a0;
+            a.bp.red_bc += r0;
+            a.bp.red_chunk += r0;
+            a.bp.app_bc += a0;
+            a.bp.app_chunk += a0;
+            if (k) {
+                a.kp.step = h->step_parts + k;
+                if (!(ck(cudaStreamCreateWithFlags(&a.stream, cudaStreamNonBlocking), "streams") &&
+                      ck(cudaEventCreateWithFlags(&a.done, cudaEventDisableTiming), "events")))
+                    return bail(LBM_ERR_CUDA, h->err);
+            }
+            m = e;
+        }
+    }
     if (h->ibp.n_fil && !(ck(cudaStreamCreateWithFlags(&h->s_fil, cudaStreamNonBlocking), "streams") &&
                           ck(cudaEventCreateWithFlags(&h->ev_nodes, cudaEventDisableTiming), "events") &&
                           ck(cudaEventCreateWithFlags(&h->ev_fil, cudaEventDisableTiming), "events")))
@@ -1008,12 +1100,13 @@ lbm_status lbm_step(lbm_handle *h, int64_t n) {
     }
     if (h->small_blocks) return small_steps(h, n);
     int64_t left = n;
-    while (left >= h->graph_steps) {
+    const int per = h->parts.empty() ? h->graph_steps : h->part_steps;
+    while (left >= per) {
         lbm_status s = ensure_graph(h);
         if (s != LBM_OK) return s;
         CK(h, cudaGraphLaunch(h->graph[h->parity], h->stream));
-        left -= h->graph_steps;
-        h->steps += h->graph_steps;
+        left -= per;
+        h->steps += per;
     }
     for (; left > 0; left--) {
         lbm_status s = ensure_graph1(h);
@@ -1535,7 +1628,8 @@ lbm_status lbm_get_info(lbm_handle *h, lbm_info_t *info) {
     info->launches_first_step = info->launches_per_step;
     if (h->overlap)  // band velocities as the two lists (an empty list launches nothing)
         info->launches_per_step += (h->n_band_ind > 0) + (h->n_band_dep > 0) - 1;
-    info->graph_steps = h->graph_steps;
+    info->graph_steps = h->parts.empty() ? h->graph_steps : h->part_steps;
+    info->parts = std::max(1, (int)h->parts.size());
     info->steps_per_launch = h->small_blocks ? SMALL_MAX_STEPS : 0;
     return LBM_OK;
 }
@@ -1559,6 +1653,11 @@ void lbm_destroy(lbm_handle *h) {
     for (auto e : {h->ev_ofork, h->ev_oband, h->ev_obc, h->ev_nodes, h->ev_fil})
         if (e) cudaEventDestroy(e);
     if (h->s_fil) cudaStreamDestroy(h->s_fil);
+    for (auto &a : h->parts) {
+        if (a.stream) cudaStreamDestroy(a.stream);
+        if (a.done) cudaEventDestroy(a.done);
+    }
+    if (h->ev_parts) cudaEventDestroy(h->ev_parts);
     if (h->s_band) cudaStreamDestroy(h->s_band);
     if (h->s_bc) cudaStreamDestroy(h->s_bc);
     if (h->s_node) cudaStreamDestroy(h->s_node);

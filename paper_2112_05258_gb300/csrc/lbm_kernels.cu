@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(BS) k_boundary(S *__restrict__ f, KParams p, B
     __shared__ int s_euler;
     cluster.barrier_arrive();  // waited for before the first block writes into the others
     let_next_start();
-    const int CL = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), b = blockIdx.x / CL;
+    const int CL = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), b = q.bc0 + blockIdx.x / CL;
     const int tid = threadIdx.x;
     const size_t N = (size_t)p.n;
     const R *aux = static_cast<const R *>(p.aux);
@@ -534,21 +534,23 @@ __global__ void k_cycle_change(BcKParams q, const int *bc_first, const int *n_bc
 template <class S, int BS>
 static cudaError_t boundary_in_one(void *f, const KParams &p, const BcKParams &q, const BcIo &io, cudaStream_t s) {
     cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at[2] = {};
+    cudaLaunchAttribute at[3] = {};
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim = {(unsigned)q.cluster, 1, 1};
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_early
     at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)(q.n_bc_total * q.cluster));
+    cfg.gridDim = dim3((unsigned)(q.n_bc * q.cluster));
     cfg.blockDim = dim3(BS);
     cfg.stream = s;
+    at[2].id = cudaLaunchAttributePriority;
+    at[2].val.priority = q.priority;
     cfg.attrs = at;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = q.priority ? 3 : 2;
     return cudaLaunchKernelEx(&cfg, k_boundary<S, BS>, as<S>(f), p, q, io);
 }
 
 cudaError_t launch_boundary(int prec, void *f, const KParams &p, const BcKParams &q, const BcIo &io, cudaStream_t s) {
-    if (q.n_bc_total == 0) return cudaSuccess;
+    if (q.n_bc == 0) return cudaSuccess;
     if (q.cluster) {
         cudaError_t e = cudaSuccess;
         if (q.wide) {
@@ -558,14 +560,25 @@ cudaError_t launch_boundary(int prec, void *f, const KParams &p, const BcKParams
         }
         return e;
     }
-    if (prec == 3) k_bc_reduce<double><<<q.n_red_blocks, BC_CHUNK, 0, s>>>(p, q);
-    else k_bc_reduce<float><<<q.n_red_blocks, BC_CHUNK, 0, s>>>(p, q);
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributePriority;
+    at.val.priority = q.priority;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)q.n_red_blocks);
+    cfg.blockDim = dim3(BC_CHUNK);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = q.priority ? 1 : 0;
+    cudaError_t e = prec == 3 ? cudaLaunchKernelEx(&cfg, k_bc_reduce<double>, p, q)
+                              : cudaLaunchKernelEx(&cfg, k_bc_reduce<float>, p, q);
+    if (e != cudaSuccess) return e;
+    cfg.gridDim = dim3((unsigned)q.n_app_blocks);
     if (q.step_in_reduce) {
-        DISPATCH(prec, (k_bc_apply<S, false><<<q.n_app_blocks, BC_CHUNK, 0, s>>>(as<S>(f), p, q)));
+        DISPATCH(prec, (e = cudaLaunchKernelEx(&cfg, k_bc_apply<S, false>, as<S>(f), p, q)));
     } else {
-        DISPATCH(prec, (k_bc_apply<S, true><<<q.n_app_blocks, BC_CHUNK, 0, s>>>(as<S>(f), p, q)));
+        DISPATCH(prec, (e = cudaLaunchKernelEx(&cfg, k_bc_apply<S, true>, as<S>(f), p, q)));
     }
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_gather(int prec, const void *fin, const KParams &p, int c0, int c1, double *f19, double *mac4,
@@ -643,6 +656,16 @@ cudaError_t launch_state_rows(const BcState *st, const BcParam *par, const doubl
 __global__ void k_copy_words(const unsigned long long *__restrict__ src, unsigned long long *__restrict__ dst,
                              int n) {
     for (int k = threadIdx.x; k < n; k += blockDim.x) dst[k] = src[k];
+}
+
+// the step counter, copied for each part of a step graph
+__global__ void k_spread_step(const long long *step, long long *out, int n) {
+    if ((int)threadIdx.x < n) out[threadIdx.x] = *step;
+}
+
+cudaError_t launch_spread_step(const long long *step, long long *out, int n, cudaStream_t s) {
+    k_spread_step<<<1, 32, 0, s>>>(step, out, n);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_copy_words(const void *src, void *dst, size_t bytes, cudaStream_t s) {

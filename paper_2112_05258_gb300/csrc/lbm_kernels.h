@@ -59,6 +59,7 @@ struct BcStepResult {
 };
 struct BcKParams {
     int n_bc_total;
+    int bc0, n_bc;              // the boundaries [bc0, bc0 + n_bc) that k_boundary takes (red_*, app_*: the two kernels')
     const BcParam *par;
     BcState *state;             // [2][n_bc_total]: step n reads state[n & 1], writes state[(n + 1) & 1]
     const int32_t *xf;
@@ -73,6 +74,7 @@ struct BcKParams {
     int step_in_reduce;         // 1: the 0D step once per boundary in k_bc_reduce; 0: in every k_bc_apply block
     int *arrived;               // per boundary: reduce CTAs done in this step (back to 0 after it)
     BcStepResult *result;       // per boundary
+    int priority;               // of the launches, where not the stream's (0)
     int cluster, wide;          // blocks per boundary of k_boundary (0: the two kernels), and whether they have 512 threads
     int n_red_blocks, n_app_blocks;
     const int32_t *red_bc, *red_chunk;  // per reduce block
@@ -168,6 +170,7 @@ cudaError_t launch_wall_shear(int prec, const void *fin, const KParams &p, int c
                               cudaStream_t s);
 cudaError_t launch_state_rows(const BcState *st, const BcParam *par, const double *etab, int b0, int nb,
                               int nbc_total, long long steps, double *out8, cudaStream_t s);
+cudaError_t launch_spread_step(const long long *step, long long *out, int n, cudaStream_t s);
 cudaError_t launch_copy_words(const void *src, void *dst, size_t bytes, cudaStream_t s);
 // per-step 0D input and output of lbm_step_io (see k_io_params, k_io_state, k_io_base)
 cudaError_t launch_io_base(const long long *step, long long *base, cudaStream_t s);

@@ -4,6 +4,8 @@
 
 namespace lbm {
 
+constexpr int LINE_CELLS = 64;  // a cache line of 16-bit populations, two of FP32
+
 // One base pointer per direction of the input and output population arrays
 // (f_i = f + i N, structure of arrays), passed in the kernel's parameter
 // space: every pull and store then forms its address with one wide
@@ -43,8 +45,10 @@ template <class S> struct PopDirs {
 // them is consumed.  The variants are kept for the run-time autotuner.
 // desc = 1 maps the blocks to the cells in descending order, so that a
 // launch starts on the lines the previous kernel touched last (still in L2).
-// The launch covers the stored cells [c0, c1); the launch with bump = 1
-// advances the step counter.
+// The launch covers the stored cells [c0, c1), its blocks beginning on whole
+// cache lines (a batch in two parts, the second from an odd cell: 500 us per
+// step, from its cache line 486); the launch with bump = 1 advances the step
+// counter.
 // EARLY: launched while its predecessor, the boundary kernel, still runs (see
 // launch_stream_collide); only tables that no step writes are read before the
 // wait.
@@ -54,7 +58,7 @@ __global__ void __launch_bounds__(256, MINB)
                      int c1, int bump) {
     using R = typename Storage<S>::R;
     const int bid = desc ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
-    const int t = c0 + bid * blockDim.x + threadIdx.x;
+    const int t = (c0 & ~(LINE_CELLS - 1)) + bid * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
     if (!EARLY && bump && t == c0 && p.step) *p.step += 1;  // the step index t_n seen by the boundary kernels
     const int N = (int)p.n;  // 19 N < 2^31 is checked at creation
@@ -64,7 +68,7 @@ __global__ void __launch_bounds__(256, MINB)
 #pragma unroll
     for (int u = 0; u < CPT; u++) {
         const int c = t + u * stride;
-        fl[u] = c < c1 ? __ldg(&p.flags[c]) : 0u;
+        fl[u] = c >= c0 && c < c1 ? __ldg(&p.flags[c]) : 0u;
         om[u] = R(0);
         const bool active = (fl[u] & FL_ACTIVE) != 0;
         if (!EARLY && !active) continue;
@@ -131,7 +135,7 @@ cudaError_t launch_stream_collide(int prec, const void *fin, void *fout, const K
     if (c1 <= c0) return cudaSuccess;
     if (block % 32) return cudaErrorInvalidValue;  // whole warps: the forcing branch is a warp vote
     const int cpt = kVariants[variant][1];
-    const int grid = (int)((c1 - c0 + (long long)block * cpt - 1) / ((long long)block * cpt));
+    const int grid = (int)((c1 - (c0 & ~(LINE_CELLS - 1)) + (long long)block * cpt - 1) / ((long long)block * cpt));
     if (early && variant == 0) {
         cudaError_t e = cudaSuccess;
         DISPATCH(prec, (e = launch_early(k_stream_collide<S, 6, 1, true>, dim3(grid), dim3(block), s,

@@ -188,3 +188,20 @@ def test_step_io_in_the_one_launch_boundary(name, bc, cols):
     assert np.array_equal(rows.numpy(), want.numpy())
     assert np.array_equal(rows.numpy()[:, 0], np.arange(4, 154))
     assert np.array_equal(a.populations(0), b.populations(0))
+
+
+PARTS = {
+    "two": lambda: [_lv(13.0, 450), _lv(12.2, 443)],
+    "one_launch": lambda: [Instance(node=geometry.closed_box(61, 47, 53), tau=0.7, name="box"), _lv(13.0, 203),
+                           _lv(6.3, 41), configs.rigid_tube(31, 31, 170, radius=11.4), _lv(12.2, 301)],
+    "two_kernels": lambda: [_lv(20.3, 171), _lv(6.0, 128), _order(_lv(12.0, 200), 4), _lv(17.7, 77), _lv(9.1, 333)],
+}
+
+
+@pytest.mark.parametrize("precision", ["f32", "bf16", "f64"])
+@pytest.mark.parametrize("name", list(PARTS))
+def test_batch_in_parts_equals_whole_steps(name, precision):
+    insts = PARTS[name]()
+    a, b = _pair(insts, precision, (64, 1, 130, 63, 7))
+    assert a.info().steps_per_launch == 0 and a.info().parts == min(4, len(insts))
+    _same(a, b, insts)
