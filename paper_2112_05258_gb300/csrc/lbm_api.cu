@@ -1012,6 +1012,14 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
             m = e;
         }
     }
+    // Shape of stream-collide, unless the caller sets or tunes one: 16-bit batches
+    // that exceed the L2 take 32 registers and more warps (96 uneven tubes FP16 348 ->
+    // 334 us per step, 48: 161.2 -> 154.6, 24 equal ones 112.5 -> 110.7; a single tube
+    // is no faster, a lattice with wall nodes slower, 183.5 -> 189.9), FP64 without wall
+    // nodes 48 registers, which halves its spills (64 tubes 211.7 -> 210.9, a tube of 1.4 M
+    // cells 338.7 -> 334.9; the aorta is slower, 2,205 -> 2,247).
+    if (h->prec == LBM_F64) h->variant = ns ? 0 : 2;
+    else if (h->sbytes == 2 && h->kp.keep && !h->parts.empty()) h->variant = 1;
     if (h->ibp.n_fil && !(ck(cudaStreamCreateWithFlags(&h->s_fil, cudaStreamNonBlocking), "streams") &&
                           ck(cudaEventCreateWithFlags(&h->ev_nodes, cudaEventDisableTiming), "events") &&
                           ck(cudaEventCreateWithFlags(&h->ev_fil, cudaEventDisableTiming), "events")))

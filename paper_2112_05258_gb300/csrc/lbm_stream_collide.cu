@@ -6,6 +6,28 @@ namespace lbm {
 
 constexpr int LINE_CELLS = 64;  // a cache line of 16-bit populations, two of FP32
 
+// Where the populations exceed the L2, one block of every AHEAD_CELLS cells has
+// the populations of as many cells fetched into the L2, AHEAD_DIST cells before
+// the blocks reach them: the loads of a block wait for the L2 instead of the
+// memory, and the bytes in flight are not bound by the warps' registers (without,
+// FP16 issued 0.55 and stalled on loads for half of its time at 43 warps an SM).
+// One bulk prefetch per direction and block of 128 cells is too many requests for
+// FP16 (364 -> 402 us per step of 96 uneven tubes, FP32 481 -> 468); of 512, 2,048,
+// 4,096, 8,192 cells: FP16 358, 351, 360, 366, FP32 467, 462, 462, 473.  8,192 to
+// 32,768 cells ahead are alike, 131,072 slower (517 with single blocks): what is
+// fetched so early takes the place of what neighbouring planes still need.  Before
+// and after: 96 uneven tubes 481 -> 462 (FP16 364 -> 348), aorta 215.5 -> 212.4 (FP16
+// 187.6 -> 184.0).  The mask comes from the host: a division per thread costs FP16,
+// which is bound by instruction issue then, all of the gain.
+constexpr int AHEAD_CELLS = 2048, AHEAD_DIST = 16384;
+// The blocks that fetch, as a mask of the block index (0: none).
+int ahead_mask(const KParams &p, int block, int cpt) {
+    if (!p.keep || cpt != 1 || p.n % LINE_CELLS) return 0;
+    int per = 1;
+    while (2 * per * block <= AHEAD_CELLS) per *= 2;
+    return per - 1;
+}
+
 // One base pointer per direction of the input and output population arrays
 // (f_i = f + i N, structure of arrays), passed in the kernel's parameter
 // space: every pull and store then forms its address with one wide
@@ -55,13 +77,19 @@ template <class S> struct PopDirs {
 template <class S, int MINB, int CPT, bool EARLY = false>
 __global__ void __launch_bounds__(256, MINB)
     k_stream_collide(const __grid_constant__ PopDirs<S> d, const __grid_constant__ KParams p, int desc, int c0,
-                     int c1, int bump) {
+                     int c1, int bump, int ahead) {
     using R = typename Storage<S>::R;
     const int bid = desc ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
     const int t = (c0 & ~(LINE_CELLS - 1)) + bid * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
     if (!EARLY && bump && t == c0 && p.step) *p.step += 1;  // the step index t_n seen by the boundary kernels
     const int N = (int)p.n;  // 19 N < 2^31 is checked at creation
+    if (CPT == 1 && threadIdx.x < NQ && ahead && (bid & ahead) == 0) {
+        const int s = t - (int)threadIdx.x + (desc ? -AHEAD_DIST : AHEAD_DIST), n = (ahead + 1) * (int)blockDim.x;
+        if (s >= c0 && s < c1 && s + n <= N)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(d.in[0] + ((long long)threadIdx.x * N + s)),
+                         "r"((unsigned)(n * sizeof(S))));
+    }
     R f[CPT][NQ];
     R om[CPT];
     uint32_t fl[CPT];
@@ -136,27 +164,28 @@ cudaError_t launch_stream_collide(int prec, const void *fin, void *fout, const K
     if (block % 32) return cudaErrorInvalidValue;  // whole warps: the forcing branch is a warp vote
     const int cpt = kVariants[variant][1];
     const int grid = (int)((c1 - (c0 & ~(LINE_CELLS - 1)) + (long long)block * cpt - 1) / ((long long)block * cpt));
+    const int ahead = ahead_mask(p, block, cpt);
     if (early && variant == 0) {
         cudaError_t e = cudaSuccess;
         DISPATCH(prec, (e = launch_early(k_stream_collide<S, 6, 1, true>, dim3(grid), dim3(block), s,
-                                         pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump)));
+                                         pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead)));
         return e;
     }
     switch (variant) {
     case 1:
-        DISPATCH(prec, (k_stream_collide<S, 8, 1><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump)));
+        DISPATCH(prec, (k_stream_collide<S, 8, 1><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead)));
         break;
     case 2:
-        DISPATCH(prec, (k_stream_collide<S, 5, 1><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump)));
+        DISPATCH(prec, (k_stream_collide<S, 5, 1><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead)));
         break;
     case 3:
-        DISPATCH(prec, (k_stream_collide<S, 4, 2><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump)));
+        DISPATCH(prec, (k_stream_collide<S, 4, 2><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead)));
         break;
     case 4:
-        DISPATCH(prec, (k_stream_collide<S, 3, 2><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump)));
+        DISPATCH(prec, (k_stream_collide<S, 3, 2><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead)));
         break;
     default:
-        DISPATCH(prec, (k_stream_collide<S, 6, 1><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump)));
+        DISPATCH(prec, (k_stream_collide<S, 6, 1><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead)));
         break;
     }
     return cudaGetLastError();
