@@ -100,7 +100,9 @@ struct lbm_handle {
     // graphs): those read no wall node, and the next node kernel waits for both.
     // The filament kernel is bound by the FP64 pipe, stream-collide by memory:
     // membrane tube of 64 x 64 x 512 with 151 filaments 109.6 -> 95.9 us per step
-    // (FP16 99.2 -> 85.7, FP64 776 -> 761).
+    // (FP16 99.2 -> 85.7), one of 45 x 45 x 24 30.1 -> 23.9.  Not in FP64, where both are
+    // bound by that pipe: 45 x 45 x 24 64.5 -> 79.1, 45 x 45 x 64 106.5 -> 120.9, 64 x 64 x 512
+    // 776 -> 760.
     cudaStream_t s_fil = nullptr;
     // A batch's step graphs advance up to four parts of its instances, each a chain
     // of its own (the instances do not meet): while one part's boundary kernels
@@ -316,7 +318,7 @@ lbm_status launch_step(lbm_handle *h, bool timed, bool band_done = false, bool n
     if (h->n_slab && !timed) return launch_step_slabs(h);
     void *fin = h->f[h->parity], *fout = h->f[1 - h->parity];
     if (h->ibp.n_nodes) CK(h, launch_ib(h->prec, fin, h->kp, h->ibp, h->stream, !band_done));
-    const bool fil_aside = h->ibp.n_fil && h->s_fil && !timed;
+    const bool fil_aside = h->ibp.n_fil && h->s_fil && h->prec != LBM_F64 && !timed;
     if (fil_aside) {
         CK(h, cudaEventRecord(h->ev_nodes, h->stream));
         CK(h, cudaStreamWaitEvent(h->s_fil, h->ev_nodes, 0));
