@@ -200,7 +200,8 @@ lbm_status lbm_init_populations(lbm_handle *h, int inst, const double *f);
 /* Advances all instances by n steps (Algorithm 1).  Asynchronous: returns
  * after enqueueing, as CUDA graphs of graph_steps steps and, for the
  * remainder, single-step graphs (each captured once per step parity); small
- * lattices without wall nodes as one kernel launch (lbm_info_t). */
+ * lattices without wall nodes as one kernel launch per steps_per_launch steps,
+ * batches in parts beside one another (lbm_info_t). */
 lbm_status lbm_step(lbm_handle *h, int64_t n);
 
 /* n steps with per-step 0D input and output and no host round trip: before
