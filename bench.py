@@ -72,7 +72,7 @@ def parse_args():
 def launches(info, steps):
     """Kernel launches of `steps` steps taken as lbm_step does them: small
     lattices in one launch per steps_per_launch steps, others in whole step
-    graphs, then single-step graphs for the rest; a graph's first step (and a
+    graphs, then short graphs and single-step ones for the rest; a graph's first step (and a
     single step) issues launches_first_step, its later steps launches_per_step; a
     batch's graphs do so once per part, after one launch more."""
     if getattr(info, "steps_per_launch", 0):
@@ -80,8 +80,12 @@ def launches(info, steps):
     g = info.graph_steps
     full, rest = divmod(steps, g)
     parts = getattr(info, "parts", 1)
-    graph = parts * (info.launches_first_step + (g - 1) * info.launches_per_step) + (parts > 1)
-    return full * graph + rest * info.launches_first_step
+    short = getattr(info, "short_graph_steps", 0)
+    short_graphs, singles = divmod(rest, short) if short and rest >= 3 * short else (0, rest)
+
+    def graph(n):
+        return parts * (info.launches_first_step + (n - 1) * info.launches_per_step) + (parts > 1)
+    return full * graph(g) + short_graphs * graph(short) + singles * info.launches_first_step
 
 
 def dist_env():

@@ -161,6 +161,8 @@ typedef struct {
                                 steps, without step graphs; 0: step graphs as above */
     int parts;               /* a batch's step graphs advance so many parts of its instances beside one another,
                               each with launches of its own, after one launch per graph (1: whole) */
+    int short_graph_steps;   /* steps of the graphs that take what is left below graph_steps, if that is three or more
+                              of them; single steps take the rest */
 } lbm_info_t;
 
 /* Sizes of the layout lbm_create would build (see lbm_check_config). */
@@ -199,7 +201,7 @@ lbm_status lbm_init_populations(lbm_handle *h, int inst, const double *f);
 
 /* Advances all instances by n steps (Algorithm 1).  Asynchronous: returns
  * after enqueueing, as CUDA graphs of graph_steps steps and, for the
- * remainder, single-step graphs (each captured once per step parity); small
+ * remainder, of short_graph_steps and of one (each captured once per step parity); small
  * lattices without wall nodes as one kernel launch per steps_per_launch steps,
  * batches in parts beside one another (lbm_info_t). */
 lbm_status lbm_step(lbm_handle *h, int64_t n);

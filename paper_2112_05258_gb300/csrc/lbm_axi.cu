@@ -69,7 +69,6 @@ struct Params {
     const float *inv_r_f;
     const double *inv_r_d;
     long long *step;       // index t_n of the step in progress (advanced by the collide kernel)
-    bool ahead;            // the populations exceed the L2: k_axi_collide has them fetched ahead
 };
 
 template <class R> struct Consts;
@@ -189,12 +188,13 @@ __device__ __forceinline__ AxiMoments<R> axi_collide_store(S *__restrict__ fout,
 // exceed it: 512 x 25,602 nodes 169.4 -> 159.5 us per step (139 at the
 // copy rate).  One request per direction and block of 256 nodes; of 512, 1,024,
 // 2,048 nodes 160.4, 161.5, 165.1; 65,536 nodes ahead are alike.  FP64 is bound by
-// its pipe and no faster (3,018 -> 3,024).
+// its pipe and no faster (3,018 -> 3,024); a kernel of its own, as the branch costs
+// grids that fit the L2 2 % (1,086 x 136 nodes).
 constexpr int AHEAD_DIST = 32768;
 
 // grid: (x-blocks, nr) of 256 nodes of a row, one row of the (x, r) grid per
 // blockIdx.y; the launch covers the x-blocks xb0 .. xb0 + gridDim.x - 1
-template <class S>
+template <class S, bool AHEAD>
 __global__ void __launch_bounds__(256, 8) k_axi_collide(const S *__restrict__ fin, S *__restrict__ fout, Params p,
                                                        int xb0) {
     using R = typename Storage<S>::R;
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(256, 8) k_axi_collide(const S *__restrict__ fi
     if (x >= p.nx) return;
     const int c = j * p.nx + x;
     const int n = p.n;
-    if (sizeof(S) == 4 && threadIdx.x < Q9 && p.ahead) {
+    if (AHEAD && threadIdx.x < Q9) {
         const int a = c - (int)threadIdx.x + AHEAD_DIST;
         if (a + 256 <= n) {  // from a 16-byte boundary
             const uintptr_t at = reinterpret_cast<uintptr_t>(fin + ((size_t)threadIdx.x * n + a)) & ~(uintptr_t)15;
@@ -691,8 +691,8 @@ struct lbm_axi_handle {
     int xb_lo = 0, xb_hi = 0;
     cudaStream_t s_bc = nullptr;
     cudaEvent_t ev_f = nullptr, ev_d = nullptr;
+    bool ahead = false;  // the populations exceed the L2: k_axi_collide has them fetched ahead
     // small grids: many steps in one launch by a cluster of blocks (0: one-step kernels)
-    bool ahead = false;
     int small_cluster = 0;
     size_t small_smem = 0;
     AxiSmall small{};
@@ -761,15 +761,14 @@ Params params(const lbm_axi_handle *h) {
     p.inv_r_f = h->inv_r_f;
     p.inv_r_d = h->inv_r_d;
     p.step = h->d_step;
-    p.ahead = h->ahead;
     return p;
 }
 
 template <class S> cudaError_t collide_blocks(lbm_axi_handle *h, const void *fin, void *fout, int b0, int b1,
                                               cudaStream_t st) {
     if (b1 <= b0) return cudaSuccess;
-    k_axi_collide<S><<<dim3(b1 - b0, h->nr), 256, 0, st>>>(static_cast<const S *>(fin), static_cast<S *>(fout),
-                                                         params(h), b0);
+    const auto k = sizeof(S) == 4 && h->ahead ? k_axi_collide<S, sizeof(S) == 4> : k_axi_collide<S, false>;
+    k<<<dim3(b1 - b0, h->nr), 256, 0, st>>>(static_cast<const S *>(fin), static_cast<S *>(fout), params(h), b0);
     return cudaGetLastError();
 }
 

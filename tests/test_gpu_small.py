@@ -205,3 +205,11 @@ def test_batch_in_parts_equals_whole_steps(name, precision):
     a, b = _pair(insts, precision, (64, 1, 130, 63, 7))
     assert a.info().steps_per_launch == 0 and a.info().parts == min(4, len(insts))
     _same(a, b, insts)
+
+
+@pytest.mark.parametrize("name", ["one_launch", "wide"])
+def test_short_graphs_equal_single_steps(name):
+    insts = PARTS["one_launch"]() if name == "one_launch" else [_lv(20.3, 171)]
+    a, b = _pair(insts, "f32", (1, 45, 15, 24, 63))
+    assert a.info().short_graph_steps == 8
+    _same(a, b, insts)
