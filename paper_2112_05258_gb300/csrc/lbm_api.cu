@@ -963,8 +963,14 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
         h->overlap = true;
     }
     if (!ck(set_up_small(h), "small-lattice tables")) return bail(LBM_ERR_CUDA, h->err);
-    if (!ns && !h->small_blocks && L.inst.size() > 1) {
-        const int K = (int)std::min<size_t>(L.inst.size(), lbm_handle::MAX_PARTS);
+    // A part needs cells: its stream-collide advances its step counter, the first
+    // part's the lattice's.  Instances without cells have no boundaries either and
+    // fall to the part before them (the first ones to the first part).
+    std::vector<size_t> filled;
+    for (size_t q = 0; q < L.inst.size(); q++)
+        if (L.inst_cell_end[q] > L.inst_cell_begin[q]) filled.push_back(q);
+    if (!ns && !h->small_blocks && filled.size() > 1) {
+        const int K = (int)std::min<size_t>(filled.size(), lbm_handle::MAX_PARTS);
         int lo = 0, hi = 0;
         if (!(ck(dalloc(h, &h->step_parts, K), "step") &&
               ck(cudaDeviceGetStreamPriorityRange(&lo, &hi), "stream priorities") &&
@@ -973,21 +979,22 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
         h->parts.reserve(K);
         h->part_steps = std::min(16, h->graph_steps);
         while (h->graph_steps % h->part_steps || h->part_steps % 2) h->part_steps++;
-        size_t m = 0;  // part k: the instances [m, e), its end where about k + 1 of K cells are
+        size_t m = 0;  // part k: the filled instances [m, e), its end where about k + 1 of K cells are
         for (int k = 0; k < K; k++) {
             size_t e = m + 1;
-            auto off = [&](size_t q) { return std::llabs(K * L.inst_cell_end[q - 1] - (k + 1) * (int64_t)n); };
-            while (e + (K - 1 - k) < L.inst.size() && off(e + 1) < off(e)) e++;
-            if (k == K - 1) e = L.inst.size();
+            auto off = [&](size_t q) { return std::llabs(K * L.inst_cell_end[filled[q - 1]] - (k + 1) * (int64_t)n); };
+            while (e + (K - 1 - k) < filled.size() && off(e + 1) < off(e)) e++;
+            if (k == K - 1) e = filled.size();
+            const size_t q0 = m ? filled[m] : 0, q1 = e < filled.size() ? filled[e] : L.inst.size();
             h->parts.emplace_back();
             lbm_handle::Part &a = h->parts.back();
-            a.c0 = (int)L.inst_cell_begin[m];
-            a.c1 = (int)L.inst_cell_end[e - 1];
+            a.c0 = (int)L.inst_cell_begin[q0];
+            a.c1 = (int)L.inst_cell_end[q1 - 1];
             a.kp = h->kp;
             a.bp = h->bp;
             a.bp.priority = hi;
-            a.bp.bc0 = L.inst[m].bc_first;
-            const int b1 = L.inst[e - 1].bc_first + L.inst[e - 1].n_bc;
+            a.bp.bc0 = L.inst[q0].bc_first;
+            const int b1 = L.inst[q1 - 1].bc_first + L.inst[q1 - 1].n_bc;
             a.bp.n_bc = b1 - a.bp.bc0;
             auto at = [](const std::vector<int32_t> &v, int bc) {
                 return (int)(std::lower_bound(v.begin(), v.end(), bc) - v.begin());

@@ -213,3 +213,28 @@ def test_short_graphs_equal_single_steps(name):
     a, b = _pair(insts, "f32", (1, 45, 15, 24, 63))
     assert a.info().short_graph_steps == 8
     _same(a, b, insts)
+
+
+def _solid():
+    return Instance(node=np.ones((5, 6, 7), np.uint8), tau=0.8, name="solid")
+
+
+# batches whose first, middle or last instances store no cells
+HOLLOW = {
+    "one_tube": lambda: [_solid(), _lv(13.0, 830)],
+    "one_tube_last": lambda: [_lv(13.0, 830), _solid(), _solid()],
+    "three_tubes": lambda: [_solid(), _lv(13.0, 450), configs.rigid_tube(31, 31, 170, radius=11.4), _lv(12.2, 443)],
+    "half_of_the_cells": lambda: [_solid(), _solid(), _lv(13.0, 600), _lv(6.3, 41), _solid(), _lv(9.1, 333), _lv(6.0, 128)],
+}
+
+
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+@pytest.mark.parametrize("name", list(HOLLOW))
+def test_batch_with_solid_instances_equals_whole_steps(name, precision):
+    # whole graphs, single-step ones and graphs again: the step counter that the
+    # inlet phase, the elastance and the waveform rows follow advances in all
+    insts = HOLLOW[name]()
+    a, b = _pair(insts, precision, (64, 3, 130, 63, 7))
+    tubes = sum(bool((i.node == 0).any()) for i in insts)
+    assert a.info().steps_per_launch == 0 and a.info().parts == min(4, tubes)
+    _same(a, b, insts)
