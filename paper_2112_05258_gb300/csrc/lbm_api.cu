@@ -1425,10 +1425,15 @@ struct CkptSection {  // rows of row_bytes on the device, pitch apart; packed in
     void *dev;
     size_t row_bytes, rows = 1, pitch = 0;
     size_t bytes() const { return row_bytes * rows; }
+    // one row by a plain copy: the documented limit of a pitch (cudaDevAttrMaxPitch, 2^31 - 1) is
+    // less than the force density of a large FP64 lattice or a long waveform ring; a direction's
+    // row stays below it
     cudaError_t copy(void *packed, bool save) const {
-        const size_t p = rows > 1 ? pitch : row_bytes;
-        return save ? cudaMemcpy2D(packed, row_bytes, dev, p, row_bytes, rows, cudaMemcpyDeviceToHost)
-                    : cudaMemcpy2D(dev, p, packed, row_bytes, row_bytes, rows, cudaMemcpyHostToDevice);
+        if (rows == 1)
+            return save ? cudaMemcpy(packed, dev, row_bytes, cudaMemcpyDeviceToHost)
+                        : cudaMemcpy(dev, packed, row_bytes, cudaMemcpyHostToDevice);
+        return save ? cudaMemcpy2D(packed, row_bytes, dev, pitch, row_bytes, rows, cudaMemcpyDeviceToHost)
+                    : cudaMemcpy2D(dev, pitch, packed, row_bytes, row_bytes, rows, cudaMemcpyHostToDevice);
     }
 };
 std::vector<CkptSection> ckpt_sections(lbm_handle *h) {

@@ -60,3 +60,15 @@ def test_checkpoint_of_another_configuration_is_refused(Lattice):
         b.restore(ck)
     with pytest.raises(LBMError):
         a.restore(ck[:100])
+
+
+def test_sections_beyond_2_gib(Lattice):
+    # a waveform ring of 2^31 + 64 bytes (2 boundaries x 4 doubles a step) is one
+    # section of the checkpoint, longer than the documented pitch of a 2D copy
+    inst = configs.lv_tube(period=300)
+    a, c = _split_run(Lattice, [inst], "f32", 173, 60, wave_capacity=2 ** 25 + 1)
+    assert np.array_equal(a.populations(0), c.populations(0))
+    for k in range(2):
+        assert np.array_equal(a.state_0d(0, k), c.state_0d(0, k))
+    rows = c.waves(0)
+    assert rows.shape[0] == 233 and np.array_equal(rows, a.waves(0))
