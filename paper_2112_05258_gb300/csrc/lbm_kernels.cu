@@ -676,26 +676,43 @@ cudaError_t launch_copy_words(const void *src, void *dst, size_t bytes, cudaStre
     return cudaGetLastError();
 }
 
-// Sums of population deviations for the FP32 read-out, about as exact as FP64
-// ones: FP32 storage adds in pairs of FP32 (two-sum, error about 2^-46 of the
-// terms), FP64 storage in FP64.
-struct PairSum {
-    float h = 0.f, l = 0.f;
-    __device__ __forceinline__ void add(float x) {
-        const float s = h + x, t = s - h;
-        l += (h - (s - t)) + (x - t);
-        h = s;
+// Sums of population deviations for the FP32 read-out, no less exact than FP64
+// ones.  FP32 and BF16 storage adds in triples of FP32 (two two-sums and a plain
+// sum, error about 2^-70 of the terms).  FP16 populations are multiples of 2^-24,
+// so that pairs of FP32 (one two-sum) hold their sums exactly (below 2^14); of
+// FP32 populations pairs lost 2^-46 of the terms, up to 25 times as much as FP64
+// where the terms cancel over many binades.  FP64 storage adds in FP64.
+template <bool TRIPLE> struct SplitSum {
+    float h = 0.f, l = 0.f, c = 0.f;
+    static __device__ __forceinline__ float two_sum(float &s, float x) {  // s += x; what the rounding left out
+        const float a = s, t = a + x, d = t - a;
+        s = t;
+        return (a - (t - d)) + (x - d);
     }
-    // an infinity or NaN in h makes l a NaN: then h alone is the sum
-    __device__ __forceinline__ float low() const { return isfinite(l) ? l : 0.f; }
-    __device__ __forceinline__ float value() const { return h + low(); }
-    __device__ __forceinline__ float pressure() const {  // (1 + h + l) / 3 to the last bit or so
-        PairSum t;
-        t.h = 1.f;
-        t.add(h);
-        const float q = t.h * (1.f / 3.f);
-        const float r = (fmaf(-3.f, q, t.h) + (t.low() + low())) * (1.f / 3.f);
-        return isfinite(r) ? q + r : q;
+    __device__ __forceinline__ void add(float x) {
+        const float e = two_sum(h, x);
+        if (TRIPLE) c += two_sum(l, e);
+        else l += e;
+    }
+    // h + l + c as a leading part and the rest; an infinity or NaN in h makes l and
+    // the rest NaNs: then h alone is the sum
+    __device__ __forceinline__ float split(float *rest) const {
+        float s = h;
+        *rest = two_sum(s, l) + c;
+        return s;
+    }
+    __device__ __forceinline__ float value() const {
+        float r;
+        const float s = split(&r);
+        return isfinite(r) ? s + r : h;
+    }
+    __device__ __forceinline__ float pressure() const {  // (1 + h + l + c) / 3 to the last bit or so
+        SplitSum t = *this;
+        t.add(1.f);
+        float r;
+        const float s = t.split(&r), q = s * (1.f / 3.f);
+        r = (fmaf(-3.f, q, s) + r) * (1.f / 3.f);
+        return isfinite(r) ? q + r : t.h * (1.f / 3.f);
     }
 };
 struct WideSum {
@@ -704,7 +721,8 @@ struct WideSum {
     __device__ __forceinline__ float value() const { return (float)h; }
     __device__ __forceinline__ float pressure() const { return (float)((1.0 + h) / 3.0); }
 };
-template <class R> struct ReadSum { using T = PairSum; };
+template <class S> struct ReadSum { using T = SplitSum<true>; };
+template <> struct ReadSum<__half> { using T = SplitSum<false>; };
 template <> struct ReadSum<double> { using T = WideSum; };
 
 // FP32 read-out of one instance in box order: thread b takes the box cells
@@ -712,11 +730,11 @@ template <> struct ReadSum<double> { using T = WideSum; };
 // fluid, and the pulls of a row's cells are coalesced too.  Bound by memory:
 // 80 B read per fluid cell (FP32 storage) and 16 B written per box cell.  The
 // sums must not lose precision against FP64, whose pipe is narrow on this
-// part (68 FP64 operations a cell took the whole time before); pairs of FP32
-// cost about 350 FP32 operations a cell and stay below the memory time.
-// Aorta (16.8M box cells, 4.0M fluid, FP32): 1,315 us as FP64 gather, four
-// memsets and a scatter, 200 us in this kernel; the 96 uneven tubes of a batch
-// (33M box cells): 576 launches and 9.3 ms before, 96 launches and 1.2 ms now.
+// part (68 FP64 operations a cell took the whole time before); triples of FP32
+// cost about 650 FP32 operations a cell, pairs (FP16) 350.
+// Aorta (16.8M box cells, 4.0M fluid): 1,315 us as FP64 gather, four memsets and
+// a scatter, in this kernel 238 us (FP16 197); the 96 uneven tubes of a batch
+// (33M box cells): 576 launches and 9.3 ms before, 96 launches and 1.42 ms (FP16 1.21).
 template <class S>
 __global__ void __launch_bounds__(256) k_fields_box(const S *__restrict__ fin, KParams p, const int32_t *__restrict__ rowid,
                                                     int nx, unsigned nbox, float *__restrict__ P, float *__restrict__ jx,
@@ -743,7 +761,7 @@ __global__ void __launch_bounds__(256) k_fields_box(const S *__restrict__ fin, K
                 const int src = ln[nbk(i)] - cx(i), own = c + ((i & 1) ? N : -N);
                 f[i] = Storage<S>::ld(fin + (size_t)i * N + (((fl >> i) & 1u) ? own : src));
             }
-            typename ReadSum<R>::T s, m[3];
+            typename ReadSum<S>::T s, m[3];
 #pragma unroll
             for (int i = 0; i < NQ; i++) {
                 s.add(f[i]);

@@ -64,3 +64,63 @@ def test_device_fields_keep_infinities_and_nan():
         at = np.isinf(e)
         assert np.array_equal(g[at], e[at].astype(np.float32))
 
+
+
+def _cancelling(node, seed, precision):
+    """Deviations s (19 x cells, exact in the storage type) whose sums cancel over
+    many binades: in every cell one of 1 + sum s, jx, jy, jz adds a small term, a
+    middle one and a large one (2^-22, 2^0, 2^10; FP16: 2^-12) before the large
+    and the middle one are taken away again, so that what the large one pushed
+    out of an FP32 sum decides."""
+    rng = np.random.default_rng(seed)
+    n = node.size
+    e = np.array([(0, 0, 0), (1, 0, 0), (-1, 0, 0), (0, 1, 0), (0, -1, 0), (0, 0, 1), (0, 0, -1),
+                  (1, 1, 0), (-1, -1, 0), (1, -1, 0), (-1, 1, 0), (1, 0, 1), (-1, 0, -1), (1, 0, -1), (-1, 0, 1),
+                  (0, 1, 1), (0, -1, -1), (0, 1, -1), (0, -1, 1)])
+
+    def stored(v):
+        v = v.astype(np.float32)
+        if precision == "f16":
+            return v.astype(np.float16).astype(np.float32)
+        return (v.view(np.uint32) & 0xffff0000).view(np.float32) if precision == "bf16" else v
+
+    def some(k):                            # +-[1/2, 1) 2^k
+        return stored(rng.uniform(0.5, 1.0, n) * rng.choice([-1.0, 1.0], n) * 2.0 ** k)
+
+    up = 10 if precision == "f16" else 0
+    s = np.zeros((19, n), np.float32)
+    kind = rng.integers(0, 4, n)
+    for a in range(4):
+        terms = [(i, 1) for i in range(1, 19)] if a == 0 else [(i, e[i, a - 1]) for i in range(19) if e[i, a - 1]]
+        m, A = some(0), some(10)
+        values = [some(up - 22), some(up - 21), m, some(up - 25), A, -A, some(up - 24), -m, some(up - 23), some(up - 26)]
+        for (i, sign), v in zip(terms, values):
+            s[i] = np.where(kind == a, sign * v, s[i])
+    s[0] = np.where(kind == 0, stored(np.float32(-1.0) + some(-12)), s[0])
+    return s, e
+
+
+@pytest.mark.parametrize("precision", ["f32", "f16", "bf16"])
+def test_device_fields_lose_no_more_than_fp64_sums(precision):
+    # the error against exact sums: half an FP32 unit in the last place of the
+    # result and 2^-53, the unit of FP64, of the terms' magnitudes (sequential
+    # FP64 sums of these terms stay below it: at most three additions are rounded,
+    # at a quarter of that each)
+    import math
+    from paper_2112_05258_gb300 import Lattice
+    inst = configs.rigid_tube()
+    s, e = _cancelling(inst.node, 9, precision)
+    w = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12)
+    lat = Lattice([inst], precision=precision)
+    f = s.astype(np.float64) + w[:, None]
+    assert np.array_equal((f - w[:, None]).astype(np.float32), s)
+    lat.init_populations(0, f)
+    got = _device_fields(lat, inst, 0)
+    for a, g in enumerate(got):
+        terms = [s[i].astype(np.float64) * (1 if a == 0 else e[i, a - 1]) for i in range(19)] + [np.full(s.shape[1], float(a == 0))]
+        T = np.array(terms)
+        for c in np.flatnonzero(inst.node.reshape(-1) == 0):
+            exact, mag = math.fsum(T[:, c]), np.abs(T[:, c]).sum()
+            if a == 0:
+                exact, mag = exact / 3, mag / 3
+            assert abs(g[c] - exact) <= 2.0 ** -24 * (1 + 2.0 ** -20) * abs(exact) + 2.0 ** -53 * mag, (a, c)
