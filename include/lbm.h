@@ -228,8 +228,17 @@ lbm_status lbm_step_io(lbm_handle *h, int inst, int bc, int64_t n, const double 
 /* Waits for the stream; returns LBM_ERR_UNSTABLE if the device status word
  * recorded NaN/Inf or |v| > 0.3 (stream-collide) or a wall node more than one
  * cell from its reference cell, i.e. outside its immersed-boundary support
- * box (node kernel), since creation.  The state stays readable. */
+ * box (node kernel), since creation.  The state stays readable.  LBM_ERR_CUDA,
+ * whatever else is recorded, if a multi-step launch gave up waiting
+ * (lbm_set_wait_limit): its blocks stopped at different steps, and the state
+ * is of no use. */
 lbm_status lbm_sync(lbm_handle *h);
+
+/* The blocks of a multi-step launch over a whole lattice wait for one another
+ * after each step.  A block gives up after so many polls (default 4,194,304,
+ * some seconds, where a step takes microseconds), and lbm_sync reports it.  For
+ * the steps enqueued from now on; a small limit serves to test that path. */
+lbm_status lbm_set_wait_limit(lbm_handle *h, int polls);
 
 /* Host outputs, box order, nx*ny*nz doubles each (non-fluid nodes 0):
  * P = c_s^2 sum_i f_i and j = sum_i e_i f_i of the current f(t_n)

@@ -616,6 +616,7 @@ cudaError_t set_up_small(lbm_handle *h) {
     h->small.bulk_off = d_off;
     h->small.done = done;
     h->small.meet = meet;
+    h->small.polls = SMALL_POLLS;
     h->small.n_inst = (int)L.inst.size();
     h->small.par = h->bc_par;
     return e;
@@ -1195,8 +1196,9 @@ lbm_status lbm_sync(lbm_handle *h) {
     CK(h, cudaStreamSynchronize(h->stream));
     unsigned s = 0;
     CK(h, cudaMemcpy(&s, h->status, sizeof s, cudaMemcpyDeviceToHost));
-    if (s & 1u) return fail(h, LBM_ERR_UNSTABLE, "NaN/Inf or |v| > 0.3 in the lattice");
+    // before the others: blocks that went on alone may have made the lattice unstable
     if (s & 4u) return fail(h, LBM_ERR_CUDA, "the blocks of a multi-step kernel did not meet in time");
+    if (s & 1u) return fail(h, LBM_ERR_UNSTABLE, "NaN/Inf or |v| > 0.3 in the lattice");
     if (s & 2u) return fail(h, LBM_ERR_UNSTABLE, "a wall node moved outside its immersed-boundary band");
     return LBM_OK;
 }
@@ -1341,6 +1343,12 @@ lbm_status lbm_set_ib_state(lbm_handle *h, int inst, const double *X, const doub
         CK(h, cudaMemcpy(h->ibD32 + o, D.data(), m * sizeof(float), cudaMemcpyHostToDevice));
         CK(h, cudaMemcpy(h->ibVs32 + o, V.data(), m * sizeof(float), cudaMemcpyHostToDevice));
     }
+    return LBM_OK;
+}
+
+lbm_status lbm_set_wait_limit(lbm_handle *h, int polls) {
+    if (!h || polls < 1) return fail(h, LBM_ERR_ARG, "the limit must be at least 1 poll");
+    h->small.polls = polls;
     return LBM_OK;
 }
 

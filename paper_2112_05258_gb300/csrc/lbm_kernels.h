@@ -123,6 +123,7 @@ struct IbKParams {
 // of blocks per instance or one grid over all (lbm_small.cu).
 constexpr int SMALL_MAX_RED = 8;          // chunks of a boundary's first layer
 constexpr int SMALL_MAX_STEPS = 4096;     // steps per launch
+constexpr int SMALL_POLLS = 1 << 22;      // grid: polls at the barrier before a block gives up
 constexpr size_t SMALL_MAX_SMEM = 212000; // dynamic shared memory of a block, beside 17 KB of static
 struct SmallKParams {
     const InstParam *inst;
@@ -130,6 +131,7 @@ struct SmallKParams {
     const int32_t *bulk_off;  // per instance, and the end
     int *done;                // blocks finished (back to 0 after the launch)
     unsigned *meet;           // grid: arrivals at the barrier (back to 0 after the launch)
+    int polls;                // grid: polls of a block there before it gives up
     int cluster;              // blocks per instance, or 0: one grid over all instances
     int n_inst;
     int n_steps;

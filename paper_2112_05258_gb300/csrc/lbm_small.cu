@@ -119,10 +119,12 @@ template <int THREADS> struct StepBarrier<true, THREADS> {
         int failed;
     };
     static constexpr int POLLER = THREADS - 32;
-    static constexpr int POLLS = 1 << 22, TRIES = 1 << 30;  // a warp never gives up before the polling thread has
+    static constexpr int TRIES = 1 << 30;  // a warp never gives up before the polling thread has
     Shared &s;
+    const int polls;
     unsigned *count, *status, target = 0, phase = 0;
-    __device__ StepBarrier(Shared &sh, const SmallKParams &sp, unsigned *st) : s(sh), count(sp.meet), status(st) {
+    __device__ StepBarrier(Shared &sh, const SmallKParams &sp, unsigned *st)
+        : s(sh), polls(sp.polls), count(sp.meet), status(st) {
         if (threadIdx.x == 0) {
             s.failed = 0;
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(address()) : "memory");
@@ -142,8 +144,8 @@ template <int THREADS> struct StepBarrier<true, THREADS> {
             unsigned v = 0;
             int k = 0;
             do asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
-            while ((int)(v - target) < 0 && ++k < POLLS);
-            if (k == POLLS) {
+            while ((int)(v - target) < 0 && ++k < polls);
+            if (k == polls) {
                 atomicOr(status, 4u);
                 s.failed = 1;
             }

@@ -238,3 +238,39 @@ def test_batch_with_solid_instances_equals_whole_steps(name, precision):
     tubes = sum(bool((i.node == 0).any()) for i in insts)
     assert a.info().steps_per_launch == 0 and a.info().parts == min(4, tubes)
     _same(a, b, insts)
+
+
+@pytest.mark.parametrize("name", ["lv", "velocity", "uneven"])
+def test_grid_that_gives_up_waiting_is_reported(name):
+    # one poll at each barrier: blocks give up while the others still work, each
+    # returns, and the launch is reported as failed whatever its populations
+    # came to; the next lattice is not touched by it
+    from paper_2112_05258_gb300 import LBMError, Lattice
+    insts = GRID[name]()
+    a = Lattice(insts, precision="f32")
+    for q, inst in enumerate(insts):
+        a.init_populations(q, configs.random_populations(inst, seed=q, amp=2e-3))
+    a.set_wait_limit(1)
+    a.step(400)
+    with pytest.raises(LBMError) as e:
+        a.sync()
+    assert e.value.status == -2 and "did not meet" in str(e.value)
+    a.close()
+    a, b = _pair(insts, "f32", (30,))
+    _same(a, b, insts)
+
+
+def test_a_launch_that_gave_up_is_not_called_unstable():
+    from paper_2112_05258_gb300 import LBMError, Lattice
+    inst = GRID["lv"]()[0]
+    f = configs.random_populations(inst, seed=1, amp=0.0)
+    f[5] += 0.4                               # |v| > 0.3 everywhere: both status bits are set
+    a = Lattice([inst], precision="f32")
+    a.init_populations(0, f)
+    a.set_wait_limit(1)
+    a.step(400)
+    with pytest.raises(LBMError) as e:
+        a.sync()
+    assert e.value.status == -2
+    with pytest.raises(LBMError):
+        a.set_wait_limit(0)
