@@ -625,6 +625,7 @@ cudaError_t set_up_small(lbm_handle *h) {
 // n steps in the multi-step kernel (launches of at most SMALL_MAX_STEPS
 // steps); io: per-step params and state rows of lbm_step_io, or null.
 lbm_status small_steps(lbm_handle *h, int64_t n, const SmallKParams *io = nullptr) {
+    if (n == 0) return LBM_OK;
     SmallKParams sp = io ? *io : h->small;
     // refused as the step graphs of the other lattices are: a replay would pass the host's step count by
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;

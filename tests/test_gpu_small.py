@@ -274,3 +274,30 @@ def test_a_launch_that_gave_up_is_not_called_unstable():
     assert e.value.status == -2
     with pytest.raises(LBMError):
         a.set_wait_limit(0)
+
+
+@pytest.mark.parametrize("inst", [lambda: configs.lv_tube(period=300), lambda: GRID["lv"]()[0], lambda: _lv(13.0, 830)])
+def test_steps_on_a_stream_that_is_captured(inst):
+    # no lattice's steps can be captured (a replay would pass the step count on
+    # the host by); a call of no steps enqueues nothing and is accepted
+    import torch
+    from paper_2112_05258_gb300 import LBMError, Lattice
+    inst, s = inst(), torch.cuda.Stream()
+    for n in (0, 1, 64):
+        lat = Lattice([inst], precision="f32", stream=s.cuda_stream)
+        lat.step(n + 1)
+        lat.sync()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(s):
+            g.capture_begin(capture_error_mode="thread_local")
+            try:
+                lat.step(n)
+                refused = False
+            except LBMError:
+                refused = True
+            try:
+                g.capture_end()
+            except RuntimeError:                # a refused graph launch ends the capture
+                assert refused
+        assert refused == (n > 0) and lat.info().steps == n + 1
+        lat.close()
