@@ -71,11 +71,12 @@ def parse_args():
 
 def launches(info, steps):
     """Kernel launches of `steps` steps taken as lbm_step does them: small
-    lattices in one launch per steps_per_launch steps, others in whole step
+    lattices in one launch per steps_per_launch steps (from multi_step_from steps
+    a call on), others in whole step
     graphs, then short graphs and single-step ones for the rest; a graph's first step (and a
     single step) issues launches_first_step, its later steps launches_per_step; a
     batch's graphs do so once per part, after one launch more."""
-    if getattr(info, "steps_per_launch", 0):
+    if getattr(info, "steps_per_launch", 0) and steps >= getattr(info, "multi_step_from", 1):
         return -(-steps // info.steps_per_launch)
     g = info.graph_steps
     full, rest = divmod(steps, g)

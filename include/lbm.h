@@ -163,6 +163,7 @@ typedef struct {
                               each with launches of its own, after one launch per graph (1: whole) */
     int short_graph_steps;   /* steps of the graphs that take what is left below graph_steps, if that is three or more
                               of them; single steps take the rest */
+    int multi_step_from;     /* where steps_per_launch is not 0: lbm_step calls of fewer steps take single-step graphs */
 } lbm_info_t;
 
 /* Sizes of the layout lbm_create would build (see lbm_check_config). */
@@ -202,7 +203,8 @@ lbm_status lbm_init_populations(lbm_handle *h, int inst, const double *f);
 /* Advances all instances by n steps (Algorithm 1).  Asynchronous: returns
  * after enqueueing, as CUDA graphs of graph_steps steps and, for the
  * remainder, of short_graph_steps and of one (each captured once per step parity); small
- * lattices without wall nodes as one kernel launch per steps_per_launch steps,
+ * lattices without wall nodes as one kernel launch per steps_per_launch steps
+ * (calls of fewer than multi_step_from steps as single-step graphs),
  * batches in parts beside one another (lbm_info_t). */
 lbm_status lbm_step(lbm_handle *h, int64_t n);
 

@@ -153,6 +153,7 @@ struct lbm_handle {
     // small lattices: many steps in one launch of so many blocks, clusters or a
     // grid (0: one-step kernels)
     int small_blocks = 0;
+    int small_from = 1;  // calls of fewer steps take the one-step kernels all the same
     size_t small_smem = 0;
     SmallKParams small{};
     // kernel timing
@@ -552,8 +553,13 @@ cudaError_t set_up_small(lbm_handle *h) {
     // kernels: launches and latencies of 12 us (FP64: 21), then bandwidth.
     const bool f64 = h->prec == LBM_F64;
     const double cells = (double)L.n_fluid;
+    // Without boundaries a one-step kernel is all there is to a step.  FP32 calls of 100 steps
+    // of closed boxes, one-step kernels -> this one: 55,000 cells 308 -> 322 us, 135,000 410 ->
+    // 455 (406 and 516 before the short graphs), 217,000 551 -> 649, 340,000 712 -> 828; of 24
+    // steps 74 -> 82, 100 -> 114, 135 -> 161, 172 -> 205.
+    if (!f64 && L.bc.empty() && cells > 170e3) return cudaSuccess;
     const double one_step = std::max(f64 ? 21.0 : 12.0, (f64 ? 16.0 : 9.0) + cells * (f64 ? 240e-6 : 30e-6));
-    double best = 0.9 * one_step;
+    double best = 0.9 * one_step, t_small = 0.0;
     for (int C : {16, 8}) {
         if (C <= most_bc) continue;
         const size_t smem = std::max(smem_b, small_smem_bulk((int)worst_bulk[C]));
@@ -569,7 +575,7 @@ cudaError_t set_up_small(lbm_handle *h) {
         const int rounds = ((int)L.inst.size() + clusters - 1) / clusters;
         const double t = rounds * std::max(owner, bulk);
         if (t >= best) continue;
-        best = t;
+        best = t_small = t;
         h->small.cluster = C;
         h->small_blocks = C * (int)L.inst.size();
         h->small_smem = smem;
@@ -594,6 +600,7 @@ cudaError_t set_up_small(lbm_handle *h) {
         const size_t smem = std::max(smem_b, small_smem_grid((int)per, f64));
         if (t < 0.95 * (h->small_blocks ? best : one_step) && smem <= SMALL_MAX_SMEM) {
             if (prepare_small(h->prec, 0, smem, &per_sm) == cudaSuccess && per_sm >= 1) {
+                t_small = t;
                 h->small.cluster = 0;
                 h->small_blocks = nb + w;
                 h->small_smem = smem;
@@ -602,6 +609,16 @@ cudaError_t set_up_small(lbm_handle *h) {
         }
     }
     if (e != cudaSuccess || !h->small_blocks) return e;
+    // A launch lays out its tables first (8.4 us), which a call of one step does not repay where
+    // the step is long: such calls take the one-step kernels.  us for a call of one step, queued
+    // and waited for, one-step kernels -> this one: FP32 2,400 cells 11.4, 26.3 -> 11.2, 27.4, 24x24x64
+    // tube 12.4, 26.2 -> 12.4, 28.2, 50,283 cells 12.4, 27.4 -> 14.4, 30.1, 324,139 cells 17.9, 32.1 ->
+    // 20.6, 36.9, 10,330 cells behind 1,029 first-layer ones 16.5, 30.0 -> 22.6, 38.7, 16 tubes of
+    // 14,112 cells 14.7, 30.9 -> 14.4, 30.7; FP64 2,400 cells 22.6, 36.7 -> 18.4, 34.8, 24x24x64 tube 22.6,
+    // 37.4 -> 26.7, 42.6, 176,407 cells 63.6, 77.5 -> 56.0, 74.6.  Two steps repay it, without boundaries
+    // (6.2 -> 8.3 to 10.3) three in FP32.
+    const double single = f64 ? 21.5 + 235e-6 * cells : 11.4 + 0.1 * ((double)L.inst.size() - 1) + 20e-6 * cells;
+    h->small_from = L.bc.empty() ? (f64 ? 2 : 3) : 8.4 + t_small > single ? 2 : 1;
     int32_t *d_bulk = nullptr, *d_off = nullptr;
     int *done = nullptr;
     unsigned *meet = nullptr;
@@ -1111,7 +1128,7 @@ lbm_status lbm_step(lbm_handle *h, int64_t n) {
         }
         return LBM_OK;
     }
-    if (h->small_blocks) return small_steps(h, n);
+    if (h->small_blocks && n >= h->small_from) return small_steps(h, n);
     int64_t left = n;
     const int per = h->parts.empty() ? h->graph_steps : h->part_steps;
     const bool use_short = n % per >= 3 * lbm_handle::SHORT_STEPS;
@@ -1654,6 +1671,7 @@ lbm_status lbm_get_info(lbm_handle *h, lbm_info_t *info) {
     info->short_graph_steps = h->small_blocks ? 0 : lbm_handle::SHORT_STEPS;
     info->parts = std::max(1, (int)h->parts.size());
     info->steps_per_launch = h->small_blocks ? SMALL_MAX_STEPS : 0;
+    info->multi_step_from = h->small_blocks ? h->small_from : 0;
     return LBM_OK;
 }
 

@@ -60,7 +60,8 @@ class Info(ctypes.Structure):
                 ("bytes_per_population", ctypes.c_int), ("slabs", ctypes.c_int),
                 ("launches_per_step", ctypes.c_int), ("launches_first_step", ctypes.c_int),
                 ("graph_steps", ctypes.c_int), ("steps_per_launch", ctypes.c_int),
-                ("parts", ctypes.c_int), ("short_graph_steps", ctypes.c_int)]
+                ("parts", ctypes.c_int), ("short_graph_steps", ctypes.c_int),
+                ("multi_step_from", ctypes.c_int)]
 
 
 class LayoutStats(ctypes.Structure):

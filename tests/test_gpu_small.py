@@ -301,3 +301,29 @@ def test_steps_on_a_stream_that_is_captured(inst):
                 assert refused
         assert refused == (n > 0) and lat.info().steps == n + 1
         lat.close()
+
+
+# lattices whose single-step calls the layout of a multi-step launch does not
+# repay: wide first layers, many cells, FP64 first layers, no boundary
+SINGLE = {
+    "flat": (lambda: [_lv(18.1, 12)], "f32"),
+    "long": (lambda: [_lv(16.2, 310)], "f16"),
+    "f64": (lambda: [configs.rigid_tube()], "f64"),
+    "box": (lambda: [Instance(node=geometry.closed_box(31, 17, 53), tau=0.7, name="box")], "bf16"),
+}
+
+
+@pytest.mark.parametrize("name", list(SINGLE))
+def test_single_step_calls_between_longer_ones(name):
+    insts, precision = SINGLE[name][0](), SINGLE[name][1]
+    a, b = _pair(insts, precision, (1, 1, 2, 1, 3, 40, 1, 2, 1))
+    info = a.info()
+    assert info.steps_per_launch > 0 and info.multi_step_from == (3 if name == "box" else 2)
+    _same(a, b, insts)
+
+
+def test_large_lattices_without_boundaries_keep_the_step_graphs():
+    insts = [Instance(node=geometry.closed_box(80, 60, 50), tau=0.7, name="box")]
+    a, b = _pair(insts, "f32", (64, 7))
+    assert a.info().steps_per_launch == 0
+    _same(a, b, insts)
