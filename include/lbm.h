@@ -236,6 +236,17 @@ lbm_status lbm_step_io(lbm_handle *h, int inst, int bc, int64_t n, const double 
  * is of no use. */
 lbm_status lbm_sync(lbm_handle *h);
 
+/* Whether a small lattice takes its steps in multi-step launches (the default)
+ * or as step graphs of one-step kernels, from the next call on; the trajectory
+ * is the same bit for bit.  A multi-step launch holds its SMs for the whole call.
+ * One lattice at a time is faster with it (176,407 cells FP32 12.8 -> 7.3 us per
+ * step); several middle-sized ones stepped at once on streams of their own
+ * overlap without it.  us per step of all, with and without: three of 176,407
+ * cells FP32 22.0 and 18.9, FP16 21.8 and 16.9, eight FP16 58.3 and 37.2; eight of
+ * 14,112 cells FP32 4.4 and 11.3, FP64 48.0 and 35.6.  As one batch in one lattice
+ * the first three take 17.6, 16.2 and 33.2. */
+lbm_status lbm_set_multi_step(lbm_handle *h, int enable);
+
 /* The blocks of a multi-step launch over a whole lattice wait for one another
  * after each step.  A block gives up after so many polls (default 4,194,304,
  * some seconds, where a step takes microseconds), and lbm_sync reports it.  For

@@ -154,6 +154,7 @@ struct lbm_handle {
     // grid (0: one-step kernels)
     int small_blocks = 0;
     int small_from = 1;  // calls of fewer steps take the one-step kernels all the same
+    bool small_on = true;  // lbm_set_multi_step
     size_t small_smem = 0;
     SmallKParams small{};
     // kernel timing
@@ -584,9 +585,9 @@ cudaError_t set_up_small(lbm_handle *h) {
     // it takes more SMs): a boundary block as above (FP32: another pass beyond 768
     // cells), and as many bulk blocks as are done a little earlier, if the shared
     // memory of those takes their cells; the other SMs stay free for other streams.
-    // (Three FP32 tubes of 176,407 cells stepped at once on three streams take turns:
-    // 7.3 to 8.7 us a step of one of them, where one-step kernels overlap to 7.1;
-    // one alone 7.2 instead of 12.4, beside a stream of long kernels 16 instead of 328.)
+    // (Lattices stepped at once on streams of their own take turns; a caller can choose
+    // the one-step kernels for them, lbm_set_multi_step, where the figures stand.  One
+    // alone 7.2 instead of 12.4 us a step, beside a stream of long kernels 16 instead of 328.)
     int sms = 0, per_sm = 0;
     const int nb = (int)L.bc.size();
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
@@ -1128,7 +1129,7 @@ lbm_status lbm_step(lbm_handle *h, int64_t n) {
         }
         return LBM_OK;
     }
-    if (h->small_blocks && n >= h->small_from) return small_steps(h, n);
+    if (h->small_blocks && h->small_on && n >= h->small_from) return small_steps(h, n);
     int64_t left = n;
     const int per = h->parts.empty() ? h->graph_steps : h->part_steps;
     const bool use_short = n % per >= 3 * lbm_handle::SHORT_STEPS;
@@ -1169,7 +1170,7 @@ lbm_status lbm_step_io(lbm_handle *h, int inst, int bc, int64_t n, const double 
         pdev = static_cast<const double *>(a.devicePointer);
         sdev = static_cast<double *>(c.devicePointer);
     }
-    if (h->small_blocks && !h->timing) {
+    if (h->small_blocks && h->small_on && !h->timing) {
         SmallKParams sp = h->small;
         sp.io_params = pdev;
         sp.io_states = sdev;
@@ -1361,6 +1362,12 @@ lbm_status lbm_set_ib_state(lbm_handle *h, int inst, const double *X, const doub
         CK(h, cudaMemcpy(h->ibD32 + o, D.data(), m * sizeof(float), cudaMemcpyHostToDevice));
         CK(h, cudaMemcpy(h->ibVs32 + o, V.data(), m * sizeof(float), cudaMemcpyHostToDevice));
     }
+    return LBM_OK;
+}
+
+lbm_status lbm_set_multi_step(lbm_handle *h, int enable) {
+    if (!h) return LBM_ERR_ARG;
+    h->small_on = enable != 0;
     return LBM_OK;
 }
 
@@ -1668,10 +1675,11 @@ lbm_status lbm_get_info(lbm_handle *h, lbm_info_t *info) {
     if (h->overlap)  // band velocities as the two lists (an empty list launches nothing)
         info->launches_per_step += (h->n_band_ind > 0) + (h->n_band_dep > 0) - 1;
     info->graph_steps = h->parts.empty() ? h->graph_steps : h->part_steps;
-    info->short_graph_steps = h->small_blocks ? 0 : lbm_handle::SHORT_STEPS;
+    const bool multi = h->small_blocks && h->small_on;
+    info->short_graph_steps = multi ? 0 : lbm_handle::SHORT_STEPS;
     info->parts = std::max(1, (int)h->parts.size());
-    info->steps_per_launch = h->small_blocks ? SMALL_MAX_STEPS : 0;
-    info->multi_step_from = h->small_blocks ? h->small_from : 0;
+    info->steps_per_launch = multi ? SMALL_MAX_STEPS : 0;
+    info->multi_step_from = multi ? h->small_from : 0;
     return LBM_OK;
 }
 

@@ -76,7 +76,8 @@ EXPORTS = ["lbm_create", "lbm_set_0d_params", "lbm_init_populations", "lbm_step"
            "lbm_init_equilibrium", "lbm_set_0d_state", "lbm_cycle_change", "lbm_autotune",
            "lbm_wall_shear", "lbm_check_config", "lbm_checkpoint_size", "lbm_checkpoint_save",
            "lbm_checkpoint_load", "lbm_read_fields_device", "lbm_set_stream_collide_shape",
-           "lbm_read_0d_state_async", "lbm_set_wait_limit"]
+           "lbm_read_0d_state_async", "lbm_set_wait_limit",
+           "lbm_set_multi_step"]
 
 _lib = None
 
@@ -98,6 +99,7 @@ def load(path: Optional[str] = None):
     L.lbm_step.argtypes = [H, ctypes.c_int64]
     L.lbm_sync.argtypes = [H]
     L.lbm_set_wait_limit.argtypes = [H, ctypes.c_int]
+    L.lbm_set_multi_step.argtypes = [H, ctypes.c_int]
     L.lbm_read_fields.argtypes = [H, ctypes.c_int, _dp, _dp, _dp, _dp]
     L.lbm_read_populations.argtypes = [H, ctypes.c_int, _dp]
     L.lbm_read_0d_state.argtypes = [H, ctypes.c_int, ctypes.c_int, _dp]
@@ -287,6 +289,11 @@ class Lattice:
 
     def sync(self):
         self._ck(load().lbm_sync(self._h))
+
+    def set_multi_step(self, enable: bool):
+        """Whether a small lattice takes its steps in multi-step launches (default) or as
+        step graphs, which overlap with those of other lattices on other streams."""
+        self._ck(load().lbm_set_multi_step(self._h, int(bool(enable))))
 
     def set_wait_limit(self, polls: int):
         """Polls after which a block of a multi-step launch gives up waiting for the others."""

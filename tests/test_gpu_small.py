@@ -327,3 +327,30 @@ def test_large_lattices_without_boundaries_keep_the_step_graphs():
     a, b = _pair(insts, "f32", (64, 7))
     assert a.info().steps_per_launch == 0
     _same(a, b, insts)
+
+
+@pytest.mark.parametrize("case", ["cluster", "grid", "batch"])
+def test_without_multi_step_launches(case):
+    # the caller's choice of step graphs (whole, short and single-step ones) for a
+    # lattice that would take multi-step launches, and back
+    import torch
+    from paper_2112_05258_gb300 import Lattice
+    insts = {"cluster": CASES["lv"], "grid": GRID["velocity"], "batch": GRID["uneven"]}[case]()
+    a, b = (Lattice(insts, precision="f32") for _ in range(2))
+    a.set_multi_step(False)
+    assert a.info().steps_per_launch == 0 and a.info().short_graph_steps == 8 and b.info().steps_per_launch > 0
+    params = torch.tensor(np.tile(insts[0].boundaries[1].params, (21, 1)), dtype=torch.float64).pin_memory()
+    rows = [torch.zeros((21, 16), dtype=torch.float64, pin_memory=True) for _ in range(2)]
+    for lat, r in zip((a, b), rows):
+        for n in (150, 1, 31):
+            lat.step(n)
+        lat.step_io(0, 1, 21, params.data_ptr(), params.shape[1], r.data_ptr())
+        lat.sync()
+    assert np.array_equal(rows[0].numpy(), rows[1].numpy())
+    _same(a, b, insts)
+    a.set_multi_step(True)
+    assert a.info().steps_per_launch == b.info().steps_per_launch
+    for lat in (a, b):
+        lat.step(9)
+        lat.sync()
+    _same(a, b, insts)
