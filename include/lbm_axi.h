@@ -56,6 +56,20 @@ lbm_status lbm_axi_create(const lbm_axi_config *cfg, lbm_axi_handle **out);
 /* Advances n steps (Algorithm 1 with Eq. Afi); asynchronous. */
 lbm_status lbm_axi_step(lbm_axi_handle *h, int64_t n);
 
+typedef struct {
+    int64_t fluid_nodes, steps;
+    int steps_per_launch;  /* small grids take the steps of an lbm_axi_step call in one launch per this many; 0: step graphs */
+    int graph_steps;       /* steps per step graph */
+    int overlapped_blocks; /* blocks of 256 nodes of a row whose next collision runs beside the boundary kernels in the graphs */
+    int fetched_ahead;     /* 1: the collision has its populations fetched into the L2 ahead of its blocks */
+} lbm_axi_info_t;
+
+lbm_status lbm_axi_get_info(lbm_axi_handle *h, lbm_axi_info_t *info);
+
+/* Whether a small grid takes its steps in multi-step launches (the default) or
+ * as the one-step kernels of larger ones; the trajectory is the same bit for bit. */
+lbm_status lbm_axi_set_multi_step(lbm_axi_handle *h, int enable);
+
 /* Waits for the stream; LBM_ERR_UNSTABLE if the device status word is set. */
 lbm_status lbm_axi_sync(lbm_axi_handle *h);
 

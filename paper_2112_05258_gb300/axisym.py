@@ -15,7 +15,8 @@ from .lbm import PRECISIONS, BoundaryDesc, LBMError, _dp, _p, _u8p, load as _loa
 
 EXPORTS = ["lbm_axi_create", "lbm_axi_step", "lbm_axi_sync", "lbm_axi_read_fields",
            "lbm_axi_read_populations", "lbm_axi_init_populations", "lbm_axi_read_0d_state",
-           "lbm_axi_read_waveforms", "lbm_axi_last_error", "lbm_axi_destroy"]
+           "lbm_axi_read_waveforms", "lbm_axi_last_error", "lbm_axi_destroy", "lbm_axi_get_info",
+           "lbm_axi_set_multi_step"]
 
 
 class AxiConfig(ctypes.Structure):
@@ -23,6 +24,11 @@ class AxiConfig(ctypes.Structure):
                 ("q_scale", ctypes.c_int), ("n_bc", ctypes.c_int), ("bc", ctypes.POINTER(BoundaryDesc)),
                 ("precision", ctypes.c_int), ("stream", ctypes.c_void_p), ("device", ctypes.c_int),
                 ("graph_steps", ctypes.c_int), ("wave_capacity", ctypes.c_int)]
+
+
+class AxiInfo(ctypes.Structure):
+    _fields_ = [("fluid_nodes", ctypes.c_int64), ("steps", ctypes.c_int64), ("steps_per_launch", ctypes.c_int),
+                ("graph_steps", ctypes.c_int), ("overlapped_blocks", ctypes.c_int), ("fetched_ahead", ctypes.c_int)]
 
 
 _ready = False
@@ -41,6 +47,8 @@ def load():
         L.lbm_axi_init_populations.argtypes = [H, _dp]
         L.lbm_axi_read_0d_state.argtypes = [H, ctypes.c_int, _dp]
         L.lbm_axi_read_waveforms.argtypes = [H, _dp, ctypes.c_int64, ctypes.POINTER(ctypes.c_int64)]
+        L.lbm_axi_get_info.argtypes = [H, ctypes.POINTER(AxiInfo)]
+        L.lbm_axi_set_multi_step.argtypes = [H, ctypes.c_int]
         L.lbm_axi_last_error.argtypes = [H]
         L.lbm_axi_last_error.restype = ctypes.c_char_p
         L.lbm_axi_destroy.argtypes = [H]
@@ -104,6 +112,15 @@ class AxiLattice:
 
     def step(self, n: int = 1):
         self._ck(load().lbm_axi_step(self._h, int(n)))
+
+    def set_multi_step(self, enable: bool):
+        """Whether a small grid takes its steps in multi-step launches (default) or as one-step kernels."""
+        self._ck(load().lbm_axi_set_multi_step(self._h, int(bool(enable))))
+
+    def info(self) -> AxiInfo:
+        i = AxiInfo()
+        self._ck(load().lbm_axi_get_info(self._h, ctypes.byref(i)))
+        return i
 
     def sync(self):
         self._ck(load().lbm_axi_sync(self._h))

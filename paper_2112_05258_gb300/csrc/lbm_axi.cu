@@ -694,10 +694,11 @@ struct lbm_axi_handle {
     bool ahead = false;  // the populations exceed the L2: k_axi_collide has them fetched ahead
     // small grids: many steps in one launch by a cluster of blocks (0: one-step kernels)
     int small_cluster = 0;
+    bool small_on = true;  // lbm_axi_set_multi_step
     size_t small_smem = 0;
     AxiSmall small{};
     int parity = 0;
-    int64_t steps = 0;
+    int64_t steps = 0, fluid = 0;
     void *f[2] = {nullptr, nullptr};
     uint16_t *flags = nullptr;
     void *aux = nullptr;
@@ -1166,6 +1167,7 @@ lbm_status lbm_axi_create(const lbm_axi_config *cfg, lbm_axi_handle **out) {
             h->xb_hi = hi;
         }
     }
+    for (uint16_t fl : flags) h->fluid += (fl & AF_FLUID) != 0;
     h->ahead = exceeds_l2((size_t)Q9 * h->n * (h->prec == LBM_F64 ? 8 : 4), h->device);
     if (set_up_small(h, flags, xf, xf_n, lk_n, node_n) != cudaSuccess) return bail("out of memory (small-grid tables)");
     if (cudaDeviceSynchronize() != cudaSuccess) return bail("initialisation failed");
@@ -1177,13 +1179,14 @@ lbm_status lbm_axi_step(lbm_axi_handle *h, int64_t nsteps) {
     if (!h || nsteps < 0) return afail(h, LBM_ERR_ARG, "bad arguments");
     ACK(h, cudaSetDevice(h->device));
     int64_t done = 0;
-    if (h->small_cluster) {  // refused where the step graph of the other grids is
+    const bool multi = h->small_cluster && h->small_on;
+    if (multi) {  // refused where the step graph of the other grids is
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
         ACK(h, cudaStreamIsCapturing(h->stream, &capture));
         if (capture != cudaStreamCaptureStatusNone && nsteps - h->parity >= h->graph_steps)
             return afail(h, LBM_ERR_CUDA, "the stream is being captured");
     }
-    while (h->small_cluster && done < nsteps) {
+    while (multi && done < nsteps) {
         const int k = (int)std::min<int64_t>(nsteps - done, AXI_MAX_STEPS);
         ACK(h, small_launch(h, nullptr, k));
         if (k & 1) h->parity ^= 1;
@@ -1217,6 +1220,23 @@ lbm_status lbm_axi_step(lbm_axi_handle *h, int64_t nsteps) {
             count_step(h);
         }
     }
+    return LBM_OK;
+}
+
+lbm_status lbm_axi_set_multi_step(lbm_axi_handle *h, int enable) {
+    if (!h) return LBM_ERR_ARG;
+    h->small_on = enable != 0;
+    return LBM_OK;
+}
+
+lbm_status lbm_axi_get_info(lbm_axi_handle *h, lbm_axi_info_t *info) {
+    if (!h || !info) return LBM_ERR_ARG;
+    info->fluid_nodes = h->fluid;
+    info->steps = h->steps;
+    info->steps_per_launch = h->small_cluster && h->small_on ? AXI_MAX_STEPS : 0;
+    info->graph_steps = h->graph_steps;
+    info->overlapped_blocks = h->xb_hi - h->xb_lo;
+    info->fetched_ahead = h->prec == LBM_F32 && h->ahead;
     return LBM_OK;
 }
 

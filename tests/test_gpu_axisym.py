@@ -155,3 +155,81 @@ def test_step_calls_of_any_length_give_the_same_bits(Axi):
     b.sync()
     assert np.array_equal(a.populations(), b.populations())
     assert np.array_equal(a.waves()[-200:], b.waves()[-200:])
+
+
+def _layered(kind, radius):
+    """A short grid with `radius` first-layer nodes at each end."""
+    nr = radius + 10
+    if kind == "velocity":
+        inst = axw.womersley_tube(nr=nr, nx=12, radius=float(radius), period=200)
+    else:
+        inst = axw.lv_tube(nr=nr, nx=12, radius=float(radius), period=60)
+    if kind == "order2":
+        for b in inst.boundaries:
+            b.params = list(b.params) + [2.0]
+    if kind == "pressure":
+        inst.boundaries[1] = Boundary(BC_PRESSURE, 0, -1, [1e-4])
+    return inst
+
+
+@pytest.mark.parametrize("prec,radius", [("f32", 6), ("f32", 256), ("f32", 257), ("f32", 600), ("f32", 800), ("f32", 1100),
+                                         ("f64", 6), ("f64", 130)])
+@pytest.mark.parametrize("kind", ["order1", "order2", "pressure", "velocity"])
+def test_multi_step_launches_equal_one_step_kernels(Axi, kind, prec, radius):
+    # first layers of one to five chunks of 256 nodes, of one or two passes of a
+    # boundary block, every kind of end: the same bits as the one-step kernels,
+    # also after a change of path at an odd step
+    inst = _layered(kind, radius)
+    a, b = Axi(inst, precision=prec), Axi(inst, precision=prec)
+    b.set_multi_step(False)
+    assert a.info().steps_per_launch > 0 and b.info().steps_per_launch == 0
+    for n in (1, 150, 32):
+        a.step(n)
+        b.step(n)
+    a.set_multi_step(False)
+    b.set_multi_step(True)
+    for n in (66, 7):
+        a.step(n)
+        b.step(n)
+    a.sync()
+    b.sync()
+    assert np.array_equal(a.populations(), b.populations())
+    assert np.array_equal(a.waves(), b.waves())
+    for k in range(2):
+        assert np.array_equal(a.state_0d(k), b.state_0d(k))
+
+
+@pytest.mark.parametrize("prec,nr", [("f64", 20), ("f32", 140)])
+def test_graph_equals_direct_on_one_step_kernels(Axi, prec, nr):
+    # too large for the multi-step launches; of the five x-blocks of a row 1 to 3
+    # hold no first-layer node, so that inside the graphs their next collision
+    # runs beside the boundary kernels
+    inst = axw.lv_tube(nr=nr, nx=1100, radius=nr - 2.0, period=300)
+    g, d = Axi(inst, precision=prec, graph_steps=8), Axi(inst, precision=prec, graph_steps=1000)
+    assert g.info().steps_per_launch == 0 and g.info().overlapped_blocks == 3
+    for lat in (g, d):
+        lat.step(203)
+        lat.sync()
+    assert np.array_equal(g.populations(), d.populations())
+    assert np.array_equal(g.waves(), d.waves())
+
+
+def test_grid_beyond_the_l2(Axi):
+    # the collision that fetches its populations ahead: graphs equal direct
+    # launches bit for bit, and 12 steps from white noise follow the FP64 lattice.
+    # Deviations stay below 0.03 = 4/9 of 1 % times 6.7; a step rounds each about 16
+    # times at 2^-24 (3e-8), 12 steps add up to 3.4e-7, and 1e-6 leaves a factor
+    # three for the terms in 1/r next to the axis.
+    inst = axw.lv_tube(nr=320, nx=12000, radius=318.0, period=300)
+    rng = np.random.default_rng(2)
+    w = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None, None]
+    f0 = w * (1 + 1e-2 * rng.standard_normal((9,) + inst.node.shape).clip(-6, 6))
+    g, d, e = (Axi(inst, precision=p, graph_steps=n) for p, n in (("f32", 4), ("f32", 1000), ("f64", 4)))
+    assert g.info().fetched_ahead == 1 and e.info().fetched_ahead == 0 and g.info().steps_per_launch == 0
+    for lat in (g, d, e):
+        lat.init_populations(f0)
+        lat.step(12)
+        lat.sync()
+    fg = g.populations()
+    assert np.array_equal(fg, d.populations())
+    assert np.abs(fg - e.populations()).max() < 1e-6
