@@ -354,3 +354,80 @@ def test_without_multi_step_launches(case):
         lat.step(9)
         lat.sync()
     _same(a, b, insts)
+
+
+@pytest.mark.parametrize("name", ["lv", "velocity", "two_chunks", "grid_lv", "grid_two_passes", "grid_uneven"])
+def test_multi_step_kernel_bf16(name):
+    insts = CASES[name]()
+    a, b = _pair(insts, "bf16", (1, 2, 150, 61))
+    assert a.info().steps_per_launch > 0
+    _same(a, b, insts)
+
+
+def _io_against_calls(inst, precision, bc, n, start, **kw):
+    """n steps with per-step 0D input and output in one call, and as calls of one
+    step between a parameter update and a state read, which are only queued."""
+    import torch
+    from paper_2112_05258_gb300 import Lattice
+    base = np.array(inst.boundaries[bc].params, dtype=np.float64)
+    par = torch.from_numpy(np.tile(base, (n, 1)) * np.where(np.arange(base.size) == 0, 1.0 + 0.2 * np.sin(np.arange(n) / 9.0)[:, None], 1.0)).pin_memory()
+    rows = [torch.zeros((n, 8 * len(inst.boundaries)), dtype=torch.float64, pin_memory=True) for _ in range(2)]
+    a, b = (Lattice([inst], precision=precision, **kw) for _ in range(2))
+    a.step(start)
+    b.step(start)
+    a.step_io(0, bc, n, par.data_ptr(), base.size, rows[0].data_ptr())
+    a.sync()
+    for k in range(n):
+        b.set_0d_params(0, bc, par[k].numpy())
+        b.step(1)
+        b.state_0d_async(0, rows[1][k].data_ptr())
+    b.sync()
+    assert np.array_equal(rows[0].numpy(), rows[1].numpy())
+    assert np.array_equal(rows[0].numpy()[:, 0], np.arange(start + 1, start + n + 1))
+    _same(a, b, [inst])
+    return a
+
+
+@pytest.mark.parametrize("make,bc", [(lambda: CASES["lv"]()[0], 1), (lambda: CASES["lv_order4"]()[0], 1),
+                                     (lambda: configs.rigid_tube(), 0),
+                                     (lambda: configs.rigid_tube(27, 27, 251, radius=10.3), 0)])  # two chunks
+def test_step_io_fp64_in_the_multi_step_kernel(make, bc):
+    assert _io_against_calls(make(), "f64", bc, 90, 5).info().steps_per_launch > 0
+
+
+# lattices without wall nodes whose boundary work is two kernels: FP64 beyond the
+# multi-step sizes, and FP32 with more links than the clusters of one launch take
+TWO_KERNELS = {
+    "f64": (lambda: _lv(20.3, 351), "f64", 1),
+    "f64_velocity": (lambda: configs.rigid_tube(41, 41, 405, radius=18.6), "f64", 0),
+    "wide": (lambda: _lv(33.0, 40), "f32", 1),
+}
+
+
+@pytest.mark.parametrize("name", list(TWO_KERNELS))
+def test_step_io_in_graphs_of_two_boundary_kernels(name):
+    # two graphs of 64 steps and a rest of 22, from an odd step on
+    make, precision, bc = TWO_KERNELS[name]
+    info = _io_against_calls(make(), precision, bc, 150, 7).info()
+    assert info.steps_per_launch == 0 and info.launches_per_step == 3
+
+
+@pytest.mark.parametrize("name", ["f64", "wide"])
+def test_queued_parameter_updates_between_step_graphs(name):
+    # updates queued between graphs of 16 steps without waiting, and the same with a
+    # wait after each call
+    from paper_2112_05258_gb300 import Lattice
+    make, precision, bc = TWO_KERNELS[name]
+    inst = make()
+    base = np.array(inst.boundaries[bc].params)
+    a, b = (Lattice([inst], precision=precision, graph_steps=16) for _ in range(2))
+    assert a.info().steps_per_launch == 0
+    for k in range(12):
+        p = base * np.where(np.arange(base.size) == 0, 1.0 + 0.05 * k, 1.0)
+        for lat, wait in ((a, False), (b, True)):
+            lat.set_0d_params(0, bc, p)
+            lat.step(16 if k % 3 else 21)
+            if wait:
+                lat.sync()
+    a.sync()
+    _same(a, b, [inst])
