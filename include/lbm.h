@@ -340,11 +340,12 @@ lbm_status lbm_cycle_change(lbm_handle *h, const int64_t *period, double *delta)
 
 /* Autotuner: times the stream-collide kernel for block sizes 64, 128, 192,
  * 256 and five register/occupancy variants ({min resident 256-thread blocks
- * per SM, cells per thread} = {6,1}, {8,1}, {5,1}, {4,2}, {3,2}), `iters`
- * launches each, on the handle's current state (which is left unchanged),
- * and keeps the fastest.  Returns the chosen block size, minimum blocks and
- * cells per thread; times_ms (NULL or 20 doubles, variant-major) receives the
- * mean launch time of every candidate. */
+ * per SM, cells per thread} = {6,1}, {8,1}, {5,1}, {4,2}, {3,2}) on the
+ * handle's current state (which is left unchanged), and keeps the fastest:
+ * `iters` steps of the step graphs each, boundary kernels and parts included,
+ * or with wall nodes `iters` launches of the kernel.  Returns the chosen block
+ * size, minimum blocks and cells per thread; times_ms (NULL or 20 doubles,
+ * variant-major) receives the mean time of every candidate. */
 /* Sets the stream-collide launch shape directly: block size (multiple of 32
  * in [32, 256]) and variant 0..4 in the order of lbm_autotune's list (for
  * reproducible timings and tests); LBM_ERR_ARG otherwise. */

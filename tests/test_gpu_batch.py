@@ -291,3 +291,36 @@ def test_step_io_rejects_bad_arguments(Lattice):
     lat.step_io(0, 1, 4, pinned.data_ptr(), 4, rows.data_ptr())
     lat.sync()
     assert lat.info().steps == 4
+
+
+@pytest.mark.parametrize("case", ["cluster", "two_kernels", "parts", "parts_two_kernels", "wall_nodes"])
+def test_autotune_leaves_every_state_as_it_was(Lattice, case):
+    # the candidates' steps write no population that is kept, no 0D state, closure
+    # velocity, waveform row or step count, whatever form the steps take; at an odd
+    # step, with the valve's closure before it
+    params = batch.draw_params(np.random.default_rng(0), 6)
+    tube = lambda q, r, l: batch.lv_tube_instance(params[q], r, l)
+    insts, precision = {
+        "cluster": ([tube(0, 13.0, 830)], "f32"),
+        "two_kernels": ([tube(0, 20.3, 351)], "f64"),
+        "parts": ([tube(q, 12.0 + q, 250) for q in range(4)], "f16"),
+        "parts_two_kernels": ([tube(q, 20.3 - q, 171) for q in range(5)], "f32"),
+        "wall_nodes": ([configs.ib_tube()], "f64"),
+    }[case]
+    a, b = (Lattice(insts, precision=precision) for _ in range(2))
+    assert a.info().steps_per_launch == 0 and (a.info().parts > 1) == case.startswith("parts")
+    for lat in (a, b):
+        lat.set_0d_state(0, 1, 2e-3)
+        lat.step(77)
+        lat.sync()
+    before = a.checkpoint()
+    (block, minb, cpt), times = a.autotune(iters=5, return_times=True)
+    assert (times > 0).all()
+    after = a.checkpoint()
+    assert np.array_equal(before, after)
+    b.set_stream_collide_shape(block, [(6, 1), (8, 1), (5, 1), (4, 2), (3, 2)].index((minb, cpt)))
+    a.step(70)
+    b.step(70)
+    assert a.info().steps == b.info().steps == 147
+    if case != "wall_nodes":                       # (its spreading adds in no fixed order)
+        assert np.array_equal(a.checkpoint(), b.checkpoint())
