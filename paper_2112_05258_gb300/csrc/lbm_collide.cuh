@@ -7,10 +7,11 @@
 namespace lbm {
 
 // out(i, c) is the address of population i of cell c; the moments of f come back.
+// LARGE: the populations exceed the L2, and the stores stay there (keep_in_l2).
 template <class R> struct Moments {
     R sd, jx, jy, jz;  // sum s, j
 };
-template <class S, class R, bool FORCED, class Out>
+template <class S, class R, bool FORCED, bool LARGE, class Out>
 __device__ __forceinline__ Moments<R> collide_store(const Out &out, const KParams &p, const R (&f)[NQ], R omega,
                                                     uint32_t fl, int c) {
     constexpr int NP = (NQ - 1) / 2;
@@ -53,7 +54,11 @@ __device__ __forceinline__ Moments<R> collide_store(const Out &out, const KParam
     const R vv = vx * vx + vy * vy + vz * vz;
     if (!(sd - sd == R(0)) || !(vv <= R(0.09))) atomicOr(p.status, 1u);
 
-    const uint64_t keep = keep_in_l2(p.keep);
+    const uint64_t keep = LARGE ? keep_in_l2(p.keep) : 0;
+    auto put = [&](S *a, R v) {
+        if (LARGE) st_keep(a, v, keep);
+        else Storage<S>::st(a, v);
+    };
     const R om1 = R(1) - omega;
     const R K = sd - R(1.5) * vv;
     // per weight class (1/18 faces, 1/36 edges): omega w K, 9/2 omega w, 3 omega w
@@ -70,7 +75,7 @@ __device__ __forceinline__ Moments<R> collide_store(const Out &out, const KParam
     }
     R post0 = om1 * f[0] + omega * R(1.0 / 3.0) * K;
     if (FORCED) post0 -= (R(1) - R(0.5) * omega) * vb;  // w_0 (1 - omega/2) (-3 v.b), w_0 = 1/3
-    st_keep(out(0, c), post0, keep);
+    put(out(0, c), post0);
 #pragma unroll
     for (int q = 0; q < NP; q++) {
         const int i = 2 * q + 1;
@@ -95,8 +100,8 @@ __device__ __forceinline__ Moments<R> collide_store(const Out &out, const KParam
             A += kw * (R(9) * eu * eb - R(3) * vb);
             B += R(3) * kw * eb;
         }
-        st_keep(out(i, c), om1 * f[i] + (A + B), keep);
-        st_keep(out(i + 1, c), om1 * f[i + 1] + (A - B), keep);
+        put(out(i, c), om1 * f[i] + (A + B));
+        put(out(i + 1, c), om1 * f[i + 1] + (A - B));
     }
     return Moments<R>{sd, jx, jy, jz};
 }

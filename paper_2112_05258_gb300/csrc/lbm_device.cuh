@@ -37,9 +37,12 @@ template <> struct Storage<__nv_bfloat16> {
 // kernel begins on the cells stored last (band velocities, or the next
 // stream-collide in the opposite order).  96 uneven tubes FP32 467 -> 455 us
 // per step, aorta 217.5 -> 215.0; FP16 343.3 -> 341.7 and 186.9 -> 185.3.  (Marking the loads to leave first is
-// slower, 467 -> 532: lines are shared between neighbouring rows.)  keep: the
-// populations exceed the L2; else the stores are ordinary ones (a membrane tube
-// of 78 MB, which mostly fits, was 0.6 to 1.3 % slower with them).
+// slower, 467 -> 532: lines are shared between neighbouring rows.)  Only where one
+// buffer of populations exceeds the L2 (LARGE): else plain stores, in kernels of
+// their own, as the hint costs something even where it says nothing.  keep is true
+// in the LARGE kernels; with the policy selected by it the 32-register ones spill
+// less than with a constant one (FP16 132 instead of 148 bytes: 100 steps of 96
+// uneven tubes 34.16 instead of 34.61 ms).
 __device__ __forceinline__ uint64_t keep_in_l2(bool keep) {
     uint64_t last, normal;
     asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(last));
@@ -98,6 +101,14 @@ cudaError_t launch_early(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s,
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
 }
+
+// the storage types with FP32 arithmetic
+#define DISPATCH_F32(prec, CALL)                               \
+    switch (prec) {                                            \
+    case 1: { using S = __half; CALL; } break;                 \
+    case 2: { using S = __nv_bfloat16; CALL; } break;          \
+    default: { using S = float; CALL; } break;                 \
+    }
 
 #define DISPATCH(prec, CALL)                                   \
     switch (prec) {                                            \

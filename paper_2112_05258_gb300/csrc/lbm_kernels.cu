@@ -551,12 +551,12 @@ static cudaError_t boundary_in_one(void *f, const KParams &p, const BcKParams &q
 
 cudaError_t launch_boundary(int prec, void *f, const KParams &p, const BcKParams &q, const BcIo &io, cudaStream_t s) {
     if (q.n_bc == 0) return cudaSuccess;
-    if (q.cluster) {
+    if (q.cluster) {  // never in FP64 (lbm_create)
         cudaError_t e = cudaSuccess;
         if (q.wide) {
-            DISPATCH(prec, (e = boundary_in_one<S, 512>(f, p, q, io, s)));
+            DISPATCH_F32(prec, (e = boundary_in_one<S, 512>(f, p, q, io, s)));
         } else {
-            DISPATCH(prec, (e = boundary_in_one<S, 256>(f, p, q, io, s)));
+            DISPATCH_F32(prec, (e = boundary_in_one<S, 256>(f, p, q, io, s)));
         }
         return e;
     }

@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
                 f[0] = PlainLoad<S>::ld(fin + c);
 #pragma unroll
                 for (int i = 1; i < NQ; i++) f[i] = PlainLoad<S>::ld(fin + tab[(i - 1) * n_cells + k]);
-                collide_store<S, R, false>(out, p, f, GRID ? om[k] : omega, 0u, c);
+                collide_store<S, R, false, false>(out, p, f, GRID ? om[k] : omega, 0u, c);
             }
             if (GRID) __syncthreads();
             __syncwarp();
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_small_steps(S *f0, S *f1, KParam
                     f[0] = PlainLoad<S>::ld(fin + c);
 #pragma unroll
                     for (int i = 1; i < NQ; i++) f[i] = PlainLoad<S>::ld(fin + tab[(i - 1) * n_cells + k]);
-                    const Moments<R> m = collide_store<S, R, false>(out, p, f, omega, 0u, c);
+                    const Moments<R> m = collide_store<S, R, false, false>(out, p, f, omega, 0u, c);
                     const R j = P.axis == 0 ? m.jx : P.axis == 1 ? m.jy : m.jz;
                     const R third = third_of(m.sd);
                     Q = (double)((R)P.sign * j / (R(1) + m.sd));

@@ -74,7 +74,12 @@ template <class S> struct PopDirs {
 // EARLY: launched while its predecessor, the boundary kernel, still runs (see
 // launch_stream_collide); only tables that no step writes are read before the
 // wait.
-template <class S, int MINB, int CPT, bool EARLY = false>
+// LARGE: one buffer of populations exceeds the L2; they are fetched ahead and their
+// stores stay in the L2.  A kernel of its own: with both switched at run time
+// lattices that fit took 1 to 2.5 % longer (tubes of 508,000, 643,000, 1.03 M cells
+// FP32 21.2 -> 21.5, 26.3 -> 26.8, 37.1 -> 37.6 us per step, FP16 18.9 -> 19.2, 20.6 -> 21.1,
+// 27.8 -> 28.6), about half from either.
+template <class S, int MINB, int CPT, bool EARLY, bool LARGE>
 __global__ void __launch_bounds__(256, MINB)
     k_stream_collide(const __grid_constant__ PopDirs<S> d, const __grid_constant__ KParams p, int desc, int c0,
                      int c1, int bump, int ahead) {
@@ -84,7 +89,7 @@ __global__ void __launch_bounds__(256, MINB)
     const int stride = gridDim.x * blockDim.x;
     if (!EARLY && bump && t == c0 && p.step) *p.step += 1;  // the step index t_n seen by the boundary kernels
     const int N = (int)p.n;  // 19 N < 2^31 is checked at creation
-    if (CPT == 1 && threadIdx.x < NQ && ahead && (bid & ahead) == 0) {
+    if (LARGE && CPT == 1 && threadIdx.x < NQ && ahead && (bid & ahead) == 0) {
         const int s = t - (int)threadIdx.x + (desc ? -AHEAD_DIST : AHEAD_DIST), n = (ahead + 1) * (int)blockDim.x;
         if (s >= c0 && s < c1 && s + n <= N)
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(d.in[0] + ((long long)threadIdx.x * N + s)),
@@ -132,9 +137,9 @@ __global__ void __launch_bounds__(256, MINB)
         const int c = t + u * stride;
         const bool band = (fl[u] & (FL_ACTIVE | FL_BAND)) == (FL_ACTIVE | FL_BAND);
         if (__any_sync(0xffffffffu, band)) {
-            if (fl[u] & FL_ACTIVE) collide_store<S, R, true>(d, p, f[u], om[u], fl[u], c);
+            if (fl[u] & FL_ACTIVE) collide_store<S, R, true, LARGE>(d, p, f[u], om[u], fl[u], c);
         } else {
-            if (fl[u] & FL_ACTIVE) collide_store<S, R, false>(d, p, f[u], om[u], fl[u], c);
+            if (fl[u] & FL_ACTIVE) collide_store<S, R, false, LARGE>(d, p, f[u], om[u], fl[u], c);
         }
     }
 }
@@ -157,6 +162,20 @@ template <class S> static PopDirs<S> pop_dirs(const void *fin, void *fout, long 
     return d;
 }
 
+template <class S, int MINB, int CPT>
+static void launch(int grid, int block, cudaStream_t s, const void *fin, void *fout, const KParams &p, int desc, int c0,
+                   int c1, int bump, int ahead) {
+    const auto k = p.keep ? k_stream_collide<S, MINB, CPT, false, true> : k_stream_collide<S, MINB, CPT, false, false>;
+    k<<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead);
+}
+
+template <class S>
+static cudaError_t early_launch(int grid, int block, cudaStream_t s, const void *fin, void *fout, const KParams &p, int desc,
+                                int c0, int c1, int bump, int ahead) {
+    const auto k = p.keep ? k_stream_collide<S, 6, 1, true, true> : k_stream_collide<S, 6, 1, true, false>;
+    return launch_early(k, dim3(grid), dim3(block), s, pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead);
+}
+
 cudaError_t launch_stream_collide(int prec, const void *fin, void *fout, const KParams &p, int block,
                                   int variant, cudaStream_t s, int desc, int c0, int c1, int bump, bool early) {
     if (c1 < 0) c1 = p.cells;
@@ -165,28 +184,17 @@ cudaError_t launch_stream_collide(int prec, const void *fin, void *fout, const K
     const int cpt = kVariants[variant][1];
     const int grid = (int)((c1 - (c0 & ~(LINE_CELLS - 1)) + (long long)block * cpt - 1) / ((long long)block * cpt));
     const int ahead = ahead_mask(p, block, cpt);
-    if (early && variant == 0) {
+    if (early && variant == 0 && prec != 3) {  // FP64 has no one-launch boundary kernel
         cudaError_t e = cudaSuccess;
-        DISPATCH(prec, (e = launch_early(k_stream_collide<S, 6, 1, true>, dim3(grid), dim3(block), s,
-                                         pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead)));
+        DISPATCH_F32(prec, (e = early_launch<S>(grid, block, s, fin, fout, p, desc, c0, c1, bump, ahead)));
         return e;
     }
     switch (variant) {
-    case 1:
-        DISPATCH(prec, (k_stream_collide<S, 8, 1><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead)));
-        break;
-    case 2:
-        DISPATCH(prec, (k_stream_collide<S, 5, 1><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead)));
-        break;
-    case 3:
-        DISPATCH(prec, (k_stream_collide<S, 4, 2><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead)));
-        break;
-    case 4:
-        DISPATCH(prec, (k_stream_collide<S, 3, 2><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead)));
-        break;
-    default:
-        DISPATCH(prec, (k_stream_collide<S, 6, 1><<<grid, block, 0, s>>>(pop_dirs<S>(fin, fout, p.n), p, desc, c0, c1, bump, ahead)));
-        break;
+    case 1: DISPATCH(prec, (launch<S, 8, 1>(grid, block, s, fin, fout, p, desc, c0, c1, bump, ahead))); break;
+    case 2: DISPATCH(prec, (launch<S, 5, 1>(grid, block, s, fin, fout, p, desc, c0, c1, bump, ahead))); break;
+    case 3: DISPATCH(prec, (launch<S, 4, 2>(grid, block, s, fin, fout, p, desc, c0, c1, bump, ahead))); break;
+    case 4: DISPATCH(prec, (launch<S, 3, 2>(grid, block, s, fin, fout, p, desc, c0, c1, bump, ahead))); break;
+    default: DISPATCH(prec, (launch<S, 6, 1>(grid, block, s, fin, fout, p, desc, c0, c1, bump, ahead))); break;
     }
     return cudaGetLastError();
 }
