@@ -23,7 +23,7 @@
 // (immersed boundary) -> k_stream_collide -> k_bc_reduce -> k_bc_apply.
 #include <cooperative_groups.h>
 
-#include "lbm_boundary.cuh"
+#include "lbm_ghost.cuh"
 #include "lbm_device.cuh"
 
 namespace lbm {

@@ -47,8 +47,8 @@
 
 #include <algorithm>
 
-#include "lbm_boundary.cuh"
 #include "lbm_collide.cuh"
+#include "lbm_ghost.cuh"
 
 namespace lbm {
 
