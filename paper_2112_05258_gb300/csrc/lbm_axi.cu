@@ -845,8 +845,12 @@ cudaError_t small_launch(lbm_axi_handle *h, int *clusters, int n_steps) {
 
 // Decides whether the grid takes its steps in the multi-step kernel.  Times of
 // a step in us, measured on GB300: this kernel the longer of a boundary block
-// (latency, and its first layer) and a bulk block; the one-step kernels 13.4
-// (FP64 21) and then bandwidth (FP64: the narrow FP64 pipe).
+// (latency, and its first layer) and a bulk block; the one-step kernels 11.5 to
+// 15 (FP64 20.5 and more) at these sizes.  One-step -> multi-step, FP32: first layers
+// of 300 nodes (nx = 12) 11.7 -> 5.7, 800 12.0 -> 12.2, 1,500 13.6 -> 19.7, 62 x 1,000
+// 12.6 -> 17.9, 762 x 95 13.9 -> 7.5; FP64: first layers of 130 17.3 -> 12.8, 180 17.3 ->
+// 14.0, bulk blocks of 515 nodes (242 x 30) 20.7 -> 16.1, 563 (258 x 32) 20.4 -> 19.7, 675 20.5 ->
+// 21.9, 963 20.8 -> 29.3.
 cudaError_t set_up_small(lbm_axi_handle *h, const std::vector<uint16_t> &flags, const std::vector<int32_t> &xf,
                          const std::vector<int32_t> &xf_n, const std::vector<int32_t> &lk_n,
                          const std::vector<int32_t> &node_n) {
@@ -871,9 +875,8 @@ cudaError_t set_up_small(lbm_axi_handle *h, const std::vector<uint16_t> &flags, 
     const int per = ((int)bulk.size() + C - nb - 1) / (C - nb);
     smem = std::max(smem, axi_smem_bulk(per, r));
     if (smem > AXI_MAX_SMEM) return cudaSuccess;
-    const double small = r == 8 ? std::max(3.5 + 0.085 * worst, 1.5 + 16e-3 * per) : std::max(2.9 + 0.006 * worst, 0.7 + 1.6e-3 * per);
-    const double one = r == 8 ? std::max(21.0, 16.0 + 120e-6 * h->n) : 13.4;
-    if (small > 0.9 * one) return cudaSuccess;
+    const double small = r == 8 ? std::max(3.5 + 0.085 * worst, 1.5 + 31e-3 * per) : std::max(2.0 + 0.0125 * worst, 0.7 + 1.6e-3 * per);
+    if (small > (r == 8 ? 20.0 : 10.8)) return cudaSuccess;
     h->small_cluster = C;
     h->small_smem = smem;
     int clusters = 0;

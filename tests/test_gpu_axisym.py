@@ -172,13 +172,12 @@ def _layered(kind, radius):
     return inst
 
 
-@pytest.mark.parametrize("prec,radius", [("f32", 6), ("f32", 256), ("f32", 257), ("f32", 600), ("f32", 800), ("f32", 1100),
+@pytest.mark.parametrize("prec,radius", [("f32", 6), ("f32", 256), ("f32", 257), ("f32", 513), ("f32", 690),
                                          ("f64", 6), ("f64", 130)])
 @pytest.mark.parametrize("kind", ["order1", "order2", "pressure", "velocity"])
 def test_multi_step_launches_equal_one_step_kernels(Axi, kind, prec, radius):
-    # first layers of one to five chunks of 256 nodes, of one or two passes of a
-    # boundary block, every kind of end: the same bits as the one-step kernels,
-    # also after a change of path at an odd step
+    # first layers of one to three chunks of 256 nodes, every kind of end: the same
+    # bits as the one-step kernels, also after a change of path at an odd step
     inst = _layered(kind, radius)
     a, b = Axi(inst, precision=prec), Axi(inst, precision=prec)
     b.set_multi_step(False)
@@ -233,3 +232,11 @@ def test_grid_beyond_the_l2(Axi):
     fg = g.populations()
     assert np.array_equal(fg, d.populations())
     assert np.abs(fg - e.populations()).max() < 1e-6
+
+
+@pytest.mark.parametrize("prec,nx,nr", [("f32", 12, 1100), ("f32", 62, 1000), ("f64", 330, 41)])
+def test_grids_whose_blocks_take_longer_than_one_step_kernels(Axi, prec, nx, nr):
+    # wide first layers, and FP64 bulk blocks of many nodes: graphs of one-step
+    # kernels, though the grid would fit the multi-step launch
+    inst = axw.lv_tube(nr=nr, nx=nx, radius=nr - 1.0, period=60)
+    assert Axi(inst, precision=prec).info().steps_per_launch == 0
