@@ -57,7 +57,7 @@ lbm_status lbm_axi_create(const lbm_axi_config *cfg, lbm_axi_handle **out);
 lbm_status lbm_axi_step(lbm_axi_handle *h, int64_t n);
 
 typedef struct {
-    int64_t fluid_nodes, steps;
+    int64_t steps;
     int steps_per_launch;  /* small grids take the steps of an lbm_axi_step call in one launch per this many; 0: step graphs */
     int graph_steps;       /* steps per step graph */
     int overlapped_blocks; /* blocks of 256 nodes of a row whose next collision runs beside the boundary kernels in the graphs */

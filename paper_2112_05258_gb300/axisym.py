@@ -27,8 +27,8 @@ class AxiConfig(ctypes.Structure):
 
 
 class AxiInfo(ctypes.Structure):
-    _fields_ = [("fluid_nodes", ctypes.c_int64), ("steps", ctypes.c_int64), ("steps_per_launch", ctypes.c_int),
-                ("graph_steps", ctypes.c_int), ("overlapped_blocks", ctypes.c_int), ("fetched_ahead", ctypes.c_int)]
+    _fields_ = [("steps", ctypes.c_int64), ("steps_per_launch", ctypes.c_int), ("graph_steps", ctypes.c_int),
+                ("overlapped_blocks", ctypes.c_int), ("fetched_ahead", ctypes.c_int)]
 
 
 _ready = False

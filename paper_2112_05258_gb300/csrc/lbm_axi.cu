@@ -698,7 +698,7 @@ struct lbm_axi_handle {
     size_t small_smem = 0;
     AxiSmall small{};
     int parity = 0;
-    int64_t steps = 0, fluid = 0;
+    int64_t steps = 0;
     void *f[2] = {nullptr, nullptr};
     uint16_t *flags = nullptr;
     void *aux = nullptr;
@@ -1170,7 +1170,6 @@ lbm_status lbm_axi_create(const lbm_axi_config *cfg, lbm_axi_handle **out) {
             h->xb_hi = hi;
         }
     }
-    for (uint16_t fl : flags) h->fluid += (fl & AF_FLUID) != 0;
     h->ahead = exceeds_l2((size_t)Q9 * h->n * (h->prec == LBM_F64 ? 8 : 4), h->device);
     if (set_up_small(h, flags, xf, xf_n, lk_n, node_n) != cudaSuccess) return bail("out of memory (small-grid tables)");
     if (cudaDeviceSynchronize() != cudaSuccess) return bail("initialisation failed");
@@ -1234,7 +1233,6 @@ lbm_status lbm_axi_set_multi_step(lbm_axi_handle *h, int enable) {
 
 lbm_status lbm_axi_get_info(lbm_axi_handle *h, lbm_axi_info_t *info) {
     if (!h || !info) return LBM_ERR_ARG;
-    info->fluid_nodes = h->fluid;
     info->steps = h->steps;
     info->steps_per_launch = h->small_cluster && h->small_on ? AXI_MAX_STEPS : 0;
     info->graph_steps = h->graph_steps;
