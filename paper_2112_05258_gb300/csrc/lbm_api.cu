@@ -952,7 +952,15 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
     h->kp.aux = h->aux;
     h->kp.step = h->step_dev;
     h->kp.status = h->status;
-    h->kp.keep = exceeds_l2((size_t)NQ * n * h->sbytes, h->device);
+    // Prefetch and kept stores of stream-collide (its LARGE kernels): where the two buffers of
+    // populations exceed the L2; in FP64, which is bound by its pipe, and with wall nodes, whose
+    // kernels want the L2 too, where one does.  us per step without -> with (one buffer of so many
+    // MB): batches FP32 33 MB 15.56 -> 15.73, 67 28.6 -> 27.0, 70 27.1 -> 26.2, 106 42.8 -> 42.0; FP16
+    // 35 MB 19.0 -> 21.5, 53 32.6 -> 33.8, 74 39.5 -> 38.6, 90 52.0 -> 48.1, 107 68.4 -> 62.2; single tubes
+    // FP32 49 MB 26.2 -> 26.9, 79 37.4 -> 37.3, FP16 39 MB 28.7 -> 29.2, 97 58.0 -> 56.7.
+    const size_t pop_bytes = (size_t)NQ * n * h->sbytes;
+    const bool one_exceeds = exceeds_l2(pop_bytes, h->device);
+    h->kp.keep = h->prec == LBM_F64 || ns ? one_exceeds : exceeds_l2(2 * pop_bytes, h->device);
     h->bp.n_bc_total = h->bp.n_bc = (int)L.bc.size();
     h->bp.par = h->bc_par;
     h->bp.state = h->bc_state;
@@ -1128,7 +1136,7 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
     // nodes 48 registers, which halves its spills (64 tubes 211.7 -> 210.9, a tube of 1.4 M
     // cells 338.7 -> 334.9; the aorta is slower, 2,205 -> 2,247).
     if (h->prec == LBM_F64) h->variant = ns ? 0 : 2;
-    else if (h->sbytes == 2 && h->kp.keep && !h->parts.empty()) h->variant = 1;
+    else if (h->sbytes == 2 && one_exceeds && !h->parts.empty()) h->variant = 1;
     if (h->ibp.n_fil && !(ck(cudaStreamCreateWithFlags(&h->s_fil, cudaStreamNonBlocking), "streams") &&
                           ck(cudaEventCreateWithFlags(&h->ev_nodes, cudaEventDisableTiming), "events") &&
                           ck(cudaEventCreateWithFlags(&h->ev_fil, cudaEventDisableTiming), "events")))

@@ -37,8 +37,8 @@ template <> struct Storage<__nv_bfloat16> {
 // kernel begins on the cells stored last (band velocities, or the next
 // stream-collide in the opposite order).  96 uneven tubes FP32 467 -> 455 us
 // per step, aorta 217.5 -> 215.0; FP16 343.3 -> 341.7 and 186.9 -> 185.3.  (Marking the loads to leave first is
-// slower, 467 -> 532: lines are shared between neighbouring rows.)  Only where one
-// buffer of populations exceeds the L2 (LARGE): else plain stores, in kernels of
+// slower, 467 -> 532: lines are shared between neighbouring rows.)  Only where the
+// populations exceed the L2 (LARGE): else plain stores, in kernels of
 // their own, as the hint costs something even where it says nothing.  keep is true
 // in the LARGE kernels; with the policy selected by it the 32-register ones spill
 // less than with a constant one (FP16 132 instead of 148 bytes: 100 steps of 96

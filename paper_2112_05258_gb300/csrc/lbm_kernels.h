@@ -34,7 +34,7 @@ struct KParams {
     void *aux;                  // first-layer macros (sum s, jx, jy, jz), compute type, 4 x n
     long long *step;            // index t_n of the step in progress
     unsigned *status;           // bit 0: NaN/Inf or |v| > 0.3 seen
-    bool keep;                  // one buffer of populations exceeds the L2 (keep_in_l2)
+    bool keep;                  // the populations exceed the L2 (LARGE kernels; the rule stands in lbm_create)
 };
 inline bool exceeds_l2(size_t bytes, int device) {
     int l2 = 0;

@@ -74,8 +74,8 @@ template <class S> struct PopDirs {
 // EARLY: launched while its predecessor, the boundary kernel, still runs (see
 // launch_stream_collide); only tables that no step writes are read before the
 // wait.
-// LARGE: one buffer of populations exceeds the L2; they are fetched ahead and their
-// stores stay in the L2.  A kernel of its own: with both switched at run time
+// LARGE: the populations exceed the L2 (the rule stands in lbm_create); they are
+// fetched ahead and their stores stay in the L2.  A kernel of its own: with both switched at run time
 // lattices that fit took 1 to 2.5 % longer (tubes of 508,000, 643,000, 1.03 M cells
 // FP32 21.2 -> 21.5, 26.3 -> 26.8, 37.1 -> 37.6 us per step, FP16 18.9 -> 19.2, 20.6 -> 21.1,
 // 27.8 -> 28.6), about half from either.
