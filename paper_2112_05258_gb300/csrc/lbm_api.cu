@@ -995,7 +995,8 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_handle **out) {
         h->bp.wide = links > 4 * 256;
         int c = 1;
         while (c < 8 && c * (h->bp.wide ? 512 : 256) < links) c *= 2;
-        if (h->prec != LBM_F64 && links > 0 && links <= 4096 && c * (int)L.bc.size() <= 300) h->bp.cluster = c;
+        const int most = h->bp.wide ? 200 : 300;  // blocks of 512 threads: one per SM
+        if (h->prec != LBM_F64 && links > 0 && links <= 4096 && c * (int)L.bc.size() <= most) h->bp.cluster = c;
     }
     h->bp.n_red_blocks = (int)L.red_bc.size();
     h->bp.n_app_blocks = (int)L.app_bc.size();

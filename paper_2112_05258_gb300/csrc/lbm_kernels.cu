@@ -194,7 +194,11 @@ __global__ void __launch_bounds__(BC_CHUNK) k_bc_apply(S *__restrict__ f, KParam
 // 64 tubes of 14k cells 36.6 -> 30.1.  A boundary of more links than its blocks
 // have threads (12.5 -> 13.0 us at 6,100 links), FP64 (whose ghosts need the FP64
 // pipes of many SMs: 25 -> 33 us) and batches with more clusters than SMs
-// take at once (96 uneven tubes 528 -> 617 us) keep the two kernels.
+// take at once (96 uneven tubes 528 -> 617 us) keep the two kernels: beyond 300
+// blocks, of 512 threads, one of which fills an SM's registers, beyond 200 (tubes of
+// 108,540 cells, 16 blocks each, two kernels -> one: 4 18.3 -> 15.7 us per step, 10 36.5 ->
+// 34.3, 12 40.0 -> 39.6, 14 44.6 -> 45.9, 18 53.2 -> 58.5; FP16 10 27.0 -> 25.2, 14 34.5 -> 40.1, 18
+// 42.3 -> 48.3).
 template <class S, int BS>
 __global__ void __launch_bounds__(BS) k_boundary(S *__restrict__ f, KParams p, BcKParams q, BcIo io) {
     using R = typename Storage<S>::R;
@@ -727,8 +731,9 @@ template <> struct ReadSum<double> { using T = WideSum; };
 
 // FP32 read-out of one instance in box order: thread b takes the box cells
 // b, so the four arrays are written once, coalesced, with the zeros off the
-// fluid, and the pulls of a row's cells are coalesced too.  Bound by memory:
-// 80 B read per fluid cell (FP32 storage) and 16 B written per box cell.  The
+// fluid, and the pulls of a row's cells are coalesced too.  80 B are read per fluid
+// cell (FP32 storage) and 16 B written per box cell, 87 us for the aorta at the
+// copy rate; bound by the sums' arithmetic in FP32 and BF16.  The
 // sums must not lose precision against FP64, whose pipe is narrow on this
 // part (68 FP64 operations a cell took the whole time before); triples of FP32
 // cost about 650 FP32 operations a cell, pairs (FP16) 350.

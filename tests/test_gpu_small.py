@@ -431,3 +431,13 @@ def test_queued_parameter_updates_between_step_graphs(name):
                 lat.sync()
     a.sync()
     _same(a, b, [inst])
+
+
+def test_batch_of_wide_boundaries_takes_two_kernels():
+    # 16 blocks of 512 threads a tube: fourteen tubes have more of them than SMs
+    from paper_2112_05258_gb300 import Lattice
+    few, many = ([_lv(13.0, 203 + q) for q in range(n)] for n in (5, 14))
+    assert Lattice(few).info().launches_per_step == 2
+    a, b = _pair(many, "f16", (64, 7))
+    assert a.info().launches_per_step == 3
+    _same(a, b, many)
