@@ -988,8 +988,10 @@ lbm_status lbm_axi_create(const lbm_axi_config *cfg, lbm_axi_handle **out) {
             for (int a = 0; a < 3 * cnt; a++) profile.push_back(b.profile[a]);
         struct Lk { int xf, ie, xb, ib, nd; };
         std::vector<Lk> lks;
+        // the boundary's nodes are in one column (checked above): its links lead to that and the next
+        const int col = b.sign > 0 ? 0 : nx - 1;
         for (int j = 0; j < nr; j++)
-            for (int x = 0; x < nx; x++) {
+            for (int x = std::max(0, col - 1); x <= std::min(nx - 1, col + 1); x++) {
                 const int c = j * nx + x;
                 if (node[c] != 0) continue;
                 for (int i = 1; i < Q9; i++) {
