@@ -45,7 +45,7 @@ BYTES_PER_BAND_CELL = {"f32": 12, "f16": 12, "bf16": 12, "f64": 24}
 PROFILE_MD = os.path.join(ROOT, "profiles", "stream_collide_tube_f32.md")
 # the sources the stream-collide kernel is compiled from
 KERNEL_SRC = [os.path.join(ROOT, "paper_2112_05258_gb300", "csrc", f)
-              for f in ("lbm_stream_collide.cu", "lbm_device.cuh")]
+              for f in ("lbm_stream_collide.cu", "lbm_collide.cuh", "lbm_device.cuh")]
 
 
 def parse_args():

@@ -12,8 +12,10 @@ multi-pass capture).  ``aorta``: the full-size elastic-wall workload.
 nodes) is also 151 axial SGFD filaments; ``spring_tube``: the same membrane
 without the filaments.  ``axi``: the axisymmetric straight aorta at 512
 nodes per diameter (12802 x 256 = 3.3M nodes, 236 MB of FP32 populations).
-Steps are launched directly (no CUDA graph) so that each kernel launch is
-visible to a profiler.
+``small``: the 24 x 24 x 64 tube, whose steps are one multi-step launch; ``long``:
+a tube of radius 13 and length 830 (0.44M cells), too large for that, with its
+boundary work in one launch.  Steps are taken as graphs of one step (runs of
+less than 24) or of eight, so that each kernel launch is visible to a profiler.
 """
 from __future__ import annotations
 
@@ -28,7 +30,7 @@ sys.path.insert(0, os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--case", default="tube",
-                    choices=["tube", "aorta", "fil_tube", "spring_tube", "axi", "batch", "mlp"])
+                    choices=["tube", "aorta", "fil_tube", "spring_tube", "axi", "batch", "mlp", "small", "long"])
     ap.add_argument("--steps", type=int, default=3)
     ap.add_argument("--precision", default="f32")
     ap.add_argument("--block", type=int, default=0)
@@ -84,6 +86,12 @@ def main():
         from workloads import batch
         insts, _ = batch.tube_batch(256, 0)
         inst = insts[0]
+    elif args.case == "small":
+        inst = configs.rigid_tube()
+    elif args.case == "long":
+        import numpy as np
+        from workloads import batch
+        inst = batch.lv_tube_instance(batch.draw_params(np.random.default_rng(0), 1)[0], 13.0, 830)
     elif args.case == "tube":
         inst = configs.rigid_tube(128, 128, 512, radius=40.0, period=4000)
     elif args.case in ("fil_tube", "spring_tube"):
@@ -92,7 +100,7 @@ def main():
     else:
         inst = aorta.build(0)
     lat = Lattice(insts or [inst], precision=args.precision, block_size=args.block,
-                  graph_steps=2 * (args.steps + 1),  # graphs longer than the run: single-step graphs only
+                  graph_steps=2 * (args.steps + 1),  # graphs longer than the run: short and single-step ones only
                   ib_slabs=args.ib_slabs)
     info = lat.info()
     t0 = time.perf_counter()
